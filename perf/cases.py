@@ -135,15 +135,20 @@ class _Rand:
     def gate(self, n):
         return torch.rand(n, generator=self.g, device=DEV)
 
-    def weights(self, K, N, r, base3=False, gates=None):
-        """A layer's packed weights and correction, as keyword values of the calls."""
-        packed, gamma = hgf.pack_ternary(self.normal((N, K), 0.02), base3=base3)
-        w = {"packed": packed, "gamma": gamma, "At": None, "Bt": None, "gate": None}
+    def latent(self, K, N, r, gates=None):
+        """A layer's fp32 weights and its correction."""
+        w = {"W": self.normal((N, K), 0.02), "At": None, "Bt": None, "gate": None}
         if r:
             w["At"] = self.normal((r, K), K ** -0.5, torch.float16)
             w["Bt"] = self.normal((N, r), r ** -0.5, torch.float16)
             w["gate"] = self.gate(gates or N)
         return w
+
+    def weights(self, K, N, r, base3=False, gates=None):
+        """A layer's packed weights and correction, as keyword values of the calls."""
+        w = self.latent(K, N, r, gates)
+        packed, gamma = hgf.pack_ternary(w.pop("W"), base3=base3)
+        return {"packed": packed, "gamma": gamma, **w}
 
     def norm(self, K):
         return {"ln_weight": 1.0 + self.normal((K,), 0.1), "ln_bias": self.normal((K,), 0.1)}
@@ -289,6 +294,105 @@ def prepare(case, seed):
 
 def run(state):
     return _KINDS[state["case"]["kind"]][1](state["case"], state)
+
+
+# ---- the same in 64 bits ----------------------------------------------------------------------------------
+# The quantisers decide in the precision that defines them (binary32 scales); every product and sum is a double's.
+def _ternary(W):
+    """(gamma_W as the nearest binary32 value, codes): the codes are those whose weight is nearest gamma_W times them."""
+    gamma = W.double().abs().mean().float().double()
+    return gamma, (W.double() > 0.5 * gamma).double() - (W.double() < -0.5 * gamma).double()
+
+
+def _dequantised(x, norm=None):
+    """The int8 values times their scale, as doubles."""
+    if norm is None:
+        g = x.double().abs().amax(1, keepdim=True).clamp_min(float(torch.tensor(1e-5)))
+        return torch.round(127.0 * x.double() / g).clamp(-127, 127) * g / 127.0
+    xd = x.double()
+    mean, var = xd.mean(1, keepdim=True), xd.var(1, unbiased=False, keepdim=True)
+    n = (x.float() - mean.float()) * (var + 1e-5).rsqrt().float() * norm["ln_weight"] + norm["ln_bias"]
+    g = n.abs().amax(1, keepdim=True).clamp_min(1e-5)
+    return torch.round(n * (127.0 / g)).clamp(-127, 127).double() * g.double() / 127.0
+
+
+def _exact_layer(x, w, norm=None, heads=1):
+    gamma, T = _ternary(w["W"])
+    y = _dequantised(x, norm) @ T.T * gamma
+    if w["At"] is not None:
+        z = x.double() @ w["At"].double().T
+        n = torch.arange(T.shape[0], device=DEV) // heads
+        y += (z * torch.sigmoid(z)) @ w["Bt"].double().T * w["gate"].double()[n]
+    return y
+
+
+def _exact_attn(c, rand):
+    B, L, h, dh = c["B"], c["L"], c["h"], c["dh"]
+    q, k, v = (rand.normal((B * L, n), 1.0, torch.bfloat16) for n in (2 * h * dh, 2 * h * dh, h * dh))
+    lam = 0.8 - 0.6 * math.exp(-0.3 * dh)
+    q, k, v = q.view(B, L, 2, h, dh), k.view(B, L, 2, h, dh), v.view(B, L, h, dh)
+    out = torch.empty((B, L, h, dh), dtype=torch.float64, device=DEV)
+    for b in range(B):
+        for hd in range(h):
+            for i in range(0, L, 2048):  # rows of the score matrix at a time
+                e = min(L, i + 2048)
+                future = torch.ones((e - i, e), dtype=torch.bool, device=DEV).triu(i + 1)
+                p = [torch.softmax((q[b, i:e, s, hd].double() @ k[b, :e, s, hd].double().T * dh ** -0.5).masked_fill(future, -math.inf), 1)
+                     for s in (0, 1)]
+                out[b, i:e, hd] = (p[0] - lam * p[1]) @ v[b, :e, hd].double()
+    return out.view(B * L, h * dh)
+
+
+def _exact_train(c, rand):
+    M, K, N, r = c["M"], c["K"], c["N"], c["r"]
+    W, x, dy = rand.normal((N, K), 0.02), rand.x(M, K), rand.normal((M, N), 1.0, torch.bfloat16).double()
+    w = {"W": W, "At": None}
+    if r:
+        w = {"W": W, "At": rand.normal((r, K), K ** -0.5, torch.float16), "Bt": rand.normal((N, r), r ** -0.5, torch.float16), "gate": rand.gate(N)}
+    gamma, T = _ternary(W)
+    out = {"y": _exact_layer(x, w), "dx": dy @ T * gamma, "dW": dy.T @ _dequantised(x)}
+    if r:
+        A, B, g, x = w["At"].double(), w["Bt"].double(), w["gate"].double(), x.double()
+        z = x @ A.T
+        s = torch.sigmoid(z)
+        dz = ((dy * g) @ B) * (s * (1 + z * (1 - s)))
+        hy = dy.T @ (z * s)
+        out["dx"] += dz @ A
+        out.update({"dAt": dz.T @ x, "dBt": hy * g[:, None], "dgate": (hy * B).sum(1)})
+    return out
+
+
+def exact(case, seed):
+    """What run() gives, from the same inputs (drawn in the order in which prepare() draws them)."""
+    c, rand = case, _Rand(seed)
+    if c["kind"] == "attn":
+        return _exact_attn(c, rand)
+    if c["kind"] == "train":
+        return _exact_train(c, rand)
+    if c["kind"] == "layer":
+        M, K, N, r = c["M"], c["K"], c["N"], c["r"]
+        heads = _head(N) if c["ln"] else 1
+        x, w = rand.x(M, K), rand.latent(K, N, r, -(-N // heads) if c["ln"] else None)
+        return _exact_layer(x, w, rand.norm(K) if c["ln"] else None, heads)
+    M, d, ffn, r, ys = c["M"], c["d"], c["ffn"], c["r"], []
+    if c["kind"] == "group":
+        for _ in range(c["blocks"]):
+            xs = {"q": rand.x(M, d), "o": rand.x(M, d), "up": rand.x(M, d), "down": rand.x(M, ffn)}
+            xs["k"] = xs["v"] = xs["q"]
+            xs["gate"] = xs["up"]
+            for p in _block(d, ffn, r):
+                ys.append(_exact_layer(xs[p.name], rand.latent(p.d_in, p.d_out, p.r)).flatten())
+        return torch.cat(ys)
+    for _ in range(c["blocks"]):
+        for N, n, ln in ((d, 3, c["ln"]), (ffn, 2, False)):
+            x = rand.x(M, d)
+            for _ in range(n):
+                w = rand.latent(d, N, r, N // 64 if ln else None)
+                ys.append(_exact_layer(x, w, rand.norm(d) if ln else None, 64 if ln else 1))
+            K = d if n == 3 else ffn  # the output projection, the down-projection
+            w = rand.latent(K, d, r)
+            ys.append(_exact_layer(rand.x(M, K), w))
+    return ys
 
 
 # ---- work and tolerance -----------------------------------------------------------------------------------
