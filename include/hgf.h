@@ -86,7 +86,8 @@ size_t hgf_packed_bytes(int64_t d_out, int64_t d_in);
  *     a weight exactly on a boundary becomes 0), then 2-bit packing as above.
  * W: device, fp32 [d_out][d_in].  packed: device, hgf_packed_bytes(d_out, d_in) bytes.
  * gamma_out: HOST pointer, receives gamma_W (sum in double, rounded once to fp32).
- * This call allocates a small temporary, synchronises `stream` and is not meant for the hot path.
+ * This call synchronises `stream`.  It takes its scratch from the library image (up to 16 calls in flight on a
+ * device; further ones allocate a small temporary).
  * Requires d_in % 64 == 0.
  */
 hgf_status hgf_pack_ternary(const float *W, int64_t d_out, int64_t d_in, void *packed,

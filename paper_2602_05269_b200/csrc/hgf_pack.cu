@@ -7,33 +7,55 @@ namespace hgf {
 constexpr int kAbsBlocks = 1024;
 constexpr int kAbsThreads = 256;
 
-// Stage 1: per-block sums of |W| in double (fixed grid-stride order, fixed tree -> deterministic).
-__global__ void __launch_bounds__(kAbsThreads) abs_sum_partial_kernel(const float4 *W4, size_t n4,
-                                                                      double *partials) {
+// Scratch of one scale computation: the blocks' partial sums, the scale, and the count of blocks that are done
+// (zero between calls: the last block puts it back).
+struct AbsScratch {
+    double partials[kAbsBlocks];
+    float gamma;
+    unsigned int done;
+    unsigned char pad[248];
+};
+
+// mean |W| into s->gamma.  Per-block sums in double (fixed grid-stride order, fixed tree), then the block that
+// finishes last adds the partials with one warp (lane-strided, then a fixed shuffle tree) and rounds the mean
+// once to fp32: the same order every time, whichever block is last.  Bound by HBM (4 bytes per weight: 7 us for 2048 x 5632) and, at that
+// size, by the start and the end of the launch: 13.7 us, one launch, against 11.1 + 2.5 us with the partials added
+// in a launch of their own.  Four 16-byte loads in flight per thread, added in index order.
+__global__ void __launch_bounds__(kAbsThreads) abs_mean_kernel(const float4 *W4, size_t n4, double count, AbsScratch *s) {
     double acc = 0.0;
-    for (size_t i = (size_t)blockIdx.x * kAbsThreads + threadIdx.x; i < n4;
-         i += (size_t)gridDim.x * kAbsThreads) {
-        float4 v = W4[i];
-        acc += (double)fabsf(v.x) + (double)fabsf(v.y) + (double)fabsf(v.z) + (double)fabsf(v.w);
+    const size_t stride = (size_t)gridDim.x * kAbsThreads;
+    auto add = [&](const float4 &v) { acc += (double)fabsf(v.x) + (double)fabsf(v.y) + (double)fabsf(v.z) + (double)fabsf(v.w); };
+    size_t i = (size_t)blockIdx.x * kAbsThreads + threadIdx.x;
+    for (; i + 3 * stride < n4; i += 4 * stride) {
+        const float4 v0 = W4[i], v1 = W4[i + stride], v2 = W4[i + 2 * stride], v3 = W4[i + 3 * stride];
+        add(v0); add(v1); add(v2); add(v3);
     }
+    for (; i < n4; i += stride) add(W4[i]);
     __shared__ double red[kAbsThreads];
+    __shared__ bool last;
     red[threadIdx.x] = acc;
     __syncthreads();
-    for (int s = kAbsThreads / 2; s > 0; s >>= 1) {
-        if (threadIdx.x < s) red[threadIdx.x] += red[threadIdx.x + s];
+    for (int k = kAbsThreads / 2; k > 0; k >>= 1) {
+        if (threadIdx.x < k) red[threadIdx.x] += red[threadIdx.x + k];
         __syncthreads();
     }
-    if (threadIdx.x == 0) partials[blockIdx.x] = red[0];
-}
-
-// Stage 2: one warp adds the partials (fixed order: lane-strided, then a fixed shuffle tree) and
-// rounds the mean once to fp32.
-__global__ void abs_sum_final_kernel(const double *partials, int n, double count, float *gamma) {
-    double acc = 0.0;
-    for (int i = threadIdx.x; i < n; i += 32) acc += partials[i];
+    if (threadIdx.x == 0) {
+        s->partials[blockIdx.x] = red[0];
+        __threadfence();
+        last = atomicAdd(&s->done, 1u) + 1u == gridDim.x;
+    }
+    __syncthreads();
+    if (!last || threadIdx.x >= 32) return;
+    __threadfence();
+    double sum = 0.0;
+#pragma unroll 8
+    for (int k = threadIdx.x; k < kAbsBlocks; k += 32) sum += __ldcg(&s->partials[k]);
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-    if (threadIdx.x == 0) *gamma = (float)(acc / count);
+    for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (threadIdx.x == 0) {
+        s->gamma = (float)(sum / count);
+        s->done = 0u;
+    }
 }
 
 // Decomposition of a packed word index into its place in the matrix.  Words are numbered in storage
@@ -190,10 +212,70 @@ cudaError_t launch_repack_b3(const void *packed_b3, int64_t d_out, int64_t d_in,
     return cudaGetLastError();
 }
 
-// gamma_W = mean |W| into *gamma_dev (two launches; partials: kAbsBlocks doubles)
-static void enqueue_gamma(const float *W, size_t n, double *partials, float *gamma_dev, cudaStream_t stream) {
-    abs_sum_partial_kernel<<<kAbsBlocks, kAbsThreads, 0, stream>>>((const float4 *)W, n / 4, partials);
-    abs_sum_final_kernel<<<1, 32, 0, stream>>>(partials, kAbsBlocks, (double)n, gamma_dev);
+// ---- scratch of the packing calls -----------------------------------------------------------------
+// Part of the library image (one copy per device that loads it), a slot per call in flight: a call synchronises
+// its stream before it returns, so its slot is free again then.  cudaMalloc and cudaFree took their place here:
+// cudaFree waits for the whole device and cost 0.1 to 3 ms a call, depending on what else the process had allocated.
+// More calls at a time than slots (from that many threads) allocate theirs.
+constexpr int kPackSlots = 16;
+static __device__ __align__(256) AbsScratch g_pack_scratch[kPackSlots];
+
+struct PackScratch {
+    AbsScratch *p = nullptr;
+    explicit PackScratch(cudaStream_t stream) {
+        dev = current_device();
+        if (dev >= 0 && dev < kMaxDevices) {
+            AbsScratch *base = slots();
+            uint32_t used = busy[dev].load(std::memory_order_relaxed);
+            while (base && slot < 0 && used != (1u << kPackSlots) - 1u) {
+                const int free_slot = __builtin_ctz(~used);
+                if (busy[dev].compare_exchange_weak(used, used | (1u << free_slot), std::memory_order_acquire)) slot = free_slot;
+            }
+            if (slot >= 0) p = base + slot;
+        }
+        if (!p) {
+            void *mem = nullptr;
+            if (cudaMalloc(&mem, sizeof(AbsScratch)) != cudaSuccess) return;
+            p = (AbsScratch *)mem;
+            if (cudaMemsetAsync(&p->done, 0, sizeof(unsigned int), stream) != cudaSuccess) { cudaFree(mem); p = nullptr; }
+        }
+    }
+    ~PackScratch() {
+        if (slot >= 0) busy[dev].fetch_and(~(1u << slot), std::memory_order_release);
+        else if (p) cudaFree(p);
+    }
+    PackScratch(const PackScratch &) = delete;
+    PackScratch &operator=(const PackScratch &) = delete;
+
+private:
+    int dev = -1, slot = -1;
+    static std::atomic<uint32_t> busy[kMaxDevices];
+    AbsScratch *slots() const {
+        static std::atomic<AbsScratch *> cache[kMaxDevices];
+        AbsScratch *ptr = cache[dev].load(std::memory_order_acquire);
+        if (!ptr) {
+            if (cudaGetSymbolAddress((void **)&ptr, g_pack_scratch) != cudaSuccess) return nullptr;
+            cache[dev].store(ptr, std::memory_order_release);
+        }
+        return ptr;
+    }
+};
+std::atomic<uint32_t> PackScratch::busy[kMaxDevices];
+
+// Both layouts: the scale, then `pack` (which enqueues the layout's kernel with the scale's device address), then
+// the scale to the host.
+template <typename Pack>
+static hgf_status pack_with_scale(const float *W, int64_t d_out, int64_t d_in, float *gamma_out, cudaStream_t stream, Pack pack) {
+    PackScratch scratch(stream);
+    if (!scratch.p) return HGF_ERR_CUDA;
+    const size_t n = (size_t)d_out * (size_t)d_in;
+    abs_mean_kernel<<<kAbsBlocks, kAbsThreads, 0, stream>>>((const float4 *)W, n / 4, (double)n, scratch.p);
+    pack(&scratch.p->gamma);
+    count_launch(2);
+    cudaError_t e = cudaMemcpyAsync(gamma_out, &scratch.p->gamma, sizeof(float), cudaMemcpyDeviceToHost, stream);
+    const cudaError_t e1 = cudaStreamSynchronize(stream);  // also after a failed copy: the slot must be idle
+    const cudaError_t e2 = cudaGetLastError();
+    return (e == cudaSuccess && e1 == cudaSuccess && e2 == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
 }
 
 }  // namespace hgf
@@ -211,20 +293,12 @@ extern "C" hgf_status hgf_pack_ternary_b3(const float *W, int64_t d_out, int64_t
     if (d_in % 64 != 0) return HGF_ERR_UNSUPPORTED_SHAPE;
     if (((uintptr_t)W | (uintptr_t)packed) & 15) return HGF_ERR_MISALIGNED;
     cudaStream_t stream = (cudaStream_t)stream_;
-    void *tmp = nullptr;
-    if (cudaMalloc(&tmp, kAbsBlocks * sizeof(double) + 256) != cudaSuccess) return HGF_ERR_CUDA;
-    float *gamma_dev = (float *)((char *)tmp + kAbsBlocks * sizeof(double));
-    enqueue_gamma(W, (size_t)d_out * (size_t)d_in, (double *)tmp, gamma_dev, stream);
     const int64_t steps = padded_k_b3(d_in) / 320;
     const size_t n_bytes = (size_t)row_tiles(d_out) * (size_t)steps * 1024;
-    ternarise_pack_b3_kernel<<<(unsigned)((n_bytes + 255) / 256), 256, 0, stream>>>(W, d_out, d_in, steps, n_bytes, gamma_dev,
-                                                                                    (uint8_t *)packed);
-    count_launch(3);
-    cudaError_t e = cudaMemcpyAsync(gamma_out, gamma_dev, sizeof(float), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    cudaError_t e2 = cudaGetLastError();
-    cudaFree(tmp);
-    return (e == cudaSuccess && e2 == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
+    return pack_with_scale(W, d_out, d_in, gamma_out, stream, [&](const float *gamma) {
+        ternarise_pack_b3_kernel<<<(unsigned)((n_bytes + 255) / 256), 256, 0, stream>>>(W, d_out, d_in, steps, n_bytes, gamma,
+                                                                                        (uint8_t *)packed);
+    });
 }
 
 extern "C" hgf_status hgf_unpack_ternary_b3(const void *packed, int64_t d_out, int64_t d_in, int8_t *T, void *stream_) {
@@ -248,23 +322,12 @@ extern "C" hgf_status hgf_pack_ternary(const float *W, int64_t d_out, int64_t d_
     if (d_in % 64 != 0) return HGF_ERR_UNSUPPORTED_SHAPE;
     if (((uintptr_t)W | (uintptr_t)packed) & 15) return HGF_ERR_MISALIGNED;
     cudaStream_t stream = (cudaStream_t)stream_;
-    size_t n = (size_t)d_out * (size_t)d_in;
-    void *tmp = nullptr;
-    if (cudaMalloc(&tmp, kAbsBlocks * sizeof(double) + 256) != cudaSuccess) return HGF_ERR_CUDA;
-    double *partials = (double *)tmp;
-    float *gamma_dev = (float *)((char *)tmp + kAbsBlocks * sizeof(double));
-    abs_sum_partial_kernel<<<kAbsBlocks, kAbsThreads, 0, stream>>>((const float4 *)W, n / 4, partials);
-    abs_sum_final_kernel<<<1, 32, 0, stream>>>(partials, kAbsBlocks, (double)n, gamma_dev);
     const int64_t steps = padded_k(d_in) / 256;
-    size_t n_words = (size_t)row_tiles(d_out) * (size_t)steps * 256;
-    ternarise_pack_kernel<<<(unsigned)((n_words + 255) / 256), 256, 0, stream>>>(W, d_out, d_in, steps, n_words, gamma_dev,
-                                                                                 (uint32_t *)packed);
-    count_launch(3);
-    cudaError_t e = cudaMemcpyAsync(gamma_out, gamma_dev, sizeof(float), cudaMemcpyDeviceToHost, stream);
-    if (e == cudaSuccess) e = cudaStreamSynchronize(stream);
-    cudaError_t e2 = cudaGetLastError();
-    cudaFree(tmp);
-    return (e == cudaSuccess && e2 == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
+    const size_t n_words = (size_t)row_tiles(d_out) * (size_t)steps * 256;
+    return pack_with_scale(W, d_out, d_in, gamma_out, stream, [&](const float *gamma) {
+        ternarise_pack_kernel<<<(unsigned)((n_words + 255) / 256), 256, 0, stream>>>(W, d_out, d_in, steps, n_words, gamma,
+                                                                                     (uint32_t *)packed);
+    });
 }
 
 extern "C" hgf_status hgf_unpack_ternary(const void *packed, int64_t d_out, int64_t d_in, int8_t *T,
