@@ -154,6 +154,42 @@ static void fill_params(const void *x, int64_t M, const void *packed, float gamm
     }
 }
 
+// The same problem for the one-launch path.
+static SmallProblem small_problem(const PrologueParams &pp, const DecodeProblem &dp, const FrontEnd &fe) {
+    SmallProblem s = {};
+    s.x = pp.x;
+    s.packed = dp.packed;
+    s.At = pp.At;
+    s.Bt = dp.Bt;
+    s.gate = dp.gate;
+    s.y = dp.y;
+    s.ln_w = fe.ln_w;
+    s.ln_b = fe.ln_b;
+    s.mean_out = fe.dbg_mean;
+    s.rstd_out = fe.dbg_rstd;
+    s.eps = fe.eps;
+    s.xq = pp.xq;
+    s.gamma_x = pp.gamma_x;
+    s.row_sum = pp.row_sum;
+    s.h = pp.h;
+    s.h_hi = pp.h_hi;
+    s.h_lo = pp.h_lo;
+    s.hpart = const_cast<float *>(dp.hpart);
+    s.nslices = dp.nslices;
+    s.dbg_xq = pp.dbg_xq;
+    s.dbg_gamma_x = pp.dbg_gamma_x;
+    s.dbg_h = pp.dbg_h;
+    s.dbg_y_int = dp.dbg_y_int;
+    s.gw_over_127 = dp.gw_over_127;
+    s.M = dp.M;
+    s.K = dp.K;
+    s.N = dp.N;
+    s.r = dp.r;
+    s.flags = dp.flags;
+    s.gate_group = dp.gate_group;
+    return s;
+}
+
 static hgf_status forward_impl(const void *x, int64_t M, const void *packed, float gamma, int64_t d_in, int64_t d_out,
                                const void *At, const void *Bt, int32_t r, const float *gate, void *y, void *workspace,
                                size_t workspace_bytes, const hgf_debug_out *dbg, const hgf_front_end *fe_in, uint32_t flags,
@@ -241,6 +277,12 @@ hgf_status hgf::forward_impl(const void *x, int64_t M, const void *packed, float
     dp.gate_group = gate_group;
 
     if (!gemm) {
+        if (do_prologue && do_main) {
+            SmallLaunch<1> sl = {};
+            sl.p[0] = small_problem(pp, dp, fe);
+            sl.n = 1;
+            if (plan_small(sl, flags)) return launch_small(sl, pdl, stream) == cudaSuccess ? HGF_OK : HGF_ERR_CUDA;
+        }
         if (do_prologue && (ln ? launch_decode_prologue_ln(pp, fe, pdl, stream) : launch_decode_prologue(pp, pdl, stream)) != cudaSuccess)
             return HGF_ERR_CUDA;
         if (!do_main) return HGF_OK;
@@ -353,6 +395,8 @@ struct hgf_group {
     int n_quant, n_lora;
     int4 *d_cta_range;        // per GEMV CTA: (first tile, end tile, first problem, 0)
     int grid;
+    bool small;               // whole forwards take the one launch `sl` describes
+    SmallLaunch<kSmallMax> sl;
 };
 
 extern "C" hgf_status hgf_group_create(const hgf_problem *problems, int32_t n, uint32_t flags, hgf_group **out) {
@@ -534,6 +578,17 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
               (ranges.empty() ||
                cudaMemcpy(g->d_cta_range, ranges.data(), sizeof(int4) * ranges.size(), cudaMemcpyHostToDevice) == cudaSuccess);
     if (!ok) { cudaFree(mem); delete g; return HGF_ERR_CUDA; }
+    g->small = false;
+    if (n <= kSmallMax) {
+        g->sl = SmallLaunch<kSmallMax>{};
+        g->sl.n = n;
+        for (int i = 0; i < n; ++i) {
+            g->sl.p[i] = small_problem(pps[i], dps[i], fes[i]);
+            for (int k = 0; k < i; ++k)
+                if (pps[k].xq == pps[i].xq) g->sl.p[i].xq = nullptr, g->sl.p[i].gamma_x = nullptr;  // the first problem with this x writes them
+        }
+        g->small = plan_small(g->sl, flags);
+    }
     g->h_probs = std::move(dps);
     *out = g;
     return HGF_OK;
@@ -545,6 +600,7 @@ extern "C" hgf_status hgf_group_debug(hgf_group *g, int32_t index, int32_t *y_in
     DecodeProblem &P = g->h_probs[(size_t)index];
     if (P.dbg_y_int != y_int) {
         P.dbg_y_int = y_int;
+        if (g->small) g->sl.p[index].dbg_y_int = y_int;
         if (cudaMemcpy(g->d_probs + index, &P, sizeof(DecodeProblem), cudaMemcpyHostToDevice) != cudaSuccess) return HGF_ERR_CUDA;
     }
     if (views) {
@@ -560,6 +616,8 @@ extern "C" hgf_status hgf_group_forward_phases(hgf_group *g, uint32_t phases, vo
     if (!g || !phases || (phases & ~(HGF_PHASE_PROLOGUE | HGF_PHASE_GEMV))) return HGF_ERR_INVALID_ARG;
     cudaStream_t stream = (cudaStream_t)stream_;
     const bool pdl = !(g->flags & HGF_FLAG_NO_PDL);
+    if (g->small && phases == (HGF_PHASE_PROLOGUE | HGF_PHASE_GEMV))
+        return launch_small(g->sl, pdl, stream) == cudaSuccess ? HGF_OK : HGF_ERR_CUDA;
     if ((phases & HGF_PHASE_PROLOGUE) &&
         launch_decode_prologue_group(g->d_quant_items, g->n_quant, g->d_lora_items, g->n_lora, g->max_M, pdl,
                                      stream) != cudaSuccess)

@@ -221,6 +221,45 @@ int decode_xq_smem_limit(uint32_t flags);
 // Grid of the decode GEMV for a launch with that many row tiles (0 if the device cannot be queried).
 int decode_grid(int total_tiles);
 
+// ---- one launch per call for small decode problems (hgf_decode_small.cu) ---------------------------
+constexpr int kSmallMax = 8;  // problems of such a launch at most (they travel as kernel parameters)
+struct SmallProblem {
+    const __nv_bfloat16 *x;
+    const uint8_t *packed;
+    const __half *At, *Bt;
+    const float *gate;
+    void *y;
+    const float *ln_w, *ln_b;        // nullable pair
+    float *mean_out, *rstd_out;      // nullable
+    // the workspace of the two-launch path, filled in the same way (nullable: a problem whose x~ another one writes)
+    int8_t *xq;
+    float *gamma_x;
+    int32_t *row_sum;
+    float *h;
+    __half *h_hi, *h_lo;
+    float *hpart;
+    int8_t *dbg_xq;                  // nullable debug copies
+    float *dbg_gamma_x, *dbg_h;
+    int32_t *dbg_y_int;
+    float gw_over_127, eps;
+    int M, K, N, r;
+    uint32_t flags;
+    int gate_group, nslices;
+    int cluster_begin, ctas;         // (plan_small) first cluster, CTAs
+};
+template <int NP>
+struct SmallLaunch {
+    SmallProblem p[NP];
+    int n;
+    int cluster_log2, clusters, nt;  // (plan_small) CTAs per cluster, clusters, 8-token tiles
+    int off_h, off_slots, off_part, off_ln, off_red, off_x, off_xq, off_at, off_bt, off_w, smem;
+};
+static_assert(sizeof(SmallLaunch<kSmallMax>) <= 4000, "kernel parameters");
+template <int NP>
+bool plan_small(SmallLaunch<NP> &L, uint32_t flags);  // false: the launch takes the two-launch path
+template <int NP>
+cudaError_t launch_small(const SmallLaunch<NP> &L, bool pdl, cudaStream_t stream);
+
 struct GemmParams {
     const int8_t *xq;        // [M][K]
     const uint8_t *packed;   // tiled layout, see above

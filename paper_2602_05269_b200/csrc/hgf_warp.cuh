@@ -1,0 +1,179 @@
+// Warp-level pieces of the decode and prologue kernels: reductions, the quantiser, the LayerNorm arithmetic, warp MMA,
+// mbarrier and bulk-copy wrappers (sm_100a).
+#pragma once
+
+#include "hgf_common.cuh"
+
+namespace hgf {
+
+constexpr unsigned long long kDecWaitLimitNs = 2000000000ull;  // bounded waits give up after two seconds
+
+__device__ __forceinline__ float warp_max(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));
+    return v;
+}
+__device__ __forceinline__ int warp_sum_i(int v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+__device__ __forceinline__ float warp_sum_f(float v) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    return v;
+}
+
+// Round-to-nearest-even of the exact quotient 127 x / gamma for a bf16 x.
+//
+// Reference form: 127 x is exact in fp32, the IEEE division is correctly rounded and k + 1/2 is
+// representable, so rintf of the rounded quotient equals the rounding of the exact one.
+__device__ __forceinline__ int quant1_div(float x, float gamma) {
+    float q = rintf(__fdiv_rn(127.0f * x, gamma));
+    q = fminf(fmaxf(q, -127.0f), 127.0f);
+    return __float2int_rn(q);
+}
+// Division- and conversion-free form, for gamma = max |x| over bf16 values (so gamma is a bf16 value
+// itself, i.e. not the 1e-5 floor).  Adding 1.5 * 2^23 in one fma rounds x * (127 / gamma) to an
+// integer (nearest, ties to even) in the low mantissa bits - a candidate that can only be wrong on
+// an exact tie of the true quotient.  The residual 127 x - q gamma is exact in one fma (127 x and
+// q gamma each have at most 15 significant bits), and the exact quotient is q + residual / gamma:
+// off a tie the candidate is always right (checked over every pair of bf16 mantissas and every
+// exponent gap in exact arithmetic), so it stands unless 2 |residual| = gamma with q odd: a tie goes
+// to the even neighbour, one step towards the residual's sign (2 |residual| > gamma cannot occur).
+// No F2I / FRND: those run at an eighth of the FMA rate and bounded the quantisation kernels.
+struct QuantScale {
+    float gamma, half_gamma, inv127;  // inv127 = 127 / gamma
+    bool fast;                        // gamma is a bf16 value
+};
+__device__ __forceinline__ QuantScale make_quant_scale(float gamma) {
+    QuantScale s;
+    s.gamma = gamma;
+    s.half_gamma = 0.5f * gamma;
+    s.inv127 = __fdiv_rn(127.0f, gamma);
+    s.fast = (__float_as_uint(gamma) & 0xffffu) == 0u;
+    return s;
+}
+// Largest magnitude of the eight bf16 values of a 16-byte unit, on the bit patterns: without the sign
+// bit a bf16 pattern orders like its magnitude, so a packed 16-bit maximum does two values at a time.
+__device__ __forceinline__ uint32_t absmax8_bits(uint32_t acc, const uint4 &v) {
+    acc = __vmaxu2(acc, v.x & 0x7fff7fffu);
+    acc = __vmaxu2(acc, v.y & 0x7fff7fffu);
+    acc = __vmaxu2(acc, v.z & 0x7fff7fffu);
+    return __vmaxu2(acc, v.w & 0x7fff7fffu);
+}
+__device__ __forceinline__ float absmax_bits_to_float(uint32_t acc) {
+    const uint32_t hi = acc >> 16, lo = acc & 0xffffu;
+    return __uint_as_float((hi > lo ? hi : lo) << 16);
+}
+// The eight values of a 16-byte unit -> eight int8 (two words), their sum added to `sum`.
+// The fast form, arranged for throughput: the candidate's low byte is already the low
+// byte of the magic-constant sum's bit pattern (its mantissa holds 2^22 + q in two's complement), so
+// the bytes are packed straight from those patterns, and the tie test of all eight values is one
+// predicate; only a unit that holds an exact tie (rare) goes back over its values to move the odd
+// candidates to their even neighbours.
+__device__ __forceinline__ uint2 quant8(const uint4 &v, const QuantScale &s, int &sum) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    uint32_t b[8];
+    if (s.fast) {
+        constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
+        float xf[8], res[8];
+        bool tie = false;
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            xf[e] = (e & 1) ? bf16hi_to_float(w[e >> 1]) : bf16lo_to_float(w[e >> 1]);
+            const float tm = fmaf(xf[e], s.inv127, kMagic);
+            res[e] = fmaf(kMagic - tm, s.gamma, 127.0f * xf[e]);  // 127 x - q gamma, exact
+            tie = tie || fabsf(res[e]) == s.half_gamma;
+            b[e] = __float_as_uint(tm);
+        }
+        if (tie) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e)
+                if (fabsf(res[e]) == s.half_gamma && (b[e] & 1u)) b[e] += res[e] > 0.0f ? 1u : 0xffffffffu;
+        }
+    } else {
+#pragma unroll
+        for (int e = 0; e < 8; ++e)
+            b[e] = (uint32_t)quant1_div((e & 1) ? bf16hi_to_float(w[e >> 1]) : bf16lo_to_float(w[e >> 1]), s.gamma);
+    }
+    uint32_t o[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t p01 = __byte_perm(b[4 * h], b[4 * h + 1], 0x0040), p23 = __byte_perm(b[4 * h + 2], b[4 * h + 3], 0x0040);
+        o[h] = __byte_perm(p01, p23, 0x5410);
+        sum = __dp4a((int)o[h], 0x01010101, sum);
+    }
+    return make_uint2(o[0], o[1]);
+}
+
+// ---- LayerNorm front end ---------------------------------------------------------------------------
+// One binary32 operation each, in this order: the rounded value decides the int8 code.
+__device__ __forceinline__ float ln_value(float x, float mean, float rstd, float w, float b) {
+    return __fadd_rn(__fmul_rn(__fmul_rn(__fsub_rn(x, mean), rstd), w), b);
+}
+__device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
+    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) f[e] = (e & 1) ? bf16hi_to_float(w[e >> 1]) : bf16lo_to_float(w[e >> 1]);
+}
+
+// ---- PTX wrappers -------------------------------------------------------------------------------
+__device__ __forceinline__ uint32_t dsmem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
+
+__device__ __forceinline__ void mma_u8s8(int (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                         uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k32.row.col.s32.u8.s8.s32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+r"(d[0]), "+r"(d[1]), "+r"(d[2]), "+r"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void mma_f16(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2, uint32_t a3,
+                                        uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k16.row.col.f32.f16.f16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ void dmbar_init(uint32_t bar, uint32_t count) {
+    asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;\n" ::"r"(bar), "r"(count));
+}
+__device__ __forceinline__ bool dmbar_try_wait(uint32_t bar, uint32_t parity) {
+    uint32_t ok;
+    asm volatile(
+        "{\n.reg .pred p;\n"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n"
+        "selp.u32 %0, 1, 0, p;\n}\n"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
+// One bulk copy global -> shared of `bytes` (a multiple of 16; both addresses 16-byte aligned),
+// completing on the mbarrier.
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+__device__ __forceinline__ void mma_tf32(float (&d)[4], uint32_t a0, uint32_t a1, uint32_t a2,
+                                         uint32_t a3, uint32_t b0, uint32_t b1) {
+    asm volatile(
+        "mma.sync.aligned.m16n8k8.row.col.f32.tf32.tf32.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, "
+        "{%0,%1,%2,%3};\n"
+        : "+f"(d[0]), "+f"(d[1]), "+f"(d[2]), "+f"(d[3])
+        : "r"(a0), "r"(a1), "r"(a2), "r"(a3), "r"(b0), "r"(b1));
+}
+__device__ __forceinline__ unsigned long long dec_timer_ns() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;\n" : "=l"(t));
+    return t;
+}
+// Programmatic dependent launch: both are no-ops when the launch carries no such attribute.
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+}  // namespace hgf

@@ -1,0 +1,94 @@
+"""The one-launch decode path against the two-launch path (the same call's two phases run apart) on the same inputs:
+codes, scales and int32 accumulators bit for bit; y within 2e-5 of its largest value (the sums of x A are added in
+another order in fp32, at most K 2^-24 relative, and both paths carry H to 2^-22).  Sizes at the edges of its split: one
+column tile and less, ragged row tiles, fewer row tiles than CTAs, more warps than column tiles, every rank."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2602_05269_b200 import inputs as syn
+
+pytestmark = pytest.mark.gpu
+
+SHAPES = [(1, 64, 1, 16), (1, 192, 40, 0), (16, 256, 17, 64), (9, 320, 1000, 48), (2, 512, 512, 16), (1, 2048, 2048, 32),
+          (4, 2048, 24, 32), (3, 1600, 1544, 64), (1, 5632, 2048, 32), (7, 1088, 4096, 0), (16, 512, 5632, 32), (2, 4096, 300, 32)]
+
+
+@pytest.fixture(scope="module")
+def hgf():
+    from paper_2602_05269_b200 import hgf as binding
+    binding.lib()
+    return binding
+
+
+def layer(hgf, M, K, N, r, seed):
+    g = torch.Generator(device="cuda").manual_seed(seed)
+    rn = lambda shape, std=1.0: torch.randn(shape, generator=g, device="cuda") * std  # noqa: E731
+    packed, gamma = hgf.pack_ternary(rn((N, K), 0.02))
+    x = rn((M, K))
+    x[:, : K // 50] *= 20.0
+    c = {"At": None, "Bt": None, "gate": None}
+    if r:
+        c = {"At": rn((r, K), K ** -0.5).half(), "Bt": rn((N, r), r ** -0.5).half(), "gate": torch.rand(N, generator=g, device="cuda")}
+    return x.bfloat16(), packed, gamma, c
+
+
+@pytest.mark.parametrize("M,K,N,r", SHAPES)
+def test_one_launch_equals_two(hgf, M, K, N, r):
+    x, packed, gamma, c = layer(hgf, M, K, N, r, 7 * K + N + M)
+    ws = torch.zeros(hgf.workspace_bytes(M, K, N, r), dtype=torch.uint8, device="cuda")
+    kw = dict(workspace=ws, debug=True, **c)
+    before = hgf.launch_count()
+    y1, d1 = hgf.linear_forward(x, packed, gamma, K, N, **kw)
+    assert hgf.launch_count() - before == 1, "this size is meant for the one-launch path"
+    _, d2 = hgf.linear_forward(x, packed, gamma, K, N, phases=1, **kw)
+    y2, d3 = hgf.linear_forward(x, packed, gamma, K, N, phases=2, **kw)
+    hgf.check_status()
+    assert torch.equal(d1["xq"], d2["xq"]) and torch.equal(d1["gamma_x"], d2["gamma_x"]) and torch.equal(d1["y_int"], d3["y_int"])
+    assert float((y1 - y2).abs().max()) <= 2e-5 * float(y2.abs().max())
+    # what a whole call leaves in the workspace serves a contraction run on its own, with and without the debug H
+    for debug in (True, False):
+        kw["debug"] = debug
+        ws.fill_(0x5a)
+        hgf.linear_forward(x, packed, gamma, K, N, **kw)
+        y3 = hgf.linear_forward(x, packed, gamma, K, N, phases=2, **kw)
+        y3 = y3[0] if debug else y3
+        assert float((y3 - y1).abs().max()) <= 2e-5 * float(y1.abs().max())
+
+
+@pytest.mark.parametrize("M,K", [(1, 64), (2, 2048), (4, 1024), (12, 320)])
+@pytest.mark.parametrize("r", [0, 32])
+def test_layernorm_group_equals_its_layers(hgf, M, K, r):
+    """A group of three projections of one x, each behind its LayerNorm, and the same three as two-launch groups of one."""
+    g = torch.Generator(device="cuda").manual_seed(K + M)
+    problems = []
+    x = (torch.randn((M, K), generator=g, device="cuda") * 3 + 1).bfloat16()
+    for i, N in enumerate((64, 208, 1024)):
+        _, packed, gamma, c = layer(hgf, M, K, N, r, 100 * K + i)
+        if r:
+            c["gate"] = c["gate"][: -(-N // 16)].contiguous()
+        stat = {n: torch.zeros(M, device="cuda") for n in ("mean_out", "rstd_out")}
+        problems.append({"x": x, "d_in": K, "d_out": N, "packed": packed, "gamma": gamma, "y": torch.empty((M, N), device="cuda"), "gate_group": 16,
+                         "eps": 1e-5, "ln_weight": 1 + 0.1 * torch.randn(K, generator=g, device="cuda"), "ln_bias": 0.1 * torch.randn(K, generator=g, device="cuda"),
+                         **stat, **c})
+    group = hgf.Group(problems)
+    yi = [torch.empty((M, p["d_out"]), dtype=torch.int32, device="cuda") for p in problems]
+    views = [group.debug(i, yi[i]) for i in range(3)]
+    before = hgf.launch_count()
+    group.forward()
+    assert hgf.launch_count() - before == 1
+    hgf.check_status()
+    y1, yi1, xq1 = [p["y"].clone() for p in problems], [t.clone() for t in yi], [v["xq"].clone() for v in views]
+    xd = x.double()
+    mean, var = xd.mean(1), xd.var(1, unbiased=False)
+    for p in problems:
+        assert float((p["mean_out"].double() - mean).abs().max()) <= 2e-7 * float(xd.square().mean().sqrt())
+        assert float((p["rstd_out"].double() * (var + 1e-5).sqrt() - 1).abs().max()) <= 3e-7
+    group.forward_phases(1)
+    group.forward_phases(2)
+    hgf.check_status()
+    for p, a, b, c, v, i in zip(problems, y1, yi1, xq1, views, yi):
+        # (the statistics are rounded to binary32 from two differently summed doubles: a last-bit tie may move a code)
+        assert float((v["xq"] != c).float().mean()) <= 1e-3 and float((i != b).float().mean()) <= 0.02
+        assert float((p["y"] - a).abs().max()) <= 2e-3 * float(a.abs().max())
+    group.close()
