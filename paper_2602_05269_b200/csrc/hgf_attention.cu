@@ -22,36 +22,50 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
     return *reinterpret_cast<const uint32_t *>(&v);
 }
 
-// One CTA of twelve warps per (batch element, head, tile of 128 queries), both streams:
-//   warp 0      TMA producer: the two query tiles once, then per key tile K of stream 1, K of stream 2 and V
-//               (KV keys: 128 for head_dim 64, 64 for head_dim 128; 128-byte swizzle, three stages)
-//   warp 1      one lane issues tcgen05.mma.kind::f16: S_s = Q_s K_s^T (128 x KV, fp32, tensor memory), and
+// Persistent, one CTA of twelve warps per SM; a tile is 128 queries of a (batch element, head), both streams, worked in
+// steps of 64 keys:
+//   warp 0      TMA producer: a tile's two query tiles, then per step K of both streams (one ring) and V (another)
+//   warps 1, 2  issue the tcgen05.mma.kind::f16 of a stream each: S_s = Q_s K_s^T (128 x 64, fp32, tensor memory), and
 //               O_s += P_s V with P_s (bf16) read from tensor memory and V read from its stored form
 //               (key rows of 128 bytes: the second operand with its row index contiguous)
-//   warps 4-7   softmax of stream 1, warps 8-11 of stream 2: a thread owns one query row; it reads S_s
-//               (tcgen05.ld), keeps a reference maximum and the sum, rescales its row of O_s in tensor memory
-//               when the maximum moved far, and writes P_s = exp2(scale (s - reference)) as bf16 pairs (tcgen05.st)
-// The issuer takes the streams in turn - P_s V of tile j, then S_s of tile j + 1 - so that one stream's
-// matrix products run under the other stream's exponentials.  Tensor-memory columns: S_1, S_2, O_1, O_2,
-// P_1, P_2 = 3 KV + 2 head_dim <= 512.  At the end O_1 / l_1 - lambda O_2 / l_2 is formed from the two
-// accumulators by the thread pair that owns the row.  Every wait is bounded.
-constexpr int kTaBM = 128, kTaThreads = 384, kTaStages = 3;
+//   warps 4-7   softmax of stream 1, warps 8-11 of stream 2: a thread owns one query row; it takes the step's 64 scores
+//               into registers (tcgen05.ld), keeps a reference maximum and the sum, rescales its row of O_s in tensor
+//               memory when the maximum moved far, and writes P_s = exp2(scale (s - reference)) as bf16 pairs
+//               (tcgen05.st) over the scores
+// The special-function pipe bounds it (2 x 128 x 64 exponentials a step at 16 a clock and SM: 1024 clocks) and, at the
+// rate that is reached, the power limit (1.7 of 1.965 GHz).  So a softmax warp must not wait for a product: each stream
+// has two score buffers, and its issuer puts the scores of step j + 2 behind P V of step j, in the buffer that P of
+// step j just left - when a softmax warp ends step j the scores of j + 1 have been there for most of a step.  The steps of
+// all tiles are one sequence, so the next tile's scores are formed under this tile's last exponentials.
+// Measured at B = 4, L = 4096, 16 heads of 64 and at B = 2, L = 1500, 16 heads of 128: one score buffer of 128 (64) keys
+// a stream, one issuing thread, a CTA per tile 502 and 79 us; two buffers, one issuing thread 645 and 80 (a thread in a
+// divergent branch takes 80 to 125 clocks an MMA, and a step of 64 keys has as many as one of 128); issued by a whole warp
+// with elect.sync 540 and 68; a warp per stream 455 and 62.5; persistent 448 and 61 to 63.  1360 clocks a step at
+// head_dim 64, 1725 at 128.  Slower: every fourth or second pair of exponentials as a polynomial on the FMA pipe (issue
+// slots are short too), four sets of softmax warps, the two streams' exponentials in turns or half a step apart.
+// Tensor-memory columns: 4 score buffers of 64, O_1, O_2 (2 head_dim, twice for head_dim 64).  At the end O_1 / l_1 -
+// lambda O_2 / l_2 is formed from the two accumulators by the thread pair that owns the row.  Every wait is bounded.
+constexpr int kTaBM = 128, kTaThreads = 384, kTaKV = 64;
 constexpr float kTaSlack = 8.0f;
 
 template <int DH>
 struct TaCfg {
-    static constexpr int KV = DH == 64 ? 128 : 64, NBLK = DH / 64;
-    static constexpr int Q_BYTES = NBLK * kTaBM * 128;             // one stream's query tile
-    static constexpr int K_BYTES = NBLK * KV * 128, V_BYTES = NBLK * KV * 128, V_BLOCK = KV * 128;
-    static constexpr int STAGE = 2 * K_BYTES + V_BYTES;
-    static constexpr int OFF_RING = 2 * Q_BYTES, OFF_BAR = OFF_RING + kTaStages * STAGE;
-    static constexpr int BAR_Q = 0, BAR_KVFULL = 1, BAR_KVEMPTY = 1 + kTaStages, BAR_SFULL = 1 + 2 * kTaStages,
-                         BAR_PFULL = BAR_SFULL + 2, BAR_FINAL = BAR_PFULL + 2, BAR_COUNT = BAR_FINAL + 1;
-    static constexpr int OFF_L = OFF_BAR + 256;                    // [2][128] floats
-    static constexpr int SMEM_BYTES = OFF_L + 2 * kTaBM * 4 + 1024;
-    static constexpr int COL_S = 0, COL_O = 2 * KV, COL_P = 2 * KV + 2 * DH;  // stream s: + s KV, + s DH, + s KV / 2
-    static constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(KV >> 3) << 17) | ((uint32_t)(kTaBM >> 4) << 24);
+    static constexpr int NBLK = DH / 64;
+    static constexpr int KST = DH == 64 ? 5 : 3, VST = DH == 64 ? 5 : 3;  // ring stages
+    static constexpr int NQ = DH == 64 ? 2 : 1, NO = DH == 64 ? 2 : 1;    // buffers of the query tiles and of O_1, O_2
+    static constexpr int Q_BYTES = NBLK * kTaBM * 128;                    // one stream's query tile
+    static constexpr int K_BYTES = NBLK * kTaKV * 128, V_BLOCK = kTaKV * 128, V_BYTES = NBLK * V_BLOCK;
+    static constexpr int OFF_K = NQ * 2 * Q_BYTES, OFF_V = OFF_K + KST * 2 * K_BYTES, OFF_BAR = OFF_V + VST * V_BYTES;
+    static constexpr int BAR_QFULL = 0, BAR_QEMPTY = 2, BAR_OEMPTY = 4, BAR_KFULL = 6, BAR_KEMPTY = BAR_KFULL + KST, BAR_VFULL = BAR_KEMPTY + KST, BAR_VEMPTY = BAR_VFULL + VST,
+                         BAR_SFULL = BAR_VEMPTY + VST,    // [stream][buffer]
+                         BAR_PFULL = BAR_SFULL + 4, BAR_L = BAR_PFULL + 4, BAR_COUNT = BAR_L + 2;
+    static constexpr int OFF_L = OFF_BAR + 384;                           // [parity of the tile][2][128] floats
+    static constexpr int SMEM_BYTES = OFF_L + 2 * 2 * kTaBM * 4 + 1024;
+    static constexpr int COL_S = 0, COL_O = 4 * kTaKV;                    // scores: + (2 stream + buffer) 64; O: + (2 buffer + stream) DH
+    static constexpr uint32_t IDESC_S = (1u << 4) | (1u << 7) | (1u << 10) | ((uint32_t)(kTaKV >> 3) << 17) | ((uint32_t)(kTaBM >> 4) << 24);
     static constexpr uint32_t IDESC_PV = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 16) | ((uint32_t)(DH >> 3) << 17) | ((uint32_t)(kTaBM >> 4) << 24);
+    static_assert(BAR_COUNT * 8 + 16 <= 384, "barrier block");
+    static_assert(COL_O + NO * 2 * DH <= 512 && SMEM_BYTES <= 227 * 1024, "tensor and shared memory");
 };
 
 __device__ __forceinline__ float ex2_approx(float x) {
@@ -59,13 +73,30 @@ __device__ __forceinline__ float ex2_approx(float x) {
     asm("ex2.approx.ftz.f32 %0, %1;\n" : "=f"(y) : "f"(x));
     return y;
 }
+// Two binary32 operations per instruction (the halves of a 64-bit register pair).
+__device__ __forceinline__ uint64_t pack_f32x2(float lo, float hi) {
+    uint64_t v;
+    asm("mov.b64 %0, {%1, %2};\n" : "=l"(v) : "f"(lo), "f"(hi));
+    return v;
+}
+__device__ __forceinline__ void unpack_f32x2(uint64_t v, float &lo, float &hi) { asm("mov.b64 {%0, %1}, %2;\n" : "=f"(lo), "=f"(hi) : "l"(v)); }
+__device__ __forceinline__ uint64_t fma_f32x2(uint64_t a, uint64_t b, uint64_t c) {
+    uint64_t d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;\n" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+__device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
+    uint64_t d;
+    asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
+    return d;
+}
 
 template <int DH>
 __global__ void __launch_bounds__(kTaThreads, 1)
 ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __grid_constant__ CUtensorMap tmap_k,
                          const __grid_constant__ CUtensorMap tmap_v, const AttnParams p, unsigned int *status) {
     using C = TaCfg<DH>;
-    constexpr int KV = C::KV;
+    constexpr int KV = kTaKV;
     extern __shared__ uint8_t ta_smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)ta_smem_raw + 1023) & ~(uintptr_t)1023);
     const uint32_t sbase = smem_u32(smem), bar0 = sbase + C::OFF_BAR;
@@ -74,25 +105,41 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_BAR + C::BAR_COUNT * 8 + 4);
     float *s_l = reinterpret_cast<float *>(smem + C::OFF_L);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const int L = p.L, h = p.h, nqt = (L + kTaBM - 1) / kTaBM;
-    const int qt = nqt - 1 - (int)(blockIdx.x / (unsigned)(p.B * h));  // the long tiles (late queries) start first
-    const int bh = (int)(blockIdx.x % (unsigned)(p.B * h)), b = bh / h, hd = bh % h;
-    const int q0 = qt * kTaBM, tok0 = b * L;
-    const int keys = q0 + kTaBM < L ? q0 + kTaBM : L;  // keys 0 .. keys - 1 are visible to this tile
-    const int J = (keys + KV - 1) / KV;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int L = p.L, h = p.h, nqt = (L + kTaBM - 1) / kTaBM, bhs = p.B * h, items = nqt * bhs, G = (int)gridDim.x;
+    // The CTA's k-th tile: the tiles in order of falling length (late queries first) are dealt in rounds, every other
+    // round backwards, so that the CTAs' sums stay close.
+    struct Tile { int q0, tok0, hd, J; };
+    auto tile_of = [&](int k, Tile &t) {
+        const int i = k * G + ((k & 1) ? G - 1 - (int)blockIdx.x : (int)blockIdx.x);
+        if (i >= items) return false;
+        const int qt = nqt - 1 - i / bhs, bh = i % bhs, keys = (qt + 1) * kTaBM < L ? (qt + 1) * kTaBM : L;  // keys visible to the tile
+        t.q0 = qt * kTaBM;
+        t.tok0 = (bh / h) * L;
+        t.hd = bh % h;
+        t.J = (keys + KV - 1) / KV;
+        return true;
+    };
 
     if (tid == 0) {
-        mbar_init(bar(C::BAR_Q), 1);
-        for (int s = 0; s < kTaStages; ++s) {
-            mbar_init(bar(C::BAR_KVFULL + s), 1);
-            mbar_init(bar(C::BAR_KVEMPTY + s), 1);
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar(C::BAR_QFULL + i), 1);
+            mbar_init(bar(C::BAR_QEMPTY + i), 2);
+            mbar_init(bar(C::BAR_OEMPTY + i), 8);
+            mbar_init(bar(C::BAR_L + i), 8);
         }
-        for (int st = 0; st < 2; ++st) {
-            mbar_init(bar(C::BAR_SFULL + st), 1);
-            mbar_init(bar(C::BAR_PFULL + st), 4);
+        for (int s = 0; s < C::KST; ++s) {
+            mbar_init(bar(C::BAR_KFULL + s), 1);
+            mbar_init(bar(C::BAR_KEMPTY + s), 2);  // a commit from each issuer
         }
-        mbar_init(bar(C::BAR_FINAL), 1);
+        for (int s = 0; s < C::VST; ++s) {
+            mbar_init(bar(C::BAR_VFULL + s), 1);
+            mbar_init(bar(C::BAR_VEMPTY + s), 2);
+        }
+        for (int i = 0; i < 4; ++i) {
+            mbar_init(bar(C::BAR_SFULL + i), 1);
+            mbar_init(bar(C::BAR_PFULL + i), 4);
+        }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
         fence_proxy_async();
@@ -104,218 +151,277 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (warp-uniform)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        uint32_t issued[kTaStages] = {};
+        uint32_t k_issued[C::KST] = {}, v_issued[C::VST] = {}, q_issued[C::NQ] = {};
         bool ok = true;
-        if (lane == 0) {
-            mbar_arrive_expect_tx(bar(C::BAR_Q), 2 * C::Q_BYTES);
-            for (int st = 0; st < 2; ++st)
-                for (int blk = 0; blk < C::NBLK; ++blk)
-                    tma_load_2d(sbase + st * C::Q_BYTES + blk * kTaBM * 128, &tmap_q, (st * h + hd) * DH + 64 * blk, tok0 + q0, bar(C::BAR_Q));
-        }
-        for (int j = 0; j < J; ++j) {
-            const int s = j % kTaStages;
-            ok = mbar_wait(bar(C::BAR_KVEMPTY + s), (uint32_t)((j / kTaStages) & 1) ^ 1u, abort_flag, status, 0xa00u + s);
+        int ks = 0, vs = 0, qb = 0;
+        uint32_t kph = 1, vph = 1, qph = 1;
+        Tile t;
+        for (int k = 0; ok && tile_of(k, t); ++k) {
+            ok = mbar_wait(bar(C::BAR_QEMPTY + qb), qph, abort_flag, status, 0xa04u + qb);
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             if (lane == 0) {
-                const uint32_t dst = sbase + C::OFF_RING + s * C::STAGE, full = bar(C::BAR_KVFULL + s);
-                mbar_arrive_expect_tx(full, C::STAGE);
-                for (int blk = 0; blk < C::NBLK; ++blk) {
-                    tma_load_2d(dst + blk * KV * 128, &tmap_k, hd * DH + 64 * blk, tok0 + j * KV, full);
-                    tma_load_2d(dst + C::K_BYTES + blk * KV * 128, &tmap_k, (h + hd) * DH + 64 * blk, tok0 + j * KV, full);
-                    tma_load_2d(dst + 2 * C::K_BYTES + blk * C::V_BLOCK, &tmap_v, hd * DH + 64 * blk, tok0 + j * KV, full);
-                }
+                const uint32_t full = bar(C::BAR_QFULL + qb);
+                mbar_arrive_expect_tx(full, 2 * C::Q_BYTES);
+                for (int st = 0; st < 2; ++st)
+                    for (int blk = 0; blk < C::NBLK; ++blk)
+                        tma_load_2d(sbase + (2 * qb + st) * C::Q_BYTES + blk * kTaBM * 128, &tmap_q, (st * h + t.hd) * DH + 64 * blk, t.tok0 + t.q0, full);
             }
-            ++issued[s];
-        }
-        for (int q = 0; q < kTaStages; ++q)  // never leave with a copy in flight
-            if (issued[q]) {
-                const uint32_t par = (issued[q] - 1u) & 1u;
-                for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar(C::BAR_KVFULL + q), par); ++i) {}
-            }
-        for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar(C::BAR_Q), 0); ++i) {}
-    } else if (warp == 1) {
-        // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
-            bool ok = true;
-            auto issue_s = [&](int st, int s) {  // S_st = Q_st K_st^T from stage s
-                const uint32_t qa = sbase + st * C::Q_BYTES, ka = sbase + C::OFF_RING + s * C::STAGE + st * C::K_BYTES;
-#pragma unroll
-                for (int blk = 0; blk < C::NBLK; ++blk) {
-                    const uint64_t adesc = make_sw128_desc(qa + blk * kTaBM * 128), bdesc = make_sw128_desc(ka + blk * KV * 128);
-#pragma unroll
-                    for (int kk = 0; kk < 4; ++kk)
-                        mma_f16(tmem_base + C::COL_S + st * KV, adesc + 2u * kk, bdesc + 2u * kk, C::IDESC_S, (blk | kk) ? 1u : 0u);
-                }
-                tc_commit(bar(C::BAR_SFULL + st));
-            };
-            auto issue_pv = [&](int st, int s, bool first) {  // O_st (+)= P_st V from stage s
-                const uint64_t bdesc = make_sw128_mn_desc(sbase + C::OFF_RING + s * C::STAGE + 2 * C::K_BYTES, C::V_BLOCK);
-#pragma unroll
-                for (int kk = 0; kk < KV / 16; ++kk)
-                    mma_f16_ts(tmem_base + C::COL_O + st * DH, tmem_base + C::COL_P + st * (KV / 2) + 8 * kk, bdesc + (uint64_t)(128 * kk),
-                               C::IDESC_PV, (!first || kk) ? 1u : 0u);
-            };
-            ok = mbar_wait(bar(C::BAR_Q), 0, abort_flag, status, 0xa10u);
-            ok = ok && mbar_wait(bar(C::BAR_KVFULL + 0), 0, abort_flag, status, 0xa11u);
-            if (ok) {
-                tc_fence_after();
-                issue_s(0, 0);
-                issue_s(1, 0);
-            }
-            for (int j = 0; ok && j < J; ++j) {
-                const int s = j % kTaStages, s1 = (j + 1) % kTaStages;
-                for (int st = 0; st < 2; ++st) {
-                    if (!(ok = mbar_wait(bar(C::BAR_PFULL + st), (uint32_t)(j & 1), abort_flag, status, 0xa20u + st))) break;
-                    tc_fence_after();
-                    issue_pv(st, s, j == 0);
-                    if (st == 1) tc_commit(bar(C::BAR_KVEMPTY + s));
-                    if (j + 1 < J) {
-                        if (st == 0 && !(ok = mbar_wait(bar(C::BAR_KVFULL + s1), (uint32_t)(((j + 1) / kTaStages) & 1), abort_flag, status, 0xa30u + s1)))
-                            break;
-                        tc_fence_after();
-                        issue_s(st, s1);
+            ++q_issued[qb];
+            if (++qb == C::NQ) { qb = 0; qph ^= 1u; }
+            for (int j = 0; j < t.J; ++j) {
+                ok = mbar_wait(bar(C::BAR_KEMPTY + ks), kph, abort_flag, status, 0xa00u + ks);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                if (lane == 0) {
+                    const uint32_t dst = sbase + C::OFF_K + ks * 2 * C::K_BYTES, full = bar(C::BAR_KFULL + ks);
+                    mbar_arrive_expect_tx(full, 2 * C::K_BYTES);
+                    for (int blk = 0; blk < C::NBLK; ++blk) {
+                        tma_load_2d(dst + blk * KV * 128, &tmap_k, t.hd * DH + 64 * blk, t.tok0 + j * KV, full);
+                        tma_load_2d(dst + C::K_BYTES + blk * KV * 128, &tmap_k, (h + t.hd) * DH + 64 * blk, t.tok0 + j * KV, full);
                     }
                 }
+                ++k_issued[ks];
+                if (++ks == C::KST) { ks = 0; kph ^= 1u; }
+                ok = mbar_wait(bar(C::BAR_VEMPTY + vs), vph, abort_flag, status, 0xa08u + vs);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                if (lane == 0) {
+                    const uint32_t full = bar(C::BAR_VFULL + vs);
+                    mbar_arrive_expect_tx(full, C::V_BYTES);
+                    for (int blk = 0; blk < C::NBLK; ++blk)
+                        tma_load_2d(sbase + C::OFF_V + vs * C::V_BYTES + blk * C::V_BLOCK, &tmap_v, t.hd * DH + 64 * blk, t.tok0 + j * KV, full);
+                }
+                ++v_issued[vs];
+                if (++vs == C::VST) { vs = 0; vph ^= 1u; }
             }
-            if (ok) tc_commit(bar(C::BAR_FINAL));
+        }
+        // never leave with a copy in flight
+        for (int q = 0; q < C::KST; ++q)
+            if (k_issued[q])
+                for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar(C::BAR_KFULL + q), (k_issued[q] - 1u) & 1u); ++i) {}
+        for (int q = 0; q < C::VST; ++q)
+            if (v_issued[q])
+                for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar(C::BAR_VFULL + q), (v_issued[q] - 1u) & 1u); ++i) {}
+        for (int q = 0; q < C::NQ; ++q)
+            if (q_issued[q])
+                for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar(C::BAR_QFULL + q), (q_issued[q] - 1u) & 1u); ++i) {}
+    } else if (warp < 3) {
+        // ------------------------------------------------------------------ MMA issuers, one warp per stream
+        // The whole warp walks the loop, so that descriptors live in uniform registers; elect.sync picks the issuing
+        // lane (one thread in a divergent branch took 80 to 125 clocks an MMA).  A warp per stream, because the
+        // book-keeping of a step shares its scheduler with the exponentials.
+        const int st = warp - 1;
+        auto wait = [&](int i, uint32_t par, unsigned int code) {
+            return __all_sync(0xffffffffu, mbar_wait_poll(bar(i), par, abort_flag, status, code)) != 0;
+        };
+        const uint64_t q_desc = make_sw128_desc(sbase + st * C::Q_BYTES), k_desc = make_sw128_desc(sbase + C::OFF_K + st * C::K_BYTES);
+        const uint64_t v_desc = make_sw128_mn_desc(sbase + C::OFF_V, C::V_BLOCK);
+        const uint32_t s_col = tmem_base + C::COL_S + 2 * st * KV;
+        auto issue_s = [&](int buf, int s, int qb) {  // the stream's scores from K stage s
+            const uint64_t qd = q_desc + (uint64_t)(qb * (2 * C::Q_BYTES >> 4)), kd = k_desc + (uint64_t)(s * (2 * C::K_BYTES >> 4));
+#pragma unroll
+            for (int blk = 0; blk < C::NBLK; ++blk)
+#pragma unroll
+                for (int kk = 0; kk < 4; ++kk)
+                    warp_mma_f16(s_col + buf * KV, qd + (uint64_t)(blk * (kTaBM * 128 >> 4) + 2 * kk), kd + (uint64_t)(blk * (KV * 128 >> 4) + 2 * kk),
+                                 C::IDESC_S, (blk | kk) ? 1u : 0u);
+        };
+        auto issue_pv = [&](int buf, int s, int ob, bool first) {  // O (+)= P V from V stage s
+            const uint32_t o_col = tmem_base + C::COL_O + (2 * ob + st) * DH;
+            const uint64_t vd = v_desc + (uint64_t)(s * (C::V_BYTES >> 4));
+#pragma unroll
+            for (int kk = 0; kk < KV / 16; ++kk)
+                warp_mma_f16_ts(o_col, s_col + buf * KV + 8 * kk, vd + (uint64_t)(128 * kk), C::IDESC_PV, (!first || kk) ? 1u : 0u);
+        };
+        // The steps of all tiles are one sequence, g: the scores of step g + 2 follow P V of step g also across
+        // the end of a tile, while its outputs are still being written.  (sj, sk, stile: the score side, two steps ahead.)
+        bool ok = true, s_more, p_more;
+        int ks = 0, vs = 0, sqb = 0, sk = 0, sj = 0, pk_ = 0, pob = 0, g = 0;
+        uint32_t kph = 0, vph = 0, sqph = 0, poph = 1;
+        Tile stile, ptile;
+        s_more = tile_of(0, stile);
+        p_more = tile_of(0, ptile);
+        auto next_scores = [&](int buf) {  // false if a wait gave up
+            if (sj == 0 && !wait(C::BAR_QFULL + sqb, sqph, 0xa10u + sqb)) return false;
+            if (!wait(C::BAR_KFULL + ks, kph, 0xa30u + ks)) return false;
+            tc_fence_after();
+            issue_s(buf, ks, sqb);
+            warp_commit(bar(C::BAR_SFULL + 2 * st + buf));  // also: P V of two steps before is complete
+            warp_commit(bar(C::BAR_KEMPTY + ks));
+            if (++ks == C::KST) { ks = 0; kph ^= 1u; }
+            if (++sj == stile.J) {
+                warp_commit(bar(C::BAR_QEMPTY + sqb));
+                if (++sqb == C::NQ) { sqb = 0; sqph ^= 1u; }
+                sj = 0;
+                s_more = tile_of(++sk, stile);
+            }
+            return true;
+        };
+        for (int i = 0; ok && i < 2 && s_more; ++i) ok = next_scores(i);
+        while (ok && p_more) {
+            if (!(ok = wait(C::BAR_OEMPTY + pob, poph, 0xa18u + pob))) break;
+            for (int j = 0; j < ptile.J; ++j, ++g) {
+                const int buf = g & 1;
+                if (!(ok = wait(C::BAR_VFULL + vs, vph, 0xa28u + vs))) break;
+                if (!(ok = wait(C::BAR_PFULL + 2 * st + buf, (uint32_t)(g >> 1) & 1u, 0xa20u + st))) break;
+                tc_fence_after();
+                issue_pv(buf, vs, pob, j == 0);
+                warp_commit(bar(C::BAR_VEMPTY + vs));
+                if (++vs == C::VST) { vs = 0; vph ^= 1u; }
+                // the products execute in issue order: P of this step has been read when those scores replace it
+                if (s_more) { if (!(ok = next_scores(buf))) break; }
+                else warp_commit(bar(C::BAR_SFULL + 2 * st + buf));
+            }
+            if (++pob == C::NO) { pob = 0; poph ^= 1u; }
+            p_more = tile_of(++pk_, ptile);
         }
     } else if (warp >= 4) {
         // ------------------------------------------------------------------ softmax of one stream, one row per thread
-        const int st = warp >= 8 ? 1 : 0, quarter = warp & 3, row = 32 * quarter + lane, qi = q0 + row;
+        const int st = warp >= 8 ? 1 : 0, quarter = warp & 3, row = 32 * quarter + lane;
         const uint32_t lane_base = tmem_base + ((uint32_t)(32 * quarter) << 16);
-        const uint32_t s_addr = lane_base + C::COL_S + st * KV, o_addr = lane_base + C::COL_O + st * DH, p_addr = lane_base + C::COL_P + st * (KV / 2);
         const float c = p.scale_log2;
-        float m = -1e30f, l = 0.0f;
         bool ok = true;
-        for (int j = 0; j < J; ++j) {
-            ok = mbar_wait(bar(C::BAR_SFULL + st), (uint32_t)(j & 1), abort_flag, status, 0xa40u + st);
-            if (!(ok = __all_sync(0xffffffffu, ok))) break;
-            tc_fence_after();
-            const int k0 = j * KV;
-            const bool diag = k0 + KV - 1 > q0;  // some key of the tile lies after some query of the tile
-            // pass 1: the row's maximum (two chunks of 32 scores in flight)
-            float mx = -1e30f;
+        int g = 0, ob = 0;
+        Tile t;
+        for (int k = 0; ok && tile_of(k, t); ++k) {
+            const int qi = t.q0 + row, w0 = t.q0 + 32 * quarter;  // w0: the warp's first query
+            const uint32_t o_addr = lane_base + C::COL_O + (2 * ob + st) * DH;
+            float m = -1e30f;
+            uint64_t l2a = 0, l2b = 0;  // the row's sum, four partial sums
+            for (int j = 0; j < t.J; ++j, ++g) {
+                const int buf = g & 1, k0 = j * KV;
+                const uint32_t s_addr = lane_base + C::COL_S + (2 * st + buf) * KV;
+                ok = mbar_wait_poll(bar(C::BAR_SFULL + 2 * st + buf), (uint32_t)(g >> 1) & 1u, abort_flag, status, 0xa40u + st);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                tc_fence_after();
+                uint32_t pk[32];
+                if (k0 > w0 + 31) {  // every key of the step lies after every query of the warp
 #pragma unroll
-            for (int cc = 0; cc < KV; cc += 64) {
-                uint32_t v0[32], v1[32];
-                tmem_ld32(s_addr + cc, v0);
-                tmem_ld32(s_addr + cc + 32, v1);
-                tmem_ld_wait();
-                if (diag) {
-#pragma unroll
-                    for (int u = 0; u < 32; ++u) {
-                        if (k0 + cc + u <= qi) mx = fmaxf(mx, __uint_as_float(v0[u]));
-                        if (k0 + cc + 32 + u <= qi) mx = fmaxf(mx, __uint_as_float(v1[u]));
-                    }
+                    for (int u = 0; u < 32; ++u) pk[u] = 0u;
                 } else {
-                    float m0 = __uint_as_float(v0[0]), m1 = __uint_as_float(v1[0]);
-#pragma unroll
-                    for (int u = 1; u < 32; ++u) {
-                        m0 = fmaxf(m0, __uint_as_float(v0[u]));
-                        m1 = fmaxf(m1, __uint_as_float(v1[u]));
-                    }
-                    mx = fmaxf(mx, fmaxf(m0, m1));
-                }
-            }
-            // The reference point of the exponentials follows the maximum only when the maximum has moved by more
-            // than kTaSlack (in log2 units): probabilities then stay below 2^kTaSlack, and O and l are rescaled
-            // rarely instead of at nearly every tile.  (The final O / l does not depend on the reference point.)
-            float m_new = m;
-            if ((mx - m) * c > (j == 0 ? -1.0f : kTaSlack)) m_new = mx;
-            if (j > 0 && __any_sync(0xffffffffu, m_new != m)) {
-                const float alpha = ex2_approx((m - m_new) * c);
-                l *= alpha;
-#pragma unroll
-                for (int cc = 0; cc < DH; cc += 32) {
-                    uint32_t v[32];
-                    tmem_ld32(o_addr + cc, v);
+                    uint32_t v0[32], v1[32];
+                    tmem_ld32(s_addr, v0);
+                    tmem_ld32(s_addr + 32, v1);
                     tmem_ld_wait();
+                    if (k0 + KV - 1 > w0) {  // some key of the step lies after some query of the warp
 #pragma unroll
-                    for (int u = 0; u < 32; ++u) v[u] = __float_as_uint(__uint_as_float(v[u]) * alpha);
-                    tmem_st32(o_addr + cc, v);
-                }
-            }
-            // pass 2: probabilities as bf16 pairs, 64 keys at a time
-            const float mc = m_new * c;
+                        for (int u = 0; u < 32; ++u) {
+                            if (k0 + u > qi) v0[u] = 0xff800000u;       // -inf: probability 0
+                            if (k0 + 32 + u > qi) v1[u] = 0xff800000u;
+                        }
+                    }
+                    float m0 = -1e30f, m1 = -1e30f, m2 = -1e30f, m3 = -1e30f;
 #pragma unroll
-            for (int cc = 0; cc < KV; cc += 64) {
-                uint32_t v0[32], v1[32], pk[32];
-                tmem_ld32(s_addr + cc, v0);
-                tmem_ld32(s_addr + cc + 32, v1);
-                tmem_ld_wait();
-                if (diag) {
+                    for (int u = 0; u < 32; u += 4) {
+                        m0 = fmaxf(m0, fmaxf(__uint_as_float(v0[u]), __uint_as_float(v0[u + 1])));
+                        m1 = fmaxf(m1, fmaxf(__uint_as_float(v0[u + 2]), __uint_as_float(v0[u + 3])));
+                        m2 = fmaxf(m2, fmaxf(__uint_as_float(v1[u]), __uint_as_float(v1[u + 1])));
+                        m3 = fmaxf(m3, fmaxf(__uint_as_float(v1[u + 2]), __uint_as_float(v1[u + 3])));
+                    }
+                    const float mx = fmaxf(fmaxf(m0, m1), fmaxf(m2, m3));
+                    // The reference point of the exponentials follows the maximum only when the maximum has moved by more
+                    // than kTaSlack (in log2 units): probabilities then stay below 2^kTaSlack, and O and l are rescaled
+                    // rarely instead of at nearly every tile.  (The final O / l does not depend on the reference point.)
+                    float m_new = m;
+                    if ((mx - m) * c > (j == 0 ? -1.0f : kTaSlack)) m_new = mx;
+                    if (j > 0 && __any_sync(0xffffffffu, m_new != m)) {
+                        // O_s is at rest once P V of the step before is complete: the barrier of the next step's scores follows it
+                        ok = mbar_wait_poll(bar(C::BAR_SFULL + 2 * st + (buf ^ 1)), (uint32_t)((g + 1) >> 1) & 1u, abort_flag, status, 0xa48u + st);
+                        if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                        tc_fence_after();
+                        const float alpha = ex2_approx((m - m_new) * c);
+                        const uint64_t a2 = pack_f32x2(alpha, alpha);
+                        l2a = fma_f32x2(l2a, a2, 0ull);
+                        l2b = fma_f32x2(l2b, a2, 0ull);
 #pragma unroll
-                    for (int u = 0; u < 32; ++u) {
-                        if (k0 + cc + u > qi) v0[u] = 0xff800000u;       // -inf: probability 0
-                        if (k0 + cc + 32 + u > qi) v1[u] = 0xff800000u;
+                        for (int cc = 0; cc < DH; cc += 16) {
+                            uint32_t o[16];
+                            tmem_ld16(o_addr + cc, o);
+                            tmem_ld_wait();
+#pragma unroll
+                            for (int u = 0; u < 16; ++u) o[u] = __float_as_uint(__uint_as_float(o[u]) * alpha);
+                            tmem_st16(o_addr + cc, o);
+                        }
+                    }
+                    m = m_new;
+                    // probabilities as bf16 pairs
+                    const uint64_t c2 = pack_f32x2(c, c), nmc2 = pack_f32x2(-m_new * c, -m_new * c);
+                    auto pair = [&](uint32_t a, uint32_t b, uint64_t &sum) {
+                        float x0, x1;
+                        unpack_f32x2(fma_f32x2(pack_f32x2(__uint_as_float(a), __uint_as_float(b)), c2, nmc2), x0, x1);
+                        const float p0 = ex2_approx(x0), p1 = ex2_approx(x1);
+                        sum = add_f32x2(sum, pack_f32x2(p0, p1));
+                        return pack_bf16(p0, p1);
+                    };
+#pragma unroll
+                    for (int u = 0; u < 32; u += 2) {
+                        pk[u >> 1] = pair(v0[u], v0[u + 1], l2a);
+                        pk[16 + (u >> 1)] = pair(v1[u], v1[u + 1], l2b);
                     }
                 }
-                float l0 = 0.0f, l1 = 0.0f;
-#pragma unroll
-                for (int u = 0; u < 32; u += 2) {
-                    const float pa0 = ex2_approx(fmaf(__uint_as_float(v0[u]), c, -mc)), pa1 = ex2_approx(fmaf(__uint_as_float(v0[u + 1]), c, -mc));
-                    const float pb0 = ex2_approx(fmaf(__uint_as_float(v1[u]), c, -mc)), pb1 = ex2_approx(fmaf(__uint_as_float(v1[u + 1]), c, -mc));
-                    l0 += pa0 + pa1;
-                    l1 += pb0 + pb1;
-                    pk[u >> 1] = pack_bf16(pa0, pa1);
-                    pk[16 + (u >> 1)] = pack_bf16(pb0, pb1);
-                }
-                l += l0 + l1;
-                tmem_st32(p_addr + (cc >> 1), pk);
+                tmem_st32(s_addr, pk);
+                tmem_st_wait();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(bar(C::BAR_PFULL + 2 * st + buf));
             }
-            tmem_st_wait();
+            if (!ok) break;
+            // ---- outputs of the tile: (O_1 / l_1 - lambda O_2 / l_2) out_scale; stream s's thread of a row writes half s
+            // of the row's columns.  The stream's last P V is complete when the barrier of two steps on says so (of
+            // the other stream's barriers this warp does not know the phase), both streams' when all eight warps say so.
+            ok = mbar_wait_poll(bar(C::BAR_SFULL + 2 * st + ((g - 1) & 1)), (uint32_t)((g + 1) >> 1) & 1u, abort_flag, status, 0xa50u + st);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            float la, lb, lc, ld;
+            unpack_f32x2(l2a, la, lb);
+            unpack_f32x2(l2b, lc, ld);
+            float *sl = s_l + (k & 1) * 2 * kTaBM;
+            sl[st * kTaBM + row] = (la + lb) + (lc + ld);
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar(C::BAR_PFULL + st));
-            m = m_new;
-        }
-        if (ok) {
-            ok = mbar_wait(bar(C::BAR_FINAL), 0, abort_flag, status, 0xa50u);
-            ok = __all_sync(0xffffffffu, ok);
-        }
-        s_l[st * kTaBM + row] = l;
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    if (warp >= 4 && !*abort_flag) {
-        // (O_1 / l_1 - lambda O_2 / l_2) out_scale: stream s's thread of a row writes half s of the row's columns
-        const int st = warp >= 8 ? 1 : 0, quarter = warp & 3, row = 32 * quarter + lane, qi = q0 + row;
-        const uint32_t lane_base = tmem_base + ((uint32_t)(32 * quarter) << 16);
-        const float w1 = p.out_scale / s_l[row], w2 = p.out_scale * p.lambda / s_l[kTaBM + row];
-        const size_t obase = (size_t)(tok0 + qi) * ((size_t)h * DH) + (size_t)hd * DH;
+            if (lane == 0) mbar_arrive(bar(C::BAR_L + (k & 1)));
+            ok = mbar_wait_poll(bar(C::BAR_L + (k & 1)), (uint32_t)(k >> 1) & 1u, abort_flag, status, 0xa52u);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            tc_fence_after();
+            const float w1 = p.out_scale / sl[row], w2 = p.out_scale * p.lambda / sl[kTaBM + row];
+            const size_t obase = (size_t)(t.tok0 + qi) * ((size_t)h * DH) + (size_t)t.hd * DH;
+            const uint32_t o_base = lane_base + C::COL_O + 2 * ob * DH;
 #pragma unroll
-        for (int cc = st * (DH / 2); cc < (st + 1) * (DH / 2); cc += 32) {
-            uint32_t v1[32], v2[32];
-            tmem_ld32(lane_base + C::COL_O + cc, v1);
-            tmem_ld32(lane_base + C::COL_O + DH + cc, v2);
-            tmem_ld_wait();
-            if (qi < L) {
-                if (p.flags & HGF_FLAG_OUT_BF16) {
-                    uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) + obase + cc);
+            for (int cc = st * (DH / 2); cc < (st + 1) * (DH / 2); cc += 32) {
+                uint32_t v1[32], v2[32];
+                tmem_ld32(o_base + cc, v1);
+                tmem_ld32(o_base + DH + cc, v2);
+                tmem_ld_wait();
+                if (cc + 32 == (st + 1) * (DH / 2)) {  // all of the accumulators is in registers
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(C::BAR_OEMPTY + ob));
+                }
+                if (qi < L) {
+                    if (p.flags & HGF_FLAG_OUT_BF16) {
+                        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) + obase + cc);
 #pragma unroll
-                    for (int u = 0; u < 32; u += 8) {
-                        uint32_t o[4];
+                        for (int u = 0; u < 32; u += 8) {
+                            uint32_t o[4];
 #pragma unroll
-                        for (int e = 0; e < 4; ++e)
-                            o[e] = pack_bf16(__uint_as_float(v1[u + 2 * e]) * w1 - __uint_as_float(v2[u + 2 * e]) * w2,
-                                             __uint_as_float(v1[u + 2 * e + 1]) * w1 - __uint_as_float(v2[u + 2 * e + 1]) * w2);
-                        dst[u >> 3] = make_uint4(o[0], o[1], o[2], o[3]);
+                            for (int e = 0; e < 4; ++e)
+                                o[e] = pack_bf16(__uint_as_float(v1[u + 2 * e]) * w1 - __uint_as_float(v2[u + 2 * e]) * w2,
+                                                 __uint_as_float(v1[u + 2 * e + 1]) * w1 - __uint_as_float(v2[u + 2 * e + 1]) * w2);
+                            dst[u >> 3] = make_uint4(o[0], o[1], o[2], o[3]);
+                        }
+                    } else {
+                        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.out) + obase + cc);
+#pragma unroll
+                        for (int u = 0; u < 32; u += 4)
+                            dst[u >> 2] = make_float4(__uint_as_float(v1[u]) * w1 - __uint_as_float(v2[u]) * w2,
+                                                      __uint_as_float(v1[u + 1]) * w1 - __uint_as_float(v2[u + 1]) * w2,
+                                                      __uint_as_float(v1[u + 2]) * w1 - __uint_as_float(v2[u + 2]) * w2,
+                                                      __uint_as_float(v1[u + 3]) * w1 - __uint_as_float(v2[u + 3]) * w2);
                     }
-                } else {
-                    float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.out) + obase + cc);
-#pragma unroll
-                    for (int u = 0; u < 32; u += 4)
-                        dst[u >> 2] = make_float4(__uint_as_float(v1[u]) * w1 - __uint_as_float(v2[u]) * w2,
-                                                  __uint_as_float(v1[u + 1]) * w1 - __uint_as_float(v2[u + 1]) * w2,
-                                                  __uint_as_float(v1[u + 2]) * w1 - __uint_as_float(v2[u + 2]) * w2,
-                                                  __uint_as_float(v1[u + 3]) * w1 - __uint_as_float(v2[u + 3]) * w2);
                 }
             }
+            if (++ob == C::NO) ob = 0;
         }
     }
     tc_fence_before();
@@ -337,10 +443,12 @@ static cudaError_t launch_attention_tc(const AttnParams &p, cudaStream_t stream)
     const uint64_t rows = (uint64_t)p.B * p.L, dq = (uint64_t)2 * p.h * DH, dv = (uint64_t)p.h * DH;
     CUtensorMap mq, mk, mv;
     if (!make_map_2d(&mq, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.q, dq, rows, dq * 2, 64, kTaBM, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&mk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.k, dq, rows, dq * 2, 64, C::KV, CU_TENSOR_MAP_SWIZZLE_128B) ||
-        !make_map_2d(&mv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.v, dv, rows, dv * 2, 64, C::KV, CU_TENSOR_MAP_SWIZZLE_128B))
+        !make_map_2d(&mk, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.k, dq, rows, dq * 2, 64, kTaKV, CU_TENSOR_MAP_SWIZZLE_128B) ||
+        !make_map_2d(&mv, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, p.v, dv, rows, dv * 2, 64, kTaKV, CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
-    const unsigned grid = (unsigned)(((p.L + kTaBM - 1) / kTaBM) * p.B * p.h);
+    const int sms = device_sm_count();
+    if (!sms) return cudaErrorInvalidDevice;
+    const unsigned items = (unsigned)(((p.L + kTaBM - 1) / kTaBM) * p.B * p.h), grid = items < (unsigned)sms ? items : (unsigned)sms;
     ta_diff_attention_kernel<DH><<<grid, kTaThreads, C::SMEM_BYTES, stream>>>(mq, mk, mv, p, status);
     count_launch();
     return cudaGetLastError();

@@ -55,6 +55,13 @@ def test_shapes_and_ragged_lengths(hgf, B, L, h, dh):
     check(hgf, B, L, h, dh, 0.8, seed=L)
 
 
+@pytest.mark.parametrize("B,L,h,dh", [(1, 300, 149, 64), (3, 129, 53, 128), (2, 257, 60, 64), (7, 64, 43, 128)])
+def test_more_tiles_than_sms(hgf, B, L, h, dh):
+    """Every CTA works several tiles one after the other - odd and even numbers of 64-key steps, fully and partly hidden
+    steps, a last round that not every CTA takes part in - so both buffers of scores, outputs and sums change hands."""
+    check(hgf, B, L, h, dh, 0.8, seed=L + h)
+
+
 def test_listing_scale_bf16_output_and_peaked_scores(hgf):
     check(hgf, 2, 300, 2, 64, float(oracle.lambda0(64)), out_scale=0.5, seed=1)
     check(hgf, 1, 256, 2, 64, 0.8, flags=hgf.FLAG_OUT_BF16, seed=2)
