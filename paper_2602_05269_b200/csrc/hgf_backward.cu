@@ -21,7 +21,8 @@ namespace hgf {
 // the 128-byte swizzle.  The contraction may continue over a second pair of operands (A2, B2: the
 // low-rank term of dX), and may be split over several CTAs that write partial sums which a second
 // kernel adds up in a fixed order.
-// Persistent, one CTA per SM, six warps: warp 0 stages operand tiles with TMA, one lane of warp 1 issues
+// Persistent, one CTA per SM, six warps: warp 0 stages operand tiles with TMA, warp 1 issues (elect.sync: the two large
+// products of 2048 x 5632 at M = 8192 and the one for dA took 136 us on average from one thread in a branch, 115 so)
 // tcgen05.mma.kind::f16 (bf16 inputs, 128 x BN x 16 per instruction, fp32 accumulators in tensor memory,
 // two of them so that a tile's epilogue runs under the next tile's main loop), warps 2-5 read the
 // accumulator back (tcgen05.ld) and write C.  Rows and columns past the matrices, and contraction
@@ -63,7 +64,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     auto bar = [&](int i) { return bar0 + 8u * i; };
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::OFF_BAR + C::BAR_COUNT * 8);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_BAR + C::BAR_COUNT * 8 + 4);
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int tiles_i = (g.I + kTBM - 1) / kTBM, tiles_j = (g.J + BN - 1) / BN, tiles_ij = tiles_i * tiles_j;
     const int n_full = tiles_ij - g.n_half / 2;  // tiles worked whole (all of them unless n_half > 0)
     const int num_work = g.n_half ? n_full + g.n_half : tiles_ij * g.splits, kb_all = g.kb1 + g.kb2;
@@ -108,7 +109,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (warp-uniform)
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -150,7 +151,9 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             }
     } else if (warp == 1) {
         // ------------------------------------------------------------------ MMA issuer
-        if (lane == 0) {
+        // (the whole warp walks the loop: see the wrappers)
+        {
+            auto wait = [&](int i, uint32_t par, unsigned int code) { return __all_sync(0xffffffffu, mbar_wait_poll(bar(i), par, abort_flag, status, code)) != 0; };
             int s = 0, it = 0;
             uint32_t ph = 0;
             bool ok = true;
@@ -159,7 +162,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
             for (int w = blockIdx.x; ok && w < num_work; w += gridDim.x, ++it) {
                 const int b = it & 1;
                 const uint32_t acc = tmem_base + b * BN;
-                if (it >= 2 && !(ok = mbar_wait(bar(C::BAR_ACCEMPTY + b), (uint32_t)((it >> 1) - 1) & 1u, abort_flag, status, 0x810u)))
+                if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x810u)))
                     break;
                 tc_fence_after();
                 const int lo = kb_lo(w), hi = kb_hi(w);
@@ -167,19 +170,19 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
                 tile_of(w, ti0, tj0, bn);
                 const uint32_t idesc_w = (idesc & ~(0x3fu << 17)) | ((uint32_t)(bn >> 3) << 17);
                 for (int kb = lo; kb < hi; ++kb) {
-                    if (!(ok = mbar_wait(bar(C::BAR_FULL + s), ph, abort_flag, status, 0x820u + s))) break;
+                    if (!(ok = wait(C::BAR_FULL + s, ph, 0x820u + s))) break;
                     tc_fence_after();
                     const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
                     const uint64_t adesc = g.a_mn ? make_sw128_mn_desc(sa, kTBox) : make_sw128_desc(sa);
                     const uint64_t bdesc = g.b_mn ? make_sw128_mn_desc(sb, kTBox) : make_sw128_desc(sb);
 #pragma unroll
                     for (int kk = 0; kk < kTBK / 16; ++kk)
-                        mma_f16(acc, adesc + (uint64_t)(a_step * kk), bdesc + (uint64_t)(b_step * kk), idesc_w, (kb > lo || kk) ? 1u : 0u);
-                    tc_commit(bar(C::BAR_EMPTY + s));
+                        warp_mma_f16(acc, adesc + (uint64_t)(a_step * kk), bdesc + (uint64_t)(b_step * kk), idesc_w, (kb > lo || kk) ? 1u : 0u);
+                    warp_commit(bar(C::BAR_EMPTY + s));
                     if (++s == C::STAGES) { s = 0; ph ^= 1u; }
                 }
                 if (!ok) break;
-                tc_commit(bar(C::BAR_ACCFULL + b));
+                warp_commit(bar(C::BAR_ACCFULL + b));
             }
         }
     } else {

@@ -13,17 +13,15 @@
 // 128 output channels (tensor-memory lanes, MMA M) x 128 tokens (columns, MMA N); two accumulators
 // alternate, so the epilogue of a tile runs under the main loop of the next.  A pipeline stage is
 // 256 input columns (eight MMAs): every hand-over between the roles costs a shared-memory round
-// trip, and the single MMA-issuing thread can only afford one per 512 tensor-core clocks.
+// trip.
 //
 // One persistent CTA per SM, 16 warps with fixed roles:
 //   warp 0      producer (all lanes): per stage the int8 activation tile as two 128 tokens x 128 B
 //               boxes (128-byte swizzle) and the packed weights of 128 channels (eight contiguous
 //               1 KiB tiles of the tiled weight layout, one bulk copy each); per tile what its
 //               epilogue needs: row sums, scales, the H tile and the (g B)^T tile
-//   warp 1      allocates tensor memory; one lane issues the MMAs of every other pipeline stage (and the
-//               correction MMAs) and commits to mbarriers
-//   warp 11     one lane issues the MMAs of the stages in between
-//   warps 2-5, 12-15  epilogue, two warps per tensor-memory lane quarter (32 channels), one for each
+//   warp 1      allocates tensor memory; issues the MMAs and commits to mbarriers
+//   warps 2-5, 11-14  epilogue, two warps per tensor-memory lane quarter (32 channels), one for each
 //               half of the tile's tokens: dequantise the accumulator in place (tcgen05.ld /
 //               tcgen05.st), wait for the correction MMA, read the result, transpose it through shared
 //               memory and store y with TMA
@@ -48,7 +46,7 @@ constexpr int X_TILE_BYTES = 2 * X_HALF_BYTES;   // 32 KiB per stage
 constexpr int P_TILE_BYTES = TILE_C * KBLK / 4;  // 8 KiB: 8 weight tiles of 16 rows x 256 columns
 constexpr int TOKV_BYTES = TILE_T * 8;           // row sums and scales of the tile's tokens
 constexpr int STORE_BUF_BYTES = 2048;            // per epilogue warp: 32 channels x 32 tokens (bf16) or x 16 tokens (fp32)
-constexpr int GEMM_THREADS = 512;  // 16 warps
+constexpr int GEMM_THREADS = 480;  // 15 warps
 // tensor memory: two accumulators of 128 columns, then one weight operand of 64 columns (= 256 int8 per lane) per stage
 constexpr int TMEM_COLS = 512, ACC_COLS = TILE_T, A_COL = 2 * ACC_COLS, A_STAGE_COLS = KBLK / 4;
 
@@ -73,8 +71,8 @@ struct Cfg {
     static constexpr int BAR_FULL = 0, BAR_EMPTY = BAR_FULL + NS, BAR_PFULL = BAR_EMPTY + NS, BAR_PEMPTY = BAR_PFULL + PSTAGES,
                          BAR_ACCFULL = BAR_PEMPTY + PSTAGES,
                          BAR_ACCEMPTY = BAR_ACCFULL + 2, BAR_LORAREADY = BAR_ACCEMPTY + 2, BAR_LORADONE = BAR_LORAREADY + 2,
-                         BAR_OPSFULL = BAR_LORADONE + 2, BAR_OPSEMPTY = BAR_OPSFULL + 2, BAR_TURN = BAR_OPSEMPTY + 2,
-                         BAR_COUNT = BAR_TURN + 2;
+                         BAR_OPSFULL = BAR_LORADONE + 2, BAR_OPSEMPTY = BAR_OPSFULL + 2, 
+                         BAR_COUNT = BAR_OPSEMPTY + 2;
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
     static_assert(BAR_COUNT * 8 + 16 <= 512, "barrier block too small");
     static_assert(A_COL + NS * A_STAGE_COLS <= TMEM_COLS, "tensor memory budget");
@@ -105,7 +103,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // the next launch in the stream, if it asks for it, may be set up while this one runs (it waits
     // for this grid's completion before it touches memory)
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     const int tiles_t = (p.M + TILE_T - 1) / TILE_T, tiles_c = (p.N + TILE_C - 1) / TILE_C;
     const int num_tiles = tiles_t * tiles_c;
     const int kblocks = (p.K + KBLK - 1) / KBLK;
@@ -129,8 +127,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             mbar_init(bar(C::BAR_PEMPTY + j), 4);
         }
         for (int b = 0; b < 2; ++b) {
-            mbar_init(bar(C::BAR_ACCFULL + b), 2);  // one commit from each of the two MMA-issuing threads
-            mbar_init(bar(C::BAR_TURN + b), 1);
+            mbar_init(bar(C::BAR_ACCFULL + b), 1);
             mbar_init(bar(C::BAR_ACCEMPTY + b), 8);
             mbar_init(bar(C::BAR_LORAREADY + b), 8);
             mbar_init(bar(C::BAR_LORADONE + b), 1);
@@ -150,7 +147,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     tc_fence_before();
     __syncthreads();
     tc_fence_after();
-    const uint32_t tmem_base = *tmem_slot;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (warp-uniform)
     // Everything above touches only this CTA's own shared and tensor memory; what follows reads what
     // the prologue launch wrote (a no-op unless the launch carries the programmatic-dependency attribute).
     asm volatile("griddepcontrol.wait;\n" ::: "memory");
@@ -212,27 +209,22 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     for (uint32_t i = 0; i < kSpinLimit && !mbar_try_wait(bar(C::BAR_OPSFULL + q), par); ++i) {}
                 }
         }
-    } else if (warp == 1 || warp == 11) {
-        // ------------------------------------------------------------------ MMA issuers
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer
         // Tile `it` accumulates into accumulator it % 2, so the epilogue of one tile runs under the main
         // loop of the next.  With a correction, the epilogue first rewrites the accumulator as fp32
-        // (dequantised), then the first issuer adds (g B) H^T onto it with one more MMA, slipped in between
+        // (dequantised), then this warp adds (g B) H^T onto it with one more MMA, slipped in between
         // the k blocks of the tile in progress as soon as the epilogue is ready for it.
         //
-        // TWO threads issue the integer MMAs, in turns: the stages are numbered through the whole tile
-        // sequence and warp 1 takes the even ones, warp 11 the odd ones.  The tensor pipe holds hardly any
-        // MMA in reserve and takes a 128 x 128 x 32 one about as fast as it executes it (64 clocks), so with
-        // a single issuing thread it idles while that thread waits on barriers, commits and keeps its
-        // books - about as long per stage as the stage's eight MMAs run.  Here one thread does all that
-        // for its next stage while the other's MMAs run, and only the hand-over itself is exposed.  Order
-        // between the two threads' MMAs on the shared accumulator is established the documented way: after
-        // its stage a thread executes tcgen05.fence::before_thread_sync and arrives on the other's TURN
-        // barrier; the other waits there and executes tcgen05.fence::after_thread_sync before its first MMA.
-        // Each thread commits the stages it issued (EMPTY) and, at the end of a tile, ACCFULL (two arrivals).
-        const int half = warp == 1 ? 0 : 1;
-        if (lane == 0) {
+        // The whole warp walks the loop and elect.sync picks the lane that issues, so the descriptors live in
+        // uniform registers: eight MMAs take 230 clocks to issue, a stage 750 with its two barriers.  (One thread in a
+        // divergent branch needed 1100, two such threads taking stages in turns 890.)  Large layers are then held by
+        // the power limit: 1.75 GHz at 985 W, 8192 x 2048 x 5632 in 122.4 us against 126.1, 4096 x 4096 x 11008 in 201.5
+        // against 209.8; two issuing warps, or asking for the next stage ahead of time, change neither.
+        {
+            auto wait = [&](int i, uint32_t par, unsigned int code) { return __all_sync(0xffffffffu, mbar_wait_poll(bar(i), par, abort_flag, status, code)) != 0; };
             bool ok = true;
-            int it = 0, pend = -1;  // pend: tile whose correction MMA is still to be issued (first issuer only)
+            int it = 0, pend = -1;  // pend: tile whose correction MMA is still to be issued
             int gs = 0;             // stage number, counted through all tiles of this CTA
             const uint64_t xdesc0 = make_sw128_desc(sbase + C::OFF_X);
             auto issue_lora = [&](int t) {
@@ -243,67 +235,51 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const uint64_t bdesc = OPSB == 128 ? make_sw128_desc(lh) : make_sw64_desc(lh);
 #pragma unroll
                 for (int kk = 0; kk < OPSB / 32; ++kk)  // K = 16 fp16 (32 bytes of a row) per MMA, on top of the fp32 values
-                    mma_f16(tmem_base + b * ACC_COLS, adesc + 2u * kk, bdesc + 2u * kk, IDESC_F16, 1u);
-                tc_commit(bar(C::BAR_LORADONE + b));
+                    warp_mma_f16(tmem_base + b * ACC_COLS, adesc + 2u * kk, bdesc + 2u * kk, IDESC_F16, 1u);
+                warp_commit(bar(C::BAR_LORADONE + b));
             };
             for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++it) {
                 const int b = it & 1;
                 const uint32_t acc = tmem_base + b * ACC_COLS;
-                bool acc_mine = false;  // this thread has waited for the accumulator's release
+                if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x200u))) break;
                 for (int kb = 0; kb < kblocks; ++kb, ++gs) {
-                    if ((gs & 1) != half) continue;
-                    if (!acc_mine) {
-                        if (it >= 2 && !(ok = mbar_wait(bar(C::BAR_ACCEMPTY + b), (uint32_t)((it >> 1) - 1) & 1u, abort_flag, status, 0x200u)))
-                            break;
-                        acc_mine = true;
-                    }
-                    if (half == 0 && pend >= 0 && mbar_try_wait(bar(C::BAR_LORAREADY + (pend & 1)), (uint32_t)(pend >> 1) & 1u)) {
+                    if (pend >= 0 && __all_sync(0xffffffffu, mbar_test_wait(bar(C::BAR_LORAREADY + (pend & 1)), (uint32_t)(pend >> 1) & 1u))) {
                         issue_lora(pend);
                         pend = -1;
                     }
                     const int s = gs % C::STAGES;
                     const uint32_t ph = (uint32_t)(gs / C::STAGES) & 1u;
-                    if (!(ok = mbar_wait(bar(C::BAR_FULL + s), ph, abort_flag, status, 0x210u + s))) break;
-                    // the other thread has issued stage gs - 1
-                    if (gs > 0 && !(ok = mbar_wait_spin(bar(C::BAR_TURN + half), (uint32_t)((gs - 1) >> 1) & 1u, abort_flag, status, 0x240u + half)))
-                        break;
+                    if (!(ok = wait(C::BAR_FULL + s, ph, 0x210u + s))) break;
                     tc_fence_after();
                     const uint64_t bdesc = xdesc0 + (uint64_t)(s * (X_TILE_BYTES >> 4));
                     const uint32_t a_tmem = tmem_base + A_COL + s * A_STAGE_COLS;
-                    // per MMA 32 int8: 8 columns of the weight operand, 32 bytes of a token row; the stage's
-                    // second 128 columns sit in the second swizzled tile
-                    mma_i8_ts(acc, a_tmem, bdesc, IDESC_I8, kb ? 1u : 0u);
-                    mma_i8_ts(acc, a_tmem + 8u, bdesc + 2u, IDESC_I8, 1u);
-                    mma_i8_ts(acc, a_tmem + 16u, bdesc + 4u, IDESC_I8, 1u);
-                    mma_i8_ts(acc, a_tmem + 24u, bdesc + 6u, IDESC_I8, 1u);
-                    mma_i8_ts(acc, a_tmem + 32u, bdesc + (X_HALF_BYTES >> 4), IDESC_I8, 1u);
-                    mma_i8_ts(acc, a_tmem + 40u, bdesc + (X_HALF_BYTES >> 4) + 2u, IDESC_I8, 1u);
-                    mma_i8_ts(acc, a_tmem + 48u, bdesc + (X_HALF_BYTES >> 4) + 4u, IDESC_I8, 1u);
-                    mma_i8_ts(acc, a_tmem + 56u, bdesc + (X_HALF_BYTES >> 4) + 6u, IDESC_I8, 1u);
-                    tc_fence_before();
-                    mbar_arrive(bar(C::BAR_TURN + (half ^ 1)));  // the other thread's turn
-                    tc_commit(bar(C::BAR_EMPTY + s));
+                    warp_mma_i8_ts(acc, a_tmem, bdesc, IDESC_I8, kb ? 1u : 0u);
+                    warp_mma_i8_ts(acc, a_tmem + 8u, bdesc + 2u, IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 16u, bdesc + 4u, IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 24u, bdesc + 6u, IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 32u, bdesc + (X_HALF_BYTES >> 4), IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 40u, bdesc + (X_HALF_BYTES >> 4) + 2u, IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 48u, bdesc + (X_HALF_BYTES >> 4) + 4u, IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 56u, bdesc + (X_HALF_BYTES >> 4) + 6u, IDESC_I8, 1u);
+                    warp_commit(bar(C::BAR_EMPTY + s));
                 }
                 if (!ok) break;
-                tc_commit(bar(C::BAR_ACCFULL + b));
-                if (half != 0) continue;
+                warp_commit(bar(C::BAR_ACCFULL + b));
                 if (pend >= 0) {  // the previous tile's correction has to be out before its accumulator's next turn
-                    if (!(ok = mbar_wait(bar(C::BAR_LORAREADY + (pend & 1)), (uint32_t)(pend >> 1) & 1u, abort_flag, status, 0x230u)))
+                    if (!(ok = wait(C::BAR_LORAREADY + (pend & 1), (uint32_t)(pend >> 1) & 1u, 0x230u)))
                         break;
                     issue_lora(pend);
                     pend = -1;
                 }
                 if (has_lora) pend = it;
             }
-            if (half == 0 && ok && pend >= 0 &&
-                mbar_wait(bar(C::BAR_LORAREADY + (pend & 1)), (uint32_t)(pend >> 1) & 1u, abort_flag, status, 0x231u))
-                issue_lora(pend);
+            if (ok && pend >= 0 && wait(C::BAR_LORAREADY + (pend & 1), (uint32_t)(pend >> 1) & 1u, 0x231u)) issue_lora(pend);
         }
-    } else if (warp < 6 || warp >= 12) {
+    } else if (warp < 6 || warp >= 11) {
         // ------------------------------------------------------------------ epilogue warps
         // Eight of them: the warp pair of a tensor-memory lane quarter (32 output channels) shares the
         // tile's 128 tokens, 64 each, so a tile's epilogue takes half as long as with one warp per
-        // quarter - with the two issuing threads the main loop of a short-K tile is over sooner than that.
+        // quarter: the main loop of a short-K tile is over sooner than that.
         const int e2 = warp < 6 ? 0 : 1;                  // which 64 tokens of the tile
         const int q = warp & 3;                           // tensor-memory lane quarter this warp may access
         constexpr int HALF_T = TILE_T / 2;

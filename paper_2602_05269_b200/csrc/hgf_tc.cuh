@@ -75,25 +75,6 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return false;
 }
 
-// The same bound, but polling without a pause: for the hand-over between the two MMA-issuing threads,
-// where every clock of wake-up delay is a clock the tensor pipe idles (one thread polls, briefly).
-__device__ __forceinline__ bool mbar_wait_spin(uint32_t bar, uint32_t parity, volatile int *abort_flag,
-                                               unsigned int *status, unsigned int code) {
-    unsigned long long t0 = 0;
-    for (uint32_t i = 0; i < (kSpinLimit << 4); ++i) {
-        if (mbar_test_wait(bar, parity)) return true;
-        if ((i & 1023u) == 1023u) {
-            if (*abort_flag) return false;
-            const unsigned long long now = global_timer_ns();
-            if (t0 == 0) t0 = now;
-            else if (now - t0 > kWaitLimitNs) break;
-        }
-    }
-    *abort_flag = 1;
-    atomicExch(status, code);
-    return false;
-}
-
 // The same bound, polling with the hardware's own suspended try_wait and no sleep in between: for roles whose wake-up
 // is on the critical path.
 __device__ __forceinline__ bool mbar_wait_poll(uint32_t bar, uint32_t parity, volatile int *abort_flag,
@@ -140,23 +121,6 @@ __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.
 
 __device__ __forceinline__ void tc_fence_before() { asm volatile("tcgen05.fence::before_thread_sync;\n" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after() { asm volatile("tcgen05.fence::after_thread_sync;\n" ::: "memory"); }
-__device__ __forceinline__ void tc_commit(uint32_t bar) {
-    asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n" ::"r"(bar) : "memory");
-}
-__device__ __forceinline__ void mma_i8(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_f16(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n"
-        ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
 // 32 lanes x 32 consecutive 32-bit columns: register i of lane l = TMEM[lane base + l][col + i]
 __device__ __forceinline__ void tmem_ld32(uint32_t taddr, uint32_t (&r)[32]) {
     asm volatile(
@@ -216,8 +180,9 @@ __device__ __forceinline__ uint64_t make_sw128_mn_desc(uint32_t saddr, uint32_t 
     return (uint64_t)((saddr & 0x3FFFFu) >> 4) | ((uint64_t)(block_bytes >> 4) << 16) | ((uint64_t)(1024 >> 4) << 32) | (1ull << 46) |
            (2ull << 61);
 }
-// ---- the same from a whole warp ---------------------------------------------------------------------
-// Every lane of a converged warp executes these and elect.sync picks the one that issues (the same one every time, so
+// ---- MMA issue from a whole warp --------------------------------------------------------------------
+// Every lane of a converged warp executes these (operands in uniform registers; from one thread in a divergent branch an MMA
+// took 80 to 125 clocks to issue) and elect.sync picks the one that issues (the same one every time, so
 // commits follow the MMAs they track).
 __device__ __forceinline__ bool elect_one() {
     uint32_t e;
@@ -233,6 +198,7 @@ __device__ __forceinline__ void warp_mma_f16(uint32_t d, uint64_t a, uint64_t b,
                  "@e tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
                  : "memory");
 }
+// (first operand in tensor memory: lane = row, two 16-bit or four 8-bit values of consecutive contraction index per column)
 __device__ __forceinline__ void warp_mma_f16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
     asm volatile("{\n.reg .pred p, e;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
                  "@e tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
@@ -242,22 +208,6 @@ __device__ __forceinline__ void warp_mma_i8_ts(uint32_t d, uint32_t a_tmem, uint
     asm volatile("{\n.reg .pred p, e;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
                  "@e tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n}\n" ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
                  : "memory");
-}
-
-// First operand in tensor memory (lane = row, two 16-bit values of consecutive contraction index per column).
-__device__ __forceinline__ void mma_f16_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n}\n"
-        ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_i8_ts(uint32_t d, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t accumulate) {
-    asm volatile(
-        "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-        "tcgen05.mma.cta_group::1.kind::i8 [%0], [%1], %2, %3, p;\n}\n"
-        ::"r"(d), "r"(a_tmem), "l"(b), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 
 // The same for K-major rows of 64 bytes with 64-byte swizzle (groups of 8 rows 512 bytes apart, layout type 4).
