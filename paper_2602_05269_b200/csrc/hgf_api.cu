@@ -312,17 +312,9 @@ hgf_status hgf::forward_impl(const void *x, int64_t M, const void *packed, float
     gx.gw_over_127 = dp.gw_over_127;
     gx.N = (int)d_out;
     gx.gate_group = gate_group;
-    if (do_prologue && ln) {
-        // the correction path's part of the prologue on the raw tokens (its own quantisation switched off),
-        // then one launch that normalises and quantises
-        if (r) {
-            PrologueParams lora_only = pp;
-            lora_only.xq = nullptr;
-            if (launch_gemm_prologue(lora_only, gx, stream) != cudaSuccess) return HGF_ERR_CUDA;
-        }
-        if (launch_ln_quant(pp, gx, fe, stream) != cudaSuccess) return HGF_ERR_CUDA;
-    } else if (do_prologue && (r ? launch_gemm_prologue(pp, gx, stream) : launch_quant(pp, gx, stream)) != cudaSuccess) {
-        return HGF_ERR_CUDA;
+    if (do_prologue) {
+        const cudaError_t e = ln ? launch_gemm_prologue_ln(pp, gx, fe, stream) : (r ? launch_gemm_prologue(pp, gx, stream) : launch_quant(pp, gx, stream));
+        if (e != cudaSuccess) return HGF_ERR_CUDA;
     }
     if (!do_main) return HGF_OK;
     GemmParams gp = {};

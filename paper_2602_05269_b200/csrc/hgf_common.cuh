@@ -183,9 +183,8 @@ cudaError_t launch_quant(const PrologueParams &p, const GemmPrologueExtra &x, cu
 cudaError_t launch_decode_prologue(const PrologueParams &p, bool pdl, cudaStream_t stream);
 // The same with the LayerNorm front end: the row blocks normalise before they quantise.
 cudaError_t launch_decode_prologue_ln(const PrologueParams &p, const FrontEnd &fe, bool pdl, cudaStream_t stream);
-// GEMM path with the front end: normalise + quantise every token (one block per row); the LoRA part
-// runs in launch_gemm_prologue with p.xq == nullptr (its quantisation switched off).
-cudaError_t launch_ln_quant(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, cudaStream_t stream);
+// GEMM path with the front end: x A on the raw tokens, normalise + quantise.
+cudaError_t launch_gemm_prologue_ln(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, cudaStream_t stream);
 // Group prologue.  A quantisation item is one token row.  A LoRA item is 16 columns of H (rows
 // 16 jt .. 16 jt + 15 of A^T) over one K slice of a problem; its 16 x 16 partial sums of x A go to
 // `hpart` as [8 accumulator registers][32 lanes] floats, and the GEMV adds the slices of a tile in

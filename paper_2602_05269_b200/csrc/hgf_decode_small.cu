@@ -31,36 +31,6 @@ struct SmHead {                // per-token values at the start of shared memory
     float mean[16], rstd[16];
 };
 
-__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory"); }
-__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
-// Stores v at the same shared-memory address of another CTA of the cluster; its bytes count towards that CTA's barrier.
-__device__ __forceinline__ void st_async_f32(uint32_t addr, uint32_t bar, uint32_t rank, float v) {
-    asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
-                 "st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [ra], %3, [rb];\n}\n" ::"r"(addr), "r"(bar), "r"(rank), "f"(v)
-                 : "memory");
-}
-__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
-__device__ __forceinline__ void prefetch_l2(const void *ptr) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(ptr)); }
-__device__ __forceinline__ void announce(uint32_t bar, uint32_t bytes) {
-    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
-}
-// Bulk copy whose bytes were announced to the barrier already.
-__device__ __forceinline__ void bulk_load_announced(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
-    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
-                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
-                 : "memory");
-}
-// The whole block waits (bounded) until the barrier's copies have landed.
-__device__ __forceinline__ bool sm_wait(uint32_t bar, unsigned int *status) {
-    bool got = dmbar_try_wait(bar, 0);
-    if (__all_sync(0xffffffffu, got)) return true;  // the warp goes on together
-    const unsigned long long t0 = dec_timer_ns();
-    for (uint32_t polls = 1; !got && !(got = dmbar_try_wait(bar, 0)); ++polls)
-        if ((polls & 255u) == 0 && dec_timer_ns() - t0 > kDecWaitLimitNs) break;
-    if (!got) atomicExch(status, 0x600u);
-    return __all_sync(0xffffffffu, got);
-}
-
 template <int NT, int NP>
 __global__ void __launch_bounds__(kSmThreads, NT == 1 ? 2 : 1)
 decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *status) {
@@ -145,7 +115,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
     if (r > 0 && warp < nt) load_gates(warp);
     __syncthreads();
     pdl_wait();  // (every thread: what it stores to global memory may belong to earlier work)
-    bool ok = sm_wait(bar_x, status);
+    bool ok = warp_wait(bar_x, status, 0x600u);
 
     // ---- x, in segments of 256 columns of one token (32 units of 16 bytes), dealt to the warps in turn -----------
     // Few segments (one or two tokens): the first eight warps quantise while the others compute x A; else every warp
@@ -246,7 +216,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
     // every CTA of the cluster. ---------------------------------------------------------------------------------
     const int J = jts <= 1 ? 1 : (jts == 2 ? 2 : 4), parts = a_warps / J;
     if (multiplies) {
-        ok = sm_wait(bar_a, status) && ok;
+        ok = warp_wait(bar_a, status, 0x600u) && ok;
         const int jt = a_warp & (J - 1), cw = a_warp / J;
         if (jt < jts) {
             float acc[NT][4];
@@ -308,16 +278,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
                 float xn[8];
                 ln_unit(m, i, u, xn);
                 const float scale = __fdiv_rn(127.0f, gm);
-                uint32_t c[8];
-#pragma unroll
-                for (int k = 0; k < 8; ++k) {
-                    float q = rintf(__fmul_rn(xn[k], scale));
-                    q = fminf(fmaxf(q, -127.0f), 127.0f);
-                    c[k] = (uint32_t)__float2int_rn(q);
-                }
-                o.x = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
-                o.y = __byte_perm(__byte_perm(c[4], c[5], 0x0040), __byte_perm(c[6], c[7], 0x0040), 0x5410);
-                sum = __dp4a((int)o.x, 0x01010101, __dp4a((int)o.y, 0x01010101, 0));
+                o = ln_codes8(xn, scale, sum);
             } else {
                 o = quant8(u, make_quant_scale(gm), sum);
             }
@@ -336,7 +297,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
     __syncthreads();
 
     // ---- the ternary contraction: warp (kw, rw) takes column tiles kw, kw + KS, ... of row tiles rw, rw + RS, ... --
-    ok = sm_wait(bar_w, status) && ok;
+    ok = warp_wait(bar_w, status, 0x600u) && ok;
     {
         const int ks_log2 = steps >= 16 ? 4 : 31 - __clz(steps), KS = 1 << ks_log2, RS = kSmWarps >> ks_log2;
         const int kw = warp & (KS - 1), rw = warp >> ks_log2;
@@ -394,7 +355,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
 
     // ---- H: the cluster's partial sums in rank order, SiLU, fp16 value and fp16 residual ---------------------
     if (r > 0) {
-        ok = sm_wait(bar_h, status) && ok;
+        ok = warp_wait(bar_h, status, 0x600u) && ok;
         const bool no_silu = (P.flags & HGF_FLAG_NO_SILU) != 0;
 #pragma unroll 1
         for (int e = tid; e < E; e += kSmThreads) {

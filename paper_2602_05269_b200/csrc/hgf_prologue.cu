@@ -595,6 +595,7 @@ decode_prologue_group_kernel(const QuantItem *quant_items, int n_quant, const Lo
 }
 
 static cudaLaunchConfig_t prologue_cfg(int blocks, bool pdl, cudaStream_t stream, cudaLaunchAttribute *attr);
+constexpr int kRpSmemLimit = 200 * 1024;
 
 // ---- GEMM-path prologue in one kernel -------------------------------------------------------------
 // Quantisation (Algorithm 1, steps 1-2) and the LoRA down-projection (steps 5-6) of a block of 32
@@ -617,6 +618,24 @@ __host__ __device__ constexpr int fp_smem_bytes(int r) {
                                                                          : kFpWarps * kFpTokens * r * 4;
 }
 
+// The up-projection's operand: row n of B^T times its channel's gate, fp16, padded to 64 columns; piece `idx` is 16 bytes.
+__device__ __forceinline__ void gate_operand(const GemmPrologueExtra &x, int r, int idx) {
+    const int n = idx >> 3, c = idx & 7;
+    if (n >= x.N) return;
+    uint4 v = make_uint4(0u, 0u, 0u, 0u);
+    if (c * 8 < r) {
+        v = *reinterpret_cast<const uint4 *>(x.Bt + (size_t)n * r + c * 8);
+        const float g = x.gate[x.gate_group > 1 ? n / x.gate_group : n];
+        __half2 *h2 = reinterpret_cast<__half2 *>(&v);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const float2 f = __half22float2(h2[k]);
+            h2[k] = __floats2half2_rn(g * f.x, g * f.y);
+        }
+    }
+    *reinterpret_cast<uint4 *>(x.gb16 + (size_t)n * 64 + c * 8) = v;
+}
+
 template <int JT>
 __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x) {
     extern __shared__ __align__(128) uint8_t fp_smem[];
@@ -627,24 +646,9 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
     const int tpb = x.tokens_per_block;  // tokens this launch gives a block (at most kFpTokens)
     const int token_blocks = (p.M + tpb - 1) / tpb;
     if ((int)blockIdx.x >= token_blocks) {
-        // the remaining blocks prepare the up-projection's operand: row n of B^T times its channel's
-        // gate, fp16, padded to 64 columns (one 16-byte piece per thread)
+        // the remaining blocks prepare the up-projection's operand
         if constexpr (JT > 0) {
-            const int idx = ((int)blockIdx.x - token_blocks) * kFpThreads + (int)threadIdx.x, n = idx >> 3, c = idx & 7;
-            if (n < x.N) {
-                uint4 v = make_uint4(0u, 0u, 0u, 0u);
-                if (c * 8 < r) {
-                    v = *reinterpret_cast<const uint4 *>(x.Bt + (size_t)n * r + c * 8);
-                    const float g = x.gate[x.gate_group > 1 ? n / x.gate_group : n];
-                    __half2 *h2 = reinterpret_cast<__half2 *>(&v);
-#pragma unroll
-                    for (int k = 0; k < 4; ++k) {
-                        const float2 f = __half22float2(h2[k]);
-                        h2[k] = __floats2half2_rn(g * f.x, g * f.y);
-                    }
-                }
-                *reinterpret_cast<uint4 *>(x.gb16 + (size_t)n * 64 + c * 8) = v;
-            }
+            gate_operand(x, r, ((int)blockIdx.x - token_blocks) * kFpThreads + (int)threadIdx.x);
         }
         return;
     }
@@ -866,6 +870,344 @@ __global__ void __launch_bounds__(kThreads, 4) round_rows_kernel(const PrologueP
     if (lane == 0 && p.row_sum) p.row_sum[m] = sum;
 }
 
+// ---- GEMM-path prologue for batches that leave the kernel above short of blocks -----------------------
+// A cluster takes 16 tokens and each of its C CTAs a slice of their columns, small enough to stay in shared memory: x is
+// read once, by one bulk copy per row, and statistics, x A and rounding all work from there.  The CTAs exchange
+// partial maxima (with a LayerNorm also sums), partial sums of x A and row sums through distributed shared memory
+// (st.async, counted by the receiver's mbarrier); the 16 / C tokens a CTA owns get their H and scales from it.
+// What it replaces there: a block walked its tokens' columns in a chain of 256-column chunks (a barrier and most of
+// a memory latency each, K / 256 of them, on M / 8 blocks), rounded in a second pass from L2, and a LayerNorm took a
+// launch of its own.
+constexpr int kRpThreads = 256, kRpWarps = kRpThreads / 32, kRpTokens = 16;
+struct RpLayout {
+    int per, pitch;              // columns of a slice (a multiple of 64), bytes per staged row
+    int off_stat, off_amax, off_sum, off_slots, off_part, off_x, smem;
+};
+__host__ __device__ inline RpLayout rp_layout(int K, int r, int log2_c) {
+    const int C = 1 << log2_c;
+    RpLayout L;
+    L.per = ((K / 64 + C - 1) >> log2_c) * 64;
+    L.pitch = 2 * L.per + 64;    // neighbouring rows on different halves of the banks
+    L.off_stat = 64;                                      // [rank][token] double2
+    L.off_amax = L.off_stat + C * kRpTokens * 16;         // [rank][token] patterns
+    L.off_sum = L.off_amax + C * kRpTokens * 4;           // [rank][token] ints
+    L.off_slots = L.off_sum + C * kRpTokens * 4;          // [rank][token][r]
+    L.off_part = L.off_slots + C * kRpTokens * r * 4;     // [warp][token][r]
+    L.off_x = (L.off_part + kRpWarps * kRpTokens * r * 4 + 127) / 128 * 128;
+    L.smem = L.off_x + kRpTokens * L.pitch;
+    return L;
+}
+
+template <int JT, bool LN>
+__global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x, const FrontEnd fe,
+                                                                   const int log2_c, unsigned int *status) {
+    extern __shared__ __align__(128) uint8_t rp_smem[];
+    constexpr int r = 8 * JT;
+    const int C = 1 << log2_c, token_blocks = (p.M + kRpTokens - 1) / kRpTokens;
+    const int cluster = (int)blockIdx.x >> log2_c, rank = (int)blockIdx.x & (C - 1);
+    if (cluster >= token_blocks) {
+        // the remaining blocks prepare the up-projection's operand (see gemm_prologue_kernel)
+        pdl_wait();
+        if constexpr (JT > 0) gate_operand(x, r, ((int)blockIdx.x - token_blocks * C) * kRpThreads + (int)threadIdx.x);
+        return;
+    }
+    const int K = p.K, M = p.M, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const RpLayout L = rp_layout(K, r, log2_c);
+    const int m0 = cluster * kRpTokens, k0 = rank * L.per < K ? rank * L.per : K, cols = K - k0 < L.per ? K - k0 : L.per;
+    const int rows = M - m0 < kRpTokens ? M - m0 : kRpTokens;
+    const uint32_t s0 = dsmem_u32(rp_smem), bar_x = s0, bar_stat = s0 + 8, bar_amax = s0 + 16, bar_h = s0 + 24, bar_sum = s0 + 32;
+    const uint8_t *x_s = rp_smem + L.off_x;
+
+    if (warp == 0) {
+        if (lane == 0) {
+            for (int i = 0; i < 5; ++i) dmbar_init(s0 + 8 * i, 1);
+            asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+            announce(bar_stat, LN ? (uint32_t)(C * kRpTokens * 16) : 0u);
+            announce(bar_amax, (uint32_t)(C * kRpTokens * 4));
+            announce(bar_h, (uint32_t)(kRpTokens * r * 4));      // C ranks x 16 / C tokens
+            announce(bar_sum, (uint32_t)(kRpTokens * 4));
+        }
+        __syncwarp();
+        cluster_arrive_relaxed();
+        pdl_wait();  // x, and the workspace this kernel overwrites, belong to earlier work
+        if (lane == 0) announce(bar_x, (uint32_t)(rows * cols * 2));
+        __syncwarp();
+        if (lane < rows && cols > 0)
+            bulk_load_announced(s0 + L.off_x + lane * L.pitch, p.x + (size_t)(m0 + lane) * K + k0, (uint32_t)(cols * 2), bar_x);
+        __syncwarp();
+    } else {
+        cluster_arrive_relaxed();
+    }
+    // (A^T is not written by pending work) this warp's first chunk of it
+    const int nch = cols >> 5;
+    const __half *arow = JT > 0 ? p.At + (size_t)g * K + k0 + 8 * t : nullptr;
+    uint4 av[JT > 0 ? JT : 1];
+    auto load_a = [&](int c) {
+        if constexpr (JT > 0)
+#pragma unroll
+            for (int jt = 0; jt < JT; ++jt) av[jt] = c < nch ? *reinterpret_cast<const uint4 *>(arow + (size_t)8 * jt * K + 32 * c) : make_uint4(0u, 0u, 0u, 0u);
+    };
+    load_a(warp);
+    __syncthreads();
+    pdl_wait();
+    bool ok = warp_wait(bar_x, status, 0x680u);
+    cluster_wait_acquire();  // every CTA of the cluster has started
+
+    // ---- statistics: warp w works tokens w and w + 8 of the block --------------------------------------------
+    const int nu = cols >> 3;  // 16-byte units of a row's slice
+    auto unit = [&](int ml, int i) { return *reinterpret_cast<const uint4 *>(x_s + ml * L.pitch + 16 * i); };
+    float mean[2] = {0.0f, 0.0f}, rstd[2] = {0.0f, 0.0f};
+    // the normalised values of unit i of both tokens (the weights are read once for the two)
+    auto ln_both = [&](int i, auto &&body) {
+        const float4 *w4 = reinterpret_cast<const float4 *>(fe.ln_w + k0 + 8 * i), *b4 = reinterpret_cast<const float4 *>(fe.ln_b + k0 + 8 * i);
+        const float4 w0 = w4[0], w1 = w4[1], b0 = b4[0], b1 = b4[1];
+        const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            if (warp + kRpWarps * q >= rows) continue;
+            float f[8], xn[8];
+            unpack8(unit(warp + kRpWarps * q, i), f);
+#pragma unroll
+            for (int e = 0; e < 8; ++e) xn[e] = ln_value(f[e], mean[q], rstd[q], w[e], b[e]);
+            body(q, xn);
+        }
+    };
+    if constexpr (LN) {
+        // Mean and variance in one pass, in double, of x - x[0]: see hgf_decode_small.cu.  A bf16 pattern moved to the top
+        // of a double is x 2^-896 (subnormals too), so one fused multiply-add gives x - x[0] without a conversion; infinities and
+        // NaNs, which that would miss, make the sum a NaN.
+        double first[2], sum[2] = {0.0, 0.0}, sum2[2] = {0.0, 0.0};
+        uint32_t top[2] = {0u, 0u};
+#pragma unroll
+        for (int q = 0; q < 2; ++q) first[q] = warp + kRpWarps * q < rows ? (double)__bfloat162float(p.x[(size_t)(m0 + warp + kRpWarps * q) * K]) : 0.0;
+        for (int i = lane; i < nu; i += 32)
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                if (warp + kRpWarps * q >= rows) continue;
+                const uint4 u = unit(warp + kRpWarps * q, i);
+                top[q] = absmax8_bits(top[q], u);
+                const uint32_t w[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+                for (int e = 0; e < 8; ++e) {
+                    const uint32_t hi = (e & 1) ? (w[e >> 1] & 0x80000000u) | ((w[e >> 1] & 0x7fff0000u) >> 3)
+                                                : ((w[e >> 1] & 0x8000u) << 16) | ((w[e >> 1] & 0x7fffu) << 13);
+                    const double d = fma(__hiloint2double((int)hi, 0), 0x1p896, -first[q]);
+                    sum[q] += d;
+                    sum2[q] = fma(d, d, sum2[q]);
+                }
+            }
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int ml = warp + kRpWarps * q;
+            double s = (top[q] & 0xffffu) >= 0x7f80u || top[q] >= 0x7f800000u ? __longlong_as_double(0x7ff8000000000000ll) : sum[q], ss = sum2[q];
+#pragma unroll
+            for (int o = 16; o > 0; o >>= 1) {
+                s += __shfl_xor_sync(0xffffffffu, s, o);
+                ss += __shfl_xor_sync(0xffffffffu, ss, o);
+            }
+            if (lane < C) {
+                const uint32_t dst = s0 + L.off_stat + (rank * kRpTokens + ml) * 16;
+                st_async_b64(dst, bar_stat, (uint32_t)lane, (uint64_t)__double_as_longlong(s));
+                st_async_b64(dst + 8, bar_stat, (uint32_t)lane, (uint64_t)__double_as_longlong(ss));
+            }
+        }
+        ok = warp_wait(bar_stat, status, 0x681u) && ok;
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            const int ml = warp + kRpWarps * q;
+            double s = 0.0, ss = 0.0;
+            for (int k = 0; k < C; ++k) {
+                const double2 v = *reinterpret_cast<const double2 *>(rp_smem + L.off_stat + (k * kRpTokens + ml) * 16);
+                s += v.x;
+                ss += v.y;
+            }
+            const double dm = s / (double)K, v0 = ss / (double)K - dm * dm, var = v0 < 0.0 ? 0.0 : v0;  // (NaN stays NaN)
+            mean[q] = (float)(first[q] + dm);
+            rstd[q] = (float)rsqrt(var + (double)fe.eps);
+        }
+    }
+    uint32_t bits[2] = {0u, 0u};
+    if constexpr (LN) {
+        float a[2] = {0.0f, 0.0f};
+#pragma unroll 2
+        for (int i = lane; i < nu; i += 32)
+            ln_both(i, [&](int q, const float (&xn)[8]) {
+#pragma unroll
+                for (int e = 0; e < 8; ++e) a[q] = fmaxf(a[q], fabsf(xn[e]));
+            });
+#pragma unroll
+        for (int q = 0; q < 2; ++q) bits[q] = __float_as_uint(a[q]);
+    } else {
+        uint32_t acc[2] = {0u, 0u};
+        for (int i = lane; i < nu; i += 32)
+#pragma unroll
+            for (int q = 0; q < 2; ++q)
+                if (warp + kRpWarps * q < rows) acc[q] = absmax8_bits(acc[q], unit(warp + kRpWarps * q, i));
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+            bits[q] = __float_as_uint(absmax_bits_to_float(acc[q]));
+            if (bits[q] > 0x7f800000u) bits[q] = 0u;  // a NaN does not count, as in fmaxf
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        bits[q] = __reduce_max_sync(0xffffffffu, bits[q]);
+        if (lane < C) st_async_f32(s0 + L.off_amax + (rank * kRpTokens + warp + kRpWarps * q) * 4, bar_amax, (uint32_t)lane, __uint_as_float(bits[q]));
+    }
+
+    // ---- x A over the slice, while the maxima travel: tokens are the 16-row operand, 8 columns of H the 8-column operand --
+    if constexpr (JT > 0) {
+        float acc[JT][4];
+#pragma unroll
+        for (int jt = 0; jt < JT; ++jt)
+#pragma unroll
+            for (int c = 0; c < 4; ++c) acc[jt][c] = 0.0f;
+        for (int c = warp; c < nch; c += kRpWarps) {
+            const uint8_t *xr = x_s + g * L.pitch + 64 * c + 16 * t;
+            const uint4 x0 = *reinterpret_cast<const uint4 *>(xr), x1 = *reinterpret_cast<const uint4 *>(xr + 8 * L.pitch);
+            uint4 a_now[JT];
+#pragma unroll
+            for (int jt = 0; jt < JT; ++jt) a_now[jt] = av[jt];
+            load_a(c + kRpWarps);
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                // elements 2 i and 2 i + 1 of this lane's eight take the k slots t and t + 4 of MMA i
+                const uint32_t w0 = (&x0.x)[i], w1 = (&x1.x)[i];
+#pragma unroll
+                for (int jt = 0; jt < JT; ++jt) {
+                    const float2 bf = __half22float2(*reinterpret_cast<const __half2 *>(&(&a_now[jt].x)[i]));
+                    mma_tf32(acc[jt], w0 << 16, w1 << 16, w0 & 0xffff0000u, w1 & 0xffff0000u, __float_as_uint(bf.x), __float_as_uint(bf.y));
+                }
+            }
+        }
+        float *part = reinterpret_cast<float *>(rp_smem + L.off_part) + (size_t)warp * kRpTokens * r;
+#pragma unroll
+        for (int jt = 0; jt < JT; ++jt) {
+            *reinterpret_cast<float2 *>(part + g * r + 8 * jt + 2 * t) = make_float2(acc[jt][0], acc[jt][1]);
+            *reinterpret_cast<float2 *>(part + (g + 8) * r + 8 * jt + 2 * t) = make_float2(acc[jt][2], acc[jt][3]);
+        }
+        __syncthreads();
+        const float *all = reinterpret_cast<const float *>(rp_smem + L.off_part);
+        for (int e = tid; e < kRpTokens * r; e += kRpThreads) {  // to the CTA that owns the token, in warp order
+            float z = 0.0f;
+#pragma unroll
+            for (int w = 0; w < kRpWarps; ++w) z += all[w * kRpTokens * r + e];
+            st_async_f32(s0 + L.off_slots + (rank * kRpTokens * r + e) * 4, bar_h, (uint32_t)((e / r) >> (4 - log2_c)), z);
+        }
+        __syncwarp();
+    }
+
+    // ---- codes ------------------------------------------------------------------------------------------------
+    ok = warp_wait(bar_amax, status, 0x682u) && ok;
+    float gm[2], scale[2];
+    int sums[2] = {0, 0};
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        uint32_t most = 0u;
+        for (int k = 0; k < C; ++k) {
+            const uint32_t v = *reinterpret_cast<const uint32_t *>(rp_smem + L.off_amax + (k * kRpTokens + warp + kRpWarps * q) * 4);
+            most = v > most ? v : most;
+        }
+        gm[q] = fmaxf(__uint_as_float(most), 1e-5f);
+        scale[q] = __fdiv_rn(127.0f, gm[q]);
+    }
+    auto store = [&](int q, int i, const uint2 &o) {
+        const size_t at = ((size_t)(m0 + warp + kRpWarps * q) * K + k0) / 8 + i;
+        reinterpret_cast<uint2 *>(p.xq)[at] = o;
+        if (p.dbg_xq) reinterpret_cast<uint2 *>(p.dbg_xq)[at] = o;
+    };
+    if (ok) {
+        if constexpr (LN) {
+#pragma unroll 2
+            for (int i = lane; i < nu; i += 32) ln_both(i, [&](int q, const float (&xn)[8]) { store(q, i, ln_codes8(xn, scale[q], sums[q])); });
+        } else {
+            const QuantScale qs[2] = {make_quant_scale(gm[0]), make_quant_scale(gm[1])};
+            for (int i = lane; i < nu; i += 32)
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    if (warp + kRpWarps * q < rows) store(q, i, quant8(unit(warp + kRpWarps * q, i), qs[q], sums[q]));
+        }
+    }
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+        const int ml = warp + kRpWarps * q;
+        int sum = sums[q];
+        sum = __reduce_add_sync(0xffffffffu, sum);
+        if (lane == 0)
+            st_async_f32(s0 + L.off_sum + (rank * kRpTokens + ml) * 4, bar_sum, (uint32_t)(ml >> (4 - log2_c)), __int_as_float(sum));
+        // (the CTA that owns the token writes its values)
+        if (lane == 0 && (ml >> (4 - log2_c)) == rank && ml < rows && ok) {
+            const int m = m0 + ml;
+            p.gamma_x[m] = gm[q];
+            if (x.tok_sc) x.tok_sc[m] = gm[q] * x.gw_over_127;
+            if (p.dbg_gamma_x) p.dbg_gamma_x[m] = gm[q];
+            if constexpr (LN) {
+                if (fe.dbg_mean) fe.dbg_mean[m] = mean[q];
+                if (fe.dbg_rstd) fe.dbg_rstd[m] = rstd[q];
+            }
+        }
+    }
+    pdl_launch_dependents();  // late: see gemm_prologue_kernel
+
+    const int own = kRpTokens >> log2_c, t0 = rank * own;  // this CTA's tokens of the block
+    if constexpr (JT > 0) {
+        ok = warp_wait(bar_h, status, 0x683u) && ok;
+        const float *slots = reinterpret_cast<const float *>(rp_smem + L.off_slots);
+        for (int e = tid; e < own * 64; e += kRpThreads) {
+            const int ml = t0 + (e >> 6), j = e & 63, m = m0 + ml;
+            float h = 0.0f;
+            if (j < r) {
+                float z = 0.0f;
+                for (int k = 0; k < C; ++k) z += slots[(k * kRpTokens + ml) * r + j];
+                h = (p.flags & HGF_FLAG_NO_SILU) ? z : silu_f(z);
+            }
+            if (ml < rows && ok) {
+                if (j < r) {
+                    p.h[(size_t)m * r + j] = h;
+                    if (p.dbg_h) p.dbg_h[(size_t)m * r + j] = h;
+                }
+                if (p.h16) p.h16[(size_t)m * 64 + j] = __float2half_rn(h);  // (zeros past r)
+            }
+        }
+    }
+    ok = warp_wait(bar_sum, status, 0x684u) && ok;
+    if (tid < own && t0 + tid < rows && ok && p.row_sum) {
+        int sum = 0;
+        for (int k = 0; k < C; ++k) sum += *reinterpret_cast<const int *>(rp_smem + L.off_sum + (k * kRpTokens + t0 + tid) * 4);
+        p.row_sum[m0 + t0 + tid] = sum;
+    }
+    if (!ok)  // bounded drain of what is still on its way into this CTA's memory
+        for (uint32_t i = 0; i < (1u << 16); ++i) {
+            bool all = true;
+            for (int b = 0; b < 5; ++b) all = all && dmbar_try_wait(s0 + 8 * b, 0);
+            if (all) break;
+        }
+}
+
+// Where it is used, and the cluster size: see launch_rows_prologue.
+template <int JT, bool LN>
+static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, int log2_c, cudaStream_t stream) {
+    static std::atomic<unsigned long long> attr_done{0};
+    const RpLayout L = rp_layout(p.K, p.r, log2_c);
+    cudaError_t e = ensure_dynamic_smem(rows_prologue_kernel<JT, LN>, kRpSmemLimit, attr_done);
+    if (e != cudaSuccess) return e;
+    unsigned int *status = device_status_word();
+    if (!status) return cudaErrorMemoryAllocation;
+    const int C = 1 << log2_c, gate_blocks = (p.r > 0 && x.gb16) ? (x.N * 8 + kRpThreads - 1) / kRpThreads : 0;
+    cudaLaunchAttribute attr[2];
+    cudaLaunchConfig_t cfg = prologue_cfg(((p.M + kRpTokens - 1) / kRpTokens) * C + (gate_blocks + C - 1) / C * C, !(p.flags & HGF_FLAG_NO_PDL), stream, attr);
+    cfg.blockDim = dim3(kRpThreads);
+    cfg.dynamicSmemBytes = (size_t)L.smem;
+    attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    attr[cfg.numAttrs].val.clusterDim.x = (unsigned)C;
+    attr[cfg.numAttrs].val.clusterDim.y = 1;
+    attr[cfg.numAttrs].val.clusterDim.z = 1;
+    ++cfg.numAttrs;
+    e = cudaLaunchKernelEx(&cfg, rows_prologue_kernel<JT, LN>, p, x, fe, log2_c, status);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+
 template <int JT>
 static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPrologueExtra &x, int blocks, cudaStream_t stream) {
     // Never more than two blocks per SM (the launcher spreads the rows over twice the SM count of
@@ -885,8 +1227,42 @@ static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPr
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
+// The cluster form above where it is the better one; cudaErrorNotSupported where it is not.  Microseconds of the whole layer
+// call in a captured chain, the other kernels / this one:
+//  - 2048 -> 2048, r = 32: 16.0 / 12.4 at M = 17, 18.4 / 14.8 at M = 512, 25.9 / 24.7 at M = 2000, 38.0 / 40.0 at 4096 (its slices
+//    then come in several waves and read A^T more often than 32-token blocks do); K = 512: 9.2 / 9.5 at M = 17;
+//  - 5632 -> 2048: 29.6 / 19.1 at M = 17, 34.5 / 23.1 at M = 512; 11008 -> 4096, r = 64: 69 / 32 at M = 17, 94 / 82 at M = 1024,
+//    133 / 142 at M = 2000 (eight CTAs a cluster for its size alone: above four CTAs an SM it is left);
+//  - with a LayerNorm, 2048 -> 2048: 23.8 / 14.3 at M = 64, 51.2 / 52.2 at M = 4096; without a correction, 4096 -> 1024:
+//    14.0 / 16.7 at M = 17, 25.2 / 16.7 at M = 64, 82.6 / 62.4 at M = 4096.
+// Cluster size: CTAs for every SM, two of them on one if they fit.
+static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd *fe, cudaStream_t stream) {
+    const int sms = device_sm_count();
+    if (!sms) return cudaErrorInvalidDevice;
+    const int blocks = (p.M + kRpTokens - 1) / kRpTokens;
+    int c = 0;
+    while (c < 3 && (blocks << c) < sms) ++c;
+    while (c < 3 && rp_layout(p.K, p.r, c).smem > 110 * 1024) ++c;  // two CTAs on an SM
+    if (rp_layout(p.K, p.r, c).smem > kRpSmemLimit) return cudaErrorNotSupported;
+    const bool few = p.M <= 2048 && p.K >= 1024 && (fe || (blocks << c) <= 4 * sms);
+    if (!(p.r > 0 ? few : p.M >= 64)) return cudaErrorNotSupported;
+    const FrontEnd none = {};
+    switch (p.r) {
+        case 0: return fe ? launch_rows_prologue_jt<0, true>(p, x, *fe, c, stream) : cudaErrorNotSupported;
+        case 16: return fe ? launch_rows_prologue_jt<2, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<2, false>(p, x, none, c, stream);
+        case 32: return fe ? launch_rows_prologue_jt<4, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<4, false>(p, x, none, c, stream);
+        case 48: return fe ? launch_rows_prologue_jt<6, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<6, false>(p, x, none, c, stream);
+        case 64: return fe ? launch_rows_prologue_jt<8, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<8, false>(p, x, none, c, stream);
+        default: return cudaErrorInvalidValue;
+    }
+}
+
 // Quantisation and (r > 0) LoRA down-projection of the GEMM path, plus gate * B^T for its epilogue.
 cudaError_t launch_gemm_prologue(const PrologueParams &p, const GemmPrologueExtra &x, cudaStream_t stream) {
+    if (p.xq && p.r > 0) {
+        const cudaError_t e = launch_rows_prologue(p, x, nullptr, stream);
+        if (e != cudaErrorNotSupported) return e;
+    }
     // Tokens per block: as many blocks as are resident at once share the rows evenly; beyond that a
     // block takes its full 32.
     const int sm_count = device_sm_count();
@@ -976,7 +1352,15 @@ cudaError_t launch_decode_prologue_ln(const PrologueParams &p, const FrontEnd &f
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_ln_quant(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, cudaStream_t stream) {
+cudaError_t launch_gemm_prologue_ln(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, cudaStream_t stream) {
+    const cudaError_t whole = launch_rows_prologue(p, x, &fe, stream);
+    if (whole != cudaErrorNotSupported) return whole;
+    if (p.r) {  // the correction path's part on the raw tokens, its own quantisation switched off
+        PrologueParams lora_only = p;
+        lora_only.xq = nullptr;
+        const cudaError_t e = launch_gemm_prologue(lora_only, x, stream);
+        if (e != cudaSuccess) return e;
+    }
     cudaLaunchAttribute attr[1];
     const bool by_warp = p.row_sum != nullptr && p.M >= 64;  // many rows: one warp each; few: one block each
     cudaLaunchConfig_t cfg = prologue_cfg(by_warp ? (p.M + kWarps - 1) / kWarps : p.M, !(p.flags & HGF_FLAG_NO_PDL), stream, attr);

@@ -118,6 +118,25 @@ __device__ __forceinline__ void unpack8(const uint4 &v, float (&f)[8]) {
     for (int e = 0; e < 8; ++e) f[e] = (e & 1) ? bf16hi_to_float(w[e >> 1]) : bf16lo_to_float(w[e >> 1]);
 }
 
+// Codes of eight normalised values, rint(xn * scale) clipped to +-127, as eight int8; their sum is added to `sum`.
+__device__ __forceinline__ uint2 ln_codes8(const float (&xn)[8], float scale, int &sum) {
+    uint32_t c[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) {
+        float q = rintf(__fmul_rn(xn[e], scale));
+        q = fminf(fmaxf(q, -127.0f), 127.0f);
+        c[e] = (uint32_t)__float2int_rn(q);
+    }
+    uint32_t o[2];
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        const uint32_t p01 = __byte_perm(c[4 * h], c[4 * h + 1], 0x0040), p23 = __byte_perm(c[4 * h + 2], c[4 * h + 3], 0x0040);
+        o[h] = __byte_perm(p01, p23, 0x5410);
+        sum = __dp4a((int)o[h], 0x01010101, sum);
+    }
+    return make_uint2(o[0], o[1]);
+}
+
 // ---- PTX wrappers -------------------------------------------------------------------------------
 __device__ __forceinline__ uint32_t dsmem_u32(const void *p) { return (uint32_t)__cvta_generic_to_shared(p); }
 
@@ -175,5 +194,41 @@ __device__ __forceinline__ unsigned long long dec_timer_ns() {
 // Programmatic dependent launch: both are no-ops when the launch carries no such attribute.
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory"); }
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\n" ::: "memory"); }
+
+// ---- clusters, distributed shared memory ------------------------------------------------------------
+__device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
+// Stores v at the same shared-memory address of another CTA of the cluster; its bytes count towards that CTA's barrier.
+__device__ __forceinline__ void st_async_f32(uint32_t addr, uint32_t bar, uint32_t rank, float v) {
+    asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
+                 "st.async.shared::cluster.mbarrier::complete_tx::bytes.f32 [ra], %3, [rb];\n}\n" ::"r"(addr), "r"(bar), "r"(rank), "f"(v)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async_b64(uint32_t addr, uint32_t bar, uint32_t rank, uint64_t v) {
+    asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
+                 "st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [ra], %3, [rb];\n}\n" ::"r"(addr), "r"(bar), "r"(rank), "l"(v)
+                 : "memory");
+}
+__device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }
+__device__ __forceinline__ void prefetch_l2(const void *ptr) { asm volatile("prefetch.global.L2 [%0];\n" ::"l"(ptr)); }
+__device__ __forceinline__ void announce(uint32_t bar, uint32_t bytes) {
+    asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;\n" ::"r"(bar), "r"(bytes) : "memory");
+}
+// Bulk copy whose bytes were announced to the barrier already.
+__device__ __forceinline__ void bulk_load_announced(uint32_t dst, const void *src, uint32_t bytes, uint32_t bar) {
+    asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];\n"
+                 ::"r"(dst), "l"(src), "r"(bytes), "r"(bar)
+                 : "memory");
+}
+// A warp waits (bounded) until the barrier's first phase is complete.
+__device__ __forceinline__ bool warp_wait(uint32_t bar, unsigned int *status, unsigned int code) {
+    bool got = dmbar_try_wait(bar, 0);
+    if (__all_sync(0xffffffffu, got)) return true;  // the warp goes on together
+    const unsigned long long t0 = dec_timer_ns();
+    for (uint32_t polls = 1; !got && !(got = dmbar_try_wait(bar, 0)); ++polls)
+        if ((polls & 255u) == 0 && dec_timer_ns() - t0 > kDecWaitLimitNs) break;
+    if (!got) atomicExch(status, code);
+    return __all_sync(0xffffffffu, got);
+}
 
 }  // namespace hgf
