@@ -272,6 +272,7 @@ struct GemmParams {
     float gw_over_127;
     int M, K, N, r;
     uint32_t flags;
+    int split_log2;          // (set by the launcher) CTAs a tile's K is divided over, as a power of two
 };
 cudaError_t launch_prefill_gemm(const GemmParams &p, cudaStream_t stream);
 cudaError_t launch_wait_timeout_selftest(unsigned long long limit_ns, cudaStream_t stream);

@@ -35,6 +35,7 @@
 // roles leave their loops, in-flight bulk copies are drained, tensor memory is freed and the
 // kernel returns.
 #include "hgf_tc.cuh"
+#include "hgf_warp.cuh"
 
 namespace hgf {
 
@@ -72,7 +73,7 @@ struct Cfg {
                          BAR_ACCFULL = BAR_PEMPTY + PSTAGES,
                          BAR_ACCEMPTY = BAR_ACCFULL + 2, BAR_LORAREADY = BAR_ACCEMPTY + 2, BAR_LORADONE = BAR_LORAREADY + 2,
                          BAR_OPSFULL = BAR_LORADONE + 2, BAR_OPSEMPTY = BAR_OPSFULL + 2, 
-                         BAR_COUNT = BAR_OPSEMPTY + 2;
+                         BAR_SPLIT = BAR_OPSEMPTY + 2, BAR_COUNT = BAR_SPLIT + 1;
     static_assert(SMEM_BYTES <= 227 * 1024, "shared memory budget");
     static_assert(BAR_COUNT * 8 + 16 <= 512, "barrier block too small");
     static_assert(A_COL + NS * A_STAGE_COLS <= TMEM_COLS, "tensor memory budget");
@@ -85,7 +86,11 @@ constexpr uint32_t IDESC_I8 = (2u << 4) /*s32*/ | (1u << 7) /*A s8*/ | (1u << 10
 constexpr uint32_t IDESC_F16 = (1u << 4) /*f32*/ | (0u << 7) /*A f16*/ | (0u << 10) /*B f16*/ |
                                ((uint32_t)(TILE_T >> 3) << 17) | ((uint32_t)(TILE_C >> 4) << 24);
 
-template <bool OUT_BF16, int NS, int OPSB>
+// SPLIT: a layer with fewer tiles than half the SMs has each tile's K divided over a cluster of 2, 4 or 8 CTAs (one tile a
+// cluster, the tile loops below run once).  The CTAs keep their int32 sums in tensor memory, hand each other
+// the token chunks the others own through distributed shared memory (st.async into the spent operand ring, counted
+// by the receiver's mbarrier), and each finishes its own 128 / S tokens; the sums are exact in any order.
+template <bool OUT_BF16, int NS, int OPSB, bool SPLIT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_h,
                     const __grid_constant__ CUtensorMap tmap_gb, const __grid_constant__ CUtensorMap tmap_y,
@@ -104,9 +109,12 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     // for this grid's completion before it touches memory)
     asm volatile("griddepcontrol.launch_dependents;\n" ::: "memory");
     const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
+    const int S = SPLIT ? 1 << p.split_log2 : 1, rank = SPLIT ? (int)blockIdx.x & (S - 1) : 0;
+    const int tile_first = SPLIT ? (int)blockIdx.x >> p.split_log2 : (int)blockIdx.x, tile_step = SPLIT ? (int)gridDim.x >> p.split_log2 : (int)gridDim.x;
+    bool arrived = false, waited = false;  // (SPLIT) the cluster barrier that frees the operand rings
     const int tiles_t = (p.M + TILE_T - 1) / TILE_T, tiles_c = (p.N + TILE_C - 1) / TILE_C;
     const int num_tiles = tiles_t * tiles_c;
-    const int kblocks = (p.K + KBLK - 1) / KBLK;
+    const int kblocks = (p.K + KBLK - 1) / KBLK, kb0 = SPLIT ? rank * kblocks / S : 0, kb1 = SPLIT ? (rank + 1) * kblocks / S : kblocks;
     const bool has_lora = p.r > 0;
 
     if (tid == 0) {
@@ -133,6 +141,10 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             mbar_init(bar(C::BAR_LORADONE + b), 1);
             mbar_init(bar(C::BAR_OPSFULL + b), 1);
             mbar_init(bar(C::BAR_OPSEMPTY + b), 8);
+        }
+        if (SPLIT) {
+            mbar_init(bar(C::BAR_SPLIT), 1);
+            mbar_arrive_expect_tx(bar(C::BAR_SPLIT), (uint32_t)((S - 1) * (8 / S) * TILE_C * 16 * 4));
         }
         *abort_flag = 0;
         asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
@@ -163,7 +175,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             uint32_t issued[C::STAGES] = {}, ops_issued[2] = {};
             int pit = 0;
             bool ok = true;
-            for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+            for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
                 const int t0 = (tile % tiles_t) * TILE_T, c0 = (tile / tiles_t) * TILE_C;
                 {
                     // what the tile's epilogue needs, into the buffer of the tile's accumulator: row sums and
@@ -183,7 +195,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     ++ops_issued[b];
                     ++pit;
                 }
-                for (int kb = 0; kb < kblocks; ++kb) {
+                for (int kb = kb0; kb < kb1; ++kb) {
                     ok = mbar_wait(bar(C::BAR_EMPTY + s), ph ^ 1u, abort_flag, status, 0x100u + s);
                     if (!(ok = __all_sync(0xffffffffu, ok))) break;
                     if (lane == 0) {
@@ -238,11 +250,11 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     warp_mma_f16(tmem_base + b * ACC_COLS, adesc + 2u * kk, bdesc + 2u * kk, IDESC_F16, 1u);
                 warp_commit(bar(C::BAR_LORADONE + b));
             };
-            for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++it) {
+            for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++it) {
                 const int b = it & 1;
                 const uint32_t acc = tmem_base + b * ACC_COLS;
                 if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x200u))) break;
-                for (int kb = 0; kb < kblocks; ++kb, ++gs) {
+                for (int kb = kb0; kb < kb1; ++kb, ++gs) {
                     if (pend >= 0 && __all_sync(0xffffffffu, mbar_test_wait(bar(C::BAR_LORAREADY + (pend & 1)), (uint32_t)(pend >> 1) & 1u))) {
                         issue_lora(pend);
                         pend = -1;
@@ -253,7 +265,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     tc_fence_after();
                     const uint64_t bdesc = xdesc0 + (uint64_t)(s * (X_TILE_BYTES >> 4));
                     const uint32_t a_tmem = tmem_base + A_COL + s * A_STAGE_COLS;
-                    warp_mma_i8_ts(acc, a_tmem, bdesc, IDESC_I8, kb ? 1u : 0u);
+                    warp_mma_i8_ts(acc, a_tmem, bdesc, IDESC_I8, kb > kb0 ? 1u : 0u);
                     warp_mma_i8_ts(acc, a_tmem + 8u, bdesc + 2u, IDESC_I8, 1u);
                     warp_mma_i8_ts(acc, a_tmem + 16u, bdesc + 4u, IDESC_I8, 1u);
                     warp_mma_i8_ts(acc, a_tmem + 24u, bdesc + 6u, IDESC_I8, 1u);
@@ -265,6 +277,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 }
                 if (!ok) break;
                 warp_commit(bar(C::BAR_ACCFULL + b));
+                if (SPLIT) { cluster_arrive_release(); arrived = true; }
                 if (pend >= 0) {  // the previous tile's correction has to be out before its accumulator's next turn
                     if (!(ok = wait(C::BAR_LORAREADY + (pend & 1), (uint32_t)(pend >> 1) & 1u, 0x230u)))
                         break;
@@ -287,7 +300,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         uint8_t *buf = smem + C::OFF_ST + (4 * e2 + q) * STORE_BUF_BYTES;
         bool ok = true;
         int it = 0;
-        for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x, ++it) {
+        for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++it) {
             const int t0 = (tile % tiles_t) * TILE_T, c0 = (tile / tiles_t) * TILE_C;
             const int b = it & 1;
             const uint32_t par = (uint32_t)(it >> 1) & 1u;
@@ -325,6 +338,72 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     ai[4 * v + 3] = __float_as_uint((float)((int)ai[4 * v + 3] - rs4.w) * sc4.w);
                 }
             };
+            if constexpr (SPLIT) {
+                // chunks of 16 tokens: chunk c belongs to CTA c / (8 / S); this warp works those of its parity
+                cluster_arrive_release();
+                arrived = waited = true;
+                cluster_wait_acquire();  // every CTA's MMAs are complete: the operand rings are free
+                const int per = 8 / S;
+                for (int c = e2; c < 8; c += 2) {
+                    const int owner = c / per;
+                    if (owner == rank) continue;
+                    uint32_t ai[16];
+                    tmem_ld16(lane_base + 16 * c, ai);
+                    tmem_ld_wait();
+                    const uint32_t dst = sbase + C::OFF_X + ((rank * per + c % per) * 4 + q) * 2048 + 16 * lane;
+#pragma unroll
+                    for (int v = 0; v < 4; ++v)
+                        st_async_v4(dst + 512 * v, bar(C::BAR_SPLIT), (uint32_t)owner, ai[4 * v], ai[4 * v + 1], ai[4 * v + 2], ai[4 * v + 3]);
+                }
+                ok = mbar_wait_poll(bar(C::BAR_SPLIT), 0u, abort_flag, status, 0x330u);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                for (int c = rank * per; c < (rank + 1) * per; ++c) {
+                    if ((c & 1) != e2) continue;
+                    uint32_t ai[16];
+                    tmem_ld16(lane_base + 16 * c, ai);
+                    tmem_ld_wait();
+                    for (int o = 0; o < S; ++o) {
+                        if (o == rank) continue;
+                        const uint8_t *src = smem + C::OFF_X + ((o * per + c % per) * 4 + q) * 2048 + 16 * lane;
+#pragma unroll
+                        for (int v = 0; v < 4; ++v) {
+                            const uint4 a = *reinterpret_cast<const uint4 *>(src + 512 * v);
+                            ai[4 * v] += a.x; ai[4 * v + 1] += a.y; ai[4 * v + 2] += a.z; ai[4 * v + 3] += a.w;
+                        }
+                    }
+                    dequant_chunk(16 * c, ai);
+                    tmem_st16(lane_base + 16 * c, ai);
+                }
+                tmem_st_wait();
+                if (has_lora) {
+                    tc_fence_before();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar(C::BAR_LORAREADY + b));
+                    ok = mbar_wait_poll(bar(C::BAR_LORADONE + b), par, abort_flag, status, 0x310u);
+                    if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                    tc_fence_after();
+                }
+                for (int c = rank * per; c < (rank + 1) * per; ++c) {
+                    if ((c & 1) != e2) continue;
+                    uint32_t ai[16];
+                    tmem_ld16(lane_base + 16 * c, ai);
+                    tmem_ld_wait();
+                    if (lane == 0) bulk_wait_read<0>();
+                    __syncwarp();
+#pragma unroll
+                    for (int j = 0; j < 16; ++j) {
+                        if (OUT_BF16) reinterpret_cast<__nv_bfloat16 *>(buf)[j * 32 + lane] = __float2bfloat16_rn(__uint_as_float(ai[j]));
+                        else reinterpret_cast<uint32_t *>(buf)[j * 32 + lane] = ai[j];
+                    }
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) {
+                        tma_store_2d(&tmap_y, c0 + 32 * q, t0 + 16 * c, smem_u32(buf));
+                        bulk_commit();
+                    }
+                }
+                break;  // one tile a cluster
+            }
             if (has_lora) {
                 // first pass: dequantise in place (int32 -> fp32), then let the MMA warp add the correction
                 for (int cc = HALF_T * e2; cc < HALF_T * (e2 + 1); cc += 32) {
@@ -389,11 +468,11 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         uint32_t pissued[C::PSTAGES] = {};
         bool ok = true;
         const int steps = (p.K + 255) >> 8, n_row_tiles = (p.N + 15) >> 4;
-        for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
+        for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
             const int rt0 = ((tile / tiles_t) * TILE_C) >> 4;
             const int nrt = n_row_tiles - rt0 < TILE_C / 16 ? n_row_tiles - rt0 : TILE_C / 16;
             const uint8_t *psrc = p.packed + (size_t)(rt0 + (lane < nrt ? lane : 0)) * steps * 1024;
-            for (int kb = 0; kb < kblocks; ++kb) {
+            for (int kb = kb0; kb < kb1; ++kb) {
                 ok = mbar_wait(bar(C::BAR_PEMPTY + pj), pph ^ 1u, abort_flag, status, 0x110u + pj);
                 if (!(ok = __all_sync(0xffffffffu, ok))) break;
                 if (lane == 0) mbar_arrive_expect_tx(bar(C::BAR_PFULL + pj), (uint32_t)nrt * 1024u);
@@ -416,8 +495,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         int s = 0, pj = 0;
         uint32_t ph = 0, pph = 0;
         bool ok = true;
-        for (int tile = blockIdx.x; ok && tile < num_tiles; tile += gridDim.x) {
-            for (int kb = 0; kb < kblocks; ++kb) {
+        for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
+            for (int kb = kb0; kb < kb1; ++kb) {
                 // the stage's packed codes have landed, and the MMAs that read this stage's previous operand
                 // are complete
                 ok = mbar_wait(bar(C::BAR_PFULL + pj), pph, abort_flag, status, 0x400u + pj) &&
@@ -452,6 +531,14 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         }
     }
 
+    if constexpr (SPLIT) {
+        // every thread arrives once, whatever happened above; then no CTA leaves while another may still write into it
+        __syncwarp();
+        if (!arrived) cluster_arrive_release();
+        if (!waited) cluster_wait_acquire();
+        cluster_arrive_release();
+        cluster_wait_acquire();
+    }
     tc_fence_before();
     __syncthreads();
     if (warp == 1) {
@@ -484,13 +571,13 @@ cudaError_t launch_wait_timeout_selftest(unsigned long long limit_ns, cudaStream
 }
 
 // ---- host side: tensor maps and launch -----------------------------------------------------------
-template <bool OUT_BF16, int NS, int OPSB>
-static cudaError_t launch_variant(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my,
+template <bool OUT_BF16, int NS, int OPSB, bool SPLIT>
+static cudaError_t launch_split(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my,
                                   const GemmParams &p, int grid, unsigned int *status, cudaStream_t stream) {
     static std::atomic<unsigned long long> attr_done{0};
     constexpr int smem = Cfg<NS, OPSB>::SMEM_BYTES;
     {
-        cudaError_t e = ensure_dynamic_smem(prefill_gemm_kernel<OUT_BF16, NS, OPSB>, smem, attr_done);
+        cudaError_t e = ensure_dynamic_smem(prefill_gemm_kernel<OUT_BF16, NS, OPSB, SPLIT>, smem, attr_done);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchConfig_t cfg = {};
@@ -498,20 +585,47 @@ static cudaError_t launch_variant(const CUtensorMap &mx, const CUtensorMap &mh, 
     cfg.blockDim = dim3(GEMM_THREADS);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
-    cudaLaunchAttribute attr[1];
+    cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = (p.flags & HGF_FLAG_NO_PDL) ? 0 : 1;  // set-up (barriers, tensor memory) may overlap the prologue's tail
-    cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<OUT_BF16, NS, OPSB>, mx, mh, mgb, my, p, status);
+    if (SPLIT) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = 1u << p.split_log2;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs].val.clusterDim.z = 1;
+        ++cfg.numAttrs;
+    }
+    cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<OUT_BF16, NS, OPSB, SPLIT>, mx, mh, mgb, my, p, status);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_prefill_gemm(const GemmParams &p, cudaStream_t stream) {
+template <bool OUT_BF16, int NS, int OPSB>
+static cudaError_t launch_variant(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my,
+                                  const GemmParams &p, int grid, unsigned int *status, cudaStream_t stream) {
+    return p.split_log2 ? launch_split<OUT_BF16, NS, OPSB, true>(mx, mh, mgb, my, p, grid, status, stream)
+                        : launch_split<OUT_BF16, NS, OPSB, false>(mx, mh, mgb, my, p, grid, status, stream);
+}
+
+cudaError_t launch_prefill_gemm(const GemmParams &p_in, cudaStream_t stream) {
+    GemmParams p = p_in;
     const int sm_count = device_sm_count();
     if (!sm_count) return cudaErrorInvalidDevice;
     const bool bf16 = (p.flags & HGF_FLAG_OUT_BF16) != 0;
     const bool narrow = p.r <= 32;  // 64-byte operand rows for the correction, and room for a fourth stage
+    const int tiles = ((p.M + TILE_T - 1) / TILE_T) * ((p.N + TILE_C - 1) / TILE_C), kblocks = (p.K + KBLK - 1) / KBLK;
+    // K divided over a cluster where tiles leave SMs idle and K is long (at least 16 blocks of 256, four a CTA).  Microseconds of the
+    // layer call in a captured chain, whole / over 2 / 4 / 8 CTAs: 5632 -> 2048 23.1 / 20.3 at M = 512 (64 tiles), 18.9 / 16.1 /
+    // 14.4 at M = 64 (16 tiles); 11008 -> 1024 35.6 / 28.8 / 24.6 / 23.1 at M = 17 (8 tiles); 2048 -> 2048 12.0 / 11.7 / 11.3 at M = 64,
+    // 15.6 / 15.3 / 17.5 at M = 256.  Clusters of four or eight do not fill the chip (an SM count that is no multiple of their
+    // size in every part of it: 128 CTAs by eights took two rounds, 22.2 for 14.4), so they stop at half of it, except fours
+    // with a very long K: 11008 -> 4096 32.6 / 28.6 / 25.8 at M = 128 (32 tiles).
+    auto may_split = [&](int log2) {
+        return kblocks >= (log2 == 1 ? 16 : 4 << log2) && (tiles << log2) <= (log2 == 1 || (log2 == 2 && kblocks >= 32) ? sm_count : sm_count / 2);
+    };
+    for (int log2 = 1; log2 <= 3; ++log2)
+        if (may_split(log2)) p.split_log2 = log2;
     CUtensorMap mx, mh, mgb, my;
     if (!make_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.xq, (uint64_t)p.K, (uint64_t)p.M, (uint64_t)p.K, 128, TILE_T,
                      CU_TENSOR_MAP_SWIZZLE_128B))
@@ -526,10 +640,9 @@ cudaError_t launch_prefill_gemm(const GemmParams &p, cudaStream_t stream) {
         mgb = mx;
     }
     if (!make_map_2d(&my, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, p.y, (uint64_t)p.N,
-                     (uint64_t)p.M, (uint64_t)p.N * (bf16 ? 2 : 4), 32, bf16 ? 32 : 16, CU_TENSOR_MAP_SWIZZLE_NONE))
+                     (uint64_t)p.M, (uint64_t)p.N * (bf16 ? 2 : 4), 32, bf16 && !p.split_log2 ? 32 : 16, CU_TENSOR_MAP_SWIZZLE_NONE))
         return cudaErrorInvalidValue;
-    const int tiles = ((p.M + TILE_T - 1) / TILE_T) * ((p.N + TILE_C - 1) / TILE_C);
-    const int grid = tiles < sm_count ? tiles : sm_count;
+    const int grid = p.split_log2 ? tiles << p.split_log2 : (tiles < sm_count ? tiles : sm_count);
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
     cudaError_t e;

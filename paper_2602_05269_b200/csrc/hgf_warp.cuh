@@ -197,6 +197,7 @@ __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;\
 
 // ---- clusters, distributed shared memory ------------------------------------------------------------
 __device__ __forceinline__ void cluster_arrive_relaxed() { asm volatile("barrier.cluster.arrive.relaxed.aligned;\n" ::: "memory"); }
+__device__ __forceinline__ void cluster_arrive_release() { asm volatile("barrier.cluster.arrive.release.aligned;\n" ::: "memory"); }
 __device__ __forceinline__ void cluster_wait_acquire() { asm volatile("barrier.cluster.wait.acquire.aligned;\n" ::: "memory"); }
 // Stores v at the same shared-memory address of another CTA of the cluster; its bytes count towards that CTA's barrier.
 __device__ __forceinline__ void st_async_f32(uint32_t addr, uint32_t bar, uint32_t rank, float v) {
@@ -207,6 +208,12 @@ __device__ __forceinline__ void st_async_f32(uint32_t addr, uint32_t bar, uint32
 __device__ __forceinline__ void st_async_b64(uint32_t addr, uint32_t bar, uint32_t rank, uint64_t v) {
     asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
                  "st.async.shared::cluster.mbarrier::complete_tx::bytes.b64 [ra], %3, [rb];\n}\n" ::"r"(addr), "r"(bar), "r"(rank), "l"(v)
+                 : "memory");
+}
+__device__ __forceinline__ void st_async_v4(uint32_t addr, uint32_t bar, uint32_t rank, uint32_t a, uint32_t b, uint32_t c, uint32_t d) {
+    asm volatile("{\n.reg .b32 ra, rb;\nmapa.shared::cluster.u32 ra, %0, %2;\nmapa.shared::cluster.u32 rb, %1, %2;\n"
+                 "st.async.shared::cluster.mbarrier::complete_tx::bytes.v4.b32 [ra], {%3, %4, %5, %6}, [rb];\n}\n"
+                 ::"r"(addr), "r"(bar), "r"(rank), "r"(a), "r"(b), "r"(c), "r"(d)
                  : "memory");
 }
 __device__ __forceinline__ void bar_sync(int id, int threads) { asm volatile("bar.sync %0, %1;\n" ::"r"(id), "r"(threads) : "memory"); }

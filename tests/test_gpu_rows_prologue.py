@@ -50,3 +50,28 @@ def test_rows_prologue(M, K, r, ln):
     if r:
         assert np.abs(dbg["h"].cpu().numpy() - ref["h"]).max() <= 1e-5 * np.abs(ref["h"]).max()
     assert np.abs(y.cpu().numpy() - ref["y"]).max() <= 6e-4 * np.abs(ref["y"]).max()
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+@pytest.mark.parametrize("M,K,N,r", [(17, 11008, 1024, 16), (100, 11008, 1000, 0), (64, 5632, 2048, 32), (129, 5632, 1032, 64), (512, 5632, 2048, 32),
+                                     (300, 4096, 3000, 48), (2000, 4160, 512, 32), (33, 4288, 128, 16), (128, 11008, 4096, 64)])
+def test_contraction_divided_over_a_cluster(M, K, N, r, bf16):
+    """Few output tiles and a long K: two, four and eight CTAs a tile, uneven shares of the K blocks, tiles that end inside
+    a token chunk and inside a channel quarter.  The int32 sums are exact (against float64 products of the same codes), y is the
+    dequantised sum plus the correction in float64 (6e-4: H enters in fp16; half a bf16 ulp more in bf16)."""
+    from paper_2602_05269_b200 import hgf
+    g = torch.Generator(device="cuda").manual_seed(M + K)
+    rn = lambda shape, std=1.0: torch.randn(shape, generator=g, device="cuda") * std  # noqa: E731
+    packed, gamma = hgf.pack_ternary(rn((N, K), 0.02))
+    x = rn((M, K)).bfloat16()
+    At, Bt, gate = (rn((r, K), K ** -0.5).half(), rn((N, r), r ** -0.5).half(), torch.rand(N, generator=g, device="cuda")) if r else (None,) * 3
+    y, dbg = hgf.linear_forward(x, packed, gamma, K, N, At, Bt, gate, debug=True, flags=hgf.FLAG_OUT_BF16 if bf16 else 0)
+    hgf.check_status()
+    T = hgf.unpack_ternary(packed, N, K).double()
+    y_int = dbg["xq"].double() @ T.T
+    assert torch.equal(dbg["y_int"].double(), y_int)
+    ref = y_int * dbg["gamma_x"].double()[:, None] * gamma / 127.0
+    if r:
+        z = x.double() @ At.double().T
+        ref = ref + (z * torch.sigmoid(z)) @ Bt.double().T * gate.double()
+    assert float((y.double() - ref).abs().max()) <= (6e-4 + (2.0 ** -8 if bf16 else 0.0)) * float(ref.abs().max())
