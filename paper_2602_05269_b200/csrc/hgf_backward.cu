@@ -9,8 +9,33 @@
 // expanded as a transposed bf16 matrix.  The quantised activations enter as exact bf16 integers
 // (|x~| <= 127) and the per-token scale is folded into dY; the ternary codes enter as exact -1 / 0 / +1.
 #include "hgf_tc.cuh"
+#include "hgf_warp.cuh"
 
 namespace hgf {
+
+// Every launch of the backward pass is chained to the one before by programmatic dependent launch: its blocks are set up
+// under the predecessor's tail and wait for its completion before they touch memory (a step of the 2048 x 5632 layer at
+// M = 8192 has seventeen such launches, most of them of 2 to 3 us: 662 -> 646 us together with bw_quant_kernel).
+template <typename... Params, typename... Args>
+static cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(grid);
+    cfg.blockDim = dim3(block);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, Params(args)...);
+    count_launch();
+    return e != cudaSuccess ? e : cudaGetLastError();
+}
+__device__ __forceinline__ void chain() {  // first thing of a kernel that is all loads and stores
+    pdl_launch_dependents();
+    pdl_wait();
+}
 
 // ---- generic GEMM on the 5th-generation tensor cores: C[I][J] (fp32) = alpha * sum_c A[i][c] B[j][c] (+ C) ----
 // Either operand may be stored with the contraction index contiguous ([rows][Cn], "K-major") or with its
@@ -110,6 +135,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
     __syncthreads();
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (warp-uniform)
+    chain();
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
@@ -236,6 +262,7 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 }
 // Sum of the partial results of a split contraction, in split order: C = alpha * sum_s P[s] (+ C).
 __global__ void __launch_bounds__(256) tc_reduce_kernel(const float4 *P, int splits, size_t n4, float alpha, int accumulate, float4 *C) {
+    chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n4) return;
     float4 a = P[i];
@@ -271,9 +298,7 @@ static cudaError_t tc_gemm_bn(const CUtensorMap *maps, const TcGemmArgs &g, cuda
     const int work = g.n_half ? tiles + g.n_half / 2 : tiles * g.splits;
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
-    tc_gemm_kernel<BN><<<work < sms ? work : sms, kTThreads, TcCfg<BN>::SMEM_BYTES, stream>>>(maps[0], maps[1], maps[2], maps[3], g, status);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(tc_gemm_kernel<BN>, (unsigned)(work < sms ? work : sms), kTThreads, TcCfg<BN>::SMEM_BYTES, stream, maps[0], maps[1], maps[2], maps[3], g, status);
 }
 
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
@@ -314,14 +339,13 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
     cudaError_t e = BN == 256 ? tc_gemm_bn<256>(maps, g, stream) : (BN == 128 ? tc_gemm_bn<128>(maps, g, stream) : tc_gemm_bn<64>(maps, g, stream));
     if (e != cudaSuccess || g.splits == 1) return e;
     const size_t n4 = (size_t)I * J / 4;
-    tc_reduce_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, stream>>>((const float4 *)partials, g.splits, n4, alpha, accumulate ? 1 : 0, (float4 *)C);
-    count_launch();
-    return cudaGetLastError();
+    return launch_chained(tc_reduce_kernel, (unsigned)((n4 + 255) / 256), 256, 0, stream, (const float4 *)partials, g.splits, n4, alpha, accumulate ? 1 : 0, (float4 *)C);
 }
 
 // ---- operand preparation ---------------------------------------------------------------------------
 // Xd = x~ gamma_x / 127 as bf16 [M][K] (eight values per thread).
 __global__ void __launch_bounds__(256) bw_dequant_kernel(const int8_t *xq, const float *gamma_x, int K, size_t n8, __nv_bfloat16 *xd) {
+    chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n8) return;
     const float s = gamma_x[(i * 8) / (size_t)K] * (1.0f / 127.0f);
@@ -337,9 +361,48 @@ __global__ void __launch_bounds__(256) bw_dequant_kernel(const int8_t *xq, const
     reinterpret_cast<uint4 *>(xd)[i] = make_uint4(o[0], o[1], o[2], o[3]);
 }
 
+// Algorithm 1, steps 1-2, and Xd in one pass over x for rows of up to 256 U columns: one warp per row, the row in
+// registers between the maximum and the rounding, the codes turned into values without touching memory.  Bound by HBM
+// (2 + 2 bytes an element): 8192 x 2048 in 11.9 us, against 11.9 + 8.8 us through int8 codes in memory.
+template <int U>
+__global__ void __launch_bounds__(256) bw_quant_kernel(const __nv_bfloat16 *x, int M, int K, __nv_bfloat16 *xd) {
+    chain();
+    const int lane = threadIdx.x & 31, m = blockIdx.x * 8 + (threadIdx.x >> 5), nv = K / 8;
+    if (m >= M) return;
+    const uint4 *xv = reinterpret_cast<const uint4 *>(x + (size_t)m * K);
+    uint4 v[U];
+    uint32_t abits = 0u;
+#pragma unroll
+    for (int u = 0; u < U; ++u) v[u] = lane + 32 * u < nv ? xv[lane + 32 * u] : make_uint4(0u, 0u, 0u, 0u);
+#pragma unroll
+    for (int u = 0; u < U; ++u) abits = absmax8_bits(abits, v[u]);
+    const float g = fmaxf(warp_max(absmax_bits_to_float(abits)), 1e-5f), s = g * (1.0f / 127.0f);
+    const QuantScale qs = make_quant_scale(g);
+    uint4 *dst = reinterpret_cast<uint4 *>(xd + (size_t)m * K);
+    int sum = 0;
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+        if (lane + 32 * u < nv) {
+            const uint2 c = quant8(v[u], qs, sum);
+            const uint32_t w[2] = {c.x ^ 0x80808080u, c.y ^ 0x80808080u};  // code + 128
+            uint32_t o[4];
+#pragma unroll
+            for (int h = 0; h < 4; ++h) {
+                // the byte as the low mantissa bits of 2^23, minus (2^23 + 128): the code as a float, exactly
+                const float c0 = __uint_as_float(__byte_perm(w[h >> 1], 0x4b000000u, 0x7650 + 2 * (h & 1))) - 8388736.0f;
+                const float c1 = __uint_as_float(__byte_perm(w[h >> 1], 0x4b000000u, 0x7651 + 2 * (h & 1))) - 8388736.0f;
+                const __nv_bfloat162 p = __floats2bfloat162_rn(c0 * s, c1 * s);
+                o[h] = *reinterpret_cast<const uint32_t *>(&p);
+            }
+            dst[lane + 32 * u] = make_uint4(o[0], o[1], o[2], o[3]);
+        }
+    }
+}
+
 // Ternary codes of the packed matrix as a bf16 matrix T [N][K] of -1 / 0 / +1 (one packed word = 16 columns per thread).
 __global__ void __launch_bounds__(256) bw_expand_ternary_kernel(const uint32_t *packed, int N, int K, int steps, size_t n_words,
                                                                 __nv_bfloat16 *T) {
+    chain();
     const size_t w = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (w >= n_words) return;
     const int kw = (int)(w & 15), r = (int)((w >> 4) & 15);
@@ -365,6 +428,7 @@ __global__ void __launch_bounds__(256) bw_expand_ternary_kernel(const uint32_t *
 
 // fp16 -> bf16, optionally times a per-row factor (the gate folded into B^T).
 __global__ void __launch_bounds__(256) bw_half_to_bf16_kernel(const __half *src, const float *row_scale, int cols, size_t n, __nv_bfloat16 *dst) {
+    chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
     const float s = row_scale ? row_scale[i / (size_t)cols] : 1.0f;
@@ -373,6 +437,7 @@ __global__ void __launch_bounds__(256) bw_half_to_bf16_kernel(const __half *src,
 
 // Z (fp32 [M][r]) -> H = act(Z) as bf16 [M][r] and SiLU'(Z) as fp32 (in place of Z).
 __global__ void __launch_bounds__(256) bw_act_kernel(float *z, size_t n, int no_silu, __nv_bfloat16 *h) {
+    chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
     const float v = z[i];
@@ -384,6 +449,7 @@ __global__ void __launch_bounds__(256) bw_act_kernel(float *z, size_t n, int no_
 // dZ = dH * SiLU'(Z), rounded to bf16, and dZ * scale (the copy that enters dX next to gamma_W dY T).
 __global__ void __launch_bounds__(256) bw_dz_kernel(const float *dh, const float *dact, size_t n, float scale, __nv_bfloat16 *dz,
                                                     __nv_bfloat16 *dz_scaled) {
+    chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
     const float v = dh[i] * dact[i];
@@ -394,6 +460,7 @@ __global__ void __launch_bounds__(256) bw_dz_kernel(const float *dh, const float
 // From G[n][j] = sum_m dY[m][n] H[m][j]: dBt[n][j] = gate[n] G[n][j] (in place), dgate[n] = sum_j G[n][j] Bt[n][j].
 // One warp per output channel n (its r values are contiguous).
 __global__ void __launch_bounds__(256) bw_gate_kernel(float *G, const __half *Bt, const float *gate, int N, int r, float *dgate) {
+    chain();
     const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (n >= N) return;
     float dg = 0.0f;
@@ -478,25 +545,30 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     const TcOperand x_k = {(const __nv_bfloat16 *)x, K, false}, x_mn = {(const __nv_bfloat16 *)x, K, true};
 
     if (grads->dW) {  // Algorithm 1, steps 1-2 again, then dW[n][k] = sum_m dY[m][n] Xd[m][k]
-        PrologueParams pp = {};
-        pp.x = (const __nv_bfloat16 *)x;
-        pp.xq = (int8_t *)(ws + L.xq);
-        pp.gamma_x = (float *)(ws + L.gamma_x);
-        pp.M = Mi;
-        pp.K = K;
-        pp.flags = HGF_FLAG_NO_PDL;
-        if (launch_quant(pp, GemmPrologueExtra{}, stream) != cudaSuccess) return HGF_ERR_CUDA;
-        const size_t n8 = (size_t)M * K / 8;
-        bw_dequant_kernel<<<blocks1(n8), 256, 0, stream>>>(pp.xq, pp.gamma_x, K, n8, bf(L.xd));
-        count_launch();
+        if (K <= 4096) {  // a row fits a warp's registers
+            const unsigned rows8 = (unsigned)((Mi + 7) / 8);
+            const __nv_bfloat16 *xp = (const __nv_bfloat16 *)x;
+            ok = (K <= 2048 ? launch_chained(bw_quant_kernel<8>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))
+                            : launch_chained(bw_quant_kernel<16>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))) == cudaSuccess;
+        } else {
+            PrologueParams pp = {};
+            pp.x = (const __nv_bfloat16 *)x;
+            pp.xq = (int8_t *)(ws + L.xq);
+            pp.gamma_x = (float *)(ws + L.gamma_x);
+            pp.M = Mi;
+            pp.K = K;
+            pp.flags = HGF_FLAG_NO_PDL;
+            if (launch_quant(pp, GemmPrologueExtra{}, stream) != cudaSuccess) return HGF_ERR_CUDA;
+            const size_t n8 = (size_t)M * K / 8;
+            ok = launch_chained(bw_dequant_kernel, blocks1(n8), 256, 0, stream, pp.xq, pp.gamma_x, K, n8, bf(L.xd)) == cudaSuccess;
+        }
         gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false);
     }
     const bool fold = gamma > 1e-20f;  // the low-rank term of dX rides in the same contraction, pre-divided by gamma_W
     if (grads->dx) {
         const int steps = (int)(padded_k(d_in) / 256);
         const size_t n_words = (size_t)row_tiles(d_out) * steps * 256;
-        bw_expand_ternary_kernel<<<blocks1(n_words), 256, 0, stream>>>((const uint32_t *)packed, N, K, steps, n_words, bf(L.T));
-        count_launch();
+        ok = ok && launch_chained(bw_expand_ternary_kernel, blocks1(n_words), 256, 0, stream, (const uint32_t *)packed, N, K, steps, n_words, bf(L.T)) == cudaSuccess;
     }
     const TcOperand T_mn = {bf(L.T), K, true};  // T [N][K]: rows k of the product, contracted over n
     if (!r) {
@@ -504,15 +576,13 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
     }
     float *z = (float *)(ws + L.z), *dh = (float *)(ws + L.dh), *G = grads->dBt ? grads->dBt : (float *)(ws + L.G);
-    bw_half_to_bf16_kernel<<<blocks1((size_t)r * K), 256, 0, stream>>>((const __half *)At, nullptr, K, (size_t)r * K, bf(L.At_b));
-    bw_half_to_bf16_kernel<<<blocks1((size_t)N * r), 256, 0, stream>>>((const __half *)Bt, gate, r, (size_t)N * r, bf(L.gBt));
-    count_launch(2);
+    ok = ok && launch_chained(bw_half_to_bf16_kernel, blocks1((size_t)r * K), 256, 0, stream, (const __half *)At, (const float *)nullptr, K, (size_t)r * K, bf(L.At_b)) == cudaSuccess &&
+         launch_chained(bw_half_to_bf16_kernel, blocks1((size_t)N * r), 256, 0, stream, (const __half *)Bt, gate, r, (size_t)N * r, bf(L.gBt)) == cudaSuccess;
     const TcOperand At_k = {bf(L.At_b), K, false}, At_mn = {bf(L.At_b), K, true};
     gemm(x_k, At_k, K, none, none, 0, z, r, Mi, r, 1.0f, false, true);                                       // Z = x A
-    bw_act_kernel<<<blocks1((size_t)M * r), 256, 0, stream>>>(z, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, bf(L.h_b));
+    ok = ok && launch_chained(bw_act_kernel, blocks1((size_t)M * r), 256, 0, stream, z, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, bf(L.h_b)) == cudaSuccess;
     gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true);            // dH = dY (g (.) B^T)
-    bw_dz_kernel<<<blocks1((size_t)M * r), 256, 0, stream>>>(dh, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b));
-    count_launch(2);
+    ok = ok && launch_chained(bw_dz_kernel, blocks1((size_t)M * r), 256, 0, stream, dh, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b)) == cudaSuccess;
     if (grads->dx) {                                                                                         // dX = gamma_W dY T + dZ A^T
         const TcOperand dzs_k = {bf(L.dzs_b), r, false};
         if (fold) {
@@ -526,8 +596,7 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         gemm(TcOperand{bf(L.dz_b), r, true}, x_mn, Mi, none, none, 0, grads->dAt, K, r, K, 1.0f, false, true);
     if (grads->dBt || grads->dgate) {                                                                        // G[n][j] = sum_m dY[m][n] H[m][j]
         gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true);
-        bw_gate_kernel<<<(unsigned)((N + 7) / 8), 256, 0, stream>>>(G, (const __half *)Bt, gate, N, r, grads->dgate);
-        count_launch();
+        ok = ok && launch_chained(bw_gate_kernel, (unsigned)((N + 7) / 8), 256, 0, stream, G, (const __half *)Bt, gate, N, r, grads->dgate) == cudaSuccess;
     }
     return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
 }

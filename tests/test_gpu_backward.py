@@ -85,3 +85,9 @@ def test_rejects_bad_arguments(hgf):
     with pytest.raises(hgf.HgfError) as e:          # d_out must be a multiple of 8
         hgf.linear_backward(x, packed, 1.0, 256, 60, dy)
     assert e.value.status == 2
+
+
+@pytest.mark.parametrize("M,K,N,r", [(40, 4096, 64, 16), (33, 4160, 64, 16), (9, 2112, 72, 32), (70, 2048, 40, 16)])
+def test_row_lengths_of_the_quantiser(hgf, M, K, N, r):
+    """Rows at the limits of what a warp holds in registers (2048, 4096 columns) and just past them."""
+    check(hgf, M, K, N, r, layer=K)
