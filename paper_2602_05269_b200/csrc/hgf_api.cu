@@ -1,6 +1,7 @@
 // C-ABI entry points: argument validation, workspace carving, routing between the decode GEMV
 // path (M <= 16) and the tcgen05 GEMM path.  No compute happens on the host and there is no CPU
 // fallback: without a CUDA device every forward call fails with HGF_ERR_CUDA.
+#include <algorithm>
 #include <atomic>
 #include <new>
 #include <unordered_map>
@@ -384,7 +385,7 @@ struct hgf_group {
     PrologueParams *d_pps;
     QuantItem *d_quant_items; // prologue: one per (problem, token)
     LoraItem *d_lora_items;   // prologue: one per (problem, 16 columns of H, K slice)
-    int n_quant, n_lora;
+    int n_ln, n_quant, n_lora;  // (rows behind a LayerNorm come first)
     int4 *d_cta_range;        // per GEMV CTA: (first tile, end tile, first problem, 0)
     int grid;
     bool small;               // whole forwards take the one launch `sl` describes
@@ -532,6 +533,7 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
     g->d_pps = (PrologueParams *)((char *)mem + off_pps);
     g->d_quant_items = (QuantItem *)((char *)mem + off_qit);
     g->d_lora_items = (LoraItem *)((char *)mem + off_lit);
+    g->n_ln = (int)(std::stable_partition(qitems.begin(), qitems.end(), [](const QuantItem &q) { return q.ln_w != nullptr; }) - qitems.begin());
     g->n_quant = (int)qitems.size();
     g->n_lora = (int)litems.size();
     g->d_cta_range = (int4 *)((char *)mem + off_cta);
@@ -611,7 +613,7 @@ extern "C" hgf_status hgf_group_forward_phases(hgf_group *g, uint32_t phases, vo
     if (g->small && phases == (HGF_PHASE_PROLOGUE | HGF_PHASE_GEMV))
         return launch_small(g->sl, pdl, stream) == cudaSuccess ? HGF_OK : HGF_ERR_CUDA;
     if ((phases & HGF_PHASE_PROLOGUE) &&
-        launch_decode_prologue_group(g->d_quant_items, g->n_quant, g->d_lora_items, g->n_lora, g->max_M, pdl,
+        launch_decode_prologue_group(g->d_quant_items, g->n_ln, g->n_quant, g->d_lora_items, g->n_lora, g->max_M, pdl,
                                      stream) != cudaSuccess)
         return HGF_ERR_CUDA;
     if (!(phases & HGF_PHASE_GEMV)) return HGF_OK;

@@ -207,7 +207,8 @@ struct QuantItem {
     float *mean_out, *rstd_out;  // nullable: where this row's statistics go
 };
 __host__ __device__ inline int prologue_slice_k(int max_M) { return max_M <= 8 ? 512 : 256; }
-cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_quant,
+// (the first n_ln quantisation items are the ones behind a LayerNorm)
+cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_ln, int n_quant,
                                          const LoraItem *d_lora_items, int n_lora, int max_M, bool pdl,
                                          cudaStream_t stream);
 cudaError_t launch_gemm_prologue(const PrologueParams &p, const GemmPrologueExtra &x, cudaStream_t stream);

@@ -497,9 +497,87 @@ __global__ void __launch_bounds__(kThreads) ln_quant_rows_kernel(const PrologueP
     }
 }
 
+// A row behind the LayerNorm front end by a whole CTA: brought into shared memory once, mean and variance in one pass in
+// double of x - x[0] (see hgf_decode_small.cu), the largest |xn|, the codes.  A decode launch has a few of these and
+// one warp alone took 20 us over a row of 2048 (four passes, a memory latency in each of their steps).
+__device__ void block_quant_row_ln(const QuantItem &q, uint8_t *buf, int tid) {
+    __shared__ double2 s_sum[kPgWarps];
+    __shared__ uint32_t s_max[kPgWarps];
+    __shared__ int s_codes[kPgWarps];
+    const int K = q.K, nv = K / 8, lane = tid & 31, warp = tid >> 5;
+    const uint32_t buf_u32 = (uint32_t)__cvta_generic_to_shared(buf);
+    for (int i = tid; i < nv; i += kPgThreads) cp_async_16(buf_u32 + 16 * i, q.x + 8 * i, 16u);
+    asm volatile("cp.async.commit_group;\n" ::: "memory");
+    asm volatile("cp.async.wait_all;\n" ::: "memory");
+    __syncthreads();
+    const double first = (double)__bfloat162float(*reinterpret_cast<const __nv_bfloat16 *>(buf));
+    double s = 0.0, ss = 0.0;
+    for (int i = tid; i < nv; i += kPgThreads) {
+        float f[8];
+        unpack8(*reinterpret_cast<const uint4 *>(buf + 16 * i), f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) {
+            const double d = (double)f[e] - first;
+            s += d;
+            ss = fma(d, d, ss);
+        }
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        s += __shfl_xor_sync(0xffffffffu, s, o);
+        ss += __shfl_xor_sync(0xffffffffu, ss, o);
+    }
+    if (lane == 0) s_sum[warp] = make_double2(s, ss);
+    __syncthreads();
+    s = ss = 0.0;
+#pragma unroll
+    for (int w = 0; w < kPgWarps; ++w) { s += s_sum[w].x; ss += s_sum[w].y; }
+    const double dm = s / (double)K, v0 = ss / (double)K - dm * dm, var = v0 < 0.0 ? 0.0 : v0;  // (NaN stays NaN)
+    const float mean = (float)(first + dm), rstd = (float)rsqrt(var + (double)q.eps);
+    auto normal = [&](int i, float (&xn)[8]) {
+        const float4 *w4 = reinterpret_cast<const float4 *>(q.ln_w + 8 * i), *b4 = reinterpret_cast<const float4 *>(q.ln_b + 8 * i);
+        const float4 w0 = w4[0], w1 = w4[1], b0 = b4[0], b1 = b4[1];
+        const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
+        float f[8];
+        unpack8(*reinterpret_cast<const uint4 *>(buf + 16 * i), f);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) xn[e] = ln_value(f[e], mean, rstd, w[e], b[e]);
+    };
+    float a = 0.0f, xn[8];
+    for (int i = tid; i < nv; i += kPgThreads) {
+        normal(i, xn);
+#pragma unroll
+        for (int e = 0; e < 8; ++e) a = fmaxf(a, fabsf(xn[e]));
+    }
+    const uint32_t most = __reduce_max_sync(0xffffffffu, __float_as_uint(a));
+    if (lane == 0) s_max[warp] = most;
+    __syncthreads();
+    uint32_t top = s_max[0];
+#pragma unroll
+    for (int w = 1; w < kPgWarps; ++w) top = s_max[w] > top ? s_max[w] : top;
+    const float g = fmaxf(__uint_as_float(top), 1e-5f), scale = __fdiv_rn(127.0f, g);
+    int sum = 0;
+    for (int i = tid; i < nv; i += kPgThreads) {
+        normal(i, xn);
+        reinterpret_cast<uint2 *>(q.xq)[i] = ln_codes8(xn, scale, sum);
+    }
+    sum = __reduce_add_sync(0xffffffffu, sum);
+    if (lane == 0) s_codes[warp] = sum;
+    __syncthreads();  // (also: the row's buffer is free)
+    if (tid == 0) {
+        int all = 0;
+#pragma unroll
+        for (int w = 0; w < kPgWarps; ++w) all += s_codes[w];
+        *q.row_sum = all;
+        *q.gamma_x = g;
+        if (q.mean_out) *q.mean_out = mean;
+        if (q.rstd_out) *q.rstd_out = rstd;
+    }
+}
+
 template <int NT>
 __global__ void __launch_bounds__(kPgThreads, 1)
-decode_prologue_group_kernel(const QuantItem *quant_items, int n_quant, const LoraItem *lora, int n_lora) {
+decode_prologue_group_kernel(const QuantItem *quant_items, int n_ln, int n_quant, const LoraItem *lora, int n_lora) {
     constexpr int CH = 16 / NT;                       // 32-column chunks per item
     constexpr int kWarpBytes = CH * (1024 + 512 * NT);  // per chunk: two rows of A^T and NT rows of x, 16 bytes per lane
     extern __shared__ __align__(128) uint8_t pg_smem[];
@@ -516,16 +594,22 @@ decode_prologue_group_kernel(const QuantItem *quant_items, int n_quant, const Lo
     }
     // LoRA items are dealt from the first warp up, quantisation items from the last warp down, so the
     // warps with one LoRA item fewer take the rows
-    const int q_first = nw - 1 - gw;
+    const int q_first = n_ln + nw - 1 - gw;
     QuantItem q = {};
     if (q_first < n_quant) q = quant_items[q_first];
     pdl_wait();  // x, and the scratch this kernel overwrites, belong to earlier work
 
+    // rows behind a LayerNorm (the first n_ln items): a CTA each, from the last CTA down
+    for (int i = gridDim.x - 1 - blockIdx.x; i < n_ln; i += gridDim.x) {
+        const QuantItem row = quant_items[i];
+        block_quant_row_ln(row, pg_smem, threadIdx.x);
+        __syncthreads();
+    }
+
     for (int i = q_first; i < n_quant; i += nw) {
         QuantItem q_next = q;
         if (i + nw < n_quant) q_next = quant_items[i + nw];  // travels while this row is worked on
-        if (q.ln_w) warp_quant_row_ln(q, lane);
-        else warp_quant_row(q, buf - 16 * lane, pg_smem + warp * kWarpBytes, kWarpBytes, lane);
+        warp_quant_row(q, buf - 16 * lane, pg_smem + warp * kWarpBytes, kWarpBytes, lane);
         q = q_next;
     }
 
@@ -1369,7 +1453,7 @@ cudaError_t launch_gemm_prologue_ln(const PrologueParams &p, const GemmPrologueE
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_quant, const LoraItem *d_lora_items, int n_lora, int max_M, bool pdl,
+cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_ln, int n_quant, const LoraItem *d_lora_items, int n_lora, int max_M, bool pdl,
                                          cudaStream_t stream) {
     static std::atomic<unsigned long long> attr_done1{0}, attr_done2{0};
     const int sm_count = device_sm_count();
@@ -1381,8 +1465,9 @@ cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_q
         e = ensure_dynamic_smem(decode_prologue_group_kernel<2>, smem2, attr_done2);
         if (e != cudaSuccess) return e;
     }
-    const int most = n_lora > n_quant ? n_lora : n_quant;
+    const int most = n_lora > n_quant - n_ln ? n_lora : n_quant - n_ln;
     int blocks = (most + kPgWarps - 1) / kPgWarps;
+    if (n_ln) blocks = (most + kPgWarps - 1) / kPgWarps + n_ln;  // CTAs of their own for the rows behind a LayerNorm
     blocks = blocks < sm_count ? blocks : sm_count;
     if (blocks < 1) blocks = 1;
     cudaLaunchAttribute attr[1];
@@ -1391,10 +1476,10 @@ cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_q
     cudaError_t e;
     if (max_M <= 8) {
         cfg.dynamicSmemBytes = smem1;
-        e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<1>, d_quant_items, n_quant, d_lora_items, n_lora);
+        e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<1>, d_quant_items, n_ln, n_quant, d_lora_items, n_lora);
     } else {
         cfg.dynamicSmemBytes = smem2;
-        e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<2>, d_quant_items, n_quant, d_lora_items, n_lora);
+        e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<2>, d_quant_items, n_ln, n_quant, d_lora_items, n_lora);
     }
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
