@@ -22,6 +22,7 @@ namespace hgf {
 
 constexpr int kSmThreads = 512, kSmWarps = kSmThreads / 32;
 constexpr int kSmSmemLimit = 113 * 1024;  // two CTAs on an SM (228 KB, 1 KB of each CTA's reserved)
+constexpr int kSmSmemMax = 200 * 1024;
 constexpr int kSmHPitch = 72;  // halves per row of H in shared memory (r <= 64, + 8 bank spread)
 
 struct SmHead {                // per-token values at the start of shared memory
@@ -294,7 +295,10 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
         sum = __reduce_add_sync(0xffffffffu, sum);
         if (lane == 0) atomicAdd(&head->row_sum[m], sum);
     });
-    __syncthreads();
+    // the codes are there; the quantising warps go on without the others
+    if (!apart) __syncthreads();
+    else if (quantises) { bar_arrive(3, kSmThreads); bar_sync(1, 32 * q_warps); }
+    else bar_sync(3, kSmThreads);
 
     // ---- the ternary contraction: warp (kw, rw) takes column tiles kw, kw + KS, ... of row tiles rw, rw + RS, ... --
     ok = warp_wait(bar_w, status, 0x600u) && ok;
@@ -353,12 +357,13 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
         if (P.dbg_gamma_x) P.dbg_gamma_x[tid] = gm;
     }
 
-    // ---- H: the cluster's partial sums in rank order, SiLU, fp16 value and fp16 residual ---------------------
-    if (r > 0) {
+    // ---- H: the cluster's partial sums in rank order, SiLU, fp16 value and fp16 residual; by the warps that computed x A,
+    // which have a smaller part in the products above (none where the CTA has one row tile) ----------------------------------
+    if (multiplies) {
         ok = warp_wait(bar_h, status, 0x600u) && ok;
         const bool no_silu = (P.flags & HGF_FLAG_NO_SILU) != 0;
 #pragma unroll 1
-        for (int e = tid; e < E; e += kSmThreads) {
+        for (int e = 32 * a_warp + lane; e < E; e += 32 * a_warps) {
             float z = 0.0f;
             for (int q = 0; q < C; ++q) z += slots[q * E + e];
             // accumulator register c of lane (g, t): row g + 8 (c >> 1), token 8 n + 2 t + (c & 1)
@@ -443,7 +448,8 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
 //    LayerNorm 6.7 / 9.0, 8.2 / 9.0, 10.9 / 9.0 at M = 1, 2, 4; 512 -> 512: 4.1 / 7.6 at M = 1, 6.4 / 9.1 at M = 16;
 //  - more shared memory than lets two CTAs share an SM: the next call's copies then wait for this one's end.
 //    2048 -> 5632 8.4 / 9.1 within (M = 4); 5632 -> 2048 14.6 / 9.9 (M = 2), 4096 -> 4096 at r = 64 13.7 / 9.6 beyond;
-//    Q, K and V of 2048 (three problems, LayerNorms) 7.7 / 20.1, two up-projections 2048 -> 5632 6.9 / 11.9 at M = 1;
+//    Q, K and V of 2048 (three problems, LayerNorms) 7.7 / 14, two up-projections 2048 -> 5632 6.9 / 11.9 at M = 1.  Groups of four
+//    problems and more take it all the same: seven of 2048 -> 2048 12.5 / 16.3 at M = 1, 16.0 / 16.9 at M = 4;
 //  - base-3 weights (no such kernel).
 template <int NP>
 bool plan_small(SmallLaunch<NP> &L, uint32_t flags) {
@@ -516,7 +522,7 @@ bool plan_small(SmallLaunch<NP> &L, uint32_t flags) {
     L.off_bt = take(bt);
     L.off_w = take(w);
     L.smem = (int)off;
-    return off <= (size_t)kSmSmemLimit;
+    return off <= (size_t)(L.n >= 4 ? kSmSmemMax : kSmSmemLimit);
 }
 template bool plan_small<1>(SmallLaunch<1> &, uint32_t);
 template bool plan_small<kSmallMax>(SmallLaunch<kSmallMax> &, uint32_t);
@@ -524,7 +530,7 @@ template bool plan_small<kSmallMax>(SmallLaunch<kSmallMax> &, uint32_t);
 template <int NT, int NP>
 static cudaError_t launch_small_nt(const SmallLaunch<NP> &L, bool pdl, cudaStream_t stream) {
     static std::atomic<unsigned long long> attr_done{0};
-    cudaError_t e = ensure_dynamic_smem(decode_small_kernel<NT, NP>, kSmSmemLimit, attr_done);
+    cudaError_t e = ensure_dynamic_smem(decode_small_kernel<NT, NP>, kSmSmemMax, attr_done);
     if (e != cudaSuccess) return e;
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
