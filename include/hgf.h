@@ -151,8 +151,8 @@ size_t hgf_workspace_bytes(int64_t M, int64_t d_in, int64_t d_out, int32_t r, ui
  * 104 KiB (no shape of the paper's model classes at M <= 16) takes the GEMM path as well.
  * Calls on the same workspace must not overlap on the device.
  * Launch overlap: the decode kernels are launched with programmatic stream serialization and start
- * fetching `packed` before the preceding work on `stream` has finished (they wait for that work
- * before touching x, the workspace or y).  packed, At, Bt and gate must therefore not be written
+ * fetching packed, At, Bt and gate before the preceding work on `stream` has finished (they wait for
+ * that work before touching x, the workspace or y).  packed, At, Bt and gate must therefore not be written
  * by work still pending on `stream`; pass HGF_FLAG_NO_PDL if they might be.
  */
 hgf_status hgf_linear_forward(const void *x, int64_t M, const void *packed, float gamma,
@@ -264,7 +264,9 @@ hgf_status hgf_linear_forward_static(const void *x, int64_t M, const void *packe
  * stay owned by the caller and must stay valid) and allocates the group's descriptors and
  * workspace on the current device; it is a set-up call, not for the hot path.
  * hgf_group_forward only enqueues: one prologue launch and one GEMV launch for the whole group,
- * which streams the packed weights of all its problems as one sequence split evenly over the SMs.
+ * which streams the packed weights of all its problems as one sequence split evenly over the SMs;
+ * up to eight problems whose weights fit the chip's shared memory are one launch in all, as is a
+ * small hgf_linear_forward.
  * Forward calls of one group must not overlap on the device.  hgf_group_destroy frees the group
  * (the caller makes sure no forward is still running).
  */

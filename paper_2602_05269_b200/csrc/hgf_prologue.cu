@@ -1022,7 +1022,6 @@ __global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const Prologu
     } else {
         cluster_arrive_relaxed();
     }
-    // (A^T is not written by pending work) this warp's first chunk of it
     const int nch = cols >> 5;
     const __half *arow = JT > 0 ? p.At + (size_t)g * K + k0 + 8 * t : nullptr;
     uint4 av[JT > 0 ? JT : 1];
@@ -1031,9 +1030,9 @@ __global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const Prologu
 #pragma unroll
             for (int jt = 0; jt < JT; ++jt) av[jt] = c < nch ? *reinterpret_cast<const uint4 *>(arow + (size_t)8 * jt * K + 32 * c) : make_uint4(0u, 0u, 0u, 0u);
     };
-    load_a(warp);
     __syncthreads();
     pdl_wait();
+    load_a(warp);  // this warp's first chunk of A^T (like every read of this path, after the wait)
     bool ok = warp_wait(bar_x, status, 0x680u);
     cluster_wait_acquire();  // every CTA of the cluster has started
 

@@ -184,11 +184,6 @@ __device__ __forceinline__ uint64_t make_sw128_mn_desc(uint32_t saddr, uint32_t 
 // Every lane of a converged warp executes these (operands in uniform registers; from one thread in a divergent branch an MMA
 // took 80 to 125 clocks to issue) and elect.sync picks the one that issues (the same one every time, so
 // commits follow the MMAs they track).
-__device__ __forceinline__ bool elect_one() {
-    uint32_t e;
-    asm volatile("{\n.reg .pred p;\nelect.sync _|p, 0xffffffff;\nselp.u32 %0, 1, 0, p;\n}\n" : "=r"(e));
-    return e != 0;
-}
 __device__ __forceinline__ void warp_commit(uint32_t bar) {
     asm volatile("{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
                  "@e tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n}\n" ::"r"(bar) : "memory");
