@@ -58,7 +58,8 @@ struct TaCfg {
     static constexpr int OFF_K = NQ * 2 * Q_BYTES, OFF_V = OFF_K + KST * 2 * K_BYTES, OFF_BAR = OFF_V + VST * V_BYTES;
     static constexpr int BAR_QFULL = 0, BAR_QEMPTY = 2, BAR_OEMPTY = 4, BAR_KFULL = 6, BAR_KEMPTY = BAR_KFULL + KST, BAR_VFULL = BAR_KEMPTY + KST, BAR_VEMPTY = BAR_VFULL + VST,
                          BAR_SFULL = BAR_VEMPTY + VST,    // [stream][buffer]
-                         BAR_PFULL = BAR_SFULL + 4, BAR_L = BAR_PFULL + 4, BAR_COUNT = BAR_L + 2;
+                         BAR_PFULL = BAR_SFULL + 4, BAR_L = BAR_PFULL + 4, BAR_END = BAR_L + 2,  // [parity of the tile], [stream]
+                         BAR_COUNT = BAR_END + 2;
     static constexpr int OFF_L = OFF_BAR + 384;                           // [parity of the tile][2][128] floats
     static constexpr int SMEM_BYTES = OFF_L + 2 * 2 * kTaBM * 4 + 1024;
     static constexpr int COL_S = 0, COL_O = 4 * kTaKV;                    // scores: + (2 stream + buffer) 64; O: + (2 buffer + stream) DH
@@ -89,6 +90,25 @@ __device__ __forceinline__ uint64_t add_f32x2(uint64_t a, uint64_t b) {
     uint64_t d;
     asm("add.rn.f32x2 %0, %1, %2;\n" : "=l"(d) : "l"(a), "l"(b));
     return d;
+}
+
+// Four lanes (lane / 4 alike) with four 16-byte blocks each: afterwards block q of lane 4 i + t is what block t of lane
+// 4 i + q was.
+__device__ __forceinline__ void exchange_blocks(uint32_t (&v)[16], int lane) {
+#pragma unroll
+    for (int step = 1; step <= 2; step *= 2) {
+        const bool upper = (lane & step) != 0;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) {
+            if (b & step) continue;
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                uint32_t &lo = v[4 * b + e], &hi = v[4 * (b + step) + e];
+                const uint32_t got = __shfl_xor_sync(0xffffffffu, upper ? lo : hi, step);
+                if (upper) lo = got; else hi = got;
+            }
+        }
+    }
 }
 
 template <int DH>
@@ -127,6 +147,7 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
             mbar_init(bar(C::BAR_QEMPTY + i), 2);
             mbar_init(bar(C::BAR_OEMPTY + i), 8);
             mbar_init(bar(C::BAR_L + i), 8);
+            mbar_init(bar(C::BAR_END + i), 1);
         }
         for (int s = 0; s < C::KST; ++s) {
             mbar_init(bar(C::BAR_KFULL + s), 1);
@@ -269,6 +290,7 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
                 tc_fence_after();
                 issue_pv(buf, vs, pob, j == 0);
                 warp_commit(bar(C::BAR_VEMPTY + vs));
+                if (C::NQ == 1 && j + 1 == ptile.J) warp_commit(bar(C::BAR_END + st));
                 if (++vs == C::VST) { vs = 0; vph ^= 1u; }
                 // the products execute in issue order: P of this step has been read when those scores replace it
                 if (s_more) { if (!(ok = next_scores(buf))) break; }
@@ -369,9 +391,11 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
             }
             if (!ok) break;
             // ---- outputs of the tile: (O_1 / l_1 - lambda O_2 / l_2) out_scale; stream s's thread of a row writes half s
-            // of the row's columns.  The stream's last P V is complete when the barrier of two steps on says so (of
-            // the other stream's barriers this warp does not know the phase), both streams' when all eight warps say so.
-            ok = mbar_wait_poll(bar(C::BAR_SFULL + 2 * st + ((g - 1) & 1)), (uint32_t)((g + 1) >> 1) & 1u, abort_flag, status, 0xa50u + st);
+            // of the row's columns.  This stream's last P V is complete when the barrier of the scores two steps on says so (with one
+            // query buffer those wait for the next tile's queries, so it has a barrier of its own); of the other stream's barriers
+            // this warp does not know the phase: both streams' are complete when all eight warps have said so.
+            if (C::NQ == 1) ok = mbar_wait_poll(bar(C::BAR_END + st), (uint32_t)k & 1u, abort_flag, status, 0xa50u + st);
+            else ok = mbar_wait_poll(bar(C::BAR_SFULL + 2 * st + ((g - 1) & 1)), (uint32_t)((g + 1) >> 1) & 1u, abort_flag, status, 0xa50u + st);
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             float la, lb, lc, ld;
             unpack_f32x2(l2a, la, lb);
@@ -385,7 +409,6 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
             if (!(ok = __all_sync(0xffffffffu, ok))) break;
             tc_fence_after();
             const float w1 = p.out_scale / sl[row], w2 = p.out_scale * p.lambda / sl[kTaBM + row];
-            const size_t obase = (size_t)(t.tok0 + qi) * ((size_t)h * DH) + (size_t)t.hd * DH;
             const uint32_t o_base = lane_base + C::COL_O + 2 * ob * DH;
 #pragma unroll
             for (int cc = st * (DH / 2); cc < (st + 1) * (DH / 2); cc += 32) {
@@ -398,26 +421,62 @@ ta_diff_attention_kernel(const __grid_constant__ CUtensorMap tmap_q, const __gri
                     __syncwarp();
                     if (lane == 0) mbar_arrive(bar(C::BAR_OEMPTY + ob));
                 }
-                if (qi < L) {
+                if constexpr (DH == 128) {
+                    // Four neighbouring rows exchange 16-byte blocks, so that four lanes store 64 consecutive bytes of one row:
+                    // a lane storing along its own row touches 32 lines with every instruction.  (With the barrier above
+                    // 59.7 -> 56.3 us at B = 2, L = 1500, 16 heads of 128, fp32; at head_dim 64, half the bytes a row, the exchange
+                    // cost 1 to 5 %.)
+                    const int quad = t.q0 + 32 * quarter + (lane & ~3);  // the first of the four rows
+                    const size_t at = (size_t)(t.tok0 + quad) * ((size_t)h * DH) + (size_t)t.hd * DH + cc;
                     if (p.flags & HGF_FLAG_OUT_BF16) {
-                        uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) + obase + cc);
+                        uint32_t o[16];
 #pragma unroll
-                        for (int u = 0; u < 32; u += 8) {
-                            uint32_t o[4];
+                        for (int e = 0; e < 16; ++e)
+                            o[e] = pack_bf16(__uint_as_float(v1[2 * e]) * w1 - __uint_as_float(v2[2 * e]) * w2,
+                                             __uint_as_float(v1[2 * e + 1]) * w1 - __uint_as_float(v2[2 * e + 1]) * w2);
+                        exchange_blocks(o, lane);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e)
+                            if (quad + e < L)
+                                *reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) + at + (size_t)e * h * DH + 8 * (lane & 3)) =
+                                    make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
+                    } else {
+#pragma unroll
+                        for (int u = 0; u < 32; u += 16) {
+                            uint32_t o[16];
+#pragma unroll
+                            for (int e = 0; e < 16; ++e) o[e] = __float_as_uint(__uint_as_float(v1[u + e]) * w1 - __uint_as_float(v2[u + e]) * w2);
+                            exchange_blocks(o, lane);
 #pragma unroll
                             for (int e = 0; e < 4; ++e)
-                                o[e] = pack_bf16(__uint_as_float(v1[u + 2 * e]) * w1 - __uint_as_float(v2[u + 2 * e]) * w2,
-                                                 __uint_as_float(v1[u + 2 * e + 1]) * w1 - __uint_as_float(v2[u + 2 * e + 1]) * w2);
-                            dst[u >> 3] = make_uint4(o[0], o[1], o[2], o[3]);
+                                if (quad + e < L)
+                                    *reinterpret_cast<uint4 *>(reinterpret_cast<float *>(p.out) + at + (size_t)e * h * DH + u + 4 * (lane & 3)) =
+                                        make_uint4(o[4 * e], o[4 * e + 1], o[4 * e + 2], o[4 * e + 3]);
                         }
-                    } else {
-                        float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.out) + obase + cc);
+                    }
+                } else {
+                    const size_t obase = (size_t)(t.tok0 + qi) * ((size_t)h * DH) + (size_t)t.hd * DH;
+                    if (qi < L) {
+                        if (p.flags & HGF_FLAG_OUT_BF16) {
+                            uint4 *dst = reinterpret_cast<uint4 *>(reinterpret_cast<__nv_bfloat16 *>(p.out) + obase + cc);
 #pragma unroll
-                        for (int u = 0; u < 32; u += 4)
-                            dst[u >> 2] = make_float4(__uint_as_float(v1[u]) * w1 - __uint_as_float(v2[u]) * w2,
-                                                      __uint_as_float(v1[u + 1]) * w1 - __uint_as_float(v2[u + 1]) * w2,
-                                                      __uint_as_float(v1[u + 2]) * w1 - __uint_as_float(v2[u + 2]) * w2,
-                                                      __uint_as_float(v1[u + 3]) * w1 - __uint_as_float(v2[u + 3]) * w2);
+                            for (int u = 0; u < 32; u += 8) {
+                                uint32_t o[4];
+#pragma unroll
+                                for (int e = 0; e < 4; ++e)
+                                    o[e] = pack_bf16(__uint_as_float(v1[u + 2 * e]) * w1 - __uint_as_float(v2[u + 2 * e]) * w2,
+                                                     __uint_as_float(v1[u + 2 * e + 1]) * w1 - __uint_as_float(v2[u + 2 * e + 1]) * w2);
+                                dst[u >> 3] = make_uint4(o[0], o[1], o[2], o[3]);
+                            }
+                        } else {
+                            float4 *dst = reinterpret_cast<float4 *>(reinterpret_cast<float *>(p.out) + obase + cc);
+#pragma unroll
+                            for (int u = 0; u < 32; u += 4)
+                                dst[u >> 2] = make_float4(__uint_as_float(v1[u]) * w1 - __uint_as_float(v2[u]) * w2,
+                                                          __uint_as_float(v1[u + 1]) * w1 - __uint_as_float(v2[u + 1]) * w2,
+                                                          __uint_as_float(v1[u + 2]) * w1 - __uint_as_float(v2[u + 2]) * w2,
+                                                          __uint_as_float(v1[u + 3]) * w1 - __uint_as_float(v2[u + 3]) * w2);
+                        }
                     }
                 }
             }
