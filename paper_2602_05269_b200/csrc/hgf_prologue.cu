@@ -1059,7 +1059,8 @@ __global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const Prologu
         // Mean and variance in one pass, in double, of x - x[0]: see hgf_decode_small.cu.  A bf16 pattern moved to the top
         // of a double is x 2^-896 (subnormals too), so one fused multiply-add gives x - x[0] without a conversion; infinities and
         // NaNs, which that would miss, make the sum a NaN.
-        double first[2], sum[2] = {0.0, 0.0}, sum2[2] = {0.0, 0.0};
+        // (four partial sums each: the additions of one are a chain)
+        double first[2], sum[2][4] = {}, sum2[2][4] = {};
         uint32_t top[2] = {0u, 0u};
 #pragma unroll
         for (int q = 0; q < 2; ++q) first[q] = warp + kRpWarps * q < rows ? (double)__bfloat162float(p.x[(size_t)(m0 + warp + kRpWarps * q) * K]) : 0.0;
@@ -1075,14 +1076,16 @@ __global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const Prologu
                     const uint32_t hi = (e & 1) ? (w[e >> 1] & 0x80000000u) | ((w[e >> 1] & 0x7fff0000u) >> 3)
                                                 : ((w[e >> 1] & 0x8000u) << 16) | ((w[e >> 1] & 0x7fffu) << 13);
                     const double d = fma(__hiloint2double((int)hi, 0), 0x1p896, -first[q]);
-                    sum[q] += d;
-                    sum2[q] = fma(d, d, sum2[q]);
+                    sum[q][e & 3] += d;
+                    sum2[q][e & 3] = fma(d, d, sum2[q][e & 3]);
                 }
             }
 #pragma unroll
         for (int q = 0; q < 2; ++q) {
             const int ml = warp + kRpWarps * q;
-            double s = (top[q] & 0xffffu) >= 0x7f80u || top[q] >= 0x7f800000u ? __longlong_as_double(0x7ff8000000000000ll) : sum[q], ss = sum2[q];
+            double s = (top[q] & 0xffffu) >= 0x7f80u || top[q] >= 0x7f800000u ? __longlong_as_double(0x7ff8000000000000ll)
+                                                                                         : (sum[q][0] + sum[q][1]) + (sum[q][2] + sum[q][3]),
+                   ss = (sum2[q][0] + sum2[q][1]) + (sum2[q][2] + sum2[q][3]);
 #pragma unroll
             for (int o = 16; o > 0; o >>= 1) {
                 s += __shfl_xor_sync(0xffffffffu, s, o);
