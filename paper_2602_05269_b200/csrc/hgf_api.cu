@@ -278,7 +278,7 @@ hgf_status hgf::forward_impl(const void *x, int64_t M, const void *packed, float
     dp.gate_group = gate_group;
 
     if (!gemm) {
-        if (do_prologue && do_main) {
+        if (do_prologue && do_main && M * d_in <= 8192) {  // (plan_small's first limit, before its set-up)
             SmallLaunch<1> sl = {};
             sl.p[0] = small_problem(pp, dp, fe);
             sl.n = 1;
