@@ -108,3 +108,25 @@ def test_rejects_bad_arguments(hgf):
     # more token rows than the kernel's 32-bit row index covers: refused before anything is touched
     ptr = q.data_ptr()
     assert hgf.lib().hgf_diff_attention_forward(ptr, ptr, ptr, 40000, 1 << 20, 1, 64, 0.5, 1.0, ptr, 0, None) == 2
+
+
+@pytest.mark.parametrize("bf16", [False, True])
+def test_largest_score_among_the_first_keys_has_probability_one(hgf, bf16):
+    """A row whose largest score lies in its second 64 keys, at most 2^8 times as probable as the others: the
+    exponentials are relative to the maximum of the first 128 keys, so that probability is exactly 1 and enters the
+    second product unrounded.  Only that key has a value, so nothing else is rounded to bf16 and the output is
+    p / l in fp32: a few 2^-22 from the exponentials and the score's scaling, far below the 2^-9 of a rounded
+    probability (bf16 output: half an ulp of the result more)."""
+    L, h, dh, lam, key = 300, 4, 64, 0.5, 100
+    rng = np.random.default_rng(71)
+    q, k = np.zeros((L, 2 * h, dh), np.float32), np.zeros((L, 2 * h, dh), np.float32)
+    q[:, :, 0] = rng.uniform(3.0, 40.0, (L, 2 * h))          # score / 8 * log2(e): 0.5 to 7.3 above the others
+    k[key, :, 0] = 1.0
+    v = np.zeros((L, h * dh), np.float32)
+    v[key] = rng.standard_normal(h * dh)
+    q, k, v = (syn.f32_to_bf16_bits(a.reshape(L, -1)) for a in (q, k, v))
+    out = hgf.diff_attention_forward(_dev(q), _dev(k), _dev(v), 1, L, h, dh, lam, flags=hgf.FLAG_OUT_BF16 if bf16 else 0)
+    ref = oracle.diff_attention(q, k, v, 1, L, h, dh, lam)
+    vmax = np.abs(syn.bf16_bits_to_f32(v)).max()
+    err = np.abs(out.float().cpu().numpy() - ref)
+    assert (err <= 2e-5 * vmax + (2.0 ** -8 * np.abs(ref) if bf16 else 0.0)).all(), err.max() / vmax
