@@ -85,7 +85,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
             bulk_load_announced(s0 + L.off_w + i * steps * 1024, P.packed + (size_t)(tile0 + i) * steps * 1024, (uint32_t)steps * 1024u, bar_w);
         __syncwarp();
         if (r > 0) cluster_arrive_relaxed();  // (the other warps below)
-        pdl_wait();                           // x, the workspace and y belong to earlier work
+        pdl_wait();                           // x, the gates, the workspace and y belong to earlier work
         if (lane == 0) announce(bar_x, (uint32_t)(2 * M * K));
         __syncwarp();
         if (lane < M) bulk_load_announced(s0 + L.off_x + lane * xpitch, P.x + (size_t)lane * K, (uint32_t)(2 * K), bar_x);
@@ -113,9 +113,9 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
             gate_b = __ldg(P.gate + (n0 + g + 8 < N ? n0 + g + 8 : N - 1));
         }
     };
-    if (r > 0 && warp < nt) load_gates(warp);
     __syncthreads();
     pdl_wait();  // (every thread: what it stores to global memory may belong to earlier work)
+    if (r > 0 && warp < nt) load_gates(warp);
     bool ok = warp_wait(bar_x, status, 0x600u);
 
     // ---- x, in segments of 256 columns of one token (32 units of 16 bytes), dealt to the warps in turn -----------

@@ -92,3 +92,24 @@ def test_layernorm_group_equals_its_layers(hgf, M, K, r):
         assert float((v["xq"] != c).float().mean()) <= 1e-3 and float((i != b).float().mean()) <= 0.02
         assert float((p["y"] - a).abs().max()) <= 2e-3 * float(a.abs().max())
     group.close()
+
+
+@pytest.mark.parametrize("M,K,N,r", [(1, 2048, 2048, 32), (4, 512, 512, 16), (16, 320, 1000, 64)])
+def test_gate_written_by_the_launch_before(hgf, M, K, N, r):
+    """The gates are the outputs of a layer call still pending on the stream, which lets the next launch start early: the
+    result is that of the same gates at rest."""
+    x, packed, gamma, c = layer(hgf, M, K, N, r, 5 * K + r)
+    xg, pg, gg, cg = layer(hgf, 1, 512, N, 16, 11)
+    gates = torch.empty((1, N), device="cuda")
+
+    def pair():
+        hgf.linear_forward(xg, pg, gg, 512, N, y=gates, **cg)
+        return hgf.linear_forward(x, packed, gamma, K, N, c["At"], c["Bt"], gates[0])
+
+    pair()
+    torch.cuda.synchronize()
+    ref = hgf.linear_forward(x, packed, gamma, K, N, c["At"], c["Bt"], gates[0])
+    for _ in range(20):
+        gates.fill_(float("nan"))
+        assert torch.equal(pair(), ref)
+    hgf.check_status()
