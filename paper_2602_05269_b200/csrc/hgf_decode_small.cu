@@ -441,16 +441,47 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
 }
 
 // ---- host side ----------------------------------------------------------------------------------------------
+// Clusters that run at the same time with one CTA an SM.  They do not fill the chip: a cluster stays within a part of it whose
+// SM count is no multiple of its size.
+static int clusters_at_once(int cluster_log2) {
+    static std::atomic<int> cache[kMaxDevices][4];
+    const int dev = current_device();
+    if (dev < 0 || dev >= kMaxDevices) return 0;
+    int n = cache[dev][cluster_log2].load(std::memory_order_acquire);
+    if (n) return n;
+    static std::atomic<unsigned long long> attr_done{0};
+    auto kernel = decode_small_kernel<1, kSmallMax>;
+    if (ensure_dynamic_smem(kernel, kSmSmemMax, attr_done) != cudaSuccess) return 0;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeClusterDimension;
+    attr[0].val.clusterDim.x = 1u << cluster_log2;
+    attr[0].val.clusterDim.y = 1;
+    attr[0].val.clusterDim.z = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(1u << cluster_log2);
+    cfg.blockDim = dim3(kSmThreads);
+    cfg.dynamicSmemBytes = kSmSmemMax;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess || n <= 0) return 0;
+    cache[dev][cluster_log2].store(n, std::memory_order_release);
+    return n;
+}
+
 // Cuts the launch into clusters and lays out shared memory.  False where the two-launch path is the better one
 // (microseconds a call in a captured chain of layers with weights of their own, this path / two launches):
 //  - M K above 8192 (4096 behind a LayerNorm): every CTA quantises all of x, which the two-launch path does once.
 //    2048 -> 2048, r = 32: 5.2 / 8.0 at M = 1, 6.0 / 7.8 at M = 2, 7.5 / 7.9 at M = 4, 9.6 / 7.9 at M = 8; with a
 //    LayerNorm 6.7 / 9.0, 8.2 / 9.0, 10.9 / 9.0 at M = 1, 2, 4; 512 -> 512: 4.1 / 7.6 at M = 1, 6.4 / 9.1 at M = 16;
 //  - more shared memory than lets two CTAs share an SM: the next call's copies then wait for this one's end.
-//    2048 -> 5632 8.4 / 9.1 within (M = 4); 5632 -> 2048 14.6 / 9.9 (M = 2), 4096 -> 4096 at r = 64 13.7 / 9.6 beyond;
-//    Q, K and V of 2048 (three problems, LayerNorms) 7.7 / 14, two up-projections 2048 -> 5632 6.9 / 11.9 at M = 1.  Groups of four
-//    problems and more take it all the same: seven of 2048 -> 2048 12.5 / 16.3 at M = 1, 16.0 / 16.9 at M = 4;
+//    2048 -> 5632 8.4 / 9.1 within (M = 4); Q, K and V of 2048 (three problems, LayerNorms) 7.7 / 14, two up-projections
+//    2048 -> 5632 6.9 / 11.9 at M = 1.  Groups of four problems and more take it all the same: seven of 2048 -> 2048 12.5 / 16.3 at M = 1.
 //  - base-3 weights (no such kernel).
+// With one CTA an SM (that, and every launch of two token tiles, for its registers) a launch is cut into the clusters that run at
+// once, 33 of four or 15 of eight on 148 SMs: 37 and 18 took a second round.  In two rounds / in one / two launches: 512 -> 5632,
+// r = 32, M = 16 14.1 / 8.3 / 10.4; behind a LayerNorm 64 -> 5632 at M = 12 16.6 / 9.3 / 10.4; four of 2048 -> 2048, r = 64, M = 4 16.5 / 10.3 /
+// 12.9; seven 11.4 in one round, 18.1 as two launches.  Where the larger shares don't fit, five problems and more run in
+// two rounds: eight of 4096 -> 1536, r = 32 15.6 / - / 20.3; but four of 3072 -> 3072, r = 64 15.7 / - / 14.0.
 template <int NP>
 bool plan_small(SmallLaunch<NP> &L, uint32_t flags) {
     const int sms = device_sm_count();
@@ -470,59 +501,70 @@ bool plan_small(SmallLaunch<NP> &L, uint32_t flags) {
     L.nt = max_M <= 8 ? 1 : 2;
     L.cluster_log2 = lora <= 4 * 36 * 1024 ? 2 : 3;
     const int cluster = 1 << L.cluster_log2;
-    const int total = sms / cluster;
-    if (L.n > total) return false;
-    // clusters per problem: the largest remaining cost per cluster gets the next one; never more CTAs than row tiles
-    int cl[NP > 1 ? NP : 1], left = total - L.n;
-    for (int i = 0; i < L.n; ++i) cl[i] = 1;
-    while (left > 0) {
-        int best = -1;
-        double most = 0.0;
-        for (int i = 0; i < L.n; ++i) {
-            const SmallProblem &P = L.p[i];
-            const double per = (double)row_tiles(P.N) * ((P.K + 255) / 256) / cl[i];
-            if ((long long)cl[i] * cluster < row_tiles(P.N) && per > most) { most = per; best = i; }
+    // Clusters per problem: the largest remaining cost per cluster gets the next one; never more CTAs than row tiles.
+    // Returns the shared memory that a CTA then needs.
+    auto cut = [&](int total) -> size_t {
+        if (L.n > total) return (size_t)-1;
+        int cl[NP > 1 ? NP : 1], left = total - L.n;
+        for (int i = 0; i < L.n; ++i) cl[i] = 1;
+        if (NP == 1) {  // (what the loop comes to; this runs on every call)
+            const int most = (int)((row_tiles(L.p[0].N) + cluster - 1) >> L.cluster_log2);
+            cl[0] = most < total ? most : total;
+            left = 0;
         }
-        if (best < 0) break;
-        ++cl[best];
-        --left;
-    }
-    int begin = 0;
-    size_t h = 0, slots = 0, part = 0, lnb = 0, red = 0, x = 0, xq = 0, at = 0, bt = 0, w = 0;
-    auto up = [](size_t &v, size_t x) { v = x > v ? x : v; };
-    for (int i = 0; i < L.n; ++i) {
-        SmallProblem &P = L.p[i];
-        P.cluster_begin = begin;
-        P.ctas = cl[i] * cluster;
-        begin += cl[i];
-        const size_t steps = (size_t)((P.K + 255) / 256), tiles = (size_t)((row_tiles(P.N) + P.ctas - 1) / P.ctas);
-        const size_t E = (size_t)(P.r / 16) * L.nt * 128, per = (size_t)((P.K / 32 + cluster - 1) / cluster);
-        up(h, (size_t)2 * L.nt * 8 * kSmHPitch * 2);
-        up(slots, (size_t)cluster * E * 4);
-        up(part, (size_t)(kSmWarps / (P.r <= 16 ? 1 : (P.r == 32 ? 2 : 4))) * E * 4);
-        if (P.ln_w) up(lnb, (size_t)P.M * steps * 16);
-        up(x, (size_t)P.M * (2 * (size_t)P.K + 64));
-        up(red, tiles * L.nt * 512);
-        up(xq, (size_t)(P.M + (P.M < 8 * L.nt ? 1 : 0)) * (steps * 256 + 64));
-        up(at, (size_t)P.r * (per * 64 + ((per & 1) ? 0 : 64)));
-        up(bt, tiles * 16 * P.r * 2);
-        up(w, tiles * steps * 1024);
-    }
-    L.clusters = begin;
-    size_t off = align_up(sizeof(SmHead), 128);
-    auto take = [&](size_t bytes) { const size_t o = off; off += align_up(bytes, 128); return (int)o; };
-    L.off_h = take(h);
-    L.off_slots = take(slots);
-    L.off_part = take(part);
-    L.off_ln = take(lnb);
-    L.off_red = take(red);
-    L.off_x = take(x);
-    L.off_xq = take(xq);
-    L.off_at = take(at);
-    L.off_bt = take(bt);
-    L.off_w = take(w);
-    L.smem = (int)off;
-    return off <= (size_t)(L.n >= 4 ? kSmSmemMax : kSmSmemLimit);
+        while (left > 0) {
+            int best = -1;
+            double most = 0.0;
+            for (int i = 0; i < L.n; ++i) {
+                const SmallProblem &P = L.p[i];
+                const double per = (double)row_tiles(P.N) * ((P.K + 255) / 256) / cl[i];
+                if ((long long)cl[i] * cluster < row_tiles(P.N) && per > most) { most = per; best = i; }
+            }
+            if (best < 0) break;
+            ++cl[best];
+            --left;
+        }
+        int begin = 0;
+        size_t h = 0, slots = 0, part = 0, lnb = 0, red = 0, x = 0, xq = 0, at = 0, bt = 0, w = 0;
+        auto up = [](size_t &v, size_t x) { v = x > v ? x : v; };
+        for (int i = 0; i < L.n; ++i) {
+            SmallProblem &P = L.p[i];
+            P.cluster_begin = begin;
+            P.ctas = cl[i] * cluster;
+            begin += cl[i];
+            const size_t steps = (size_t)((P.K + 255) / 256), tiles = (size_t)((row_tiles(P.N) + P.ctas - 1) / P.ctas);
+            const size_t E = (size_t)(P.r / 16) * L.nt * 128, per = (size_t)((P.K / 32 + cluster - 1) / cluster);
+            up(h, (size_t)2 * L.nt * 8 * kSmHPitch * 2);
+            up(slots, (size_t)cluster * E * 4);
+            up(part, (size_t)(kSmWarps / (P.r <= 16 ? 1 : (P.r == 32 ? 2 : 4))) * E * 4);
+            if (P.ln_w) up(lnb, (size_t)P.M * steps * 16);
+            up(x, (size_t)P.M * (2 * (size_t)P.K + 64));
+            up(red, tiles * L.nt * 512);
+            up(xq, (size_t)(P.M + (P.M < 8 * L.nt ? 1 : 0)) * (steps * 256 + 64));
+            up(at, (size_t)P.r * (per * 64 + ((per & 1) ? 0 : 64)));
+            up(bt, tiles * 16 * P.r * 2);
+            up(w, tiles * steps * 1024);
+        }
+        L.clusters = begin;
+        size_t off = align_up(sizeof(SmHead), 128);
+        auto take = [&](size_t bytes) { const size_t o = off; off += align_up(bytes, 128); return (int)o; };
+        L.off_h = take(h);
+        L.off_slots = take(slots);
+        L.off_part = take(part);
+        L.off_ln = take(lnb);
+        L.off_red = take(red);
+        L.off_x = take(x);
+        L.off_xq = take(xq);
+        L.off_at = take(at);
+        L.off_bt = take(bt);
+        L.off_w = take(w);
+        L.smem = (int)off;
+        return off;
+    };
+    if (L.nt == 1 && cut(sms / cluster) <= (size_t)kSmSmemLimit) return true;  // two CTAs an SM
+    if (L.nt == 1 && L.n < 4) return false;
+    if (cut(clusters_at_once(L.cluster_log2)) <= (size_t)(L.n >= 4 ? kSmSmemMax : kSmSmemLimit)) return true;
+    return L.n >= 5 && cut(sms / cluster) <= (size_t)kSmSmemMax;  // in two rounds
 }
 template bool plan_small<1>(SmallLaunch<1> &, uint32_t);
 template bool plan_small<kSmallMax>(SmallLaunch<kSmallMax> &, uint32_t);

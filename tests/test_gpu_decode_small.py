@@ -113,3 +113,36 @@ def test_gate_written_by_the_launch_before(hgf, M, K, N, r):
         gates.fill_(float("nan"))
         assert torch.equal(pair(), ref)
     hgf.check_status()
+
+
+# One CTA an SM: two token tiles with more row tiles than run at once, more shared memory than lets two share an SM - in one round
+# and, where the larger shares don't fit, in two.
+ONE_ROUND = [[(16, 512, 5632, 32)], [(12, 64, 4096, 0)], [(9, 640, 3000, 64)] * 2, [(4, 2048, 2048, 64)] * 4, [(2, 1024, 2816, 16)] * 5, [(1, 4096, 1536, 32)] * 8]
+
+
+@pytest.mark.parametrize("shapes", ONE_ROUND)
+def test_one_cta_an_sm(hgf, shapes):
+    """A group against its two phases run apart: int32 accumulators bit for bit, y to 2e-5."""
+    problems = []
+    for i, (M, K, N, r) in enumerate(shapes):
+        x, packed, gamma, c = layer(hgf, M, K, N, r, 17 * i + K)
+        problems.append({"x": x, "d_in": K, "d_out": N, "packed": packed, "gamma": gamma, "y": torch.empty((M, N), device="cuda"), **c})
+    group = hgf.Group(problems)
+    yi = [torch.empty(p["y"].shape, dtype=torch.int32, device="cuda") for p in problems]
+    for i, t in enumerate(yi):
+        group.debug(i, t)
+    before = hgf.launch_count()
+    group.forward()
+    assert hgf.launch_count() - before == 1
+    hgf.check_status()
+    y1, yi1 = [p["y"].clone() for p in problems], [t.clone() for t in yi]
+    for p, t in zip(problems, yi):
+        p["y"].fill_(float("nan"))
+        t.fill_(-1)
+    group.forward_phases(1)
+    group.forward_phases(2)
+    hgf.check_status()
+    for p, t, a, b in zip(problems, yi, y1, yi1):
+        assert torch.equal(t, b)
+        assert float((p["y"] - a).abs().max()) <= 2e-5 * float(a.abs().max())
+    group.close()
