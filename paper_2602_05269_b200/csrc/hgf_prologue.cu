@@ -982,8 +982,11 @@ __host__ __device__ inline RpLayout rp_layout(int K, int r, int log2_c) {
     return L;
 }
 
-template <int JT, bool LN>
-__global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x, const FrontEnd fe,
+// PER_SM: CTAs an SM that its registers leave room for (0: as they come).  All forms fit two but the widest behind a LayerNorm, which takes 154 registers
+// and spills 36 bytes at 128: in launches of more CTAs than SMs two an SM are worth that (r = 64, 2048 -> 1024: 26.3 -> 21.1 us
+// at M = 1000, 34.5 -> 27.8 at M = 2048), in smaller ones not (22.1 -> 26.4 at M = 1184).
+template <int JT, bool LN, int PER_SM>
+__global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x, const FrontEnd fe,
                                                                    const int log2_c, unsigned int *status) {
     extern __shared__ __align__(128) uint8_t rp_smem[];
     constexpr int r = 8 * JT;
@@ -1271,11 +1274,11 @@ __global__ void __launch_bounds__(kRpThreads) rows_prologue_kernel(const Prologu
 }
 
 // Where it is used, and the cluster size: see launch_rows_prologue.
-template <int JT, bool LN>
+template <int JT, bool LN, int PER_SM = 0>
 static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, int log2_c, cudaStream_t stream) {
     static std::atomic<unsigned long long> attr_done{0};
     const RpLayout L = rp_layout(p.K, p.r, log2_c);
-    cudaError_t e = ensure_dynamic_smem(rows_prologue_kernel<JT, LN>, kRpSmemLimit, attr_done);
+    cudaError_t e = ensure_dynamic_smem(rows_prologue_kernel<JT, LN, PER_SM>, kRpSmemLimit, attr_done);
     if (e != cudaSuccess) return e;
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
@@ -1289,7 +1292,7 @@ static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPr
     attr[cfg.numAttrs].val.clusterDim.y = 1;
     attr[cfg.numAttrs].val.clusterDim.z = 1;
     ++cfg.numAttrs;
-    e = cudaLaunchKernelEx(&cfg, rows_prologue_kernel<JT, LN>, p, x, fe, log2_c, status);
+    e = cudaLaunchKernelEx(&cfg, rows_prologue_kernel<JT, LN, PER_SM>, p, x, fe, log2_c, status);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1319,26 +1322,44 @@ static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPr
 //    then come in several waves and read A^T more often than 32-token blocks do); K = 512: 9.2 / 9.5 at M = 17;
 //  - 5632 -> 2048: 29.6 / 19.1 at M = 17, 34.5 / 23.1 at M = 512; 11008 -> 4096, r = 64: 69 / 32 at M = 17, 94 / 82 at M = 1024,
 //    133 / 142 at M = 2000 (eight CTAs a cluster for its size alone: above four CTAs an SM it is left);
-//  - with a LayerNorm, 2048 -> 2048: 23.8 / 14.3 at M = 64, 51.2 / 52.2 at M = 4096; without a correction, 4096 -> 1024:
-//    14.0 / 16.7 at M = 17, 25.2 / 16.7 at M = 64, 82.6 / 62.4 at M = 4096.
-// Cluster size: CTAs for every SM, two of them on one if they fit.
+//  - rank 16, short rows, K -> 1024: 19.6 / 18.2 at K = 2048 and M = 1200, but 19.9 / 20.7 at M = 1600, 16.0 / 17.1 at K = 1280;
+//    32.3 / 25.3 at K = 4096 and M = 1600;
+//  - with a LayerNorm, 2048 -> 2048: 23.8 / 14.3 at M = 64, 51.2 / 52.2 at M = 4096; r = 64, 11008 -> 1024: 105 / 26 at M = 64,
+//    127 / 123 at M = 2048 (no limit of CTAs there: the other kernels take two launches);
+//  - with a LayerNorm and without a correction, 4096 -> 1024: 14.0 / 16.7 at M = 17, 25.2 / 16.7 at M = 64, 82.6 / 62.4 at
+//    M = 4096.  Short rows: K = 512 9.6 / 10.2 at M = 130, 10.6 / 11.1 at 700, 13.5 / 12.2 at 2000; K = 768 11.5 / 10.8 at M = 130, 15.4 /
+//    18.1 at 1500, 22.9 / 21.4 at 3000; K = 1024 12.8 / 11.1 at M = 130.  Long ones in one CTA: K = 3072 72 / 68 at M = 5000, 80.4 / 82.6
+//    at 8192.
+// Cluster size: CTAs for every SM, two of them on one if they fit; one step smaller where that many don't run at once: 1024 -> 1024,
+// M = 1168, r = 48 16.4 -> 15.0 us, M = 570 15.4 -> 13.9; 8192 -> 1024, M = 525 26.6 -> 28.5.
 static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd *fe, cudaStream_t stream) {
     const int sms = device_sm_count();
     if (!sms) return cudaErrorInvalidDevice;
     const int blocks = (p.M + kRpTokens - 1) / kRpTokens;
     int c = 0;
     while (c < 3 && (blocks << c) < sms) ++c;
+    // (registers: two CTAs an SM at most; 33 clusters of eight or 71 of four run at once on 148 SMs, more take a second round, which
+    // only long slices are worth)
+    if ((p.r >= 48 || (fe && p.r == 32)) && ((c == 3 && p.K <= 2048 && (blocks << c) > 2 * sms - sms / 4) || (c == 2 && (blocks << c) > 2 * sms - sms / 16))) --c;
     while (c < 3 && rp_layout(p.K, p.r, c).smem > 110 * 1024) ++c;  // two CTAs on an SM
     if (rp_layout(p.K, p.r, c).smem > kRpSmemLimit) return cudaErrorNotSupported;
-    const bool few = p.M <= 2048 && p.K >= 1024 && (fe || (blocks << c) <= 4 * sms);
-    if (!(p.r > 0 ? few : p.M >= 64)) return cudaErrorNotSupported;
+    bool take;
+    if (p.r == 0) {
+        take = p.M >= 64 && p.K >= (p.M <= 1024 ? 768 : (p.M < 1920 ? 1024 : 0)) && (p.M <= 7168 || c > 0 || p.K <= 2048);
+    } else {
+        take = p.M <= 2048 && p.K >= 1024;
+        if (!fe) take = take && (blocks << c) <= 4 * sms && (p.r > 16 || p.K > 2048 || p.M <= 1280);
+    }
+    if (!take) return cudaErrorNotSupported;
     const FrontEnd none = {};
     switch (p.r) {
         case 0: return fe ? launch_rows_prologue_jt<0, true>(p, x, *fe, c, stream) : cudaErrorNotSupported;
         case 16: return fe ? launch_rows_prologue_jt<2, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<2, false>(p, x, none, c, stream);
         case 32: return fe ? launch_rows_prologue_jt<4, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<4, false>(p, x, none, c, stream);
         case 48: return fe ? launch_rows_prologue_jt<6, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<6, false>(p, x, none, c, stream);
-        case 64: return fe ? launch_rows_prologue_jt<8, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<8, false>(p, x, none, c, stream);
+        case 64:
+            if (!fe) return launch_rows_prologue_jt<8, false>(p, x, none, c, stream);
+            return (blocks << c) <= sms ? launch_rows_prologue_jt<8, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<8, true, 2>(p, x, *fe, c, stream);
         default: return cudaErrorInvalidValue;
     }
 }
