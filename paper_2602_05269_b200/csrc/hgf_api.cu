@@ -385,7 +385,8 @@ struct hgf_group {
     PrologueParams *d_pps;
     QuantItem *d_quant_items; // prologue: one per (problem, token)
     LoraItem *d_lora_items;   // prologue: one per (problem, 16 columns of H, K slice)
-    int n_ln, n_quant, n_lora;  // (rows behind a LayerNorm come first)
+    int n_ln, n_quant, n_lora;  // (the rows that get a CTA each come first)
+    bool ln_warps;            // rows behind a LayerNorm get a warp each, like the others
     int4 *d_cta_range;        // per GEMV CTA: (first tile, end tile, first problem, 0)
     int grid;
     bool small;               // whole forwards take the one launch `sl` describes
@@ -534,6 +535,8 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
     g->d_quant_items = (QuantItem *)((char *)mem + off_qit);
     g->d_lora_items = (LoraItem *)((char *)mem + off_lit);
     g->n_ln = (int)(std::stable_partition(qitems.begin(), qitems.end(), [](const QuantItem &q) { return q.ln_w != nullptr; }) - qitems.begin());
+    g->ln_warps = !group_rows_by_cta(qitems.data(), g->n_ln);
+    if (g->ln_warps) g->n_ln = 0;
     g->n_quant = (int)qitems.size();
     g->n_lora = (int)litems.size();
     g->d_cta_range = (int4 *)((char *)mem + off_cta);
@@ -613,7 +616,7 @@ extern "C" hgf_status hgf_group_forward_phases(hgf_group *g, uint32_t phases, vo
     if (g->small && phases == (HGF_PHASE_PROLOGUE | HGF_PHASE_GEMV))
         return launch_small(g->sl, pdl, stream) == cudaSuccess ? HGF_OK : HGF_ERR_CUDA;
     if ((phases & HGF_PHASE_PROLOGUE) &&
-        launch_decode_prologue_group(g->d_quant_items, g->n_ln, g->n_quant, g->d_lora_items, g->n_lora, g->max_M, pdl,
+        launch_decode_prologue_group(g->d_quant_items, g->n_ln, g->ln_warps, g->n_quant, g->d_lora_items, g->n_lora, g->max_M, pdl,
                                      stream) != cudaSuccess)
         return HGF_ERR_CUDA;
     if (!(phases & HGF_PHASE_GEMV)) return HGF_OK;

@@ -207,8 +207,10 @@ struct QuantItem {
     float *mean_out, *rstd_out;  // nullable: where this row's statistics go
 };
 __host__ __device__ inline int prologue_slice_k(int max_M) { return max_M <= 8 ? 512 : 256; }
-// (the first n_ln quantisation items are the ones behind a LayerNorm)
-cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_ln, int n_quant,
+// Whether n rows behind a LayerNorm get a CTA each (true) or a warp each.
+bool group_rows_by_cta(const QuantItem *items, int n);
+// (the first n_ln quantisation items are rows that get a CTA each; ln_warps: rows behind a LayerNorm are among the others)
+cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_ln, bool ln_warps, int n_quant,
                                          const LoraItem *d_lora_items, int n_lora, int max_M, bool pdl,
                                          cudaStream_t stream);
 cudaError_t launch_gemm_prologue(const PrologueParams &p, const GemmPrologueExtra &x, cudaStream_t stream);

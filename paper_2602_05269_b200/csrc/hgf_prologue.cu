@@ -575,7 +575,8 @@ __device__ void block_quant_row_ln(const QuantItem &q, uint8_t *buf, int tid) {
     }
 }
 
-template <int NT>
+// LN_WARPS: rows behind a LayerNorm are among the warps' rows (without them the kernel goes without their code).
+template <int NT, bool LN_WARPS>
 __global__ void __launch_bounds__(kPgThreads, 1)
 decode_prologue_group_kernel(const QuantItem *quant_items, int n_ln, int n_quant, const LoraItem *lora, int n_lora) {
     constexpr int CH = 16 / NT;                       // 32-column chunks per item
@@ -599,7 +600,7 @@ decode_prologue_group_kernel(const QuantItem *quant_items, int n_ln, int n_quant
     if (q_first < n_quant) q = quant_items[q_first];
     pdl_wait();  // x, and the scratch this kernel overwrites, belong to earlier work
 
-    // rows behind a LayerNorm (the first n_ln items): a CTA each, from the last CTA down
+    // the first n_ln items, rows behind a LayerNorm: a CTA each, from the last CTA down
     for (int i = gridDim.x - 1 - blockIdx.x; i < n_ln; i += gridDim.x) {
         const QuantItem row = quant_items[i];
         block_quant_row_ln(row, pg_smem, threadIdx.x);
@@ -609,7 +610,8 @@ decode_prologue_group_kernel(const QuantItem *quant_items, int n_ln, int n_quant
     for (int i = q_first; i < n_quant; i += nw) {
         QuantItem q_next = q;
         if (i + nw < n_quant) q_next = quant_items[i + nw];  // travels while this row is worked on
-        warp_quant_row(q, buf - 16 * lane, pg_smem + warp * kWarpBytes, kWarpBytes, lane);
+        if (LN_WARPS && q.ln_w) warp_quant_row_ln(q, lane);
+        else warp_quant_row(q, buf - 16 * lane, pg_smem + warp * kWarpBytes, kWarpBytes, lane);
         q = q_next;
     }
 
@@ -1476,36 +1478,46 @@ cudaError_t launch_gemm_prologue_ln(const PrologueParams &p, const GemmPrologueE
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_ln, int n_quant, const LoraItem *d_lora_items, int n_lora, int max_M, bool pdl,
-                                         cudaStream_t stream) {
-    static std::atomic<unsigned long long> attr_done1{0}, attr_done2{0};
+// A CTA works one row after the other, eight warps eight rows at a time but each slowly: microseconds of a group's forward, r = 32,
+// rows by warps / by CTAs: K = 512 19.4 / 18.6 with 240 rows, 20.3 / 20.7 with 320, 25.0 / 41.3 with 1728; K = 1024 22.9 / 22.3 with 400,
+// 23.3 / 24.4 with 448; K = 2048 30.0 / 26.7 with 320, 29.0 / 27.6 with 448, 30.4 / 30.7 with 576, 73 / 85 with 1728; K = 3072
+// 37.5 / 36.7 with 576, 41.0 / 41.9 with 720.
+bool group_rows_by_cta(const QuantItem *items, int n) {
+    const int sms = device_sm_count();
+    int K = 0;
+    for (int i = 0; i < n; ++i) K = items[i].K > K ? items[i].K : K;
+    return 4 * n <= sms * (K >= 3072 ? 18 : (K >= 2048 ? 14 : (K >= 1024 ? 11 : 8)));
+}
+
+template <int NT, bool LN_WARPS>
+static cudaError_t launch_prologue_group_nt(const QuantItem *d_quant_items, int n_ln, int n_quant, const LoraItem *d_lora_items, int n_lora, bool pdl,
+                                            cudaStream_t stream) {
+    static std::atomic<unsigned long long> attr_done{0};
     const int sm_count = device_sm_count();
     if (!sm_count) return cudaErrorInvalidDevice;
-    const int smem1 = kPgWarps * 16 * (1024 + 512), smem2 = kPgWarps * 8 * (1024 + 1024);
-    {
-        cudaError_t e = ensure_dynamic_smem(decode_prologue_group_kernel<1>, smem1, attr_done1);
-        if (e != cudaSuccess) return e;
-        e = ensure_dynamic_smem(decode_prologue_group_kernel<2>, smem2, attr_done2);
-        if (e != cudaSuccess) return e;
-    }
+    constexpr int smem = kPgWarps * (16 / NT) * (1024 + 512 * NT);
+    cudaError_t e = ensure_dynamic_smem(decode_prologue_group_kernel<NT, LN_WARPS>, smem, attr_done);
+    if (e != cudaSuccess) return e;
     const int most = n_lora > n_quant - n_ln ? n_lora : n_quant - n_ln;
-    int blocks = (most + kPgWarps - 1) / kPgWarps;
-    if (n_ln) blocks = (most + kPgWarps - 1) / kPgWarps + n_ln;  // CTAs of their own for the rows behind a LayerNorm
+    int blocks = (most + kPgWarps - 1) / kPgWarps + n_ln;  // CTAs of their own for the first n_ln rows
     blocks = blocks < sm_count ? blocks : sm_count;
     if (blocks < 1) blocks = 1;
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = prologue_cfg(blocks, pdl, stream, attr);
     cfg.blockDim = dim3(kPgThreads);
-    cudaError_t e;
-    if (max_M <= 8) {
-        cfg.dynamicSmemBytes = smem1;
-        e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<1>, d_quant_items, n_ln, n_quant, d_lora_items, n_lora);
-    } else {
-        cfg.dynamicSmemBytes = smem2;
-        e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<2>, d_quant_items, n_ln, n_quant, d_lora_items, n_lora);
-    }
+    cfg.dynamicSmemBytes = smem;
+    e = cudaLaunchKernelEx(&cfg, decode_prologue_group_kernel<NT, LN_WARPS>, d_quant_items, n_ln, n_quant, d_lora_items, n_lora);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
+}
+
+cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_ln, bool ln_warps, int n_quant, const LoraItem *d_lora_items, int n_lora,
+                                         int max_M, bool pdl, cudaStream_t stream) {
+    if (max_M <= 8)
+        return ln_warps ? launch_prologue_group_nt<1, true>(d_quant_items, n_ln, n_quant, d_lora_items, n_lora, pdl, stream)
+                        : launch_prologue_group_nt<1, false>(d_quant_items, n_ln, n_quant, d_lora_items, n_lora, pdl, stream);
+    return ln_warps ? launch_prologue_group_nt<2, true>(d_quant_items, n_ln, n_quant, d_lora_items, n_lora, pdl, stream)
+                    : launch_prologue_group_nt<2, false>(d_quant_items, n_ln, n_quant, d_lora_items, n_lora, pdl, stream);
 }
 
 }  // namespace hgf

@@ -171,3 +171,32 @@ def test_attention_projections_as_one_group(hgf, M):
     # Q, K and V have LayerNorms of their own: three quantisations of the same x, all different
     assert not np.array_equal(views[0]["xq"].cpu().numpy(), views[1]["xq"].cpu().numpy())
     group.close()
+
+
+@pytest.mark.parametrize("n,M,K,N", [(18, 16, 192, 16), (19, 16, 192, 16), (26, 16, 1088, 24), (40, 1, 64, 8)])
+def test_group_with_many_rows_behind_layernorms(hgf, n, M, K, N):
+    """More LayerNorm rows than CTAs are given to them, and fewer: a warp or a CTA a row, codes and int32 accumulators bit for
+    bit under the library's statistics."""
+    probs, hosts = [], []
+    for i in range(n):
+        L = syn.make_layer(syn.LayerShape("rows", K, N, 16), M, config=29, layer=i)
+        packed, gamma = hgf.pack_ternary(dev(L["W"]))
+        w, b = ln_params(K, 70 + i)
+        probs.append({"x": dev(L["x"], torch.bfloat16), "packed": packed, "gamma": gamma, "d_in": K, "d_out": N, "y": torch.zeros((M, N), device="cuda"),
+                      "At": dev(L["At"], torch.float16), "Bt": dev(L["Bt"], torch.float16), "gate": dev(L["gate"]), "gate_group": 1,
+                      "ln_weight": dev(w), "ln_bias": dev(b), "eps": 1e-5, "mean_out": torch.zeros(M, device="cuda"), "rstd_out": torch.zeros(M, device="cuda")})
+        hosts.append((L, oracle.ternarise(L["W"], np.float32(gamma)), gamma, w, b))
+    group = hgf.Group(probs)
+    y_ints = [torch.full((M, N), -1, dtype=torch.int32, device="cuda") for _ in probs]
+    views = [group.debug(i, t) for i, t in enumerate(y_ints)]
+    group.forward()
+    hgf.check_status()
+    for q, view, y_int, (L, T, gamma, w, b) in zip(probs, views, y_ints, hosts):
+        mean_g, rstd_g = q["mean_out"].cpu().numpy(), q["rstd_out"].cpu().numpy()
+        mean_o, rstd_o = oracle.ln_stats(L["x"], 1e-5)
+        assert np.all(np.abs(mean_g - mean_o) <= 2e-7 * np.sqrt(1.0 / rstd_o ** 2 + mean_o ** 2)) and np.all(np.abs(rstd_g / rstd_o - 1) <= 3e-7)
+        own = oracle.forward_ln(L["x"], T, gamma, w, b, 1e-5, L["At"], L["Bt"], L["gate"], mean=mean_g, rstd=rstd_g)
+        assert np.array_equal(view["xq"].cpu().numpy(), own["xq"]) and np.array_equal(view["gamma_x"].cpu().numpy(), own["gamma_x"])
+        assert np.array_equal(y_int.cpu().numpy(), own["y_int"])
+        assert np.abs(q["y"].cpu().numpy() - own["y"]).max() <= TOL_DECODE * np.abs(own["y"]).max()
+    group.close()
