@@ -581,6 +581,7 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
         g->sl.n = n;
         for (int i = 0; i < n; ++i) {
             g->sl.p[i] = small_problem(pps[i], dps[i], fes[i]);
+            g->sl.p[i].dbg_y_int_at = &g->d_probs[i].dbg_y_int;
             for (int k = 0; k < i; ++k)
                 if (pps[k].xq == pps[i].xq) g->sl.p[i].xq = nullptr, g->sl.p[i].gamma_x = nullptr;  // the first problem with this x writes them
         }
@@ -597,7 +598,6 @@ extern "C" hgf_status hgf_group_debug(hgf_group *g, int32_t index, int32_t *y_in
     DecodeProblem &P = g->h_probs[(size_t)index];
     if (P.dbg_y_int != y_int) {
         P.dbg_y_int = y_int;
-        if (g->small) g->sl.p[index].dbg_y_int = y_int;
         if (cudaMemcpy(g->d_probs + index, &P, sizeof(DecodeProblem), cudaMemcpyHostToDevice) != cudaSuccess) return HGF_ERR_CUDA;
     }
     if (views) {

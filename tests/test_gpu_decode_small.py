@@ -115,6 +115,39 @@ def test_gate_written_by_the_launch_before(hgf, M, K, N, r):
     hgf.check_status()
 
 
+@pytest.mark.parametrize("n", [3, 30])
+def test_captured_group_follows_the_debug_buffer(hgf, n):
+    """A captured forward writes the integer accumulators where hgf_group_debug last said, also when that was after the
+    capture - one launch and two."""
+    M, K, N, r = 2, 512, 72, 16
+    problems = []
+    for i in range(n):
+        x, packed, gamma, c = layer(hgf, M, K, N, r, i)
+        problems.append({"x": x, "d_in": K, "d_out": N, "packed": packed, "gamma": gamma, "y": torch.empty((M, N), device="cuda"), **c})
+    group = hgf.Group(problems)
+    before = hgf.launch_count()
+    group.forward()
+    assert hgf.launch_count() - before == (1 if n == 3 else 2)
+    torch.cuda.synchronize()
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        group.forward()
+    y_int = torch.full((M, N), -7, dtype=torch.int32, device="cuda")
+    xq = group.debug(1, y_int)["xq"]
+    graph.replay()
+    torch.cuda.synchronize()
+    T = hgf.unpack_ternary(problems[1]["packed"], N, K)
+    assert torch.equal(y_int.double(), xq.double() @ T.double().T)
+    group.debug(1, None)
+    y_int.fill_(-7)
+    graph.replay()
+    torch.cuda.synchronize()
+    assert bool((y_int == -7).all())
+    hgf.check_status()
+    del graph
+    group.close()
+
+
 # One CTA an SM: two token tiles with more row tiles than run at once, more shared memory than lets two share an SM - in one round
 # and, where the larger shares don't fit, in two.
 ONE_ROUND = [[(16, 512, 5632, 32)], [(12, 64, 4096, 0)], [(9, 640, 3000, 64)] * 2, [(4, 2048, 2048, 64)] * 4, [(2, 1024, 2816, 16)] * 5, [(1, 4096, 1536, 32)] * 8]
