@@ -4,10 +4,9 @@
 //     dW = dY^T Xd,  dX = dY Wd + dZ A^T,  dZ = ((dY (.) g) B^T) (.) SiLU'(x A),
 //     dA = x^T dZ,   dB = g (.) (H^T dY),   dg = sum_m dY (.) (H B)
 // with Xd = x~ gamma_x / 127 and Wd = gamma_W t.  Seven matrix products on one generic tcgen05 bf16 GEMM
-// (C = A B^T, both operands with the contraction index contiguous), plus preparation kernels that bring
-// the operands into that form: transposes of dY, x, x~ and of the small matrices, and the ternary codes
-// expanded as a transposed bf16 matrix.  The quantised activations enter as exact bf16 integers
-// (|x~| <= 127) and the per-token scale is folded into dY; the ternary codes enter as exact -1 / 0 / +1.
+// (C = A B^T, each operand read in the form it is stored in), plus preparation kernels: Xd as a bf16 matrix (the
+// quantiser again, its codes times their scale), the ternary codes as a bf16 matrix of exact -1 / 0 / +1, A and
+// g (.) B in bf16.  gamma_W is applied to the fp32 accumulator.
 #include "hgf_tc.cuh"
 #include "hgf_warp.cuh"
 
@@ -476,6 +475,7 @@ __global__ void __launch_bounds__(256) bw_gate_kernel(float *G, const __half *Bt
 }
 
 constexpr int kBwSplitsMax = 16;
+constexpr int kBwQuantMaxK = 4096;  // up to here a row fits a warp's registers (bw_quant_kernel): no codes and scales in memory
 
 struct BwLayout {
     size_t xq, gamma_x, xd, T, At_b, gBt, z, h_b, dh, dz_b, dzs_b, G, partials, total;
@@ -485,8 +485,8 @@ static BwLayout bw_layout(int64_t M, int64_t K, int64_t N, int32_t r) {
     size_t off = 0;
     auto take = [&](size_t bytes) { const size_t o = off; off += align_up(bytes, 256); return o; };
     const size_t rr = (size_t)(r > 0 ? r : 16);
-    L.xq = take((size_t)M * K);
-    L.gamma_x = take((size_t)M * 4);
+    L.xq = take(K > kBwQuantMaxK ? (size_t)M * K : 0);
+    L.gamma_x = take(K > kBwQuantMaxK ? (size_t)M * 4 : 0);
     L.xd = take((size_t)M * K * 2);
     L.T = take((size_t)N * K * 2);
     L.At_b = take(rr * K * 2);
@@ -545,10 +545,10 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     const TcOperand x_k = {(const __nv_bfloat16 *)x, K, false}, x_mn = {(const __nv_bfloat16 *)x, K, true};
 
     if (grads->dW) {  // Algorithm 1, steps 1-2 again, then dW[n][k] = sum_m dY[m][n] Xd[m][k]
-        if (K <= 4096) {  // a row fits a warp's registers
+        if (K <= kBwQuantMaxK) {
             const unsigned rows8 = (unsigned)((Mi + 7) / 8);
             const __nv_bfloat16 *xp = (const __nv_bfloat16 *)x;
-            ok = (K <= 2048 ? launch_chained(bw_quant_kernel<8>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))
+            ok = (K <= kBwQuantMaxK / 2 ? launch_chained(bw_quant_kernel<8>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))
                             : launch_chained(bw_quant_kernel<16>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))) == cudaSuccess;
         } else {
             PrologueParams pp = {};

@@ -42,6 +42,18 @@ def test_packed_bytes_and_workspace(hgf):
     assert hgf.workspace_bytes(512, 2048, 2048, 32) >= 512 * 2048 + 512 * 64 * 2
 
 
+def test_backward_workspace_holds_what_the_pass_uses(hgf):
+    """Up to 4096 columns the quantiser goes straight to bf16: no room for codes and scales is asked for."""
+    def rest(M, K, N, r):       # every other section: bf16 Xd, T, A, g B, H, dZ (twice); fp32 Z, dH, G, 16 partial results
+        up = lambda n: -(-n // 256) * 256  # noqa: E731
+        return sum(map(up, (2 * M * K, 2 * N * K, 2 * r * K, 2 * N * r, 4 * M * r, 2 * M * r, 4 * M * r, 2 * M * r, 2 * M * r, 4 * N * r,
+                            16 * 4 * max(M, N, K) * r)))
+    for M, K, N, r in ((8192, 2048, 5632, 32), (100, 4096, 72, 16), (17, 64, 8, 64)):
+        assert hgf.backward_workspace_bytes(M, K, N, r) == rest(M, K, N, r)
+    for M, K, N, r in ((100, 4160, 72, 16), (8192, 5632, 2048, 32)):
+        assert hgf.backward_workspace_bytes(M, K, N, r) == rest(M, K, N, r) + -(-M * K // 256) * 256 + -(-4 * M // 256) * 256
+
+
 def test_tmax_matches_paper_example(hgf):
     # 7B parameters, FP16, 500 GB/s -> about 35 tokens/s (paper, introduction)
     t = hgf.tmax_tokens_per_s(500e9, 7e9, 16)
