@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 import torch
 
-from paper_2602_05269_b200 import inputs as syn
+import oracle
 
 pytestmark = pytest.mark.gpu
 
@@ -31,6 +31,13 @@ def layer(hgf, M, K, N, r, seed):
     if r:
         c = {"At": rn((r, K), K ** -0.5).half(), "Bt": rn((N, r), r ** -0.5).half(), "gate": torch.rand(N, generator=g, device="cuda")}
     return x.bfloat16(), packed, gamma, c
+
+
+def host(t):
+    """A device tensor as the oracle takes it: 16-bit floats by their bit patterns, None as it is."""
+    if t is None:
+        return None
+    return t.cpu().view(torch.int16).numpy().view(np.uint16) if t.dtype in (torch.bfloat16, torch.float16) else t.cpu().numpy()
 
 
 @pytest.mark.parametrize("M,K,N,r", SHAPES)
@@ -59,7 +66,8 @@ def test_one_launch_equals_two(hgf, M, K, N, r):
 @pytest.mark.parametrize("M,K", [(1, 64), (2, 2048), (4, 1024), (12, 320)])
 @pytest.mark.parametrize("r", [0, 32])
 def test_layernorm_group_equals_its_layers(hgf, M, K, r):
-    """A group of three projections of one x, each behind its LayerNorm, and the same three as two-launch groups of one."""
+    """A group of three projections of one x, each behind its LayerNorm, in one launch: against the oracle, codes, scales
+    and int32 accumulators bit for bit under the library's own statistics; and against the same group's two phases."""
     g = torch.Generator(device="cuda").manual_seed(K + M)
     problems = []
     x = (torch.randn((M, K), generator=g, device="cuda") * 3 + 1).bfloat16()
@@ -81,9 +89,15 @@ def test_layernorm_group_equals_its_layers(hgf, M, K, r):
     y1, yi1, xq1 = [p["y"].clone() for p in problems], [t.clone() for t in yi], [v["xq"].clone() for v in views]
     xd = x.double()
     mean, var = xd.mean(1), xd.var(1, unbiased=False)
-    for p in problems:
+    for p, view, i, y in zip(problems, views, yi, y1):
         assert float((p["mean_out"].double() - mean).abs().max()) <= 2e-7 * float(xd.square().mean().sqrt())
         assert float((p["rstd_out"].double() * (var + 1e-5).sqrt() - 1).abs().max()) <= 3e-7
+        T = hgf.unpack_ternary(p["packed"], p["d_out"], K).cpu().numpy()
+        ref = oracle.forward_ln(host(x), T, p["gamma"], host(p["ln_weight"]), host(p["ln_bias"]), 1e-5, host(p["At"]), host(p["Bt"]),
+                                host(p["gate"]), gate_group=16, mean=host(p["mean_out"]), rstd=host(p["rstd_out"]))
+        assert np.array_equal(host(view["xq"]), ref["xq"]) and np.array_equal(host(view["gamma_x"]), ref["gamma_x"])
+        assert np.array_equal(host(i), ref["y_int"])
+        assert np.abs(host(y) - ref["y"]).max() <= 2e-5 * np.abs(ref["y"]).max()
     group.forward_phases(1)
     group.forward_phases(2)
     hgf.check_status()
@@ -178,4 +192,41 @@ def test_one_cta_an_sm(hgf, shapes):
     for p, t, a, b in zip(problems, yi, y1, yi1):
         assert torch.equal(t, b)
         assert float((p["y"] - a).abs().max()) <= 2e-5 * float(a.abs().max())
+    group.close()
+
+
+# In the first two groups one problem asks for two token tiles: in the others the second tile has no token and reads the row of zeros.
+UNEQUAL = [[(12, 320, 200, 32), (3, 640, 56, 16), (8, 512, 1000, 64), (1, 64, 24, 0)], [(9, 192, 72, 48), (16, 512, 512, 16), (1, 256, 17, 32)],
+           [(5, 1024, 100, 16), (1, 1088, 300, 32), (7, 64, 2048, 64), (2, 704, 8, 0), (3, 320, 640, 48)]]
+
+
+@pytest.mark.parametrize("shapes", UNEQUAL)
+def test_group_of_unequal_problems(hgf, shapes):
+    """Problems of unequal token counts, lengths and ranks in one launch, against the oracle: codes, scales and int32
+    accumulators bit for bit, y to the decode path's 2e-5."""
+    problems = []
+    for i, (M, K, N, r) in enumerate(shapes):
+        x, packed, gamma, c = layer(hgf, M, K, N, r, 31 * i + K)
+        problems.append({"x": x, "d_in": K, "d_out": N, "packed": packed, "gamma": gamma, "y": torch.empty((M, N), device="cuda"), **c})
+    group = hgf.Group(problems)
+    yi = [torch.full((p["x"].shape[0], p["d_out"]), -1, dtype=torch.int32, device="cuda") for p in problems]
+    views = [group.debug(i, t) for i, t in enumerate(yi)]
+    before = hgf.launch_count()
+    group.forward()
+    assert hgf.launch_count() - before == 1
+    hgf.check_status()
+    whole = [p["y"].clone() for p in problems]
+    for p, view, i in zip(problems, views, yi):
+        T = hgf.unpack_ternary(p["packed"], p["d_out"], p["d_in"]).cpu().numpy()
+        ref = oracle.forward(host(p["x"]), T, p["gamma"], host(p["At"]), host(p["Bt"]), host(p["gate"]))
+        assert np.array_equal(host(view["xq"]), ref["xq"]) and np.array_equal(host(view["gamma_x"]), ref["gamma_x"])
+        assert np.array_equal(host(i), ref["y_int"])
+        assert np.abs(host(p["y"]) - ref["y"]).max() <= 2e-5 * np.abs(ref["y"]).max()
+    # what the launch left in the workspace serves the group's contraction run on its own
+    for p in problems:
+        p["y"].fill_(float("nan"))
+    group.forward_phases(2)
+    hgf.check_status()
+    for p, y in zip(problems, whole):
+        assert float((p["y"] - y).abs().max()) <= 2e-5 * float(y.abs().max())
     group.close()
