@@ -242,8 +242,10 @@ struct SmallProblem {
     float *hpart;
     int8_t *dbg_xq;                  // nullable debug copies
     float *dbg_gamma_x, *dbg_h;
-    int32_t *dbg_y_int;
-    int32_t *const *dbg_y_int_at;    // (groups) the device word that holds it: a captured launch follows hgf_group_debug
+    union {
+        int32_t *dbg_y_int;
+        int32_t *const *dbg_y_int_at;  // (groups) the device word that holds it: a captured launch follows hgf_group_debug
+    };
     float gw_over_127, eps;
     int M, K, N, r;
     uint32_t flags;

@@ -116,8 +116,8 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
     __syncthreads();
     pdl_wait();  // (every thread: what it stores to global memory may belong to earlier work)
     if (r > 0 && warp < nt) load_gates(warp);
-    int32_t *dbg_y_int = P.dbg_y_int;
-    if constexpr (NP > 1) dbg_y_int = *P.dbg_y_int_at;
+    int32_t *group_dbg_y_int = nullptr;
+    if constexpr (NP > 1) group_dbg_y_int = *P.dbg_y_int_at;
     bool ok = warp_wait(bar_x, status, 0x600u);
 
     // ---- x, in segments of 256 columns of one token (32 units of 16 bytes), dealt to the warps in turn -----------
@@ -436,7 +436,7 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
                     const size_t o = (size_t)m * N + row;
                     if (out_bf16) reinterpret_cast<__nv_bfloat16 *>(P.y)[o] = __float2bfloat16_rn(y);
                     else reinterpret_cast<float *>(P.y)[o] = y;
-                    if (dbg_y_int) dbg_y_int[o] = y_int;
+                    if (int32_t *dbg = NP > 1 ? group_dbg_y_int : P.dbg_y_int) dbg[o] = y_int;
                 }
             }
     }
