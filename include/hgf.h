@@ -148,12 +148,12 @@ size_t hgf_workspace_bytes(int64_t M, int64_t d_in, int64_t d_out, int32_t r, ui
  * pointers.  M <= HGF_DECODE_MAX_M runs the bandwidth-bound GEMV path, larger M the tcgen05
  * int8 GEMM path (which additionally needs d_out % 8 == 0).  The GEMV path keeps the layer's
  * quantised activations in shared memory; a problem with (M + 1) * (d_in_padded + 64) above about
- * 104 KiB (no shape of the paper's model classes at M <= 16) takes the GEMM path as well.
+ * 104 KiB takes the GEMM path as well (of the paper's shapes d_in = 8640 from M = 12 and 11008 from M = 9 on).
  * Calls on the same workspace must not overlap on the device.
  * Launch overlap: the decode kernels are launched with programmatic stream serialization and start
- * fetching packed, At, Bt and gate before the preceding work on `stream` has finished (they wait for
- * that work before touching x, the workspace or y).  packed, At, Bt and gate must therefore not be written
- * by work still pending on `stream`; pass HGF_FLAG_NO_PDL if they might be.
+ * fetching packed, At and Bt before the preceding work on `stream` has finished (they wait for that work
+ * before touching x, gate, the workspace or y).  packed, At and Bt must therefore not be written by work
+ * still pending on `stream`; pass HGF_FLAG_NO_PDL if they might be.
  */
 hgf_status hgf_linear_forward(const void *x, int64_t M, const void *packed, float gamma,
                               int64_t d_in, int64_t d_out, const void *At, const void *Bt,
@@ -162,12 +162,14 @@ hgf_status hgf_linear_forward(const void *x, int64_t M, const void *packed, floa
                               void *stream);
 
 /*
- * The two launches of hgf_linear_forward separately (both bits together are hgf_linear_forward):
+ * The two halves of hgf_linear_forward as launches of their own (both bits together are hgf_linear_forward):
  * HGF_PHASE_PROLOGUE runs Algorithm 1 steps 1-2 and 5-6 (activation quantisation, H = SiLU(x A))
  * into the workspace; HGF_PHASE_GEMV runs steps 3-4 and 7-8 (the ternary contraction - GEMV or
  * tensor-core GEMM, whichever path the problem takes - with dequantisation, up-projection and gated
- * fusion) from what the last prologue call with the same arguments left in the workspace.  For
- * timing the two kernels apart, and for callers that re-run the contraction of an unchanged input.
+ * fusion) from what the last prologue call with the same arguments, or the last whole call, left in the
+ * workspace.  For timing the halves apart, and for callers that re-run the contraction of an unchanged input.
+ * A whole call of a small decode problem is one launch of another kernel, which forms x A in another order of
+ * fp32 sums: its time is not the sum of the halves'.
  */
 #define HGF_PHASE_PROLOGUE 0x1u
 #define HGF_PHASE_GEMV 0x2u
@@ -195,7 +197,8 @@ hgf_status hgf_linear_forward_phases(const void *x, int64_t M, const void *packe
  * 0 or 1 = one per channel, d_out / n_heads = one per head, >= d_out = the paper's scalar gate;
  * it must be 1, a multiple of 16, or >= d_out.  mean_out / rstd_out: nullable device fp32 [M], receive
  * the statistics the kernels used (for parity checks).  Everything else as hgf_linear_forward, same
- * workspace size.  With a LayerNorm the GEMM path takes one more launch (normalise + quantise).
+ * workspace size.  On the GEMM path the normalisation rides in the prologue's launch or, for large batches and
+ * short rows, is one more.
  */
 typedef struct {
     const float *ln_weight;
@@ -227,7 +230,7 @@ hgf_status hgf_linear_forward_ln(const void *x, int64_t M, const void *packed, f
  * process exits).  It calls no allocator of any kind.  Arguments are those of hgf_linear_forward
  * without workspace and debug outputs; results are the same.
  *
- * Limits: only decode-sized problems (those hgf_linear_forward serves with its GEMV path, M <=
+ * Limits: only decode-sized problems (those hgf_linear_forward serves on its decode path, M <=
  * HGF_DECODE_MAX_M) with hgf_workspace_bytes(M, d_in, d_out, r, flags) <= HGF_STATIC_SCRATCH_BYTES.
  * The scratch holds M * d_in bytes of quantised activations plus (r / 16) * ceil(d_in / 256) KiB of
  * partial sums of x A and a few KiB of per-token values: with r = 64 that is every model shape of
@@ -251,7 +254,7 @@ hgf_status hgf_linear_forward_static(const void *x, int64_t M, const void *packe
                                      void *stream);
 
 /*
- * A group of independent decode-sized layer problems served by one pair of launches.  The paper's
+ * A group of independent decode-sized layer problems served by one pair of launches, or by one.  The paper's
  * blocks evaluate several HGF layers on the same or on unrelated inputs with no dependency between
  * them (Section 2.4, Definition "HGF Attention Projections": Q, K and V are three HGF layers of the
  * same X; the MLP's two up-projections likewise), and each is small against the launch latency,
@@ -265,8 +268,8 @@ hgf_status hgf_linear_forward_static(const void *x, int64_t M, const void *packe
  * workspace on the current device; it is a set-up call, not for the hot path.
  * hgf_group_forward only enqueues: one prologue launch and one GEMV launch for the whole group,
  * which streams the packed weights of all its problems as one sequence split evenly over the SMs;
- * up to eight problems whose weights fit the chip's shared memory are one launch in all, as is a
- * small hgf_linear_forward.
+ * up to eight problems with max M * max d_in <= 8192 (4096 behind a LayerNorm), two-bit weights and shares
+ * that fit the chip's shared memory are one launch in all, as is an hgf_linear_forward of that size.
  * Forward calls of one group must not overlap on the device.  hgf_group_destroy frees the group
  * (the caller makes sure no forward is still running).
  */
@@ -301,10 +304,12 @@ hgf_status hgf_group_create_ln(const hgf_problem *problems /* host array */,
                                uint32_t flags, hgf_group **out);
 hgf_status hgf_group_forward(hgf_group *group, void *stream);
 /*
- * The two launches of hgf_group_forward separately, for measurement: HGF_PHASE_PROLOGUE runs
+ * The two halves of hgf_group_forward as launches of their own, for measurement: HGF_PHASE_PROLOGUE runs
  * Algorithm 1 steps 1-2 and 5-6 (activation quantisation, H = SiLU(x A)) into the group's
- * workspace, HGF_PHASE_GEMV steps 3-4 and 7-8 from what the last prologue left there.  Both bits
- * together are hgf_group_forward.
+ * workspace, HGF_PHASE_GEMV steps 3-4 and 7-8 from what the last prologue, or the last whole forward, left
+ * there.  Both bits together are hgf_group_forward: for a small group that is one launch of another kernel,
+ * whose time is not the sum of the halves'.  Behind a LayerNorm that kernel sums the statistics in another
+ * order, so they may differ in the last bit of their binary32 value, and a code then by one.
  */
 hgf_status hgf_group_forward_phases(hgf_group *group, uint32_t phases, void *stream);
 /*
@@ -382,9 +387,9 @@ hgf_status hgf_linear_backward(const void *x, int64_t M, const void *packed, flo
                                size_t workspace_bytes, uint32_t flags, void *stream);
 
 /*
- * Device-side waits in the GEMM path are bounded; when one gives up the kernel records it and
- * returns.  This call synchronises `stream`, reads and clears that record, and returns
- * HGF_ERR_TIMEOUT if a wait gave up since the last check (HGF_OK otherwise).
+ * Device-side waits are bounded; when one gives up the kernel records it and returns.  This call
+ * synchronises `stream`, reads and clears that record, and returns HGF_ERR_TIMEOUT if a wait gave up
+ * since the last check (HGF_OK otherwise).  Outputs and workspaces of the calls since are undefined then.
  */
 hgf_status hgf_check_status(void *stream);
 

@@ -12,7 +12,7 @@
 //  - x A needs all of A^T, too much for every CTA: the CTAs of a cluster take one slice of K each and
 //    exchange their partial sums through distributed shared memory, in rank order.  The cluster barrier runs under
 //    the integer products.
-//  - the eight warps split K (column tiles of 256) and, where K is short, the row tiles; their integer sums meet in
+//  - the sixteen warps split K (column tiles of 256) and, where K is short, the row tiles; their integer sums meet in
 //    shared memory (exact, so in any order).
 // Two CTAs fit an SM when a share is small, so the next call's CTAs can be fetching their weights while this one
 // works.
@@ -121,8 +121,8 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
     bool ok = warp_wait(bar_x, status, 0x600u);
 
     // ---- x, in segments of 256 columns of one token (32 units of 16 bytes), dealt to the warps in turn -----------
-    // Few segments (one or two tokens): the first eight warps quantise while the others compute x A; else every warp
-    // does both.
+    // At most one a warp (one token up to K = 4096, two up to 2048, ...): the first eight warps quantise while the others
+    // compute x A; else every warp does both.
     const int segs = steps;
     const bool apart = r > 0 && M * segs <= kSmWarps;
     const int q_warps = apart ? kSmWarps / 2 : kSmWarps, a_warps = apart ? kSmWarps / 2 : kSmWarps, a_warp = warp - (kSmWarps - a_warps);
@@ -390,7 +390,9 @@ decode_small_kernel(const __grid_constant__ SmallLaunch<NP> L, unsigned int *sta
         }
     }
     __syncthreads();
-    if (!ok) {  // a copy never landed (reported): this warp writes nothing; bounded drain, then leave
+    // A copy never landed (reported; what the call wrote is undefined): bounded drain, then leave.  Only warps that waited for it
+    // know; telling the others through shared memory cost every call 0.1 us.
+    if (!ok) {
         for (uint32_t i = 0; i < (1u << 16) && !(dmbar_try_wait(bar_a, 0) && dmbar_try_wait(bar_w, 0) && dmbar_try_wait(bar_x, 0) && dmbar_try_wait(bar_h, 0)); ++i) {}
         return;
     }

@@ -18,9 +18,9 @@ struct AbsScratch {
 
 // mean |W| into s->gamma.  Per-block sums in double (fixed grid-stride order, fixed tree), then the block that
 // finishes last adds the partials with one warp (lane-strided, then a fixed shuffle tree) and rounds the mean
-// once to fp32: the same order every time, whichever block is last.  Bound by HBM (4 bytes per weight: 7 us for 2048 x 5632) and, at that
-// size, by the start and the end of the launch: 13.7 us, one launch, against 11.1 + 2.5 us with the partials added
-// in a launch of their own.  Four 16-byte loads in flight per thread, added in index order.
+// once to fp32: the same order every time, whichever block is last.  13.7 us for 2048 x 5632, where HBM needs 7 (4 bytes per weight):
+// the rest is the start and the end of the launch.  As long as the sums and their addition took as two launches (11.1 + 2.5 us);
+// what a packing call gained came from its scratch (below).  Four 16-byte loads in flight per thread, added in index order.
 __global__ void __launch_bounds__(kAbsThreads) abs_mean_kernel(const float4 *W4, size_t n4, double count, AbsScratch *s) {
     double acc = 0.0;
     const size_t stride = (size_t)gridDim.x * kAbsThreads;
@@ -72,7 +72,7 @@ __device__ __forceinline__ WordPos word_pos(size_t w, int64_t steps) {
     return p;
 }
 
-// Stage 3: one thread per 32-bit packed word (16 weights).  Weight k0 + 4 j + b goes to bits
+// One thread per 32-bit packed word (16 weights).  Weight k0 + 4 j + b goes to bits
 // 8 b + 2 j of the word; code = t + 1; t = sign(w) * [|w| > gamma/2].  Padding words hold code 1.
 __global__ void __launch_bounds__(256) ternarise_pack_kernel(const float *W, int64_t N, int64_t K, int64_t steps,
                                                              size_t n_words, const float *gamma, uint32_t *packed) {

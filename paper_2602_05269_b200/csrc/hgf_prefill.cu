@@ -15,11 +15,10 @@
 // 256 input columns (eight MMAs): every hand-over between the roles costs a shared-memory round
 // trip.
 //
-// One persistent CTA per SM, 16 warps with fixed roles:
+// One persistent CTA per SM, 15 warps with fixed roles:
 //   warp 0      producer (all lanes): per stage the int8 activation tile as two 128 tokens x 128 B
-//               boxes (128-byte swizzle) and the packed weights of 128 channels (eight contiguous
-//               1 KiB tiles of the tiled weight layout, one bulk copy each); per tile what its
-//               epilogue needs: row sums, scales, the H tile and the (g B)^T tile
+//               boxes (128-byte swizzle); per tile what its epilogue needs: row sums, scales, the H
+//               tile and the (g B)^T tile
 //   warp 1      allocates tensor memory; issues the MMAs and commits to mbarriers
 //   warps 2-5, 11-14  epilogue, two warps per tensor-memory lane quarter (32 channels), one for each
 //               half of the tile's tokens: dequantise the accumulator in place (tcgen05.ld /
@@ -120,9 +119,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     if (tid == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
             // FULL: the stage's activation tile has landed (producer's arrival + bytes) and the four unpack
-            // warps have put the weight operand into tensor memory, so the MMA thread waits on this one
-            // barrier only (it is a single thread and every barrier operation costs it a shared-memory
-            // round trip).  EMPTY: the MMAs that read the stage are complete (one commit; the producer
+            // warps have put the weight operand into tensor memory, so the MMA warp waits on this one
+            // barrier only (every barrier operation costs it a shared-memory round trip).  EMPTY: the MMAs that read the stage are complete (one commit; the producer
             // and the unpack warps both wait on it).
             mbar_init(bar(C::BAR_FULL + s), 1 + 4);
             mbar_init(bar(C::BAR_EMPTY + s), 1);

@@ -202,6 +202,9 @@ def linear_forward(x, packed, gamma, d_in, d_out, At=None, Bt=None, gate=None, *
 
     x bf16 [M][d_in]; packed uint8 from pack_ternary; At fp16 [r][d_in]; Bt fp16 [d_out][r];
     gate fp32 [d_out]; y fp32 (or bf16 with FLAG_OUT_BF16) [M][d_out].
+    Decode-sized calls (M <= DECODE_MAX_M) start fetching packed, At and Bt before earlier work on the stream
+    has finished: these must not be outputs of work still pending there (x, gate and the LayerNorm's parameters
+    may be); FLAG_NO_PDL lifts that.
     With ln_weight / ln_bias (fp32 [d_in]) and/or gate_group the call is hgf_linear_forward_ln: LayerNorm
     in front of the quantiser, gate fp32 [ceil(d_out / gate_group)]; debug then also returns mean and rstd.
     """
@@ -271,7 +274,8 @@ class Group:
     """A group of independent decode-sized problems (hgf_group_*).  `problems` is a list of dicts
     with keys x, packed, gamma, d_in, d_out, y and optionally At, Bt, gate (device tensors), and for
     the front end of hgf_group_create_ln: ln_weight, ln_bias (fp32 [d_in]), eps, gate_group, mean_out,
-    rstd_out; the tensors are kept alive by this object."""
+    rstd_out; the tensors are kept alive by this object.  As in linear_forward, packed, At and Bt must not be
+    outputs of work still pending on the stream of a forward, unless flags has FLAG_NO_PDL."""
 
     def __init__(self, problems, flags: int = 0):
         self._keep = problems
