@@ -389,7 +389,7 @@ def run_ours(args):
                 "achieved": gemv_bytes / (gemv_ms * 1e-3) / 1e9, "peak": peaks["hbm_gbs"],
                 "unit": "GB/s", "frac": None, "traffic": decode_traffic(gemv_bytes), "peak_source": peaks["source"],
                 "traffic_note": "ncu dram bytes per algorithmic byte of the captured launch x this launch's bytes; null "
-                                "when hgf_decode.cu differs from the captured source (sha1 %s)" % DECODE_TRAFFIC["source_sha1"][:12],
+                                "when hgf_decode.cu or hgf_warp.cuh differs from the captured source (sha1 %s)" % DECODE_TRAFFIC["source_sha1"][:12],
                 "bytes_per_launch": gemv_bytes, "us_per_launch": gemv_ms * 1e3,
                 "frac_of_nominal_8000": None,
                 "whole_step": {"GB/s": value, "frac": value / peaks["hbm_gbs"], "launches": 2,
@@ -457,19 +457,19 @@ def run_ours(args):
 # DRAM traffic of the decode GEMV launch from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum
 # of a config-1, M = 1 group launch): bytes moved per algorithmic byte.  It is only reported while the
 # kernel source is the one that was captured.
-DECODE_TRAFFIC = {"source_sha1": "7b2cc479563a0d062a4c3a356e67630e5471a690",
-                  "dram_bytes_per_algorithmic_byte": (517.347072e6 + 7.010560e6) / 518805504.0}
+DECODE_TRAFFIC = {"source_sha1": "dd008a0e3695ed629c6b1c6999618f2713341375",
+                  "dram_bytes_per_algorithmic_byte": (517.357824e6 + 5.695232e6) / 518805504.0}
 
 
 # DRAM traffic of the prefill GEMM launch from one ncu capture of the very shape the bench times
 # (2048 -> 5632, r = 32, M = 8192, bf16 y): dram__bytes_read.sum + dram__bytes_write.sum of one launch.  Below
 # the launch's algorithmic bytes because most of y is still in L2 when the kernel ends.
-PREFILL_TRAFFIC = {"source_sha1": "8ff95e068f9752902d0b321377a47b0986601768", "dram_bytes_per_launch": 21.581312e6 + 43.126016e6}
+PREFILL_TRAFFIC = {"source_sha1": "d63d4d700369fb6bb26571622ae28e0b0029d6fc", "dram_bytes_per_launch": 21.574912e6 + 43.079680e6}
 
 
 def prefill_traffic():
     import hashlib
-    srcs = [os.path.join(ROOT, "paper_2602_05269_b200", "csrc", f) for f in ("hgf_prefill.cu", "hgf_tc.cuh")]
+    srcs = [os.path.join(ROOT, "paper_2602_05269_b200", "csrc", f) for f in ("hgf_prefill.cu", "hgf_tc.cuh", "hgf_warp.cuh")]
     if not all(os.path.exists(f) for f in srcs):
         return None
     if hashlib.sha1(b"".join(open(f, "rb").read() for f in srcs)).hexdigest() != PREFILL_TRAFFIC["source_sha1"]:
@@ -479,10 +479,10 @@ def prefill_traffic():
 
 def decode_traffic(gemv_bytes):
     import hashlib
-    src = os.path.join(ROOT, "paper_2602_05269_b200", "csrc", "hgf_decode.cu")
-    if DECODE_TRAFFIC["source_sha1"] is None or not os.path.exists(src):
+    srcs = [os.path.join(ROOT, "paper_2602_05269_b200", "csrc", f) for f in ("hgf_decode.cu", "hgf_warp.cuh")]
+    if not all(os.path.exists(f) for f in srcs):
         return None
-    if hashlib.sha1(open(src, "rb").read()).hexdigest() != DECODE_TRAFFIC["source_sha1"]:
+    if hashlib.sha1(b"".join(open(f, "rb").read() for f in srcs)).hexdigest() != DECODE_TRAFFIC["source_sha1"]:
         return None
     return DECODE_TRAFFIC["dram_bytes_per_algorithmic_byte"] * gemv_bytes
 
