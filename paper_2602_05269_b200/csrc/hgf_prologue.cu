@@ -1329,9 +1329,10 @@ static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPr
 //  - with a LayerNorm, 2048 -> 2048: 23.8 / 14.3 at M = 64, 51.2 / 52.2 at M = 4096; r = 64, 11008 -> 1024: 105 / 26 at M = 64,
 //    127 / 123 at M = 2048 (no limit of CTAs there: the other kernels take two launches);
 //  - with a LayerNorm and without a correction, 4096 -> 1024: 14.0 / 16.7 at M = 17, 25.2 / 16.7 at M = 64, 82.6 / 62.4 at
-//    M = 4096.  Short rows: K = 512 9.6 / 10.2 at M = 130, 10.6 / 11.1 at 700, 13.5 / 12.2 at 2000; K = 768 11.5 / 10.8 at M = 130, 15.4 /
-//    18.1 at 1500, 22.9 / 21.4 at 3000; K = 1024 12.8 / 11.1 at M = 130.  Long ones in one CTA: K = 3072 72 / 68 at M = 5000, 80.4 / 82.6
-//    at 8192.
+//    M = 4096.  Short rows: 512 -> 1024 9.6 / 10.2 at M = 130, 10.6 / 11.1 at 700, 13.3 / 12.3 at 1280, 13.5 / 12.2 at 2000; 512 -> 3040
+//    11.1 / 13.9 at M = 500 (96 output tiles), 12.7 / 13.6 at 640 (120), 16.5 / 13.9 at 700 (144); 512 -> 5632 12.5 / 14.2 at M = 300 (132);
+//    768 -> 1024 12.9 / 11.7 at M = 700, 15.4 / 18.1 at 1500, 22.9 / 21.4 at 3000; 768 -> 3040 13.0 / 14.3 at M = 500, a quarter less
+//    at 700 to 1168.  Long rows in one CTA: K = 3072 72 / 68 at M = 5000, 80.4 / 82.6 at 8192.
 // Cluster size: CTAs for every SM, two of them on one if they fit; one step smaller where that many don't run at once: 1024 -> 1024,
 // M = 1168, r = 48 16.4 -> 15.0 us, M = 570 15.4 -> 13.9; 8192 -> 1024, M = 525 26.6 -> 28.5.
 static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd *fe, cudaStream_t stream) {
@@ -1347,7 +1348,13 @@ static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmProlo
     if (rp_layout(p.K, p.r, c).smem > kRpSmemLimit) return cudaErrorNotSupported;
     bool take;
     if (p.r == 0) {
-        take = p.M >= 64 && p.K >= (p.M <= 1024 ? 768 : (p.M < 1920 ? 1024 : 0)) && (p.M <= 7168 || c > 0 || p.K <= 2048);
+        take = p.M >= 64 && (p.M <= 7168 || c > 0 || p.K <= 2048);
+        if (p.K < 896) {  // (by the output tiles of the launch that follows: in one round of them or more)
+            const int tiles = ((p.M + 127) / 128) * ((x.N + 127) / 128);
+            if (p.M < 640) take = take && tiles > sms;
+            else if (2 * blocks < sms) take = take && (p.K >= 640 || tiles > sms * 5 / 6);
+            else take = take && (p.K <= 512 || p.M >= 1800 || tiles > sms);
+        }
     } else {
         take = p.M <= 2048 && p.K >= 1024;
         if (!fe) take = take && (blocks << c) <= 4 * sms && (p.r > 16 || p.K > 2048 || p.M <= 1280);

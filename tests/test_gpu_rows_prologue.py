@@ -21,7 +21,7 @@ def dev(a, dtype=None):
 @pytest.mark.parametrize("ln", [False, True])
 @pytest.mark.parametrize("M,K,r", [(17, 1024, 16), (31, 1088, 32), (33, 5632, 48), (64, 1024, 0), (95, 1600, 64), (200, 2048, 32), (513, 1216, 16),
                                    (1100, 2112, 64), (2048, 1024, 32), (70, 11008, 64), (130, 192, 0),
-                                   (1024, 768, 0), (1100, 768, 0), (1920, 64, 0), (1150, 1024, 64), (1184, 1024, 64), (2048, 1088, 64), (570, 1024, 48), (1300, 1024, 16)])
+                                   (1024, 768, 0), (1100, 576, 0), (1300, 576, 0), (1920, 64, 0), (1150, 1024, 64), (1184, 1024, 64), (2048, 1088, 64), (570, 1024, 48), (1300, 1024, 16)])
 def test_rows_prologue(M, K, r, ln):
     from paper_2602_05269_b200 import hgf
     N = 40
