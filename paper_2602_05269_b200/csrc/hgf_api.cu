@@ -389,9 +389,63 @@ struct hgf_group {
     bool ln_warps;            // rows behind a LayerNorm get a warp each, like the others
     int4 *d_cta_range;        // per GEMV CTA: (first tile, end tile, first problem, 0)
     int grid;
+    bool tc;                  // the contraction runs on decode_tc_kernel, in the shares below
+    DecodeTcSeg *d_tc_segs;
+    int2 *d_tc_cta;
+    int tc_grid, tc_image;    // CTAs; shared memory for the largest problem's activations
     bool small;               // whole forwards take the one launch `sl` describes
     SmallLaunch<kSmallMax> sl;
 };
+
+namespace hgf {
+// Whether a group's contraction runs on decode_tc_kernel, and its shares: base-3 weights, or more than eight tokens.  Measured over
+// one to 36 blocks, widths 512 to 4096, ranks 16 to 64 (a captured chain, warp MMA against tensor memory): base-3 1.04 to 1.30
+// times as fast, 9 to 16 tokens 1.00 to 1.29; two-bit weights with up to eight tokens 0.86 to 0.96, which stay where they were.
+// More runs of row tiles on a CTA than its table holds, or activations that leave no room for the ring, stay there too.
+static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const DecodeProblem *d_probs, int max_M, uint32_t flags,
+                           std::vector<DecodeTcSeg> *segs, std::vector<int2> *cta, int *image) {
+    const int sms = device_sm_count(), n = (int)dps.size();
+    if (sms <= 0 || sms > 1024 || (max_M <= 8 && !(flags & HGF_FLAG_BASE3))) return false;
+    // a row tile's cost: its weight tiles, and its rows of B^T (1 KiB at r = 32)
+    auto cost_of = [&](int i) { return 32ll * weight_steps(dps[i].K, flags) + dps[i].r; };
+    long long cost = 0;
+    *image = 0;
+    for (int i = 0; i < n; ++i) {
+        cost += row_tiles(dps[i].N) * cost_of(i);
+        const int b = decode_tc_image_bytes(max_M, dps[i].K, flags);
+        *image = b > *image ? b : *image;
+    }
+    int p = 0, t = 0, max_segs = 0;  // next row tile to deal out
+    long long dealt = 0;
+    for (int c = 0; c < sms; ++c) {
+        const int first = (int)segs->size();
+        const long long until = cost * (c + 1) / sms;
+        while (p < n && dealt < until) {
+            const DecodeProblem &P = dps[p];
+            const long long per = cost_of(p), tiles = row_tiles(P.N);
+            long long take = (until - dealt + per / 2) / per;
+            if (c + 1 == sms || take > tiles - t) take = tiles - t;
+            if (take <= 0) break;  // (less than half a row tile is left of this share)
+            DecodeTcSeg s = {};
+            s.steps = weight_steps(P.K, flags);
+            s.packed = P.packed + (size_t)t * s.steps * 1024;
+            s.xq = P.xq; s.gamma_x = P.gamma_x; s.row_sum = P.row_sum; s.hpart = P.hpart; s.nslices = P.nslices;
+            s.Bt = P.Bt; s.gate = P.gate; s.y = P.y;
+            s.dbg_y_int_at = &d_probs[p].dbg_y_int;
+            s.gw_over_127 = P.gw_over_127;
+            s.M = P.M; s.K = P.K; s.N = P.N; s.r = P.r; s.gate_group = P.gate_group; s.flags = P.flags;
+            s.lo = t; s.n = (int)take;
+            segs->push_back(s);
+            dealt += take * per;
+            t += (int)take;
+            if (t == tiles) { ++p; t = 0; }
+        }
+        cta->push_back(make_int2(first, (int)segs->size() - first));
+        max_segs = cta->back().y > max_segs ? cta->back().y : max_segs;
+    }
+    return p == n && decode_tc_fits(*image, max_segs);
+}
+}  // namespace hgf
 
 extern "C" hgf_status hgf_group_create(const hgf_problem *problems, int32_t n, uint32_t flags, hgf_group **out) {
     return hgf_group_create_ln(problems, nullptr, n, flags, out);
@@ -450,7 +504,9 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
     const size_t off_qit = align_up(off_pps + sizeof(PrologueParams) * (size_t)n, 256);
     const size_t off_lit = align_up(off_qit + sizeof(QuantItem) * n_quant, 256);
     const size_t off_cta = align_up(off_lit + sizeof(LoraItem) * n_lora, 256);
-    const size_t off_hpart = align_up(off_cta + sizeof(int4) * 1024, 256);
+    const size_t off_tc_cta = align_up(off_cta + sizeof(int4) * 1024, 256);
+    const size_t off_tc_segs = align_up(off_tc_cta + sizeof(int2) * 1024, 256);
+    const size_t off_hpart = align_up(off_tc_segs + sizeof(DecodeTcSeg) * ((size_t)n + 1024), 256);
     const size_t off_ws = align_up(off_hpart + n_lora * 8 * 32 * sizeof(float), 256);
     void *mem = nullptr;
     if (cudaMalloc(&mem, off_ws + ws_total) != cudaSuccess) return HGF_ERR_CUDA;
@@ -567,13 +623,22 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
     } else {
         g->d_cta_range = nullptr;  // the kernel works its share out itself
     }
+    // the same on the tensor cores: shares of 16-row tiles of equal cost, cut into their problems' runs
+    std::vector<DecodeTcSeg> tc_segs;
+    std::vector<int2> tc_cta;
+    g->d_tc_segs = (DecodeTcSeg *)((char *)mem + off_tc_segs);
+    g->d_tc_cta = (int2 *)((char *)mem + off_tc_cta);
+    g->tc = plan_decode_tc(dps, g->d_probs, max_M, flags, &tc_segs, &tc_cta, &g->tc_image);
+    g->tc_grid = (int)tc_cta.size();
     bool ok = cudaMemcpy(g->d_probs, dps.data(), sizeof(DecodeProblem) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(g->d_pps, pps.data(), sizeof(PrologueParams) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(g->d_quant_items, qitems.data(), sizeof(QuantItem) * qitems.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
               (litems.empty() || cudaMemcpy(g->d_lora_items, litems.data(), sizeof(LoraItem) * litems.size(),
                                             cudaMemcpyHostToDevice) == cudaSuccess) &&
               (ranges.empty() ||
-               cudaMemcpy(g->d_cta_range, ranges.data(), sizeof(int4) * ranges.size(), cudaMemcpyHostToDevice) == cudaSuccess);
+               cudaMemcpy(g->d_cta_range, ranges.data(), sizeof(int4) * ranges.size(), cudaMemcpyHostToDevice) == cudaSuccess) &&
+              (!g->tc || (cudaMemcpy(g->d_tc_segs, tc_segs.data(), sizeof(DecodeTcSeg) * tc_segs.size(), cudaMemcpyHostToDevice) == cudaSuccess &&
+                          cudaMemcpy(g->d_tc_cta, tc_cta.data(), sizeof(int2) * tc_cta.size(), cudaMemcpyHostToDevice) == cudaSuccess));
     if (!ok) { cudaFree(mem); delete g; return HGF_ERR_CUDA; }
     g->small = false;
     if (n <= kSmallMax) {
@@ -620,6 +685,8 @@ extern "C" hgf_status hgf_group_forward_phases(hgf_group *g, uint32_t phases, vo
                                      stream) != cudaSuccess)
         return HGF_ERR_CUDA;
     if (!(phases & HGF_PHASE_GEMV)) return HGF_OK;
+    if (g->tc)
+        return launch_decode_tc(g->d_tc_segs, g->d_tc_cta, g->tc_grid, g->tc_image, g->max_M, g->flags, pdl, stream) == cudaSuccess ? HGF_OK : HGF_ERR_CUDA;
     DecodeLaunch dl = {};
     dl.probs = g->d_probs;
     dl.n_probs = g->n;

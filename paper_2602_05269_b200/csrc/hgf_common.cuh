@@ -265,6 +265,34 @@ bool plan_small(SmallLaunch<NP> &L, uint32_t flags);  // false: the launch takes
 template <int NP>
 cudaError_t launch_small(const SmallLaunch<NP> &L, bool pdl, cudaStream_t stream);
 
+// ---- decode groups on the 5th-generation tensor cores (hgf_decode_tc.cu) --------------------------------
+// The run of 16-row tiles of one problem that falls into a CTA's share.
+struct DecodeTcSeg {
+    const uint8_t *packed;           // the run's first row tile
+    const int8_t *xq;                // [M][K]
+    const float *gamma_x;            // [M]
+    const int32_t *row_sum;          // [M]
+    const float *hpart;              // partial sums of x A, as in DecodeProblem
+    const __half *Bt;                // [N][r]
+    const float *gate;
+    void *y;                         // [M][N]
+    int32_t *const *dbg_y_int_at;    // the device word that holds the debug address (see hgf_group_debug)
+    float gw_over_127;
+    int M, K, N, r, nslices, gate_group;
+    uint32_t flags;
+    int steps, lo, n;                // column tiles of a row tile; first row tile (of the problem) and row tiles of the run
+    int reserved[2];
+};
+static_assert(sizeof(DecodeTcSeg) % 16 == 0, "copied in 16-byte units");
+struct DecodeTcLaunch {
+    const DecodeTcSeg *segs;
+    const int2 *cta;                 // per CTA: first segment, segments
+    int x_bytes, stages;             // (set by the launcher) shared memory for activations, ring stages
+};
+int decode_tc_image_bytes(int max_M, int K, uint32_t flags);  // a problem's activations in the launch's shared memory
+bool decode_tc_fits(int max_image, int max_segs);
+cudaError_t launch_decode_tc(const DecodeTcSeg *segs, const int2 *cta, int grid, int max_image, int max_M, uint32_t flags, bool pdl, cudaStream_t stream);
+
 struct GemmParams {
     const int8_t *xq;        // [M][K]
     const uint8_t *packed;   // tiled layout, see above
