@@ -45,8 +45,7 @@ __device__ __forceinline__ void chain() {  // first thing of a kernel that is al
 // the 128-byte swizzle.  The contraction may continue over a second pair of operands (A2, B2: the
 // low-rank term of dX), and may be split over several CTAs that write partial sums which a second
 // kernel adds up in a fixed order.
-// Persistent, one CTA per SM, six warps: warp 0 stages operand tiles with TMA, warp 1 issues (elect.sync: the two large
-// products of 2048 x 5632 at M = 8192 and the one for dA took 136 us on average from one thread in a branch, 115 so)
+// Persistent, one CTA per SM, six warps: warp 0 stages operand tiles with TMA, warp 1 issues (elect.sync)
 // tcgen05.mma.kind::f16 (bf16 inputs, 128 x BN x 16 per instruction, fp32 accumulators in tensor memory,
 // two of them so that a tile's epilogue runs under the next tile's main loop), warps 2-5 read the
 // accumulator back (tcgen05.ld) and write C.  Rows and columns past the matrices, and contraction
@@ -259,6 +258,227 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(C::TMEM_COLS) : "memory");
     }
 }
+
+// ---- the same by pairs of CTAs: 256 x 256 tiles ------------------------------------------------------------
+// tcgen05.mma.cta_group::2: the pair's first CTA issues for both; each CTA stages 128 rows of A and half of B's rows, and keeps 128
+// rows of C in its tensor memory.  An instruction of 128 x 256 x 16 reads 12 KiB of operands from an SM's shared memory, one of the
+// pair 8 KiB on each SM, and a tile's operands are fetched once for 256 rows instead of 128.
+// Barriers: both CTAs' copies count on the first one's FULL; its commits reach both CTAs' EMPTY and ACCFULL; both epilogues
+// arrive on its ACCEMPTY.
+// It takes every product whose output is more than 128 x 128: the tiles of 128 x 256 by single CTAs held the two large products of
+// 2048 x 5632 at M = 8192 at 1.14 and 1.22 PFLOP/s (166, 155 us), pairs at 1.25 and 1.42 (152, 133 us), where the power limit is
+// near (library bf16 products for seconds on end: 1.37).  Whole backward pass in a captured chain: 425 -> 380 us, 8192 x 5632 -> 2048
+// 547 -> 451, 2048 -> 2048 215 -> 186, 1500 x 3200 -> 2000 93 -> 75, 200 x 1024 -> 768 52.9 -> 52.5, 64 x 512 -> 512 41.6 -> 42.1.
+struct TpCfg {
+    static constexpr int STAGES = 6, A_BYTES = kTBM * 128, STAGE_BYTES = 2 * A_BYTES;
+    static constexpr int OFF_BAR = STAGES * STAGE_BYTES;
+    static constexpr int BAR_FULL = 0, BAR_EMPTY = STAGES, BAR_ACCFULL = 2 * STAGES, BAR_ACCEMPTY = 2 * STAGES + 2, BAR_COUNT = 2 * STAGES + 4;
+    static constexpr int SMEM_BYTES = OFF_BAR + 256 + 1024;
+    static constexpr uint32_t IDESC = (1u << 4) /*f32*/ | (1u << 7) /*A bf16*/ | (1u << 10) /*B bf16*/ | ((uint32_t)(256 >> 4) << 24);
+};
+constexpr int kTpTile = 256;
+
+__device__ __forceinline__ uint32_t cluster_address(uint32_t addr, uint32_t rank) {
+    uint32_t r;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;\n" : "=r"(r) : "r"(addr), "r"(rank));
+    return r;
+}
+// Into this CTA's shared memory, counted by a barrier of either CTA of the pair.
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap *map, int x, int y, uint32_t cluster_bar) {
+    asm volatile("cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%3, %4}], [%2];\n"
+                 ::"r"(dst), "l"(map), "r"(cluster_bar), "r"(x), "r"(y)
+                 : "memory");
+}
+__device__ __forceinline__ void warp_mma_f16_pair(uint32_t d, uint64_t a, uint64_t b, uint32_t idesc, uint32_t accumulate) {
+    asm volatile("{\n.reg .pred p, e;\nelect.sync _|e, 0xffffffff;\nsetp.ne.b32 p, %4, 0;\n"
+                 "@e tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(d), "l"(a), "l"(b), "r"(idesc), "r"(accumulate)
+                 : "memory");
+}
+__device__ __forceinline__ void warp_commit_pair(uint32_t bar) {  // arrives at this place in both CTAs
+    asm volatile("{\n.reg .pred e;\nelect.sync _|e, 0xffffffff;\n"
+                 "@e tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;\n}\n" ::"r"(bar), "h"((uint16_t)3)
+                 : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
+    asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_bar) : "memory");
+}
+
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTThreads, 1)
+tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
+                    const __grid_constant__ CUtensorMap tmap_a2, const __grid_constant__ CUtensorMap tmap_b2, const TcGemmArgs g,
+                    unsigned int *status) {
+    using C = TpCfg;
+    extern __shared__ uint8_t tp_smem_raw[];
+    uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)tp_smem_raw + 1023) & ~(uintptr_t)1023);
+    const uint32_t sbase = smem_u32(smem), bar0 = sbase + C::OFF_BAR;
+    auto bar = [&](int i) { return bar0 + 8u * i; };
+    uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::OFF_BAR + C::BAR_COUNT * 8);
+    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_BAR + C::BAR_COUNT * 8 + 4);
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31, rank = (int)blockIdx.x & 1;
+    const int pair = (int)blockIdx.x >> 1, pairs = (int)gridDim.x >> 1;
+    const int tiles_i = (g.I + kTpTile - 1) / kTpTile, tiles_j = (g.J + kTpTile - 1) / kTpTile, tiles = tiles_i * tiles_j;
+    const int n_full = tiles - g.n_half / 2, num_work = n_full + g.n_half, kb_all = g.kb1 + g.kb2;
+    auto tile_of = [&](int w, int &i0, int &j0, int &bn) {  // (halves of the last tiles: as in tc_gemm_kernel)
+        int tile = w, half = 0;
+        bn = kTpTile;
+        if (w >= n_full) {
+            tile = n_full + (w - n_full) / 2;
+            half = (w - n_full) & 1;
+            bn = kTpTile / 2;
+        }
+        i0 = (tile / tiles_j) * kTpTile;
+        j0 = (tile % tiles_j) * kTpTile + half * (kTpTile / 2);
+    };
+
+    if (tid == 0) {
+        for (int s = 0; s < C::STAGES; ++s) {
+            mbar_init(bar(C::BAR_FULL + s), 1);
+            mbar_init(bar(C::BAR_EMPTY + s), 1);
+        }
+        for (int b = 0; b < 2; ++b) {
+            mbar_init(bar(C::BAR_ACCFULL + b), 1);
+            mbar_init(bar(C::BAR_ACCEMPTY + b), 8);
+        }
+        *abort_flag = 0;
+        asm volatile("fence.mbarrier_init.release.cluster;\n" ::: "memory");
+        fence_proxy_async();
+    }
+    if (warp == 1) {
+        asm volatile("tcgen05.alloc.cta_group::2.sync.aligned.shared::cta.b32 [%0], %1;\n" ::"r"(smem_u32(tmem_slot)), "r"(512) : "memory");
+        asm volatile("tcgen05.relinquish_alloc_permit.cta_group::2.sync.aligned;\n" ::: "memory");
+    }
+    tc_fence_before();
+    cluster_arrive_release();  // both CTAs' barriers are there before either is reached from the other
+    cluster_wait_acquire();
+    __syncthreads();
+    tc_fence_after();
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_slot, 0);  // (warp-uniform)
+    chain();
+
+    if (warp == 0) {
+        // ------------------------------------------------------------------ TMA producer
+        int s = 0;
+        uint32_t ph = 0, issued = 0;
+        bool ok = true;
+        for (int w = pair; ok && w < num_work; w += pairs) {
+            int i0, j0, bn;
+            tile_of(w, i0, j0, bn);
+            i0 += rank * kTBM;
+            j0 += rank * (bn / 2);
+            for (int kb = 0; kb < kb_all; ++kb) {
+                ok = mbar_wait(bar(C::BAR_EMPTY + s), ph ^ 1u, abort_flag, status, 0x840u + s);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                if (lane == 0) {
+                    const bool second = kb >= g.kb1;
+                    const CUtensorMap *ma = second ? &tmap_a2 : &tmap_a, *mb = second ? &tmap_b2 : &tmap_b;
+                    const int c0 = (second ? kb - g.kb1 : kb) * kTBK;
+                    const uint32_t dst_a = sbase + s * C::STAGE_BYTES, dst_b = dst_a + C::A_BYTES, full = cluster_address(bar(C::BAR_FULL + s), 0);
+                    if (rank == 0)  // (a K-major box always has 128 rows)
+                        mbar_arrive_expect_tx(bar(C::BAR_FULL + s), 2 * (C::A_BYTES + (g.b_mn ? bn / 2 * 128 : C::A_BYTES)));
+                    if (g.a_mn) {
+                        for (int h = 0; h < kTBM / 64; ++h) tma_load_2d_pair(dst_a + h * kTBox, ma, i0 + 64 * h, c0, full);
+                    } else {
+                        tma_load_2d_pair(dst_a, ma, c0, i0, full);
+                    }
+                    if (g.b_mn) {
+                        for (int h = 0; h < bn / 128; ++h) tma_load_2d_pair(dst_b + h * kTBox, mb, j0 + 64 * h, c0, full);
+                    } else {
+                        tma_load_2d_pair(dst_b, mb, c0, j0, full);
+                    }
+                }
+                ++issued;
+                if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+            }
+        }
+        // Never leave with a copy in flight: a stage's MMAs, which follow its copies, reach this CTA's EMPTY.
+        for (uint32_t q = 0; q < (uint32_t)C::STAGES; ++q) {
+            const uint32_t rounds = (issued + C::STAGES - 1 - q) / C::STAGES;
+            if (rounds)
+                for (uint32_t i = 0; i < (ok ? kSpinLimit : 1u << 12) && !mbar_try_wait(bar(C::BAR_EMPTY + q), (rounds - 1u) & 1u); ++i)
+                    if (!ok) __nanosleep(1000);  // (after a time-out nothing may come: some milliseconds, which a copy does not take)
+        }
+    } else if (warp == 1) {
+        // ------------------------------------------------------------------ MMA issuer (the first CTA's, for both)
+        if (rank == 0) {
+            auto wait = [&](int i, uint32_t par, unsigned int code) { return __all_sync(0xffffffffu, mbar_wait_poll(bar(i), par, abort_flag, status, code)) != 0; };
+            int s = 0, it = 0;
+            uint32_t ph = 0;
+            bool ok = true;
+            const uint32_t idesc = C::IDESC | (g.a_mn ? 1u << 15 : 0u) | (g.b_mn ? 1u << 16 : 0u);
+            const uint32_t a_step = g.a_mn ? (16 * 128) >> 4 : 32 >> 4, b_step = g.b_mn ? (16 * 128) >> 4 : 32 >> 4;  // 16 contraction elements
+            for (int w = pair; ok && w < num_work; w += pairs, ++it) {
+                const int b = it & 1;
+                const uint32_t acc = tmem_base + b * kTpTile;
+                if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x850u))) break;
+                tc_fence_after();
+                int ti0, tj0, bn;
+                tile_of(w, ti0, tj0, bn);
+                const uint32_t idesc_w = idesc | ((uint32_t)(bn >> 3) << 17);
+                for (int kb = 0; kb < kb_all; ++kb) {
+                    if (!(ok = wait(C::BAR_FULL + s, ph, 0x860u + s))) break;
+                    tc_fence_after();
+                    const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+                    const uint64_t adesc = g.a_mn ? make_sw128_mn_desc(sa, kTBox) : make_sw128_desc(sa);
+                    const uint64_t bdesc = g.b_mn ? make_sw128_mn_desc(sb, kTBox) : make_sw128_desc(sb);
+#pragma unroll
+                    for (int kk = 0; kk < kTBK / 16; ++kk)
+                        warp_mma_f16_pair(acc, adesc + (uint64_t)(a_step * kk), bdesc + (uint64_t)(b_step * kk), idesc_w, (kb || kk) ? 1u : 0u);
+                    warp_commit_pair(bar(C::BAR_EMPTY + s));
+                    if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+                }
+                if (!ok) break;
+                warp_commit_pair(bar(C::BAR_ACCFULL + b));
+            }
+        }
+    } else {
+        // ------------------------------------------------------------------ epilogue warps
+        const int q = warp & 3;  // tensor-memory lane quarter this warp may access
+        bool ok = true;
+        int it = 0;
+        for (int w = pair; ok && w < num_work; w += pairs, ++it) {
+            int i0, j0, bn;
+            tile_of(w, i0, j0, bn);
+            const int b = it & 1;
+            ok = mbar_wait(bar(C::BAR_ACCFULL + b), (uint32_t)(it >> 1) & 1u, abort_flag, status, 0x870u);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            tc_fence_after();
+            const int i = i0 + rank * kTBM + 32 * q + lane;  // this thread's row of C = its tensor-memory lane
+            const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16) + b * kTpTile;
+            for (int cc = 0; cc < bn; cc += 32) {
+                if (j0 + cc >= g.J) break;  // (warp-uniform)
+                uint32_t v[32];
+                tmem_ld32(lane_base + cc, v);
+                tmem_ld_wait();
+                if (i < g.I) {
+                    float *row = g.C + (size_t)i * g.ldc + j0 + cc;
+#pragma unroll
+                    for (int u = 0; u < 8; ++u) {
+                        if (j0 + cc + 4 * u < g.J) {  // J is a multiple of 4
+                            float4 o = make_float4(g.alpha * __uint_as_float(v[4 * u]), g.alpha * __uint_as_float(v[4 * u + 1]),
+                                                   g.alpha * __uint_as_float(v[4 * u + 2]), g.alpha * __uint_as_float(v[4 * u + 3]));
+                            float4 *dst = reinterpret_cast<float4 *>(row + 4 * u);
+                            if (g.accumulate) { const float4 c = *dst; o.x += c.x; o.y += c.y; o.z += c.z; o.w += c.w; }
+                            *dst = o;
+                        }
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_address(bar(C::BAR_ACCEMPTY + b), 0));
+        }
+    }
+
+    tc_fence_before();
+    __syncwarp();
+    cluster_arrive_release();  // no CTA leaves while the other may still reach its barriers or its shared memory
+    cluster_wait_acquire();
+    if (warp == 1) {
+        tc_fence_after();
+        asm volatile("tcgen05.dealloc.cta_group::2.sync.aligned.b32 %0, %1;\n" ::"r"(tmem_base), "r"(512) : "memory");
+    }
+}
+
 // Sum of the partial results of a split contraction, in split order: C = alpha * sum_s P[s] (+ C).
 __global__ void __launch_bounds__(256) tc_reduce_kernel(const float4 *P, int splits, size_t n4, float alpha, int accumulate, float4 *C) {
     chain();
@@ -300,22 +520,53 @@ static cudaError_t tc_gemm_bn(const CUtensorMap *maps, const TcGemmArgs &g, cuda
     return launch_chained(tc_gemm_kernel<BN>, (unsigned)(work < sms ? work : sms), kTThreads, TcCfg<BN>::SMEM_BYTES, stream, maps[0], maps[1], maps[2], maps[3], g, status);
 }
 
+// Pairs of CTAs that run at once with one CTA an SM.
+static int tc_pairs_at_once() {
+    static std::atomic<int> cache[kMaxDevices];
+    const int dev = current_device();
+    if (dev < 0 || dev >= kMaxDevices) return 0;
+    int n = cache[dev].load(std::memory_order_acquire);
+    if (n) return n;
+    static std::atomic<unsigned long long> attr_done{0};
+    if (ensure_dynamic_smem(tc_pair_gemm_kernel, TpCfg::SMEM_BYTES, attr_done) != cudaSuccess) return 0;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(2);
+    cfg.blockDim = dim3(kTThreads);
+    cfg.dynamicSmemBytes = TpCfg::SMEM_BYTES;
+    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_gemm_kernel, &cfg) != cudaSuccess || n <= 0) return 0;
+    cache[dev].store(n, std::memory_order_release);
+    return n;
+}
+
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
 // operand forms.  `partials` (splits_max * I * ldc floats) enables splitting the contraction when the
 // output has fewer tiles than the device has SMs; ldc must then be J.  Bases 16-byte aligned, ld % 8 == 0.
 static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J,
                            float alpha, bool accumulate, float *partials, int splits_max, cudaStream_t stream) {
     const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64);
+    const int pairs = I > kTBM && J > 128 ? tc_pairs_at_once() : 0;
     CUtensorMap maps[4];
-    if (!tc_map(&maps[0], A, I, Cn, kTBM) || !tc_map(&maps[1], B, J, Cn, BN)) return cudaErrorInvalidValue;
+    const int rows_b = pairs ? 128 : BN;
+    if (!tc_map(&maps[0], A, I, Cn, kTBM) || !tc_map(&maps[1], B, J, Cn, rows_b)) return cudaErrorInvalidValue;
     maps[2] = maps[0];
     maps[3] = maps[1];
-    if (A2.p && (!tc_map(&maps[2], A2, I, Cn2, kTBM) || !tc_map(&maps[3], B2, J, Cn2, BN))) return cudaErrorInvalidValue;
+    if (A2.p && (!tc_map(&maps[2], A2, I, Cn2, kTBM) || !tc_map(&maps[3], B2, J, Cn2, rows_b))) return cudaErrorInvalidValue;
     TcGemmArgs g = {};
     g.I = I; g.J = J; g.ldc = ldc;
     g.kb1 = (Cn + kTBK - 1) / kTBK;
     g.kb2 = A2.p ? (Cn2 + kTBK - 1) / kTBK : 0;
     g.a_mn = A.mn; g.b_mn = B.mn;
+    if (pairs) {
+        const int tiles = ((I + kTpTile - 1) / kTpTile) * ((J + kTpTile - 1) / kTpTile);
+        if (B.mn && tiles > pairs && tiles % pairs != 0 && 2 * (tiles % pairs) <= pairs && J % kTpTile == 0) g.n_half = 2 * (tiles % pairs);
+        g.splits = 1;
+        g.C = C; g.alpha = alpha; g.accumulate = accumulate ? 1 : 0;
+        const int work = tiles + g.n_half / 2;
+        unsigned int *status = device_status_word();
+        if (!status) return cudaErrorMemoryAllocation;
+        return launch_chained(tc_pair_gemm_kernel, 2u * (unsigned)(work < pairs ? work : pairs), kTThreads, TpCfg::SMEM_BYTES, stream, maps[0], maps[1],
+                              maps[2], maps[3], g, status);
+    }
     const int kb_all = g.kb1 + g.kb2, tiles = ((I + kTBM - 1) / kTBM) * ((J + BN - 1) / BN), sms = device_sm_count();
     int splits = 1;
     if (partials && ldc == J && sms > 0 && tiles * 2 <= sms) {

@@ -91,3 +91,10 @@ def test_rejects_bad_arguments(hgf):
 def test_row_lengths_of_the_quantiser(hgf, M, K, N, r):
     """Rows at the limits of what a warp holds in registers (2048, 4096 columns) and just past them."""
     check(hgf, M, K, N, r, layer=K)
+
+
+@pytest.mark.parametrize("M,K,N,r", [(40, 192, 136, 16), (257, 320, 264, 64), (256, 256, 256, 32), (1, 192, 136, 0), (130, 2112, 384, 48)])
+def test_tiles_of_cta_pairs(hgf, M, K, N, r):
+    """Outputs just past 128 rows and columns (the second CTA of a pair has 8 rows, or none), exact 256 x 256 tiles, a contraction of
+    one element, column tiles that end inside the second CTA's half."""
+    check(hgf, M, K, N, r, layer=M + 500, lora=r > 0)
