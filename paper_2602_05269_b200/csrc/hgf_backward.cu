@@ -14,7 +14,7 @@ namespace hgf {
 
 // Every launch of the backward pass is chained to the one before by programmatic dependent launch: its blocks are set up
 // under the predecessor's tail and wait for its completion before they touch memory (a step of the 2048 x 5632 layer at
-// M = 8192 has seventeen such launches, most of them of 2 to 3 us: 662 -> 646 us together with bw_quant_kernel).
+// M = 8192 had seventeen such launches, most of them of 2 to 3 us: 662 -> 646 us together with bw_quant_kernel; now twelve).
 template <typename... Params, typename... Args>
 static cudaError_t launch_chained(void (*kernel)(Params...), unsigned grid, unsigned block, size_t smem, cudaStream_t stream, Args... args) {
     cudaLaunchAttribute attr[1];
@@ -540,9 +540,10 @@ static int tc_pairs_at_once() {
 
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
 // operand forms.  `partials` (splits_max * I * ldc floats) enables splitting the contraction when the
-// output has fewer tiles than the device has SMs; ldc must then be J.  Bases 16-byte aligned, ld % 8 == 0.
+// output has fewer tiles than the device has SMs; ldc must then be J.  With `splits_out` they are left there for the kernel that
+// reads the product next (*splits_out of them; 1: the product is in C).  Bases 16-byte aligned, ld % 8 == 0.
 static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J,
-                           float alpha, bool accumulate, float *partials, int splits_max, cudaStream_t stream) {
+                           float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, cudaStream_t stream) {
     const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64);
     const int pairs = I > kTBM && J > 128 ? tc_pairs_at_once() : 0;
     CUtensorMap maps[4];
@@ -561,6 +562,7 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
         if (B.mn && tiles > pairs && tiles % pairs != 0 && 2 * (tiles % pairs) <= pairs && J % kTpTile == 0) g.n_half = 2 * (tiles % pairs);
         g.splits = 1;
         g.C = C; g.alpha = alpha; g.accumulate = accumulate ? 1 : 0;
+        if (splits_out) *splits_out = 1;
         const int work = tiles + g.n_half / 2;
         unsigned int *status = device_status_word();
         if (!status) return cudaErrorMemoryAllocation;
@@ -587,7 +589,8 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
         g.C = partials; g.alpha = 1.0f; g.accumulate = 0;
     }
     cudaError_t e = BN == 256 ? tc_gemm_bn<256>(maps, g, stream) : (BN == 128 ? tc_gemm_bn<128>(maps, g, stream) : tc_gemm_bn<64>(maps, g, stream));
-    if (e != cudaSuccess || g.splits == 1) return e;
+    if (splits_out) *splits_out = g.splits;  // the caller adds the partial sums
+    if (e != cudaSuccess || g.splits == 1 || splits_out) return e;
     const size_t n4 = (size_t)I * J / 4;
     return launch_chained(tc_reduce_kernel, (unsigned)((n4 + 255) / 256), 256, 0, stream, (const float4 *)partials, g.splits, n4, alpha, accumulate ? 1 : 0, (float4 *)C);
 }
@@ -649,17 +652,39 @@ __global__ void __launch_bounds__(256) bw_quant_kernel(const __nv_bfloat16 *x, i
     }
 }
 
-// Ternary codes of the packed matrix as a bf16 matrix T [N][K] of -1 / 0 / +1 (one packed word = 16 columns per thread).
-__global__ void __launch_bounds__(256) bw_expand_ternary_kernel(const uint32_t *packed, int N, int K, int steps, size_t n_words,
-                                                                __nv_bfloat16 *T) {
+// The weights' side of the products, one launch: a small layer's pass is a chain of launches of 2 to 3 us (this one as three, and the
+// partial sums of three products added by launches of their own: 64 x 512 -> 512 42.1 us, now 38.8; 2048 -> 5632 at M = 2048
+// 137.9 / 136.8).  The ternary codes of the packed matrix as a bf16 matrix T [N][K] of -1 / 0 / +1 (one packed word = 16 columns
+// per thread), A^T in bf16, and B^T in bf16 with the gate folded in (an element per thread).
+struct BwWeights {
+    const uint32_t *packed;
+    const __half *At, *Bt;
+    const float *gate;
+    __nv_bfloat16 *T, *At_b, *gBt;
+    size_t n_words, n_at, n_bt;      // 0: not wanted
+    unsigned blocks_t, blocks_at;    // blocks of the first two parts
+    int N, K, r, steps;
+};
+__global__ void __launch_bounds__(256) bw_weights_kernel(const BwWeights p) {
     chain();
+    if (blockIdx.x >= p.blocks_t) {
+        const unsigned b = blockIdx.x - p.blocks_t;
+        if (b < p.blocks_at) {
+            const size_t i = (size_t)b * 256 + threadIdx.x;
+            if (i < p.n_at) p.At_b[i] = __float2bfloat16_rn(__half2float(p.At[i]));
+        } else {
+            const size_t i = (size_t)(b - p.blocks_at) * 256 + threadIdx.x;
+            if (i < p.n_bt) p.gBt[i] = __float2bfloat16_rn(__half2float(p.Bt[i]) * p.gate[i / (size_t)p.r]);
+        }
+        return;
+    }
     const size_t w = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (w >= n_words) return;
+    if (w >= p.n_words) return;
     const int kw = (int)(w & 15), r = (int)((w >> 4) & 15);
     const size_t tile = w >> 8;
-    const int n = (int)(tile / steps) * 16 + r, k0 = (int)(tile % steps) * 256 + kw * 16;
-    if (n >= N || k0 >= K) return;
-    const uint32_t word = packed[w];
+    const int n = (int)(tile / p.steps) * 16 + r, k0 = (int)(tile % p.steps) * 256 + kw * 16;
+    if (n >= p.N || k0 >= p.K) return;
+    const uint32_t word = p.packed[w];
     uint32_t o[8];
 #pragma unroll
     for (int j = 0; j < 4; ++j) {
@@ -671,54 +696,53 @@ __global__ void __launch_bounds__(256) bw_expand_ternary_kernel(const uint32_t *
             o[2 * j + (b >> 1)] = *reinterpret_cast<const uint32_t *>(&v);
         }
     }
-    uint4 *dst = reinterpret_cast<uint4 *>(T + (size_t)n * K + k0);
+    uint4 *dst = reinterpret_cast<uint4 *>(p.T + (size_t)n * p.K + k0);
     dst[0] = make_uint4(o[0], o[1], o[2], o[3]);
     dst[1] = make_uint4(o[4], o[5], o[6], o[7]);
 }
 
-// fp16 -> bf16, optionally times a per-row factor (the gate folded into B^T).
-__global__ void __launch_bounds__(256) bw_half_to_bf16_kernel(const __half *src, const float *row_scale, int cols, size_t n, __nv_bfloat16 *dst) {
-    chain();
-    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (i >= n) return;
-    const float s = row_scale ? row_scale[i / (size_t)cols] : 1.0f;
-    dst[i] = __float2bfloat16_rn(__half2float(src[i]) * s);
+// Element i of a product: the sum of its partial results in split order (n elements each), or the product itself.
+__device__ __forceinline__ float split_sum(const float *P, int splits, size_t n, size_t i) {
+    float v = P[i];
+    for (int s = 1; s < splits; ++s) v += P[(size_t)s * n + i];
+    return v;
 }
 
-// Z (fp32 [M][r]) -> H = act(Z) as bf16 [M][r] and SiLU'(Z) as fp32 (in place of Z).
-__global__ void __launch_bounds__(256) bw_act_kernel(float *z, size_t n, int no_silu, __nv_bfloat16 *h) {
+// Z (fp32 [M][r], in `splits` partial sums) -> H = act(Z) as bf16 [M][r] and SiLU'(Z) as fp32.
+__global__ void __launch_bounds__(256) bw_act_kernel(const float *P, int splits, size_t n, int no_silu, float *dact, __nv_bfloat16 *h) {
     chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
-    const float v = z[i];
+    const float v = split_sum(P, splits, n, i);
     const float sg = 1.0f / (1.0f + expf(-v));
     h[i] = __float2bfloat16_rn(no_silu ? v : v * sg);
-    z[i] = no_silu ? 1.0f : sg * (1.0f + v * (1.0f - sg));
+    dact[i] = no_silu ? 1.0f : sg * (1.0f + v * (1.0f - sg));
 }
 
-// dZ = dH * SiLU'(Z), rounded to bf16, and dZ * scale (the copy that enters dX next to gamma_W dY T).
-__global__ void __launch_bounds__(256) bw_dz_kernel(const float *dh, const float *dact, size_t n, float scale, __nv_bfloat16 *dz,
+// dZ = dH * SiLU'(Z), rounded to bf16, and dZ * scale (the copy that enters dX next to gamma_W dY T); dH in partial sums.
+__global__ void __launch_bounds__(256) bw_dz_kernel(const float *P, int splits, const float *dact, size_t n, float scale, __nv_bfloat16 *dz,
                                                     __nv_bfloat16 *dz_scaled) {
     chain();
     const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
     if (i >= n) return;
-    const float v = dh[i] * dact[i];
+    const float v = split_sum(P, splits, n, i) * dact[i];
     dz[i] = __float2bfloat16_rn(v);
     dz_scaled[i] = __float2bfloat16_rn(v * scale);
 }
 
-// From G[n][j] = sum_m dY[m][n] H[m][j]: dBt[n][j] = gate[n] G[n][j] (in place), dgate[n] = sum_j G[n][j] Bt[n][j].
+// From G[n][j] = sum_m dY[m][n] H[m][j] (in partial sums): dBt[n][j] = gate[n] G[n][j], dgate[n] = sum_j G[n][j] Bt[n][j].
 // One warp per output channel n (its r values are contiguous).
-__global__ void __launch_bounds__(256) bw_gate_kernel(float *G, const __half *Bt, const float *gate, int N, int r, float *dgate) {
+__global__ void __launch_bounds__(256) bw_gate_kernel(const float *P, int splits, const __half *Bt, const float *gate, int N, int r, float *dBt,
+                                                      float *dgate) {
     chain();
     const int n = blockIdx.x * 8 + (threadIdx.x >> 5), lane = threadIdx.x & 31;
     if (n >= N) return;
     float dg = 0.0f;
     const float gn = gate[n];
     for (int j = lane; j < r; j += 32) {
-        const float v = G[(size_t)n * r + j];
+        const float v = split_sum(P, splits, (size_t)N * r, (size_t)n * r + j);
         dg = fmaf(v, __half2float(Bt[(size_t)n * r + j]), dg);
-        G[(size_t)n * r + j] = gn * v;
+        dBt[(size_t)n * r + j] = gn * v;
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) dg += __shfl_xor_sync(0xffffffffu, dg, o);
@@ -788,8 +812,8 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     float *partials = (float *)(ws + L.partials);
     bool ok = true;
     auto gemm = [&](TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J, float alpha,
-                    bool acc, bool may_split) {
-        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, stream) == cudaSuccess;
+                    bool acc, bool may_split, int *splits_out = nullptr) {
+        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, splits_out, stream) == cudaSuccess;
     };
     const TcOperand dy_k = {(const __nv_bfloat16 *)dy, N, false};  // dY as [M rows][N contraction]
     const TcOperand dy_mn = {(const __nv_bfloat16 *)dy, N, true};  // dY as [N rows] contracted over its M stored rows
@@ -816,10 +840,21 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false);
     }
     const bool fold = gamma > 1e-20f;  // the low-rank term of dX rides in the same contraction, pre-divided by gamma_W
-    if (grads->dx) {
-        const int steps = (int)(padded_k(d_in) / 256);
-        const size_t n_words = (size_t)row_tiles(d_out) * steps * 256;
-        ok = ok && launch_chained(bw_expand_ternary_kernel, blocks1(n_words), 256, 0, stream, (const uint32_t *)packed, N, K, steps, n_words, bf(L.T)) == cudaSuccess;
+    {
+        BwWeights p = {};
+        p.packed = (const uint32_t *)packed;
+        p.T = bf(L.T);
+        p.N = N; p.K = K; p.r = r;
+        p.steps = (int)(padded_k(d_in) / 256);
+        p.n_words = grads->dx ? (size_t)row_tiles(d_out) * p.steps * 256 : 0;
+        p.blocks_t = blocks1(p.n_words);
+        if (r) {
+            p.At = (const __half *)At; p.At_b = bf(L.At_b); p.n_at = (size_t)r * K;
+            p.Bt = (const __half *)Bt; p.gate = gate; p.gBt = bf(L.gBt); p.n_bt = (size_t)N * r;
+            p.blocks_at = blocks1(p.n_at);
+        }
+        const unsigned blocks = p.blocks_t + p.blocks_at + blocks1(p.n_bt);
+        if (blocks) ok = ok && launch_chained(bw_weights_kernel, blocks, 256, 0, stream, p) == cudaSuccess;
     }
     const TcOperand T_mn = {bf(L.T), K, true};  // T [N][K]: rows k of the product, contracted over n
     if (!r) {
@@ -827,13 +862,12 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
     }
     float *z = (float *)(ws + L.z), *dh = (float *)(ws + L.dh), *G = grads->dBt ? grads->dBt : (float *)(ws + L.G);
-    ok = ok && launch_chained(bw_half_to_bf16_kernel, blocks1((size_t)r * K), 256, 0, stream, (const __half *)At, (const float *)nullptr, K, (size_t)r * K, bf(L.At_b)) == cudaSuccess &&
-         launch_chained(bw_half_to_bf16_kernel, blocks1((size_t)N * r), 256, 0, stream, (const __half *)Bt, gate, r, (size_t)N * r, bf(L.gBt)) == cudaSuccess;
     const TcOperand At_k = {bf(L.At_b), K, false}, At_mn = {bf(L.At_b), K, true};
-    gemm(x_k, At_k, K, none, none, 0, z, r, Mi, r, 1.0f, false, true);                                       // Z = x A
-    ok = ok && launch_chained(bw_act_kernel, blocks1((size_t)M * r), 256, 0, stream, z, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, bf(L.h_b)) == cudaSuccess;
-    gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true);            // dH = dY (g (.) B^T)
-    ok = ok && launch_chained(bw_dz_kernel, blocks1((size_t)M * r), 256, 0, stream, dh, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b)) == cudaSuccess;
+    int sp = 1;
+    gemm(x_k, At_k, K, none, none, 0, z, r, Mi, r, 1.0f, false, true, &sp);                                  // Z = x A
+    ok = ok && launch_chained(bw_act_kernel, blocks1((size_t)M * r), 256, 0, stream, sp > 1 ? partials : z, sp, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, z, bf(L.h_b)) == cudaSuccess;
+    gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true, &sp);       // dH = dY (g (.) B^T)
+    ok = ok && launch_chained(bw_dz_kernel, blocks1((size_t)M * r), 256, 0, stream, sp > 1 ? partials : dh, sp, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b)) == cudaSuccess;
     if (grads->dx) {                                                                                         // dX = gamma_W dY T + dZ A^T
         const TcOperand dzs_k = {bf(L.dzs_b), r, false};
         if (fold) {
@@ -846,8 +880,8 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     if (grads->dAt)                                                                                          // dA^T[j][k] = sum_m dZ[m][j] x[m][k]
         gemm(TcOperand{bf(L.dz_b), r, true}, x_mn, Mi, none, none, 0, grads->dAt, K, r, K, 1.0f, false, true);
     if (grads->dBt || grads->dgate) {                                                                        // G[n][j] = sum_m dY[m][n] H[m][j]
-        gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true);
-        ok = ok && launch_chained(bw_gate_kernel, (unsigned)((N + 7) / 8), 256, 0, stream, G, (const __half *)Bt, gate, N, r, grads->dgate) == cudaSuccess;
+        gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true, &sp);
+        ok = ok && launch_chained(bw_gate_kernel, (unsigned)((N + 7) / 8), 256, 0, stream, sp > 1 ? partials : G, sp, (const __half *)Bt, gate, N, r, G, grads->dgate) == cudaSuccess;
     }
     return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
 }
