@@ -656,13 +656,12 @@ __global__ void __launch_bounds__(DtCfg<B3, NT>::WARPS * 32, 1) decode_tc_kernel
 
 // ---- host side -----------------------------------------------------------------------------------------
 // Shared memory of a launch: the activations' region (two problems side by side where they fit beside a ring of six stages,
-// else the largest one) and the ring.  False: the largest problem leaves fewer than four stages.
+// else what six stages leave, else the largest problem) and the ring.  False: the largest problem leaves fewer than four stages.
 static bool dt_layout(int max_image, int *x_bytes, int *stages) {
     const int room = kDtSmemLimit - kDtOffX;
     max_image = (max_image + 1023) & ~1023;
-    int x = room - 6 * kDtStageBytes;
+    int x = (room - 6 * kDtStageBytes) & ~1023;  // (down: rounded up it cost the sixth stage, and with it the fifth)
     x = x < max_image ? max_image : (x > 2 * max_image ? 2 * max_image : x);
-    x = (x + 1023) & ~1023;
     *x_bytes = x;
     *stages = (room - x) / kDtStageBytes;
     if (*stages > kDtMaxStages) *stages = kDtMaxStages;
@@ -674,6 +673,12 @@ int decode_tc_image_bytes(int max_M, int K, uint32_t flags) { return (max_M <= 8
 bool decode_tc_fits(int max_image, int max_segs) {
     int x, s;
     return max_segs <= kDtMaxSegs && dt_layout(max_image, &x, &s);
+}
+// (for the tests: the layout for activations of that size; out: their region, ring stages, bytes of a stage, shared memory for both)
+extern "C" int hgf_internal_decode_tc_layout(int32_t max_image, int32_t *out) {
+    out[2] = kDtStageBytes;
+    out[3] = kDtSmemLimit - kDtOffX;
+    return dt_layout(max_image, &out[0], &out[1]) ? 1 : 0;
 }
 
 template <bool B3, int NT>
