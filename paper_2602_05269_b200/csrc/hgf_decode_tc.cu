@@ -30,7 +30,8 @@
 //     sum_e c_e x_e = Q_0 x_0 + sum_{e >= 1} (Q_e x_e - 3 Q_e x_{e-1}):
 // the operand is the quotients, not the digits, and the second operand carries x_e and x_{e-1} as two sets of columns (the
 // planes x_4 .. x_0 lie one after the other, so the rows of x_{e-1} follow those of x_e).  Q_0 is the byte itself (less 128: a
-// signed byte), the others are a 16-bit multiplication for two bytes each, exact for every byte.  18 operations give 20 weights.
+// signed byte), the others are a 16-bit multiplication for two bytes each, exact for all 256 values (a byte above 242, which no packed
+// matrix holds, has a fifth digit of 3: weight 2).  18 operations give 20 weights.
 //
 // Bank conflicts: a row tile's 64-byte rows would put the eight threads of a phase on two bank groups.  Row tiles are placed
 // 16 bytes past a multiple of 128 apart and a warp's lanes run over four row tiles, so the eight threads meet all eight groups.
@@ -388,8 +389,8 @@ __global__ void __launch_bounds__(DtCfg<B3, NT>::WARPS * 32, 1) decode_tc_kernel
                         tmem_ld8(acc + C::CORR + 8 * half, corr);
                         if (NT == 1) tmem_ld8(acc + C::CORR + 8, res);
                     }
-                    if constexpr (B3) {  // c_e x_e = Q_e x_e - 3 Q_e x_{e-1}; planes 2 and 3 hold twice, plane 4 eight times Q
-                        constexpr int at[3] = {C::C1, C::C2, C::C3}, shift[3] = {0, 1, 3};
+                    if constexpr (B3) {  // c_e x_e = Q_e x_e - 3 Q_e x_{e-1}; planes 2 and 3 hold twice Q, plane 4 thirty-two times
+                        constexpr int at[3] = {C::C1, C::C2, C::C3}, shift[3] = {0, 1, 5};
 #pragma unroll
                         for (int e = 0; e < 3; ++e) {
                             uint32_t v[8], u[8];
@@ -469,10 +470,10 @@ __global__ void __launch_bounds__(DtCfg<B3, NT>::WARPS * 32, 1) decode_tc_kernel
                             for (int k = 0; k < 8; ++k) {
                                 const uint32_t b4 = w[8 * h + k], e = b4 & 0x00ff00ffu, o = __byte_perm(b4, 0u, 0x4341);
                                 p0[k] = b4 ^ 0x80808080u;                                                          // b - 128
-                                p1[k] = __byte_perm(e * 85u + 0x00530053u, o * 85u + 0x00530053u, 0x7351);         // floor(b / 3)
+                                p1[k] = __byte_perm(e * 85u + 0x00550055u, o * 85u + 0x00550055u, 0x7351);         // floor(b / 3)
                                 p2[k] = __byte_perm(e * 57u, o * 57u, 0x7351) & 0xfefefefeu;                       // 2 floor(b / 9)
                                 p3[k] = __byte_perm(e * 19u, o * 19u, 0x7351) & 0xfefefefeu;                       // 2 floor(b / 27)
-                                p4[k] = __byte_perm(e * 25u + 0x002f002fu, o * 25u + 0x002f002fu, 0x7351) & 0x18181818u;  // 8 floor(b / 81)
+                                p4[k] = __byte_perm(e * 101u + 0x00210021u, o * 101u + 0x00210021u, 0x7351) & 0x60606060u;  // 32 floor(b / 81)
                             }
                             tmem_st8(dst + 8 * h, p0);
                             tmem_st8(dst + 16 + 8 * h, p1);

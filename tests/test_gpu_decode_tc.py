@@ -70,11 +70,49 @@ def test_group_against_oracle(hgf, shapes, base3, cap):
 
 
 def test_base3_quotients_are_exact_for_every_byte():
-    """The operand registers of the base-3 expansion, in the kernel's arithmetic (two bytes in the 16-bit halves of a word)."""
-    b = np.arange(243, dtype=np.uint32)
+    """The operand registers of the base-3 expansion, in the kernel's arithmetic (two bytes in the 16-bit halves of a word).  This is
+    the recipe on its own; test_base3_digits_of_every_byte runs the kernel."""
+    b = np.arange(256, dtype=np.uint32)
     half = lambda m, c: (b * m + c) >> 8  # noqa: E731  (the byte that the permutation takes)
-    assert ((b * 85 + 83) < 65536).all() and ((b * 57) < 65536).all()
-    assert np.array_equal(half(85, 83) & 0xff, b // 3)
+    assert ((b * 101 + 33) < 65536).all() and ((b * 85 + 85) < 65536).all()
+    assert np.array_equal(half(85, 85) & 0xff, b // 3)
     assert np.array_equal(half(57, 0) & 0xfe, 2 * (b // 9))
     assert np.array_equal(half(19, 0) & 0xfe, 2 * (b // 27))
-    assert np.array_equal(half(25, 47) & 0x18, 8 * (b // 81))
+    assert np.array_equal(half(101, 33) & 0x60, 32 * (b // 81))
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("M", [3, 16])
+def test_base3_digits_of_every_byte(hgf, M):
+    """Integer results on packed bytes of all 256 values (242 is the largest a packed matrix holds), against the digits taken apart
+    here: one column tile and two, a launch that the tensor cores take."""
+    rng = np.random.default_rng(7)
+    probs, want = [], []
+    for i, K in enumerate((320, 640)):
+        steps, N = K // 320, 4096
+        raw = rng.integers(0, 256, (N // 16, steps, 16, 64), dtype=np.uint8)
+        raw[0, 0, :4] = np.arange(256, dtype=np.uint8).reshape(4, 64)
+        q = np.arange(64)
+        t, j = q // 16, q % 16
+        c = np.empty((N // 16, steps, 16, 320), dtype=np.int64)  # the code of tile column k: a digit of byte q (hgf.h)
+        for e in range(5):
+            p = j if e < 4 else 16 + j // 4
+            k = 32 * (p // 2) + 16 * (p % 2) + 4 * t + (e if e < 4 else j % 4)
+            c[..., k] = raw.astype(np.int64) // 3 ** e - (3 * (raw.astype(np.int64) // 3 ** (e + 1)) if e < 4 else 0)
+        W = c.transpose(0, 2, 1, 3).reshape(N, K) - 1
+        x = syn.make_x(M, K, config=31, layer=70 + i)
+        xd = dev(x, torch.bfloat16)
+        want.append(hgf.act_quant(xd)[0].cpu().numpy().astype(np.int64) @ W.T)
+        packed = dev(raw.reshape(-1))
+        for _ in range(6):
+            probs.append({"x": xd, "packed": packed, "gamma": 0.5, "d_in": K, "d_out": N,
+                          "y": torch.zeros((M, N), dtype=torch.float32, device="cuda")})
+    group = hgf.Group(probs, flags=hgf.FLAG_BASE3)
+    y_ints = [torch.full(q["y"].shape, -1, dtype=torch.int32, device="cuda") for q in probs]
+    for i, yi in enumerate(y_ints):
+        group.debug(i, yi)
+    group.forward()
+    hgf.check_status()
+    for i, yi in enumerate(y_ints):
+        assert np.array_equal(yi.cpu().numpy(), want[i // 6])
+    group.close()
