@@ -267,7 +267,7 @@ cudaError_t launch_small(const SmallLaunch<NP> &L, bool pdl, cudaStream_t stream
 
 // ---- decode groups on the 5th-generation tensor cores (hgf_decode_tc.cu) --------------------------------
 // The run of 16-row tiles of one problem that falls into a CTA's share.
-struct DecodeTcSeg {
+struct alignas(16) DecodeTcSeg {       // (copied in 16-byte units)
     const uint8_t *packed;           // the run's first row tile
     const int8_t *xq;                // [M][K]
     const float *gamma_x;            // [M]
@@ -281,9 +281,7 @@ struct DecodeTcSeg {
     int M, K, N, r, nslices, gate_group;
     uint32_t flags;
     int steps, lo, n;                // column tiles of a row tile; first row tile (of the problem) and row tiles of the run
-    int reserved[2];
 };
-static_assert(sizeof(DecodeTcSeg) % 16 == 0, "copied in 16-byte units");
 struct DecodeTcLaunch {
     const DecodeTcSeg *segs;
     const int2 *cta;                 // per CTA: first segment, segments

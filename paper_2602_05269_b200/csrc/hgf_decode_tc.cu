@@ -670,7 +670,9 @@ static bool dt_layout(int max_image, int *x_bytes, int *stages) {
     return *stages >= kDtMinStages;
 }
 
-int decode_tc_image_bytes(int max_M, int K, uint32_t flags) { return (max_M <= 8 ? 8 : 16) * weight_steps(K, flags) * ((flags & HGF_FLAG_BASE3) ? 320 : 256); }
+int decode_tc_image_bytes(int max_M, int K, uint32_t flags) {
+    return (flags & HGF_FLAG_BASE3) ? (max_M <= 8 ? 8 : 16) * weight_steps(K, flags) * 320 : 16 * weight_steps(K, flags) * 256;
+}
 bool decode_tc_fits(int max_image, int max_segs) {
     int x, s;
     return max_segs <= kDtMaxSegs && dt_layout(max_image, &x, &s);
@@ -711,7 +713,7 @@ cudaError_t launch_decode_tc(const DecodeTcSeg *segs, const int2 *cta, int grid,
     if (!dt_layout(max_image, &L.x_bytes, &L.stages)) return cudaErrorInvalidValue;
     if (flags & HGF_FLAG_BASE3)
         return max_M <= 8 ? launch_decode_tc_variant<true, 1>(L, grid, pdl, stream) : launch_decode_tc_variant<true, 2>(L, grid, pdl, stream);
-    return max_M <= 8 ? launch_decode_tc_variant<false, 1>(L, grid, pdl, stream) : launch_decode_tc_variant<false, 2>(L, grid, pdl, stream);
+    return launch_decode_tc_variant<false, 2>(L, grid, pdl, stream);  // (two-bit groups of up to eight tokens do not come here)
 }
 
 }  // namespace hgf
