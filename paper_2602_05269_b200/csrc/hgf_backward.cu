@@ -265,10 +265,10 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 // pair 8 KiB on each SM, and a tile's operands are fetched once for 256 rows instead of 128.
 // Barriers: both CTAs' copies count on the first one's FULL; its commits reach both CTAs' EMPTY and ACCFULL; both epilogues
 // arrive on its ACCEMPTY.
-// It takes every product whose output is more than 128 x 128: the tiles of 128 x 256 by single CTAs held the two large products of
+// Which products it takes: tc_pairs_pay.  The tiles of 128 x 256 by single CTAs held the two large products of
 // 2048 x 5632 at M = 8192 at 1.14 and 1.22 PFLOP/s (166, 155 us), pairs at 1.25 and 1.42 (152, 133 us), where the power limit is
 // near (library bf16 products for seconds on end: 1.37).  Whole backward pass in a captured chain: 425 -> 380 us, 8192 x 5632 -> 2048
-// 547 -> 451, 2048 -> 2048 215 -> 186, 1500 x 3200 -> 2000 93 -> 75, 200 x 1024 -> 768 52.9 -> 52.5, 64 x 512 -> 512 41.6 -> 42.1.
+// 547 -> 451, 2048 -> 2048 215 -> 186, 1500 x 3200 -> 2000 93 -> 75.
 struct TpCfg {
     static constexpr int STAGES = 6, A_BYTES = kTBM * 128, STAGE_BYTES = 2 * A_BYTES;
     static constexpr int OFF_BAR = STAGES * STAGE_BYTES;
@@ -277,6 +277,7 @@ struct TpCfg {
     static constexpr uint32_t IDESC = (1u << 4) /*f32*/ | (1u << 7) /*A bf16*/ | (1u << 10) /*B bf16*/ | ((uint32_t)(256 >> 4) << 24);
 };
 constexpr int kTpTile = 256;
+constexpr int kTpMinBlocks = 7, kTpMinBlocksRounds = 10;  // 64-element blocks of the contraction: one round of tiles, several (see tc_pairs_pay)
 
 __device__ __forceinline__ uint32_t cluster_address(uint32_t addr, uint32_t rank) {
     uint32_t r;
@@ -538,14 +539,41 @@ static int tc_pairs_at_once() {
     return n;
 }
 
+// Rounds of the persistent schedule for that many tiles, in halves: the last tiles are worked as twice as many of half the width
+// where that fills their round (`halves`: the operand forms and the width allow it).
+static int tc_half_rounds(int tiles, int at_once, bool halves) {
+    const int rest = tiles % at_once;
+    return 2 * (tiles / at_once) + (rest == 0 ? 0 : (halves && tiles > at_once && 2 * rest <= at_once ? 1 : 2));
+}
+// Whether pairs of CTAs take an I x J product over kb_all blocks of 64.  An output has to be more than 128 x 128.  A short contraction
+// does not repay a pair's start and its hand-overs: over 1300 products (I 136 to 4096, J 192 to 12544; dW or dX alone in a captured
+// chain, single CTAs' time over pairs') 64 to 256 gave 0.85 to 1.03, 448 to 576 gave 0.95 to 1.06 in one round of tiles and 0.93 to 1.08
+// in several, 640 and more 0.97 to 1.54.  And 256-row tiles may need more rounds than 128-row ones: one and a half
+// instead of one gave 0.86 to 0.98 at any contraction, two and a half instead of two 0.91 to 0.99 up to 1024 and 0.98 to 1.14 from
+// 2048 on.  4096 x 4096 over 300: 32.4 us, by pairs 35.3; 384 x 9984 over 640: 21.7, 25.3; 8192 x 2048 over 5632: 155, 133.
+static bool tc_pairs_pay(int I, int J, int kb_all, bool b_mn, int sms, int pairs) {
+    if (I <= kTBM || J <= 128 || pairs <= 0 || sms <= 0) return false;
+    const int tiles_j = (J + 255) / 256, tiles = (I + kTpTile - 1) / kTpTile * tiles_j;
+    if (kb_all < (tiles <= pairs ? kTpMinBlocks : kTpMinBlocksRounds)) return false;
+    const bool halves = b_mn && J % 256 == 0;
+    const int by_pairs = tc_half_rounds(tiles, pairs, halves), by_one = tc_half_rounds((I + kTBM - 1) / kTBM * tiles_j, sms, halves);
+    return by_pairs <= by_one || (kb_all >= 16 && 4 * by_pairs <= 5 * by_one);
+}
+// (for the tests)
+extern "C" int hgf_internal_tc_pairs_pay(int32_t I, int32_t J, int32_t contraction, int32_t sms, int32_t pairs) {
+    return tc_pairs_pay(I, J, (contraction + kTBK - 1) / kTBK, true, sms, pairs) ? 1 : 0;
+}
+
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
 // operand forms.  `partials` (splits_max * I * ldc floats) enables splitting the contraction when the
 // output has fewer tiles than the device has SMs; ldc must then be J.  With `splits_out` they are left there for the kernel that
 // reads the product next (*splits_out of them; 1: the product is in C).  Bases 16-byte aligned, ld % 8 == 0.
 static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J,
                            float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, cudaStream_t stream) {
-    const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64);
-    const int pairs = I > kTBM && J > 128 ? tc_pairs_at_once() : 0;
+    const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64), sms = device_sm_count();
+    const int kb1 = (Cn + kTBK - 1) / kTBK, kb2 = A2.p ? (Cn2 + kTBK - 1) / kTBK : 0, kb_all = kb1 + kb2;
+    int pairs = I > kTBM && J > 128 && kb_all >= kTpMinBlocks && sms > 0 ? tc_pairs_at_once() : 0;
+    if (!tc_pairs_pay(I, J, kb_all, B.mn, sms, pairs)) pairs = 0;
     CUtensorMap maps[4];
     const int rows_b = pairs ? 128 : BN;
     if (!tc_map(&maps[0], A, I, Cn, kTBM) || !tc_map(&maps[1], B, J, Cn, rows_b)) return cudaErrorInvalidValue;
@@ -554,8 +582,8 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
     if (A2.p && (!tc_map(&maps[2], A2, I, Cn2, kTBM) || !tc_map(&maps[3], B2, J, Cn2, rows_b))) return cudaErrorInvalidValue;
     TcGemmArgs g = {};
     g.I = I; g.J = J; g.ldc = ldc;
-    g.kb1 = (Cn + kTBK - 1) / kTBK;
-    g.kb2 = A2.p ? (Cn2 + kTBK - 1) / kTBK : 0;
+    g.kb1 = kb1;
+    g.kb2 = kb2;
     g.a_mn = A.mn; g.b_mn = B.mn;
     if (pairs) {
         const int tiles = ((I + kTpTile - 1) / kTpTile) * ((J + kTpTile - 1) / kTpTile);
@@ -569,7 +597,7 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
         return launch_chained(tc_pair_gemm_kernel, 2u * (unsigned)(work < pairs ? work : pairs), kTThreads, TpCfg::SMEM_BYTES, stream, maps[0], maps[1],
                               maps[2], maps[3], g, status);
     }
-    const int kb_all = g.kb1 + g.kb2, tiles = ((I + kTBM - 1) / kTBM) * ((J + BN - 1) / BN), sms = device_sm_count();
+    const int tiles = ((I + kTBM - 1) / kTBM) * ((J + BN - 1) / BN);
     int splits = 1;
     if (partials && ldc == J && sms > 0 && tiles * 2 <= sms) {
         splits = sms / tiles;

@@ -94,7 +94,48 @@ def test_row_lengths_of_the_quantiser(hgf, M, K, N, r):
 
 
 @pytest.mark.parametrize("M,K,N,r", [(40, 192, 136, 16), (257, 320, 264, 64), (256, 256, 256, 32), (1, 192, 136, 0), (130, 2112, 384, 48)])
-def test_tiles_of_cta_pairs(hgf, M, K, N, r):
-    """Outputs just past 128 rows and columns (the second CTA of a pair has 8 rows, or none), exact 256 x 256 tiles, a contraction of
-    one element, column tiles that end inside the second CTA's half."""
+def test_outputs_just_past_one_tile(hgf, M, K, N, r):
+    """Outputs just past 128 rows and columns with a short contraction (single CTAs): ragged tiles, a contraction of one element."""
     check(hgf, M, K, N, r, layer=M + 500, lora=r > 0)
+
+
+# contractions that pairs take: dW contracts over M, dX over N (and r)
+@pytest.mark.parametrize("M,K,N,r", [(440, 192, 136, 16), (700, 320, 264, 64), (768, 256, 256, 32), (641, 192, 136, 0), (136, 192, 640, 16),
+                                     (257, 320, 648, 64), (256, 256, 768, 0), (650, 2112, 704, 48)])
+def test_tiles_of_cta_pairs(hgf, M, K, N, r):
+    """Outputs just past 128 rows and columns (the second CTA of a pair has 8 rows, or none), exact 256 x 256 tiles, a contraction that
+    ends inside a block, column tiles that end inside the second CTA's half."""
+    check(hgf, M, K, N, r, layer=M + 500, lora=r > 0)
+
+
+def _close(got, a, b, alpha=1.0):
+    """got = alpha a b in fp32 against 64 bits: each of the C products is exact in fp32; an addition in the tensor core's accumulator may
+    cut off instead of rounding and align its products first, so it is charged 2^-22 of the sum of magnitudes."""
+    a, b = a.double(), b.double()
+    bound = (a.shape[1] + 2) * 2.0 ** -22 * abs(alpha) * (a.abs() @ b.abs())
+    err = (got.double() - alpha * (a @ b)).abs()
+    assert bool((err <= bound).all()), float((err / bound.clamp_min(1e-30)).max())
+
+
+@pytest.mark.parametrize("C,I,J", [(648, 4088, 4160), (640, 4096, 4096), (648, 3592, 4096)])
+def test_cta_pairs_with_many_tiles_each(hgf, C, I, J):
+    """Every pair of CTAs takes at least three output tiles, so accumulators are handed back between the two CTAs and used again:
+    dW (both operands with the contraction outside) and dX (the first one with it inside), ragged in both extents, and last rounds
+    of whole and of half tiles."""
+    assert hgf.lib().hgf_internal_tc_pairs_pay(I, J, C, 148, 74) == 1
+    g = torch.Generator(device="cuda")
+    g.manual_seed(C + I)
+    W = torch.randn((I, J), generator=g, device="cuda")
+    packed, gamma = hgf.pack_ternary(W)
+    x = torch.randn((C, J), generator=g, device="cuda").to(torch.bfloat16)
+    dy = torch.randn((C, I), generator=g, device="cuda").to(torch.bfloat16)
+    got = hgf.linear_backward(x, packed, gamma, J, I, dy, want=("dW",))["dW"]
+    xq, gx, _ = hgf.act_quant(x)
+    xd = (xq.float() * (gx * (1.0 / 127.0))[:, None]).to(torch.bfloat16)
+    _close(got, dy.t(), xd)
+    packed, gamma = hgf.pack_ternary(W[:C])
+    T = hgf.unpack_ternary(packed, C, J)
+    x = torch.randn((I, J), generator=g, device="cuda").to(torch.bfloat16)
+    dy = torch.randn((I, C), generator=g, device="cuda").to(torch.bfloat16)
+    _close(hgf.linear_backward(x, packed, gamma, J, C, dy, want=("dx",))["dx"], dy, T, gamma)
+    hgf.check_status()
