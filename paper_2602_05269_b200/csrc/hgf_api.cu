@@ -398,17 +398,78 @@ struct hgf_group {
 };
 
 namespace hgf {
-// Whether a group's contraction runs on decode_tc_kernel, and its shares: base-3 weights, or more than eight tokens.  Measured over
-// one to 36 blocks, widths 512 to 4096, ranks 16 to 64 (a captured chain, warp MMA against tensor memory): base-3 1.04 to 1.30
-// times as fast, 9 to 16 tokens 1.00 to 1.29; two-bit weights with up to eight tokens 0.86 to 0.96, which stay where they were.
-// More runs of row tiles on a CTA than its table holds, or activations that leave no room for the ring, stay there too.
-static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const DecodeProblem *d_probs, int max_M, uint32_t flags,
-                           std::vector<DecodeTcSeg> *segs, std::vector<int2> *cta, int *image) {
-    const int sms = device_sm_count(), n = (int)dps.size();
-    if (sms <= 0 || sms > 1024 || (max_M <= 8 && !(flags & HGF_FLAG_BASE3))) return false;
+// The GEMV's split of the launch-wide tile sequence into contiguous shares of equal cost, one per CTA: first tile, end tile, first problem.
+static std::vector<int4> gemv_ranges(const std::vector<DecodeProblem> &dps, long long cost, int tiles, int grid, uint32_t flags) {
+    const int n = (int)dps.size();
+    std::vector<int4> ranges;
+    auto tile_of_cost = [&](long long c, int *prob) {
+        int lo = 0, hi = n - 1;
+        while (lo < hi) {  // last problem with cost_begin <= c
+            const int mid = (lo + hi + 1) >> 1;
+            if (dps[mid].cost_begin <= c) lo = mid; else hi = mid - 1;
+        }
+        const long long steps = row_tile_cost(dps[lo].K, flags), tl = row_tiles(dps[lo].N);
+        long long local = (c - dps[lo].cost_begin + steps - 1) / steps;
+        if (local > tl) local = tl;
+        *prob = lo;
+        return dps[lo].tile_begin + (int)local;
+    };
+    for (int c = 0; c < grid; ++c) {
+        int p0 = 0, p1 = 0;
+        const int t0 = tile_of_cost(cost * c / grid, &p0);
+        const int t1 = c + 1 == grid ? tiles : tile_of_cost(cost * (c + 1) / grid, &p1);
+        while (p0 + 1 < n && dps[p0 + 1].tile_begin <= t0) ++p0;  // the problem that holds tile t0
+        ranges.push_back(make_int4(t0, t1, p0, 0));
+    }
+    return ranges;
+}
+
+// Whether decode_tc_kernel is the faster one for a group that it can take (base-3 weights, or more than eight tokens).  It spends a
+// whole block of 128 rows on a run of row tiles, however few they are, and its start grows with K (x~ and H of the first problem);
+// the warp MMA splits such runs over its sixteen warps, but loses 2.5 to 5 us at every change of problem inside a CTA's share.  So:
+// the 1 KiB tiles of the GEMV's largest share against the column tiles of blocks of this kernel's (`blocks`), by the longest row
+// (`longest`, in column tiles) and by whether a GEMV share holds several problems.  Captured chains, warp MMA's time over this
+// kernel's, 1650 groups: one to three equal problems, blocks of transformers (one to twelve, 512 to 4096 wide), mixed sizes.
+//   base-3, shares of one problem:   taken 0.98 to 1.42, mean 1.19; left 0.73 to 1.16, mean 0.94  (2048 -> 2048, M = 1: 10.9 us, here 12.0)
+//   base-3, several problems:        taken 0.90 to 1.53, mean 1.20; left 0.82 to 1.50, mean 0.99
+//   two-bit, shares of one problem:  taken 0.95 to 1.18, mean 1.05; left 0.86 to 1.17, mean 0.95  (5632 -> 2048, M = 16: 19.1 us, here 22.1)
+//   two-bit, several problems:       taken 0.95 to 1.57, mean 1.27; left 0.74 to 1.49, mean 1.06  (rows longer than 4200 on average, most of them)
+// Two-bit weights with up to eight tokens: 0.86 to 0.96 on whole blocks; not taken.
+static bool decode_tc_pays(const std::vector<DecodeProblem> &dps, const std::vector<int4> &ranges, long long blocks, uint32_t flags) {
+    long long share = 0, tiles = 0, weighted = 0;
+    int several = 1, longest = 0;
+    for (const int4 &c : ranges) {
+        long long sum = 0;
+        int held = 0;
+        for (size_t p = (size_t)c.z; p < dps.size() && dps[p].tile_begin < c.y; ++p) {
+            const int lo = dps[p].tile_begin > c.x ? dps[p].tile_begin : c.x, end = dps[p].tile_begin + (int)row_tiles(dps[p].N), hi = end < c.y ? end : c.y;
+            if (lo >= hi) continue;
+            sum += (long long)(hi - lo) * weight_steps(dps[p].K, flags);
+            ++held;
+        }
+        share = sum > share ? sum : share;
+        several = held > several ? held : several;
+    }
+    for (const DecodeProblem &P : dps) {
+        const int steps = weight_steps(P.K, flags);
+        longest = steps > longest ? steps : longest;
+        tiles += row_tiles(P.N) * steps;
+        weighted += row_tiles(P.N) * steps * steps;
+    }
+    if (flags & HGF_FLAG_BASE3) return share >= (several > 1 ? 1 : 2) * blocks && 13 * share >= 2 * longest * blocks;
+    if (several > 1) return share >= blocks && 10 * share >= longest * blocks && 2 * weighted <= 33 * tiles;
+    return longest <= 8 || (longest <= 13 && 7 * share >= 2 * longest * blocks);
+}
+
+// A group's shares on decode_tc_kernel; false: its contraction stays on the GEMV (see decode_tc_pays; also more runs of row tiles on a
+// CTA than its table holds, or activations that leave no room for the ring).
+static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const std::vector<int4> &ranges, const DecodeProblem *d_probs, int max_M, uint32_t flags,
+                           int sms, std::vector<DecodeTcSeg> *segs, std::vector<int2> *cta, int *image) {
+    const int n = (int)dps.size();
+    if (sms <= 0 || sms > 1024 || ranges.empty() || (max_M <= 8 && !(flags & HGF_FLAG_BASE3))) return false;
     // a row tile's cost: its weight tiles, and its rows of B^T (1 KiB at r = 32)
     auto cost_of = [&](int i) { return 32ll * weight_steps(dps[i].K, flags) + dps[i].r; };
-    long long cost = 0;
+    long long cost = 0, slowest = 0;
     *image = 0;
     for (int i = 0; i < n; ++i) {
         cost += row_tiles(dps[i].N) * cost_of(i);
@@ -420,6 +481,7 @@ static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const DecodePr
     for (int c = 0; c < sms; ++c) {
         const int first = (int)segs->size();
         const long long until = cost * (c + 1) / sms;
+        long long blocks = 0;
         while (p < n && dealt < until) {
             const DecodeProblem &P = dps[p];
             const long long per = cost_of(p), tiles = row_tiles(P.N);
@@ -436,16 +498,41 @@ static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const DecodePr
             s.M = P.M; s.K = P.K; s.N = P.N; s.r = P.r; s.gate_group = P.gate_group; s.flags = P.flags;
             s.lo = t; s.n = (int)take;
             segs->push_back(s);
+            blocks += (take + 7) / 8 * s.steps;
             dealt += take * per;
             t += (int)take;
             if (t == tiles) { ++p; t = 0; }
         }
+        slowest = blocks > slowest ? blocks : slowest;
         cta->push_back(make_int2(first, (int)segs->size() - first));
         max_segs = cta->back().y > max_segs ? cta->back().y : max_segs;
     }
-    return p == n && decode_tc_fits(*image, max_segs);
+    return p == n && decode_tc_fits(*image, max_segs) && decode_tc_pays(dps, ranges, slowest, flags);
 }
 }  // namespace hgf
+
+// (for the tests: whether a group of these layers would run on decode_tc_kernel on a device of that many SMs, and the most problems that a
+// CTA of it would hold)
+extern "C" int hgf_internal_group_on_tensor_memory(const int32_t *K, const int32_t *N, int32_t n, int32_t r, int32_t max_M, uint32_t flags,
+                                                   int32_t sms, int32_t *most_problems) {
+    std::vector<DecodeProblem> dps((size_t)n);
+    long long cost = 0;
+    int tiles = 0, image = 0;
+    for (int i = 0; i < n; ++i) {
+        dps[i] = DecodeProblem{};
+        dps[i].K = K[i]; dps[i].N = N[i]; dps[i].r = r;
+        dps[i].tile_begin = tiles;
+        dps[i].cost_begin = cost;
+        tiles += (int)row_tiles(N[i]);
+        cost += row_tiles(N[i]) * row_tile_cost(K[i], flags);
+    }
+    std::vector<DecodeTcSeg> segs;
+    std::vector<int2> cta;
+    const bool tc = plan_decode_tc(dps, sms > 0 ? gemv_ranges(dps, cost, tiles, tiles < sms ? tiles : sms, flags) : std::vector<int4>(), dps.data(), max_M, flags, sms, &segs, &cta, &image);
+    *most_problems = 0;
+    for (const int2 &c : cta) *most_problems = c.y > *most_problems ? c.y : *most_problems;
+    return tc ? 1 : 0;
+}
 
 extern "C" hgf_status hgf_group_create(const hgf_problem *problems, int32_t n, uint32_t flags, hgf_group **out) {
     return hgf_group_create_ln(problems, nullptr, n, flags, out);
@@ -600,35 +687,14 @@ extern "C" hgf_status hgf_group_create_ln(const hgf_problem *problems, const hgf
     // the GEMV's split of the launch-wide tile sequence into equal contiguous shares, one per CTA
     g->grid = decode_grid(tiles);
     std::vector<int4> ranges;
-    if (g->grid > 0 && g->grid <= 1024) {
-        auto tile_of_cost = [&](long long c, int *prob) {
-            int lo = 0, hi = n - 1;
-            while (lo < hi) {  // last problem with cost_begin <= c
-                const int mid = (lo + hi + 1) >> 1;
-                if (dps[mid].cost_begin <= c) lo = mid; else hi = mid - 1;
-            }
-            const long long steps = row_tile_cost(dps[lo].K, flags), tl = row_tiles(dps[lo].N);
-            long long local = (c - dps[lo].cost_begin + steps - 1) / steps;
-            if (local > tl) local = tl;
-            *prob = lo;
-            return dps[lo].tile_begin + (int)local;
-        };
-        for (int c = 0; c < g->grid; ++c) {
-            int p0 = 0, p1 = 0;
-            const int t0 = tile_of_cost(cost * c / g->grid, &p0);
-            const int t1 = c + 1 == g->grid ? tiles : tile_of_cost(cost * (c + 1) / g->grid, &p1);
-            while (p0 + 1 < n && dps[p0 + 1].tile_begin <= t0) ++p0;  // the problem that holds tile t0
-            ranges.push_back(make_int4(t0, t1, p0, 0));
-        }
-    } else {
-        g->d_cta_range = nullptr;  // the kernel works its share out itself
-    }
+    if (g->grid > 0 && g->grid <= 1024) ranges = gemv_ranges(dps, cost, tiles, g->grid, flags);
+    else g->d_cta_range = nullptr;  // the kernel works its share out itself
     // the same on the tensor cores: shares of 16-row tiles of equal cost, cut into their problems' runs
     std::vector<DecodeTcSeg> tc_segs;
     std::vector<int2> tc_cta;
     g->d_tc_segs = (DecodeTcSeg *)((char *)mem + off_tc_segs);
     g->d_tc_cta = (int2 *)((char *)mem + off_tc_cta);
-    g->tc = plan_decode_tc(dps, g->d_probs, max_M, flags, &tc_segs, &tc_cta, &g->tc_image);
+    g->tc = plan_decode_tc(dps, ranges, g->d_probs, max_M, flags, device_sm_count(), &tc_segs, &tc_cta, &g->tc_image);
     g->tc_grid = (int)tc_cta.size();
     bool ok = cudaMemcpy(g->d_probs, dps.data(), sizeof(DecodeProblem) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
               cudaMemcpy(g->d_pps, pps.data(), sizeof(PrologueParams) * (size_t)n, cudaMemcpyHostToDevice) == cudaSuccess &&
