@@ -77,7 +77,8 @@ def check_group(hgf, shapes, base3, cap, *, flags=0, bf16=False, variants=5):
         ref = oracle.forward(*h, flags=oflags)
         assert np.array_equal(yi.cpu().numpy(), ref["y_int"]), (i, shapes[i])
         y, peak = ref["y"], np.abs(ref["y"]).max()
-        rounding = 1.01 * 2.0 ** -9 * np.abs(y) if bf16 else 0.0   # (bf16: half a unit in the last place)
+        # bf16 has eight significant bits: the result of the path, within TOL of y, is rounded by up to 2^-8 of itself
+        rounding = 2.0 ** -8 * (np.abs(y) + TOL * peak) if bf16 else 0.0
         over = np.abs(q["y"].float().cpu().numpy().astype(np.float64) - y) - rounding
         assert over.max() <= TOL * peak, (i, shapes[i], over.max() / peak)
     group.close()
