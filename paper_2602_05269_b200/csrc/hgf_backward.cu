@@ -534,7 +534,10 @@ static int tc_pairs_at_once() {
     cfg.gridDim = dim3(2);
     cfg.blockDim = dim3(kTThreads);
     cfg.dynamicSmemBytes = TpCfg::SMEM_BYTES;
-    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_gemm_kernel, &cfg) != cudaSuccess || n <= 0) return 0;
+    if (cudaOccupancyMaxActiveClusters(&n, tc_pair_gemm_kernel, &cfg) != cudaSuccess || n <= 0) {
+        cudaGetLastError();  // (single CTAs take the product: their launch is not to report this call's error)
+        return 0;
+    }
     cache[dev].store(n, std::memory_order_release);
     return n;
 }
