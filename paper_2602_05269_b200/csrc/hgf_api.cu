@@ -428,15 +428,17 @@ static std::vector<int4> gemv_ranges(const std::vector<DecodeProblem> &dps, long
 // whole block of 128 rows on a run of row tiles, however few they are, and its start grows with K (x~ and H of the first problem);
 // the warp MMA splits such runs over its sixteen warps, but loses 2.5 to 5 us at every change of problem inside a CTA's share.  So:
 // the 1 KiB tiles of the GEMV's largest share against the column tiles of blocks of this kernel's (`blocks`), by the longest row
-// (`longest`, in column tiles) and by whether a GEMV share holds several problems.  Captured chains, warp MMA's time over this
-// kernel's, 1650 groups: one to three equal problems, blocks of transformers (one to twelve, 512 to 4096 wide), mixed sizes.
-//   base-3, shares of one problem:   taken 0.98 to 1.42, mean 1.19; left 0.73 to 1.16, mean 0.94  (2048 -> 2048, M = 1: 10.9 us, here 12.0)
-//   base-3, several problems:        taken 0.90 to 1.53, mean 1.20; left 0.82 to 1.50, mean 0.99
+// (`longest`, in column tiles) and by whether a GEMV share holds several problems.  Where only the GEMV's shares do (`runs`: problems of
+// this kernel's largest) it is always this kernel's (1.10 to 1.53); on base-3 weights short rows on less than half of the SMs are too
+// (0.96 to 1.16, mean 1.05).  Captured chains, warp MMA's time over this kernel's, 1650 groups: one to three equal problems, blocks of
+// transformers (one to twelve, 512 to 4096 wide), mixed sizes.
+//   base-3, shares of one problem:   taken 0.96 to 1.42, mean 1.17; left 0.73 to 1.07, mean 0.91  (2048 -> 2048, M = 1: 10.9 us, here 12.0)
+//   base-3, several problems:        taken 0.90 to 1.53, mean 1.20; left 0.82 to 1.22, mean 0.96
 //   two-bit, shares of one problem:  taken 0.95 to 1.18, mean 1.05; left 0.86 to 1.17, mean 0.95  (5632 -> 2048, M = 16: 19.1 us, here 22.1)
-//   two-bit, several problems:       taken 0.95 to 1.57, mean 1.27; left 0.74 to 1.49, mean 1.06  (rows longer than 4200 on average, most of them)
+//   two-bit, several problems:       taken 0.95 to 1.57, mean 1.27; left 0.74 to 1.32, mean 1.04  (rows longer than 4200 on average, most of them)
 // Two-bit weights with up to eight tokens: 0.86 to 0.96 on whole blocks; not taken.
-static bool decode_tc_pays(const std::vector<DecodeProblem> &dps, const std::vector<int4> &ranges, long long blocks, uint32_t flags) {
-    long long share = 0, tiles = 0, weighted = 0;
+static bool decode_tc_pays(const std::vector<DecodeProblem> &dps, const std::vector<int4> &ranges, long long blocks, int runs, uint32_t flags, int sms) {
+    long long share = 0, tiles = 0, weighted = 0, rows = 0;
     int several = 1, longest = 0;
     for (const int4 &c : ranges) {
         long long sum = 0;
@@ -453,9 +455,12 @@ static bool decode_tc_pays(const std::vector<DecodeProblem> &dps, const std::vec
     for (const DecodeProblem &P : dps) {
         const int steps = weight_steps(P.K, flags);
         longest = steps > longest ? steps : longest;
+        rows += row_tiles(P.N);
         tiles += row_tiles(P.N) * steps;
         weighted += row_tiles(P.N) * steps * steps;
     }
+    if (several > 1 && runs == 1) return true;
+    if ((flags & HGF_FLAG_BASE3) && several == 1 && longest <= 4 && 2 * rows <= sms) return true;
     if (flags & HGF_FLAG_BASE3) return share >= (several > 1 ? 1 : 2) * blocks && 13 * share >= 2 * longest * blocks;
     if (several > 1) return share >= blocks && 10 * share >= longest * blocks && 2 * weighted <= 33 * tiles;
     return longest <= 8 || (longest <= 13 && 7 * share >= 2 * longest * blocks);
@@ -507,7 +512,7 @@ static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const std::vec
         cta->push_back(make_int2(first, (int)segs->size() - first));
         max_segs = cta->back().y > max_segs ? cta->back().y : max_segs;
     }
-    return p == n && decode_tc_fits(*image, max_segs) && decode_tc_pays(dps, ranges, slowest, flags);
+    return p == n && decode_tc_fits(*image, max_segs) && decode_tc_pays(dps, ranges, slowest, max_segs, flags, sms);
 }
 }  // namespace hgf
 

@@ -46,6 +46,7 @@ def block(d, ffn):
     (block(2048, 5632) * 36, 16, 32, False, 1.08), (block(4096, 11008) * 8, 1, 64, True, 1.16), (block(2048, 5632), 9, 32, False, 1.17),
     (block(512, 1408), 16, 32, False, 1.48), (block(1024, 2816), 8, 32, True, 1.08), ([(4096, 11008)] * 2, 1, 64, True, 1.18),
     ([(2048, 5632)] * 2, 16, 32, False, 1.07), ([(4096, 4096)] * 3, 16, 64, False, 1.16), ([(3200, 3200)], 1, 64, True, 1.20),
+    ([(768, 208), (3200, 312)], 9, 16, False, 1.49), ([(1024, 256)], 1, 16, True, 1.16), ([(1024, 2048)], 1, 64, True, 0.94),
     ([(5632, 2048)], 1, 32, True, 0.82), ([(5632, 2048)], 16, 32, False, 0.86), ([(11008, 4096)], 8, 64, True, 0.86),
     ([(2048, 2048)], 1, 32, True, 0.91), ([(4096, 4096)], 16, 64, False, 0.95), ([(8192, 1536)], 1, 32, True, 0.73),
     ([(5632, 2048)] * 3, 16, 32, False, 0.90), ([(2048, 2056), (320, 136), (5632, 520), (256, 128)], 16, 32, False, 0.91),
