@@ -1,6 +1,7 @@
 // Decode path, M <= 16 tokens: one pass over the packed ternary weights (Algorithm 1, step 3),
 // with the dequantisation (step 4), the LoRA up-projection (step 7) and the gated fusion (step 8)
-// fused into the epilogue.  One launch serves one layer or a group of independent layers.
+// fused into the epilogue.  One launch serves one layer or a group of independent layers (groups on base-3 weights or of more than
+// eight tokens run on hgf_decode_tc.cu where that is the faster one: decode_tc_pays in hgf_api.cu).
 //
 // The kernel is bound by the packed-weight stream from HBM, so it is built around keeping that
 // stream busy.  One persistent CTA of 16 warps per SM.  The weights of all problems of the launch
