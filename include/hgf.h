@@ -102,7 +102,8 @@ hgf_status hgf_unpack_ternary(const void *packed, int64_t d_out, int64_t d_in, i
  * c0 + 3 c1 + 9 c2 + 27 c3 + 81 c4 (0..242), the nearest byte-aligned packing to the log2(3) = 1.58
  * bits the paper counts per ternary weight (Introduction, the T_max bound; Section 4.2, the
  * effective bit-width).  It takes a fifth off the weight stream of the memory-bound decode path at
- * the price of a table look-up per byte; forward calls take it with HGF_FLAG_BASE3.  The decode
+ * the price of decoding: a table look-up per byte in single calls and small groups, arithmetic on the
+ * bytes in the others; forward calls take it with HGF_FLAG_BASE3.  The decode
  * path (M <= HGF_DECODE_MAX_M) computes straight from the base-3 bytes.  The compute-bound GEMM path
  * reads two-bit tiles: given base-3 weights, hgf_linear_forward first rewrites the layer's tiles into
  * its workspace (one small launch; hgf_workspace_bytes with the flag includes the room), so a model

@@ -1,12 +1,12 @@
 // Decode groups on the 5th-generation tensor cores (M <= 16 tokens): the contraction of Algorithm 1, step 3, with the
-// epilogue of steps 4, 7 and 8.  It takes the groups on base-3 weights and those of more than eight tokens; two-bit groups of up to
-// eight tokens stay on the warp MMA of hgf_decode.cu (the rule and its figures: plan_decode_tc).
+// epilogue of steps 4, 7 and 8.  It takes groups on base-3 weights and those of more than eight tokens where it is the faster kernel
+// (decode_tc_pays in hgf_api.cu: the rule and its figures); the others stay on the warp MMA of hgf_decode.cu.
 //
-// In hgf_decode.cu every warp carries codes, activations and accumulators through its own registers: 122 instructions a 1 KiB
-// weight tile for two sets of eight tokens, 270 on base-3 weights, and the issue slots bound it.  Here 128 output rows go
+// In hgf_decode.cu every warp carries codes, activations and accumulators through its own registers: 155 instructions a 1 KiB
+// weight tile for two sets of eight tokens (counted over a launch), and the issue slots bound it.  Here 128 output rows go
 // through one instruction: a thread owns one row, turns the row's packed bytes into int8 operands and puts them into tensor
 // memory (tcgen05.st), and tcgen05.mma.kind::i8 contracts them with the tokens, which lie in shared memory in the operand's
-// order: 35 instructions a tile for any number of tokens, 75 on base-3 weights.
+// order: the expansion of a tile is 43 instructions for any number of tokens (150 on base-3 weights), all roles with their waits 132.
 //
 // One persistent CTA per SM:
 //   warp 0 and one of the last two: producers, in turns; a stage is two column tiles of eight row tiles (128 rows), one bulk
@@ -16,10 +16,13 @@
 //   warps 2-5    epilogue: a thread owns an output channel; they also fetch the rows of B^T of the row tiles to come
 //   warps 6-     expansion, four warps an operand stage in tensor memory (three stages, two on base-3 weights)
 //   then four or eight warps that stage a problem's activations (one problem ahead where shared memory has the room), H and scales
-// What bounds it is the MMA issuer: 840 clocks a stage of 16 MMAs beside the other warps (its waits, the MMAs' operands through
-// uniform registers), 470 a column tile with the ends of the row-tile blocks, where HBM alone would take 330.  Against the warp
-// MMA, one launch with its prologue, 2048-wide blocks with r = 32: 16 tokens, 36 blocks 167 -> 155 us, 2 blocks 31.2 -> 26.2; base-3
-// weights, 4096-wide, r = 64, one token, 8 blocks 153.5 -> 133; 2048-wide, 8 tokens, 36 blocks 212 -> 165.
+// What bounds it is the chain of the MMA issuer.  Stamped on one B200, 36 blocks of 2048, 16 tokens: of 241 thousand clocks in the middle
+// CTA the issuer waits 13 for the first x~, 10 for x~ at changes of problem, 46 for operands and 33 for accumulators that the epilogue
+// still reads; the rest is 360 clocks for the 8 MMAs of a column tile, their commits and loops, where HBM alone would take 330.  The CTAs
+// end 123 to 143 us after the first one's start: shares are cut in 16-row tiles, but a run costs whole blocks of eight.  8 blocks of
+// 4096 on base-3 weights, one token: 199 thousand, 9 for x~, 50 for operands, 7 for accumulators, 490 a column tile of 10 MMAs.
+// Against the warp MMA, one launch with its prologue, 2048-wide blocks with r = 32: 16 tokens, 36 blocks 167 -> 155 us, 2 blocks
+// 31.2 -> 26.2; base-3 weights, 4096-wide, r = 64, one token, 8 blocks 153.5 -> 133; 2048-wide, 8 tokens, 36 blocks 212 -> 165.
 //
 // Two-bit codes: masked in place they are codes times 1, 4, 16 (the fourth position is shifted down by two: 64 times a code
 // would not fit a signed byte), and each scale has an accumulator; the scaled sums are exact multiples.  The order of K

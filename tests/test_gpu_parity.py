@@ -364,7 +364,7 @@ def test_group_of_independent_layers_matches_oracle_and_single_calls(hgf, M):
     for q, ref, (s, m, lora) in zip(probs, refs, shapes):
         y_single = hgf.linear_forward(q["x"], q["packed"], q["gamma"], s.d_in, s.d_out, q.get("At"), q.get("Bt"),
                                       q.get("gate"))
-        # same GEMV kernel; the two prologues add the K slices of x A in different orders (fp32)
+        # the two paths add the K slices of x A, and the parts of H, in different orders (fp32); integers are the same
         assert (y_single - q["y"]).abs().max().item() <= 2e-6 * np.abs(ref["y"]).max(), s
     group.close()
 
