@@ -1,4 +1,4 @@
-"""Build libhgf_b200.so (sm_100a) in-tree with nvcc.  Run as `python -m paper_2602_05269_b200.build`."""
+"""Build libhgf_b200.so (sm_100a, nvcc) and _hgf_python.so (the binding's native part) in-tree.  Run as `python -m paper_2602_05269_b200.build`."""
 from __future__ import annotations
 
 import os
@@ -9,6 +9,7 @@ from concurrent.futures import ThreadPoolExecutor
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhgf_b200.so")
+MODULE = os.path.join(HERE, "_hgf_python.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["hgf_api.cu", "hgf_pack.cu", "hgf_prologue.cu", "hgf_decode.cu", "hgf_decode_small.cu", "hgf_decode_tc.cu", "hgf_prefill.cu", "hgf_attention.cu", "hgf_backward.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -56,6 +57,20 @@ def build(force: bool = False, verbose: bool = False) -> str:
         tmp = LIB + f".tmp{os.getpid()}"
         run([nvcc, "-shared", "-o", tmp, *objs, "-gencode", "arch=compute_100a,code=sm_100a"])
         os.replace(tmp, LIB)
+
+    src = os.path.join(CSRC, "hgf_python.cpp")
+    newest = max(os.path.getmtime(d) for d in (src, os.path.join(HERE, "..", "include", "hgf.h")))
+    if force or not os.path.exists(MODULE) or os.path.getmtime(MODULE) < newest:
+        import sysconfig
+
+        import torch
+        t = os.path.dirname(torch.__file__)
+        cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc)) if os.path.isabs(nvcc) else "/usr/local/cuda", "include")
+        tmp = MODULE + f".tmp{os.getpid()}"
+        run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-I{t}/include", f"-I{t}/include/torch/csrc/api/include", f"-I{cuda}",
+             f"-I{sysconfig.get_paths()['include']}", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", src, "-o", tmp,
+             f"-L{t}/lib", "-ltorch_python", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda"])
+        os.replace(tmp, MODULE)
     return LIB
 
 

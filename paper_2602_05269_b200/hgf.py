@@ -1,4 +1,5 @@
-"""Thin ctypes binding of libhgf_b200.so: same names as the C ABI, argument marshalling only.
+"""Thin binding of libhgf_b200.so: same names as the C ABI, argument marshalling only (ctypes; linear_forward, the call whose GPU time
+can be shorter than that, through the native module _hgf_python, csrc/hgf_python.cpp).
 
 Tensors are torch CUDA tensors used purely as device memory; every step of the layer runs in the
 library's kernels.  If the library is missing, or a call fails, this raises: there is no fallback.
@@ -63,11 +64,12 @@ class FrontEnd(ctypes.Structure):
 
 
 _lib = None
+_native_forward = None  # linear_forward's marshalling (set with _lib)
 
 
 def lib() -> ctypes.CDLL:
     """Load the CUDA library (built in-tree by paper_2602_05269_b200.build)."""
-    global _lib
+    global _lib, _native_forward
     if _lib is None:
         if not os.path.exists(LIB_PATH):
             raise RuntimeError(f"{LIB_PATH} is missing: run `python -m paper_2602_05269_b200.build` "
@@ -132,8 +134,20 @@ def lib() -> ctypes.CDLL:
         L.hgf_group_destroy.argtypes = [vp]
         L.hgf_status_string.restype = c.c_char_p
         L.hgf_status_string.argtypes = [c.c_int]
+        native = _marshal()
+        native.bind(c.cast(L.hgf_linear_forward, vp).value, c.cast(L.hgf_linear_forward_ln, vp).value)
+        _native_forward = native.linear_forward
         _lib = L
     return _lib
+
+
+def _marshal():
+    """The native module beside the library, built with it."""
+    try:
+        from . import _hgf_python
+    except ImportError as e:
+        raise RuntimeError(f"{_HERE}/_hgf_python.so is missing or does not load ({e}): run `python -m paper_2602_05269_b200.build`") from e
+    return _hgf_python
 
 
 def _ptr(t):
@@ -209,13 +223,22 @@ def linear_forward(x, packed, gamma, d_in, d_out, At=None, Bt=None, gate=None, *
     in front of the quantiser, gate fp32 [ceil(d_out / gate_group)]; debug then also returns mean and rstd.
     """
     assert x.is_cuda and x.dtype == torch.bfloat16 and x.is_contiguous()
-    M = x.shape[0]
-    r = 0 if At is None else At.shape[0]
+    if y is None or workspace is None or debug or phases is not None:
+        M = x.shape[0]
+        r = 0 if At is None else At.shape[0]
     if y is None:
         y = torch.empty((M, d_out), dtype=torch.bfloat16 if flags & FLAG_OUT_BF16 else torch.float32,
                         device=x.device)
     if workspace is None:
         workspace = torch.empty(workspace_bytes(M, d_in, d_out, r, flags), dtype=torch.uint8, device=x.device)
+    if not debug and phases is None:
+        if _lib is None:
+            lib()
+        st = _native_forward(x, packed, gamma, d_in, d_out, At, Bt, gate, y, workspace, flags, stream, ln_weight, ln_bias, eps,
+                             None if gate_group is None else int(gate_group or 1))
+        if st != HGF_OK:
+            raise HgfError("hgf_linear_forward", st)
+        return y
     dbg_struct, dbg = None, None
     if debug:
         dbg = {"xq": torch.empty((M, d_in), dtype=torch.int8, device=x.device),

@@ -1,0 +1,67 @@
+"""The native marshalling of hgf.linear_forward (csrc/hgf_python.cpp), without a GPU: what it takes and refuses before any launch."""
+import pytest
+import torch
+
+from paper_2602_05269_b200 import build as hgf_build
+
+
+@pytest.fixture(scope="module")
+def call():
+    hgf_build.build()
+    from paper_2602_05269_b200 import hgf
+    hgf.lib()
+    return hgf._native_forward
+
+
+class Stream:
+    cuda_stream = 0
+
+
+class Array:
+    """Not a tensor, but with a tensor's methods, as the ctypes calls take it too."""
+    def __init__(self, shape, address):
+        self.shape, self.address = shape, address
+
+    def data_ptr(self):
+        return self.address
+
+    def numel(self):
+        n = 1
+        for v in self.shape:
+            n *= v
+        return n
+
+
+def arguments(**changed):
+    x = torch.zeros(4, 64, dtype=torch.bfloat16)
+    a = {"x": x, "packed": x, "gamma": 0.5, "d_in": 64, "d_out": 64, "At": None, "Bt": None, "gate": None, "y": x, "workspace": Array((16,), 4096),
+         "flags": 0, "stream": Stream(), "ln_weight": None, "ln_bias": None, "eps": 1e-5, "gate_group": None}
+    assert not set(changed) - set(a)
+    return list({**a, **changed}.values())
+
+
+# the status that hgf.h gives for each, found before the library touches a device
+@pytest.mark.parametrize("changed,status", [
+    ({"x": Array((4, 64), 0)}, 1), ({"packed": None}, 1), ({"y": None}, 1), ({"d_in": 0}, 1), ({"d_out": -1}, 1), ({"flags": 1 << 20}, 1),
+    ({"d_in": 96}, 2), ({"x": Array((1 << 23, 64), 4096)}, 2), ({"At": Array((17, 64), 4096), "Bt": Array((64, 17), 4096), "gate": Array((64,), 4096)}, 2),
+    ({"y": Array((4, 64), 4104)}, 3), ({"workspace": Array((16,), 4096)}, 4), ({"workspace": None}, None),
+    ({"workspace": Array((1 << 24,), 4096), "ln_weight": Array((64,), 4096)}, 1), ({"workspace": Array((1 << 24,), 4096), "gate_group": 24}, 2),
+    ({"workspace": Array((1 << 24,), 4096 + 128)}, 3),
+])
+def test_status_of_refused_calls(call, changed, status):
+    if status is None:
+        with pytest.raises(AttributeError):
+            call(*arguments(**changed))
+    else:
+        assert call(*arguments(**changed)) == status
+
+
+@pytest.mark.parametrize("changed", [{"d_in": 64.0}, {"gamma": "one"}, {"flags": None}, {"gate_group": 2.5}, {"x": 7}, {"stream": 7}])
+def test_arguments_of_another_type_raise(call, changed):
+    with pytest.raises((TypeError, AttributeError)):
+        call(*arguments(**changed))
+
+
+def test_wrong_number_of_arguments(call):
+    with pytest.raises(TypeError):
+        call(*arguments()[:-1])
