@@ -334,6 +334,8 @@ hgf_status hgf::forward_impl(const void *x, int64_t M, const void *packed, float
     gp.N = (int)d_out;
     gp.r = r;
     gp.flags = flags;
+    // (every block of the prologue kernels waits for the launches before it ahead of letting the next one start, and they do not write it)
+    gp.early_weights = do_prologue ? 1 : 0;
     return launch_prefill_gemm(gp, stream) == cudaSuccess ? HGF_OK : HGF_ERR_CUDA;
 }
 

@@ -304,6 +304,7 @@ struct GemmParams {
     float gw_over_127;
     int M, K, N, r;
     uint32_t flags;
+    int early_weights;       // the launch before is this layer's prologue, so work that wrote `packed` is complete when a CTA starts
     int split_log2;          // (set by the launcher) CTAs a tile's K is divided over, as a power of two
 };
 cudaError_t launch_prefill_gemm(const GemmParams &p, cudaStream_t stream);
