@@ -302,7 +302,7 @@ hgf_status hgf::forward_impl(const void *x, int64_t M, const void *packed, float
     // arithmetic, not by the weight bytes the base-3 layout saves).
     const void *packed2 = packed;
     if (do_main && (flags & HGF_FLAG_BASE3)) {
-        if (launch_repack_b3(packed, d_out, d_in, (char *)workspace + L.w2, stream) != cudaSuccess) return HGF_ERR_CUDA;
+        if (launch_repack_b3(packed, d_out, d_in, (char *)workspace + L.w2, pdl, stream) != cudaSuccess) return HGF_ERR_CUDA;
         packed2 = (char *)workspace + L.w2;
     }
     GemmPrologueExtra gx = {};

@@ -215,7 +215,7 @@ cudaError_t launch_decode_prologue_group(const QuantItem *d_quant_items, int n_l
                                          cudaStream_t stream);
 cudaError_t launch_gemm_prologue(const PrologueParams &p, const GemmPrologueExtra &x, cudaStream_t stream);
 // base-3 bytes of a layer -> its two-bit tiles (the GEMM path's weight format)
-cudaError_t launch_repack_b3(const void *packed_b3, int64_t d_out, int64_t d_in, void *packed2, cudaStream_t stream);
+cudaError_t launch_repack_b3(const void *packed_b3, int64_t d_out, int64_t d_in, void *packed2, bool pdl, cudaStream_t stream);
 cudaError_t launch_decode_gemv(const DecodeLaunch &L, const DecodeProblem *single, bool pdl, cudaStream_t stream);
 // Shared memory the decode kernel needs for one problem's activations, and the largest it accepts.
 int decode_xq_smem_bytes(int M, int K, uint32_t flags);

@@ -1,6 +1,6 @@
 // Offline weight preparation: absmean scale, ternary codes, 2-bit packing (and its inverse).
 // Paper: Section 2.2, Definition "Absmax Quantization" (the scale is the mean of |W|).
-#include "hgf_common.cuh"
+#include "hgf_warp.cuh"
 
 namespace hgf {
 
@@ -175,41 +175,71 @@ __global__ void __launch_bounds__(256) unpack_b3_kernel(const uint8_t *packed, i
     T[idx] = (int8_t)(c - 1);
 }
 
-// Base-3 bytes -> two-bit tiles (the GEMM path reads only those).  One thread per two-bit word: its sixteen
-// codes are digits of up to sixteen bytes of the row's 64 in the base-3 tile that holds those columns.
-__global__ void __launch_bounds__(256) repack_b3_kernel(const uint8_t *packed_b3, int64_t N, int64_t K, int64_t steps2, int64_t steps3,
-                                                        size_t n_words, uint32_t *packed2) {
-    const size_t w = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (w >= n_words) return;
-    const WordPos p = word_pos(w, steps2);
-    uint32_t word = 0x55555555u;
-    if (p.n < N && p.k0 < K) {
-        word = 0;
-        const uint8_t *row_base = packed_b3 + (size_t)(p.n / 16) * steps3 * 1024 + (size_t)(p.n % 16) * 64;
+// Base-3 bytes -> two-bit tiles (the GEMM path reads only those).  A thread takes a row of a base-3 tile: its 64 bytes as four vectors,
+// every byte through a table of its five digits, and its 320 columns out as five vectors of four words.  Bytes 16 t + j of the row hold
+// columns 16 j + 4 t .. + 3 (digits 0..3) and 16 (16 + j / 4) + 4 t + j % 4 (digit 4), so a two-bit word - columns 4 t + e of a group of
+// 16 at bits 8 e + 2 t - is one byte of each of the four vectors, or the fifth digits of four bytes of each.
+// Bound by the launch at these sizes (4 + 4 MB for 4096 x 4096): a layer call of 128 tokens there 63.5 -> 23.1 us, 17 tokens of 8192 x 8192 192.6 -> 35.2 against a thread per
+// two-bit word, which divided its way through up to sixteen bytes one after the other.
+__global__ void __launch_bounds__(256) repack_b3_kernel(const uint8_t *packed_b3, int64_t N, int64_t K, int64_t steps2, int64_t steps3, int64_t tiles,
+                                                        size_t n_items, uint32_t *packed2) {
+    __shared__ uint32_t digits[256];  // digit e < 4 of the byte in byte e, digit 4 in bits 4 and 5
+    {
+        const uint32_t v = threadIdx.x;
+        digits[v] = v <= 242 ? v % 3 | v / 3 % 3 << 8 | v / 9 % 3 << 16 | v / 27 % 3 << 24 | v / 81 << 4 : 0x01010111u;
+    }
+    __syncthreads();
+    pdl_wait();
+    pdl_launch_dependents();
+    const size_t i = (size_t)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n_items) return;
+    const int r = (int)(i & 15);
+    const int64_t tile = (int64_t)(i >> 4) % tiles, row_tile = (int64_t)(i >> 4) / tiles, left = K - tile * 320;  // columns of the matrix from the tile on
+    const bool inside = row_tile * 16 + r < N && left > 0;
+    uint32_t word[20];
 #pragma unroll
-        for (int i = 0; i < 16; ++i) {
-            const int64_t k = p.k0 + i;  // K is a multiple of 64: the word's sixteen columns are all inside the matrix
-            const int col = (int)(k % 320), q = 2 * (col / 32) + (col % 32) / 16, t = (col % 16) / 4, e = col % 4;
-            const int j = q < 16 ? q : 4 * (q - 16) + e, digit = q < 16 ? e : 4;
-            int v = row_base[(size_t)(k / 320) * 1024 + 16 * t + j];
-            int c = 1;
-            if (v <= 242) {
-                for (int d = 0; d < digit; ++d) v /= 3;
-                c = v % 3;
+    for (int g = 0; g < 20; ++g) word[g] = inside ? 0u : 0x55555555u;
+    if (inside) {
+        const uint4 *src = reinterpret_cast<const uint4 *>(packed_b3 + (size_t)(row_tile * steps3 + tile) * 1024 + r * 64);
+        uint4 v[4];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) v[t] = src[t];
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+            const uint32_t w[4] = {v[t].x, v[t].y, v[t].z, v[t].w};
+#pragma unroll
+            for (int j = 0; j < 16; ++j) {
+                const uint32_t d = digits[w[j >> 2] >> 8 * (j & 3) & 0xffu];
+                word[j] |= (d & 0x03030303u) << 2 * t;
+                word[16 + (j >> 2)] |= (d >> 4 & 3u) << (8 * (j & 3) + 2 * t);
             }
-            word |= (uint32_t)c << (8 * (i & 3) + 2 * (i >> 2));
         }
     }
-    packed2[w] = word;
+#pragma unroll
+    for (int u = 0; u < 5; ++u) {
+        const int64_t c = tile * 320 + 64 * u;
+        if (c >= steps2 * 256) break;
+        const bool in = 64 * u < left;  // (K is a multiple of 64)
+        *reinterpret_cast<uint4 *>(packed2 + (size_t)(row_tile * steps2 + (c >> 8)) * 256 + r * 16 + ((c & 255) >> 4)) =
+            make_uint4(in ? word[4 * u] : 0x55555555u, in ? word[4 * u + 1] : 0x55555555u, in ? word[4 * u + 2] : 0x55555555u, in ? word[4 * u + 3] : 0x55555555u);
+    }
 }
 
-cudaError_t launch_repack_b3(const void *packed_b3, int64_t d_out, int64_t d_in, void *packed2, cudaStream_t stream) {
-    const int64_t steps2 = padded_k(d_in) / 256, steps3 = padded_k_b3(d_in) / 320;
-    const size_t n_words = (size_t)row_tiles(d_out) * steps2 * 256;
-    repack_b3_kernel<<<(unsigned)((n_words + 255) / 256), 256, 0, stream>>>((const uint8_t *)packed_b3, d_out, d_in, steps2, steps3, n_words,
-                                                                            (uint32_t *)packed2);
+cudaError_t launch_repack_b3(const void *packed_b3, int64_t d_out, int64_t d_in, void *packed2, bool pdl, cudaStream_t stream) {
+    const int64_t steps2 = padded_k(d_in) / 256, steps3 = padded_k_b3(d_in) / 320, tiles = (steps2 * 256 + 319) / 320;
+    const size_t n_items = (size_t)row_tiles(d_out) * tiles * 16;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)((n_items + 255) / 256));
+    cfg.blockDim = dim3(256);
+    cfg.stream = stream;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, repack_b3_kernel, (const uint8_t *)packed_b3, d_out, d_in, steps2, steps3, tiles, n_items, (uint32_t *)packed2);
     count_launch();
-    return cudaGetLastError();
+    return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 // ---- scratch of the packing calls -----------------------------------------------------------------
