@@ -117,22 +117,12 @@ __device__ __forceinline__ void quant_row_ln(const PrologueParams &p, const Fron
         const float4 w0 = *reinterpret_cast<const float4 *>(fe.ln_w + 8 * i), w1 = *reinterpret_cast<const float4 *>(fe.ln_w + 8 * i + 4);
         const float4 b0 = *reinterpret_cast<const float4 *>(fe.ln_b + 8 * i), b1 = *reinterpret_cast<const float4 *>(fe.ln_b + 8 * i + 4);
         const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
-        uint32_t c[8];
+        float xn[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            float q = rintf(__fmul_rn(ln_value(f[e], mean, rstd, w[e], b[e]), scale));
-            q = fminf(fmaxf(q, -127.0f), 127.0f);
-            c[e] = (uint32_t)__float2int_rn(q);
-        }
-        uint32_t o[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t p01 = __byte_perm(c[4 * h], c[4 * h + 1], 0x0040), p23 = __byte_perm(c[4 * h + 2], c[4 * h + 3], 0x0040);
-            o[h] = __byte_perm(p01, p23, 0x5410);
-            sum_q = __dp4a((int)o[h], 0x01010101, sum_q);
-        }
-        qv[i] = make_uint2(o[0], o[1]);
-        if (dq) dq[i] = make_uint2(o[0], o[1]);
+        for (int e = 0; e < 8; ++e) xn[e] = ln_value(f[e], mean, rstd, w[e], b[e]);
+        const uint2 o = ln_codes8(xn, scale, sum_q);
+        qv[i] = o;
+        if (dq) dq[i] = o;
     }
     sum_q = warp_sum_i(sum_q);
     if (lane == 0) s_red_i[warp] = sum_q;
@@ -440,21 +430,10 @@ __device__ void warp_quant_row_ln(const QuantItem &q, int lane) {
     for (int i = lane; i < nv; i += 32) {
         unpack8(xv[i], f);
         load_wb(i, w, b);
-        uint32_t c[8];
+        float xn[8];
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            float v = rintf(__fmul_rn(ln_value(f[e], mean, rstd, w[e], b[e]), scale));
-            v = fminf(fmaxf(v, -127.0f), 127.0f);
-            c[e] = (uint32_t)__float2int_rn(v);
-        }
-        uint32_t o[2];
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-            const uint32_t p01 = __byte_perm(c[4 * h], c[4 * h + 1], 0x0040), p23 = __byte_perm(c[4 * h + 2], c[4 * h + 3], 0x0040);
-            o[h] = __byte_perm(p01, p23, 0x5410);
-            sum_q = __dp4a((int)o[h], 0x01010101, sum_q);
-        }
-        qv[i] = make_uint2(o[0], o[1]);
+        for (int e = 0; e < 8; ++e) xn[e] = ln_value(f[e], mean, rstd, w[e], b[e]);
+        qv[i] = ln_codes8(xn, scale, sum_q);
     }
     sum_q = warp_sum_i(sum_q);
     if (lane == 0) {
