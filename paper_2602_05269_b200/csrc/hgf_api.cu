@@ -430,8 +430,8 @@ static std::vector<int4> gemv_ranges(const std::vector<DecodeProblem> &dps, long
 // whole block of 128 rows on a run of row tiles, however few they are, and its start grows with K (x~ and H of the first problem);
 // the warp MMA splits such runs over its sixteen warps, but loses 2.5 to 5 us at every change of problem inside a CTA's share.  So:
 // the 1 KiB tiles of the GEMV's largest share against the column tiles of blocks of this kernel's (`blocks`), by the longest row
-// (`longest`, in column tiles) and by whether a GEMV share holds several problems.  Where only the GEMV's shares do (`runs`: problems of
-// this kernel's largest) it is always this kernel's (1.10 to 1.53); on base-3 weights short rows on less than half of the SMs are too
+// (`longest`, in column tiles) and by whether a GEMV share holds several problems.  Where only the GEMV's shares do (`runs`: the most
+// problems of a share if the row tiles are dealt evenly) it is always this kernel's (1.10 to 1.53); on base-3 weights short rows on less than half of the SMs are too
 // (0.96 to 1.16, mean 1.05).  Captured chains, warp MMA's time over this kernel's, 1650 groups: one to three equal problems, blocks of
 // transformers (one to twelve, 512 to 4096 wide), mixed sizes.
 //   base-3, shares of one problem:   taken 0.96 to 1.42, mean 1.17; left 0.73 to 1.07, mean 0.91  (2048 -> 2048, M = 1: 10.9 us, here 12.0)
@@ -474,47 +474,93 @@ static bool plan_decode_tc(const std::vector<DecodeProblem> &dps, const std::vec
                            int sms, std::vector<DecodeTcSeg> *segs, std::vector<int2> *cta, int *image) {
     const int n = (int)dps.size();
     if (sms <= 0 || sms > 1024 || ranges.empty() || (max_M <= 8 && !(flags & HGF_FLAG_BASE3))) return false;
-    // a row tile's cost: its weight tiles, and its rows of B^T (1 KiB at r = 32)
+    // A CTA works its runs of row tiles in blocks of eight, however few the last one holds.  So the shares are dealt under two limits:
+    // the smallest on a share's blocks that reaches the end of the sequence, and under that the smallest on its row tiles (what it
+    // streams; few blocks are spread over all SMs).  The cost of either: weight tiles, and rows of B^T (1 KiB a row tile at r = 32).
     auto cost_of = [&](int i) { return 32ll * weight_steps(dps[i].K, flags) + dps[i].r; };
-    long long cost = 0, slowest = 0;
+    long long rows = 0, blocks = 0, largest = 0;
     *image = 0;
     for (int i = 0; i < n; ++i) {
-        cost += row_tiles(dps[i].N) * cost_of(i);
+        rows += row_tiles(dps[i].N) * cost_of(i);
+        blocks += (row_tiles(dps[i].N) + 7) / 8 * cost_of(i);
+        largest = cost_of(i) > largest ? cost_of(i) : largest;
         const int b = decode_tc_image_bytes(max_M, dps[i].K, flags);
         *image = b > *image ? b : *image;
     }
-    int p = 0, t = 0, max_segs = 0;  // next row tile to deal out
-    long long dealt = 0;
-    for (int c = 0; c < sms; ++c) {
-        const int first = (int)segs->size();
-        const long long until = cost * (c + 1) / sms;
-        long long blocks = 0;
+    // one share of the sequence from (problem p, row tile t) on; for each of its runs run(p, t, row tiles)
+    auto deal = [&](long long most_blocks, long long most_rows, int *p, long long *t, auto &&run) {
+        while (*p < n) {
+            const long long cost = cost_of(*p), tiles = row_tiles(dps[*p].N);
+            const long long take = std::min({most_blocks / cost * 8, most_rows / cost, tiles - *t});
+            if (take <= 0) break;
+            run(*p, *t, take);
+            most_blocks -= (take + 7) / 8 * cost;
+            most_rows -= take * cost;
+            *t += take;
+            if (*t < tiles) break;
+            ++*p;
+            *t = 0;
+        }
+    };
+    auto reaches_the_end = [&](long long most_blocks, long long most_rows) {
+        int p = 0;
+        long long t = 0;
+        for (int c = 0; c < sms && p < n; ++c) deal(most_blocks, most_rows, &p, &t, [](int, long long, long long) {});
+        return p == n;
+    };
+    auto smallest = [](long long low, long long high, auto &&enough) {  // in (low, high], which is enough
+        while (low + 1 < high) {
+            const long long mid = low + (high - low) / 2;
+            if (enough(mid)) high = mid; else low = mid;
+        }
+        return high;
+    };
+    // (a share under the first limit alone is filled to within a block)
+    const long long most_blocks = smallest(std::max(largest, (blocks + sms - 1) / sms) - 1, blocks / sms + 1 + largest, [&](long long v) { return reaches_the_end(v, 8 * blocks); });
+    const long long most_rows = smallest(std::max(largest, rows / sms) - 1, 8 * most_blocks, [&](long long v) { return reaches_the_end(most_blocks, v); });
+    // the most problems in a share of row tiles dealt evenly (decode_tc_pays goes by it)
+    int p = 0, runs = 0;
+    long long t = 0, dealt = 0;
+    for (int c = 0; c < sms && p < n; ++c) {
+        const long long until = rows * (c + 1) / sms;
+        int held = 0;
         while (p < n && dealt < until) {
-            const DecodeProblem &P = dps[p];
-            const long long per = cost_of(p), tiles = row_tiles(P.N);
-            long long take = (until - dealt + per / 2) / per;
-            if (c + 1 == sms || take > tiles - t) take = tiles - t;
-            if (take <= 0) break;  // (less than half a row tile is left of this share)
-            DecodeTcSeg s = {};
-            s.steps = weight_steps(P.K, flags);
-            s.packed = P.packed + (size_t)t * s.steps * 1024;
-            s.xq = P.xq; s.gamma_x = P.gamma_x; s.row_sum = P.row_sum; s.hpart = P.hpart; s.nslices = P.nslices;
-            s.Bt = P.Bt; s.gate = P.gate; s.y = P.y;
-            s.dbg_y_int_at = &d_probs[p].dbg_y_int;
-            s.gw_over_127 = P.gw_over_127;
-            s.M = P.M; s.K = P.K; s.N = P.N; s.r = P.r; s.gate_group = P.gate_group; s.flags = P.flags;
-            s.lo = t; s.n = (int)take;
-            segs->push_back(s);
-            blocks += (take + 7) / 8 * s.steps;
-            dealt += take * per;
-            t += (int)take;
+            const long long cost = cost_of(p), tiles = row_tiles(dps[p].N), take = std::min(c + 1 == sms ? tiles : (until - dealt + cost / 2) / cost, tiles - t);
+            if (take <= 0) break;
+            dealt += take * cost;
+            t += take;
+            ++held;
             if (t == tiles) { ++p; t = 0; }
         }
-        slowest = blocks > slowest ? blocks : slowest;
-        cta->push_back(make_int2(first, (int)segs->size() - first));
-        max_segs = cta->back().y > max_segs ? cta->back().y : max_segs;
+        runs = std::max(runs, held);
     }
-    return p == n && decode_tc_fits(*image, max_segs) && decode_tc_pays(dps, ranges, slowest, max_segs, flags, sms);
+    p = 0;
+    t = 0;
+    int max_segs = 0;
+    long long slowest = 0;
+    for (int c = 0; c < sms; ++c) {
+        const int first = (int)segs->size();
+        long long col_tiles = 0;
+        deal(most_blocks, most_rows, &p, &t, [&](int i, long long from, long long take) {
+            const DecodeProblem &P = dps[i];
+            DecodeTcSeg s = {};
+            s.steps = weight_steps(P.K, flags);
+            s.packed = P.packed + (size_t)from * s.steps * 1024;
+            s.xq = P.xq; s.gamma_x = P.gamma_x; s.row_sum = P.row_sum; s.hpart = P.hpart; s.nslices = P.nslices;
+            s.Bt = P.Bt; s.gate = P.gate; s.y = P.y;
+            s.dbg_y_int_at = &d_probs[i].dbg_y_int;
+            s.gw_over_127 = P.gw_over_127;
+            s.M = P.M; s.K = P.K; s.N = P.N; s.r = P.r; s.gate_group = P.gate_group; s.flags = P.flags;
+            s.lo = (int)from;
+            s.n = (int)take;
+            segs->push_back(s);
+            col_tiles += (take + 7) / 8 * s.steps;
+        });
+        slowest = std::max(slowest, col_tiles);
+        cta->push_back(make_int2(first, (int)segs->size() - first));
+        max_segs = std::max(max_segs, cta->back().y);
+    }
+    return p == n && decode_tc_fits(*image, max_segs) && decode_tc_pays(dps, ranges, slowest, runs, flags, sms);
 }
 }  // namespace hgf
 
