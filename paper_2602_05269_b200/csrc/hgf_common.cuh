@@ -306,6 +306,7 @@ struct GemmParams {
     uint32_t flags;
     int early_weights;       // the launch before is this layer's prologue, so work that wrote `packed` is complete when a CTA starts
     int split_log2;          // (set by the launcher) CTAs a tile's K is divided over, as a power of two
+    int tile_t;              // (set by the launcher) tokens of a tile
 };
 cudaError_t launch_prefill_gemm(const GemmParams &p, cudaStream_t stream);
 cudaError_t launch_wait_timeout_selftest(unsigned long long limit_ns, cudaStream_t stream);

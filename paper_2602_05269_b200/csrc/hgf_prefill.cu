@@ -39,7 +39,7 @@
 namespace hgf {
 
 constexpr int TILE_C = 128;   // output channels per tile (MMA M, tensor-memory lanes)
-constexpr int TILE_T = 128;   // tokens per tile (MMA N, accumulator columns)
+constexpr int TILE_T = 128;   // tokens per tile (MMA N, accumulator columns) at most: see prefill_tile_tokens
 constexpr int KBLK = 256;      // input columns per pipeline stage: one column tile of the packed layout
 constexpr int X_HALF_BYTES = TILE_T * 128;       // 16 KiB: 128 tokens x 128 columns, one 128-byte-swizzled operand tile
 constexpr int X_TILE_BYTES = 2 * X_HALF_BYTES;   // 32 KiB per stage
@@ -80,10 +80,8 @@ struct Cfg {
 
 // Instruction descriptor: D format (bits 4-5), A format (7-9), B format (10-12), K-major A and B,
 // N >> 3 (17-22), M >> 4 (24-28).
-constexpr uint32_t IDESC_I8 = (2u << 4) /*s32*/ | (1u << 7) /*A s8*/ | (1u << 10) /*B s8*/ |
-                              ((uint32_t)(TILE_T >> 3) << 17) | ((uint32_t)(TILE_C >> 4) << 24);
-constexpr uint32_t IDESC_F16 = (1u << 4) /*f32*/ | (0u << 7) /*A f16*/ | (0u << 10) /*B f16*/ |
-                               ((uint32_t)(TILE_T >> 3) << 17) | ((uint32_t)(TILE_C >> 4) << 24);
+constexpr uint32_t IDESC_I8 = (2u << 4) /*s32*/ | (1u << 7) /*A s8*/ | (1u << 10) /*B s8*/ | ((uint32_t)(TILE_C >> 4) << 24);  // (N: the launch's)
+constexpr uint32_t IDESC_F16 = (1u << 4) /*f32*/ | (0u << 7) /*A f16*/ | (0u << 10) /*B f16*/ | ((uint32_t)(TILE_C >> 4) << 24);
 
 // SPLIT: a layer with fewer tiles than half the SMs has each tile's K divided over a cluster of 2, 4 or 8 CTAs (one tile a
 // cluster, the tile loops below run once).  The CTAs keep their int32 sums in tensor memory, hand each other
@@ -111,7 +109,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     const int S = SPLIT ? 1 << p.split_log2 : 1, rank = SPLIT ? (int)blockIdx.x & (S - 1) : 0;
     const int tile_first = SPLIT ? (int)blockIdx.x >> p.split_log2 : (int)blockIdx.x, tile_step = SPLIT ? (int)gridDim.x >> p.split_log2 : (int)gridDim.x;
     bool arrived = false, waited = false;  // (SPLIT) the cluster barrier that frees the operand rings
-    const int tiles_t = (p.M + TILE_T - 1) / TILE_T, tiles_c = (p.N + TILE_C - 1) / TILE_C;
+    const int T = SPLIT ? TILE_T : p.tile_t;  // tokens of a tile
+    const int tiles_t = (p.M + T - 1) / T, tiles_c = (p.N + TILE_C - 1) / TILE_C;
     const int num_tiles = tiles_t * tiles_c;
     const int kblocks = (p.K + KBLK - 1) / KBLK, kb0 = SPLIT ? rank * kblocks / S : 0, kb1 = SPLIT ? (rank + 1) * kblocks / S : kblocks;
     const bool has_lora = p.r > 0;
@@ -178,17 +177,17 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             int pit = 0;
             bool ok = true;
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
-                const int t0 = (tile % tiles_t) * TILE_T, c0 = (tile / tiles_t) * TILE_C;
+                const int t0 = (tile % tiles_t) * T, c0 = (tile / tiles_t) * TILE_C;
                 {
                     // what the tile's epilogue needs, into the buffer of the tile's accumulator: row sums and
-                    // scales of the 128 tokens, and with a correction the H tile and the (g B)^T tile
+                    // scales of the T tokens, and with a correction the H tile and the (g B)^T tile
                     const int b = pit & 1;
                     ok = mbar_wait(bar(C::BAR_OPSEMPTY + b), ((uint32_t)(pit >> 1) & 1u) ^ 1u, abort_flag, status, 0x120u + b);
                     if (!(ok = __all_sync(0xffffffffu, ok))) break;
                     if (lane == 0) {
-                        mbar_arrive_expect_tx(bar(C::BAR_OPSFULL + b), 2u * TILE_T * 4u + (has_lora ? C::LORA_H_BYTES + C::LORA_B_BYTES : 0));
-                        bulk_load_1d(sbase + C::OFF_TOKV + b * TOKV_BYTES, p.row_sum + t0, TILE_T * 4u, bar(C::BAR_OPSFULL + b));
-                        bulk_load_1d(sbase + C::OFF_TOKV + b * TOKV_BYTES + TILE_T * 4, p.tok_sc + t0, TILE_T * 4u, bar(C::BAR_OPSFULL + b));
+                        mbar_arrive_expect_tx(bar(C::BAR_OPSFULL + b), 2u * T * 4u + (has_lora ? T * OPSB + C::LORA_B_BYTES : 0));
+                        bulk_load_1d(sbase + C::OFF_TOKV + b * TOKV_BYTES, p.row_sum + t0, T * 4u, bar(C::BAR_OPSFULL + b));
+                        bulk_load_1d(sbase + C::OFF_TOKV + b * TOKV_BYTES + TILE_T * 4, p.tok_sc + t0, T * 4u, bar(C::BAR_OPSFULL + b));
                         if (has_lora) {
                             tma_load_2d(sbase + C::OFF_LH + b * C::LORA_H_BYTES, &tmap_h, 0, t0, bar(C::BAR_OPSFULL + b));
                             tma_load_2d(sbase + C::OFF_LB + b * C::LORA_B_BYTES, &tmap_gb, 0, c0, bar(C::BAR_OPSFULL + b));
@@ -201,8 +200,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     ok = mbar_wait(bar(C::BAR_EMPTY + s), ph ^ 1u, abort_flag, status, 0x100u + s);
                     if (!(ok = __all_sync(0xffffffffu, ok))) break;
                     if (lane == 0) {
-                        // 256 columns of 128 tokens as two 128-byte-swizzled tiles (columns past K read as zeros)
-                        mbar_arrive_expect_tx(bar(C::BAR_FULL + s), X_TILE_BYTES);
+                        // 256 columns of T tokens as two 128-byte-swizzled tiles (columns past K read as zeros)
+                        mbar_arrive_expect_tx(bar(C::BAR_FULL + s), 2u * 128u * T);
                         tma_load_2d(sbase + C::OFF_X + s * X_TILE_BYTES, &tmap_x, kb * KBLK, t0, bar(C::BAR_FULL + s));
                         tma_load_2d(sbase + C::OFF_X + s * X_TILE_BYTES + X_HALF_BYTES, &tmap_x, kb * KBLK + 128, t0, bar(C::BAR_FULL + s));
                     }
@@ -241,6 +240,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             int it = 0, pend = -1;  // pend: tile whose correction MMA is still to be issued
             int gs = 0;             // stage number, counted through all tiles of this CTA
             const uint64_t xdesc0 = make_sw128_desc(sbase + C::OFF_X);
+            const uint32_t idesc_i8 = IDESC_I8 | ((uint32_t)(T >> 3) << 17), idesc_f16 = IDESC_F16 | ((uint32_t)(T >> 3) << 17);
             auto issue_lora = [&](int t) {
                 const int b = t & 1;
                 tc_fence_after();
@@ -249,7 +249,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                 const uint64_t bdesc = OPSB == 128 ? make_sw128_desc(lh) : make_sw64_desc(lh);
 #pragma unroll
                 for (int kk = 0; kk < OPSB / 32; ++kk)  // K = 16 fp16 (32 bytes of a row) per MMA, on top of the fp32 values
-                    warp_mma_f16(tmem_base + b * ACC_COLS, adesc + 2u * kk, bdesc + 2u * kk, IDESC_F16, 1u);
+                    warp_mma_f16(tmem_base + b * ACC_COLS, adesc + 2u * kk, bdesc + 2u * kk, idesc_f16, 1u);
                 warp_commit(bar(C::BAR_LORADONE + b));
             };
             for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++it) {
@@ -267,14 +267,14 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
                     tc_fence_after();
                     const uint64_t bdesc = xdesc0 + (uint64_t)(s * (X_TILE_BYTES >> 4));
                     const uint32_t a_tmem = tmem_base + A_COL + s * A_STAGE_COLS;
-                    warp_mma_i8_ts(acc, a_tmem, bdesc, IDESC_I8, kb > kb0 ? 1u : 0u);
-                    warp_mma_i8_ts(acc, a_tmem + 8u, bdesc + 2u, IDESC_I8, 1u);
-                    warp_mma_i8_ts(acc, a_tmem + 16u, bdesc + 4u, IDESC_I8, 1u);
-                    warp_mma_i8_ts(acc, a_tmem + 24u, bdesc + 6u, IDESC_I8, 1u);
-                    warp_mma_i8_ts(acc, a_tmem + 32u, bdesc + (X_HALF_BYTES >> 4), IDESC_I8, 1u);
-                    warp_mma_i8_ts(acc, a_tmem + 40u, bdesc + (X_HALF_BYTES >> 4) + 2u, IDESC_I8, 1u);
-                    warp_mma_i8_ts(acc, a_tmem + 48u, bdesc + (X_HALF_BYTES >> 4) + 4u, IDESC_I8, 1u);
-                    warp_mma_i8_ts(acc, a_tmem + 56u, bdesc + (X_HALF_BYTES >> 4) + 6u, IDESC_I8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem, bdesc, idesc_i8, kb > kb0 ? 1u : 0u);
+                    warp_mma_i8_ts(acc, a_tmem + 8u, bdesc + 2u, idesc_i8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 16u, bdesc + 4u, idesc_i8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 24u, bdesc + 6u, idesc_i8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 32u, bdesc + (X_HALF_BYTES >> 4), idesc_i8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 40u, bdesc + (X_HALF_BYTES >> 4) + 2u, idesc_i8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 48u, bdesc + (X_HALF_BYTES >> 4) + 4u, idesc_i8, 1u);
+                    warp_mma_i8_ts(acc, a_tmem + 56u, bdesc + (X_HALF_BYTES >> 4) + 6u, idesc_i8, 1u);
                     warp_commit(bar(C::BAR_EMPTY + s));
                 }
                 if (!ok) break;
@@ -295,15 +295,15 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // Eight of them: the warp pair of a tensor-memory lane quarter (32 output channels) shares the
         // tile's 128 tokens, 64 each, so a tile's epilogue takes half as long as with one warp per
         // quarter: the main loop of a short-K tile is over sooner than that.
-        const int e2 = warp < 6 ? 0 : 1;                  // which 64 tokens of the tile
+        const int e2 = warp < 6 ? 0 : 1;                  // which half of the tile's tokens
         const int q = warp & 3;                           // tensor-memory lane quarter this warp may access
-        constexpr int HALF_T = TILE_T / 2;
+        const int half_t = T / 2;
         constexpr int W = OUT_BF16 ? 32 : 16;             // tokens per staging step (2 KiB of staging either way)
         uint8_t *buf = smem + C::OFF_ST + (4 * e2 + q) * STORE_BUF_BYTES;
         bool ok = true;
         int it = 0;
         for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step, ++it) {
-            const int t0 = (tile % tiles_t) * TILE_T, c0 = (tile / tiles_t) * TILE_C;
+            const int t0 = (tile % tiles_t) * T, c0 = (tile / tiles_t) * TILE_C;
             const int b = it & 1;
             const uint32_t par = (uint32_t)(it >> 1) & 1u;
             // the tile's row sums and scales (and the correction's operands) were fetched by the producer
@@ -408,7 +408,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
             }
             if (has_lora) {
                 // first pass: dequantise in place (int32 -> fp32), then let the MMA warp add the correction
-                for (int cc = HALF_T * e2; cc < HALF_T * (e2 + 1); cc += 32) {
+                for (int cc = half_t * e2; cc < half_t * (e2 + 1); cc += 32) {
                     uint32_t ai[32];
                     tmem_ld32(lane_base + cc, ai);
                     tmem_ld_wait();
@@ -426,7 +426,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
             // read the result, transpose it through shared memory (a thread holds one channel of W
             // tokens; y wants the channels of a token next to each other) and store with TMA
-            for (int cc = HALF_T * e2; cc < HALF_T * (e2 + 1); cc += W) {
+            for (int cc = half_t * e2; cc < half_t * (e2 + 1); cc += W) {
                 uint32_t ai[W];
                 if constexpr (W == 32) tmem_ld32(lane_base + cc, ai); else tmem_ld16(lane_base + cc, ai);
                 tmem_ld_wait();
@@ -610,6 +610,17 @@ static cudaError_t launch_variant(const CUtensorMap &mx, const CUtensorMap &mh, 
                         : launch_split<OUT_BF16, NS, OPSB, false>(mx, mh, mgb, my, p, grid, status, stream);
 }
 
+// Tokens of a tile: 64 where that many tiles still run in one round (or there are no more), else 128.  A tile of 64 halves the products, the
+// copies of x~ and the epilogue of a CTA, but not the expansion of its weights, so more rounds than one cost more than they save.
+// Microseconds of a layer call in a captured chain, tiles of 128 / 112 / 96 / 80 / 64 / 48: 1024 -> 1024 9.7 / 9.7 / 9.1 / 9.1 / 8.5 / 8.4 at M = 100
+// (16 tiles of 64), 13.5 / 14.0 / 12.6 / 12.6 / 11.4 / 12.6 at M = 512 (64), 11.9 / 11.9 / 11.5 / 11.4 / 10.9 / 12.0 at M = 1000 (128), 13.0 / 13.0 / 12.7 /
+// 14.0 / 13.1 / 13.9 at M = 1500 (192); 2048 -> 5632 11.7 / 11.5 / 11.1 / 11.0 / 10.5 / 11.6 at M = 100 (88), 12.5 / 12.4 / 12.8 / 12.7 / 14.5 / 14.6 at
+// M = 200 (176); 2048 -> 2048 14.6 / 15.6 / 15.1 / 14.7 / 14.3 / 17.5 at M = 512 (128), 19.9 / 20.9 / 20.4 / 22.6 / 23.0 / 26.3 at M = 1500.
+static int prefill_tile_tokens(int M, int N, int sms) {
+    const long long tiles = (long long)((M + 63) / 64) * ((N + TILE_C - 1) / TILE_C);
+    return M <= 64 || tiles <= sms ? 64 : TILE_T;
+}
+
 cudaError_t launch_prefill_gemm(const GemmParams &p_in, cudaStream_t stream) {
     GemmParams p = p_in;
     const int sm_count = device_sm_count();
@@ -628,14 +639,16 @@ cudaError_t launch_prefill_gemm(const GemmParams &p_in, cudaStream_t stream) {
     };
     for (int log2 = 1; log2 <= 3; ++log2)
         if (may_split(log2)) p.split_log2 = log2;
+    p.tile_t = p.split_log2 ? TILE_T : prefill_tile_tokens(p.M, p.N, sm_count);
+    const uint32_t T = (uint32_t)p.tile_t;
     CUtensorMap mx, mh, mgb, my;
-    if (!make_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.xq, (uint64_t)p.K, (uint64_t)p.M, (uint64_t)p.K, 128, TILE_T,
+    if (!make_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.xq, (uint64_t)p.K, (uint64_t)p.M, (uint64_t)p.K, 128, T,
                      CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
     if (p.r > 0) {  // H [M][64] and (g B)^T [N][64] fp16: tiles of 128 rows; the first 32 or all 64 columns
         const uint32_t cols = narrow ? 32 : 64;
         const CUtensorMapSwizzle sw = narrow ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_128B;
-        if (!make_map_2d(&mh, CU_TENSOR_MAP_DATA_TYPE_UINT16, p.h16, 64, (uint64_t)p.M, 128, cols, TILE_T, sw)) return cudaErrorInvalidValue;
+        if (!make_map_2d(&mh, CU_TENSOR_MAP_DATA_TYPE_UINT16, p.h16, 64, (uint64_t)p.M, 128, cols, T, sw)) return cudaErrorInvalidValue;
         if (!make_map_2d(&mgb, CU_TENSOR_MAP_DATA_TYPE_UINT16, p.gb16, 64, (uint64_t)p.N, 128, cols, TILE_C, sw)) return cudaErrorInvalidValue;
     } else {
         mh = mx;
@@ -644,7 +657,8 @@ cudaError_t launch_prefill_gemm(const GemmParams &p_in, cudaStream_t stream) {
     if (!make_map_2d(&my, bf16 ? CU_TENSOR_MAP_DATA_TYPE_BFLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32, p.y, (uint64_t)p.N,
                      (uint64_t)p.M, (uint64_t)p.N * (bf16 ? 2 : 4), 32, bf16 && !p.split_log2 ? 32 : 16, CU_TENSOR_MAP_SWIZZLE_NONE))
         return cudaErrorInvalidValue;
-    const int grid = p.split_log2 ? tiles << p.split_log2 : (tiles < sm_count ? tiles : sm_count);
+    const int work = ((p.M + p.tile_t - 1) / p.tile_t) * ((p.N + TILE_C - 1) / TILE_C);
+    const int grid = p.split_log2 ? tiles << p.split_log2 : (work < sm_count ? work : sm_count);
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
     cudaError_t e;
