@@ -25,8 +25,8 @@
 //               tcgen05.st), wait for the correction MMA, read the result, transpose it through shared
 //               memory and store y with TMA
 //   warps 6-9   expand the packed tile into tensor memory
-//   warp 10     producer of the packed codes (eight contiguous 1 KiB tiles of the tiled weight layout
-//               per stage, one bulk copy each), in a ring that runs ahead of the activations'
+//   warp 10     producer of the packed codes (1 KiB tiles of eight consecutive row tiles of the tiled weight
+//               layout per stage, with one TMA copy), in a ring that runs ahead of the activations'
 // Codes are c = t + 1 (both operands are declared signed 8-bit; 0, 1, 2 read the same either way);
 // sum_k t x~ = sum_k c x~ - sum_k x~ is restored in the epilogue from the row sums.
 //
@@ -91,7 +91,7 @@ template <bool OUT_BF16, int NS, int OPSB, bool SPLIT>
 __global__ void __launch_bounds__(GEMM_THREADS, 1)
 prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_constant__ CUtensorMap tmap_h,
                     const __grid_constant__ CUtensorMap tmap_gb, const __grid_constant__ CUtensorMap tmap_y,
-                    const GemmParams p, unsigned int *status) {
+                    const __grid_constant__ CUtensorMap tmap_w, const GemmParams p, unsigned int *status) {
     using C = Cfg<NS, OPSB>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -463,24 +463,22 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // ------------------------------------------------------------------ packed-code producer
         // Its own warp and ring: the codes run ahead of the activations, so the expansion into tensor
         // memory starts the moment a stage's MMAs are complete, in parallel with the reload of the
-        // activation tile.  Per stage the 1 KiB tiles (16 rows x 256 columns) of 8 consecutive row tiles,
-        // one bulk copy per lane (row tiles past the matrix are left out).
+        // activation tile.  Per stage the 1 KiB tiles (16 rows x 256 columns) of 8 consecutive row tiles with one
+        // copy (row tiles past the matrix are zeros); as eight bulk copies 512 tokens of 5632 -> 2048 took 21.0 us in place
+        // of 20.7, 64 of 2048 -> 2048 11.15 in place of 11.0.
         int pj = 0;
         uint32_t pph = 0;
         uint32_t pissued[C::PSTAGES] = {};
         bool ok = true;
-        const int steps = (p.K + 255) >> 8, n_row_tiles = (p.N + 15) >> 4;
         for (int tile = tile_first; ok && tile < num_tiles; tile += tile_step) {
             const int rt0 = ((tile / tiles_t) * TILE_C) >> 4;
-            const int nrt = n_row_tiles - rt0 < TILE_C / 16 ? n_row_tiles - rt0 : TILE_C / 16;
-            const uint8_t *psrc = p.packed + (size_t)(rt0 + (lane < nrt ? lane : 0)) * steps * 1024;
             for (int kb = kb0; kb < kb1; ++kb) {
                 ok = mbar_wait(bar(C::BAR_PEMPTY + pj), pph ^ 1u, abort_flag, status, 0x110u + pj);
                 if (!(ok = __all_sync(0xffffffffu, ok))) break;
-                if (lane == 0) mbar_arrive_expect_tx(bar(C::BAR_PFULL + pj), (uint32_t)nrt * 1024u);
-                __syncwarp();
-                if (lane < nrt)
-                    bulk_load_1d(sbase + C::OFF_P + pj * P_TILE_BYTES + lane * 1024, psrc + (size_t)kb * 1024, 1024u, bar(C::BAR_PFULL + pj));
+                if (lane == 0) {
+                    mbar_arrive_expect_tx(bar(C::BAR_PFULL + pj), P_TILE_BYTES);
+                    tma_load_2d(sbase + C::OFF_P + pj * P_TILE_BYTES, &tmap_w, kb * (1024 / 8), rt0, bar(C::BAR_PFULL + pj));
+                }
                 ++pissued[pj];
                 if (++pj == C::PSTAGES) { pj = 0; pph ^= 1u; }
             }
@@ -574,7 +572,7 @@ cudaError_t launch_wait_timeout_selftest(unsigned long long limit_ns, cudaStream
 
 // ---- host side: tensor maps and launch -----------------------------------------------------------
 template <bool OUT_BF16, int NS, int OPSB, bool SPLIT>
-static cudaError_t launch_split(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my,
+static cudaError_t launch_split(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my, const CUtensorMap &mw,
                                   const GemmParams &p, int grid, unsigned int *status, cudaStream_t stream) {
     static std::atomic<unsigned long long> attr_done{0};
     constexpr int smem = Cfg<NS, OPSB>::SMEM_BYTES;
@@ -599,15 +597,15 @@ static cudaError_t launch_split(const CUtensorMap &mx, const CUtensorMap &mh, co
         attr[cfg.numAttrs].val.clusterDim.z = 1;
         ++cfg.numAttrs;
     }
-    cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<OUT_BF16, NS, OPSB, SPLIT>, mx, mh, mgb, my, p, status);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, prefill_gemm_kernel<OUT_BF16, NS, OPSB, SPLIT>, mx, mh, mgb, my, mw, p, status);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
 template <bool OUT_BF16, int NS, int OPSB>
-static cudaError_t launch_variant(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my,
+static cudaError_t launch_variant(const CUtensorMap &mx, const CUtensorMap &mh, const CUtensorMap &mgb, const CUtensorMap &my, const CUtensorMap &mw,
                                   const GemmParams &p, int grid, unsigned int *status, cudaStream_t stream) {
-    return p.split_log2 ? launch_split<OUT_BF16, NS, OPSB, true>(mx, mh, mgb, my, p, grid, status, stream)
-                        : launch_split<OUT_BF16, NS, OPSB, false>(mx, mh, mgb, my, p, grid, status, stream);
+    return p.split_log2 ? launch_split<OUT_BF16, NS, OPSB, true>(mx, mh, mgb, my, mw, p, grid, status, stream)
+                        : launch_split<OUT_BF16, NS, OPSB, false>(mx, mh, mgb, my, mw, p, grid, status, stream);
 }
 
 // Tokens of a tile: 64 where that many tiles still run in one round (or there are no more), else 128.  A tile of 64 halves the products, the
@@ -641,7 +639,7 @@ cudaError_t launch_prefill_gemm(const GemmParams &p_in, cudaStream_t stream) {
         if (may_split(log2)) p.split_log2 = log2;
     p.tile_t = p.split_log2 ? TILE_T : prefill_tile_tokens(p.M, p.N, sm_count);
     const uint32_t T = (uint32_t)p.tile_t;
-    CUtensorMap mx, mh, mgb, my;
+    CUtensorMap mx, mh, mgb, my, mw;
     if (!make_map_2d(&mx, CU_TENSOR_MAP_DATA_TYPE_UINT8, p.xq, (uint64_t)p.K, (uint64_t)p.M, (uint64_t)p.K, 128, T,
                      CU_TENSOR_MAP_SWIZZLE_128B))
         return cudaErrorInvalidValue;
@@ -659,15 +657,19 @@ cudaError_t launch_prefill_gemm(const GemmParams &p_in, cudaStream_t stream) {
         return cudaErrorInvalidValue;
     const int work = ((p.M + p.tile_t - 1) / p.tile_t) * ((p.N + TILE_C - 1) / TILE_C);
     const int grid = p.split_log2 ? tiles << p.split_log2 : (work < sm_count ? work : sm_count);
+    // the packed codes: a row tile's 1 KiB tiles one after the other, in units of 8 bytes
+    if (!make_map_2d(&mw, CU_TENSOR_MAP_DATA_TYPE_FLOAT64, p.packed, (uint64_t)kblocks * 128, (uint64_t)((p.N + 15) / 16), (uint64_t)kblocks * 1024, 128,
+                     TILE_C / 16, CU_TENSOR_MAP_SWIZZLE_NONE))
+        return cudaErrorInvalidValue;
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
     cudaError_t e;
     if (narrow)
-        e = bf16 ? launch_variant<true, 4, 64>(mx, mh, mgb, my, p, grid, status, stream)
-                 : launch_variant<false, 4, 64>(mx, mh, mgb, my, p, grid, status, stream);
+        e = bf16 ? launch_variant<true, 4, 64>(mx, mh, mgb, my, mw, p, grid, status, stream)
+                 : launch_variant<false, 4, 64>(mx, mh, mgb, my, mw, p, grid, status, stream);
     else
-        e = bf16 ? launch_variant<true, 3, 128>(mx, mh, mgb, my, p, grid, status, stream)
-                 : launch_variant<false, 3, 128>(mx, mh, mgb, my, p, grid, status, stream);
+        e = bf16 ? launch_variant<true, 3, 128>(mx, mh, mgb, my, mw, p, grid, status, stream)
+                 : launch_variant<false, 3, 128>(mx, mh, mgb, my, mw, p, grid, status, stream);
     count_launch();
     return e;
 }
