@@ -7,6 +7,8 @@
 // (C = A B^T, each operand read in the form it is stored in), plus preparation kernels: Xd as a bf16 matrix (the
 // quantiser again, its codes times their scale), the ternary codes as a bf16 matrix of exact -1 / 0 / +1, A and
 // g (.) B in bf16.  gamma_W is applied to the fp32 accumulator.
+#include <algorithm>
+
 #include "hgf_tc.cuh"
 #include "hgf_warp.cuh"
 
@@ -61,6 +63,20 @@ struct TcGemmArgs {
     int a_mn, b_mn;    // operand forms (both pairs alike); 2: by blocks of 64 rows, two a copy (tc_map)
     float alpha;
     int accumulate;
+};
+
+// A product with one extent of at most 64 that rides in a launch by pairs (tc_pair_gemm_kernel): output tiles of 256 x 64, the
+// contraction in `splits` parts, each with partial sums of its own.  B is stored with its row index contiguous.
+struct TcThin {
+    float *P;                    // [splits][I][J], or [splits][J][I] when `across`
+    int I, J, kb, splits, kb_per_split;
+    int a_mn, across;            // (a_mn as in TcGemmArgs)
+};
+constexpr int kTcThinMax = 2;
+struct TcThinArgs {
+    TcThin job[kTcThinMax];
+    int items, items0;           // tiles times splits of all jobs, of the first
+    int busy, c_idle, c_busy;    // pairs 0 .. busy - 1, which have a product tile more than the others, take c_busy items each, the others c_idle
 };
 
 template <int BN>
@@ -313,10 +329,12 @@ __device__ __forceinline__ void mbar_arrive_cluster(uint32_t cluster_bar) {
     asm volatile("mbarrier.arrive.release.cluster.shared::cluster.b64 _, [%0];\n" ::"r"(cluster_bar) : "memory");
 }
 
+struct TcThinMaps { CUtensorMap a[kTcThinMax], b[kTcThinMax]; };
+
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kTThreads, 1)
 tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant__ CUtensorMap tmap_b,
                     const __grid_constant__ CUtensorMap tmap_a2, const __grid_constant__ CUtensorMap tmap_b2, const TcGemmArgs g,
-                    unsigned int *status) {
+                    const __grid_constant__ TcThinMaps thin_maps, const __grid_constant__ TcThinArgs thin, unsigned int *status) {
     using C = TpCfg;
     extern __shared__ uint8_t tp_smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>(((uintptr_t)tp_smem_raw + 1023) & ~(uintptr_t)1023);
@@ -339,6 +357,24 @@ tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
         i0 = (tile / tiles_j) * kTpTile;
         j0 = (tile % tiles_j) * kTpTile + half * (kTpTile / 2);
     };
+    // The pair's pieces of the thin products, after its tiles.  (Loops of their own in every role: as one loop over both kinds of work the
+    // products themselves took 3 % longer, the operands of their MMAs no longer being uniform to the compiler.)
+    struct Piece { int i0, kb0, kb1, job, part; };
+    auto piece_of = [&](int q, Piece &t) {
+        const bool busy = pair < thin.busy;
+        int e = (busy ? (pairs - thin.busy) * thin.c_idle + pair * thin.c_busy : (pair - thin.busy) * thin.c_idle) + q;
+        if (q >= (busy ? thin.c_busy : thin.c_idle) || e >= thin.items) return false;
+        t.job = e >= thin.items0 ? 1 : 0;
+        if (t.job) e -= thin.items0;
+        const TcThin &T = thin.job[t.job];
+        const int tiles_t = (T.I + kTpTile - 1) / kTpTile;
+        t.i0 = (e % tiles_t) * kTpTile;
+        t.part = e / tiles_t;
+        t.kb0 = t.part * T.kb_per_split;
+        t.kb1 = t.kb0 + T.kb_per_split < T.kb ? t.kb0 + T.kb_per_split : T.kb;
+        return true;
+    };
+    constexpr int kThinCols = kTpTile / 2;  // (the second CTA's half of the columns lies past the matrix: zeros)
 
     if (tid == 0) {
         for (int s = 0; s < C::STAGES; ++s) {
@@ -404,6 +440,30 @@ tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 if (++s == C::STAGES) { s = 0; ph ^= 1u; }
             }
         }
+        Piece t;
+        for (int q = 0; ok && piece_of(q, t); ++q) {
+            const int i0 = t.i0 + rank * kTBM, a_mn = thin.job[t.job].a_mn;
+            for (int kb = t.kb0; kb < t.kb1; ++kb) {
+                ok = mbar_wait(bar(C::BAR_EMPTY + s), ph ^ 1u, abort_flag, status, 0x880u + s);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                if (lane == 0) {
+                    const CUtensorMap *ma = &thin_maps.a[t.job];
+                    const int c0 = kb * kTBK;
+                    const uint32_t dst_a = sbase + s * C::STAGE_BYTES, dst_b = dst_a + C::A_BYTES, full = cluster_address(bar(C::BAR_FULL + s), 0);
+                    if (rank == 0) mbar_arrive_expect_tx(bar(C::BAR_FULL + s), 2 * (C::A_BYTES + kTBox));
+                    if (a_mn == 2) {
+                        tma_load_3d_pair(dst_a, ma, 0, c0, i0 / 64, full);
+                    } else if (a_mn) {
+                        for (int h = 0; h < kTBM / 64; ++h) tma_load_2d_pair(dst_a + h * kTBox, ma, i0 + 64 * h, c0, full);
+                    } else {
+                        tma_load_2d_pair(dst_a, ma, c0, i0, full);
+                    }
+                    tma_load_2d_pair(dst_b, &thin_maps.b[t.job], rank * (kThinCols / 2), c0, full);
+                }
+                ++issued;
+                if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+            }
+        }
         // Never leave with a copy in flight: a stage's MMAs, which follow its copies, reach this CTA's EMPTY.
         for (uint32_t q = 0; q < (uint32_t)C::STAGES; ++q) {
             const uint32_t rounds = (issued + C::STAGES - 1 - q) / C::STAGES;
@@ -443,6 +503,28 @@ tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 if (!ok) break;
                 warp_commit_pair(bar(C::BAR_ACCFULL + b));
             }
+            Piece t;
+            for (int q = 0; ok && piece_of(q, t); ++q, ++it) {
+                const int b = it & 1;
+                const uint32_t acc = tmem_base + b * kTpTile;
+                if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x890u))) break;
+                tc_fence_after();
+                const bool a_mn = thin.job[t.job].a_mn != 0;
+                const uint32_t idesc_w = C::IDESC | (a_mn ? 1u << 15 : 0u) | (1u << 16) | ((uint32_t)(kThinCols >> 3) << 17), step = a_mn ? (16 * 128) >> 4 : 32 >> 4;
+                for (int kb = t.kb0; kb < t.kb1; ++kb) {
+                    if (!(ok = wait(C::BAR_FULL + s, ph, 0x8a0u + s))) break;
+                    tc_fence_after();
+                    const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+                    const uint64_t adesc = a_mn ? make_sw128_mn_desc(sa, kTBox) : make_sw128_desc(sa), bdesc = make_sw128_mn_desc(sb, kTBox);
+#pragma unroll
+                    for (int kk = 0; kk < kTBK / 16; ++kk)
+                        warp_mma_f16_pair(acc, adesc + (uint64_t)(step * kk), bdesc + (uint64_t)(((16 * 128) >> 4) * kk), idesc_w, (kb > t.kb0 || kk) ? 1u : 0u);
+                    warp_commit_pair(bar(C::BAR_EMPTY + s));
+                    if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+                }
+                if (!ok) break;
+                warp_commit_pair(bar(C::BAR_ACCFULL + b));
+            }
         }
     } else {
         // ------------------------------------------------------------------ epilogue warps
@@ -474,6 +556,35 @@ tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                             if (g.accumulate) { const float4 c = *dst; o.x += c.x; o.y += c.y; o.z += c.z; o.w += c.w; }
                             *dst = o;
                         }
+                    }
+                }
+            }
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) mbar_arrive_cluster(cluster_address(bar(C::BAR_ACCEMPTY + b), 0));
+        }
+        Piece t;
+        for (int n = 0; ok && piece_of(n, t); ++n, ++it) {
+            const TcThin &T = thin.job[t.job];
+            const int b = it & 1;
+            ok = mbar_wait(bar(C::BAR_ACCFULL + b), (uint32_t)(it >> 1) & 1u, abort_flag, status, 0x8b0u);
+            if (!(ok = __all_sync(0xffffffffu, ok))) break;
+            tc_fence_after();
+            const int i = t.i0 + rank * kTBM + 32 * q + lane;
+            const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16) + b * kTpTile;
+            for (int cc = 0; cc < T.J; cc += 16) {  // (J is a multiple of 16)
+                uint32_t v[16];
+                tmem_ld16(lane_base + cc, v);
+                tmem_ld_wait();
+                if (i < T.I) {
+                    if (T.across) {
+#pragma unroll
+                        for (int u = 0; u < 16; ++u) T.P[((size_t)t.part * T.J + cc + u) * T.I + i] = __uint_as_float(v[u]);
+                    } else {
+                        float4 *dst = reinterpret_cast<float4 *>(T.P + ((size_t)t.part * T.I + i) * T.J + cc);
+#pragma unroll
+                        for (int u = 0; u < 4; ++u)
+                            dst[u] = make_float4(__uint_as_float(v[4 * u]), __uint_as_float(v[4 * u + 1]), __uint_as_float(v[4 * u + 2]), __uint_as_float(v[4 * u + 3]));
                     }
                 }
             }
@@ -588,12 +699,80 @@ extern "C" int hgf_internal_tc_pairs_pay(int32_t I, int32_t J, int32_t contracti
     return tc_pairs_pay(I, J, (contraction + kTBK - 1) / kTBK, true, sms, pairs) ? 1 : 0;
 }
 
+// A thin product as the caller describes it: P as in TcThin, room for splits_max partial sums; splits: as many as it was given.
+struct TcThinProduct {
+    TcOperand A, B;      // B.mn
+    int I, J, Cn;
+    bool across;
+    float *P;
+    int splits;
+};
+
+// The thin products' pieces over the pairs; false where launches of their own are the better way.  In half blocks of the product (64 of the
+// contraction for half a tile, 0.22 us): a piece costs 1.1 a block - its first operand is staged whole, of the second nearly nothing - and 10
+// for its start and end.  The pairs that have a tile of the last round less take pieces first; contractions are split, up to four
+// times, where that brings the last pair's end forward.  A launch of its own takes 4 us and its first operand's bytes at 4.5 TB/s; the
+// estimate has to stay below three quarters of that, since a pair streams what has left L2 by then more slowly than all SMs together do.
+// Training steps, launches of their own / this: 700 x 1024 -> 3000 130 / 112 us, 2048 x 2048 -> 2048 147 / 128, 1500 x 3200 -> 2000, r = 64 191 / 166,
+// 8000 x 768 -> 1536, r = 64 214 / 185, 4096 x 4096 -> 4096, r = 16 430 / 414, 8192 x 4096 -> 1024, r = 64 370 / 354, 8192 x 2048 -> 5632 565 / 559.
+static bool tc_deal_thin(TcThinArgs *t, const TcThinProduct *thin, int n, int num_work, int n_half, int kb_all, int pairs) {
+    const int rest = num_work % pairs, idle = pairs - rest;
+    const double extra = rest ? (n_half ? kb_all : 2.0 * kb_all) : 0.0;
+    double best = -1.0, alone = 0.0;
+    int longest = 0;
+    for (int i = 0; i < n; ++i) {
+        longest = std::max(longest, (thin[i].Cn + kTBK - 1) / kTBK);
+        alone += 4.0 + 2.0 * thin[i].I * thin[i].Cn / 4.5e6;
+    }
+    for (int parts = 1; parts <= 4; ++parts) {
+        const int piece = (longest + parts - 1) / parts;
+        TcThinArgs c = {};
+        for (int i = 0; i < n; ++i) {
+            TcThin &T = c.job[i];
+            T.P = thin[i].P;
+            T.I = thin[i].I; T.J = thin[i].J;
+            T.kb = (thin[i].Cn + kTBK - 1) / kTBK;
+            T.splits = (T.kb + piece - 1) / piece;
+            T.kb_per_split = (T.kb + T.splits - 1) / T.splits;
+            T.splits = (T.kb + T.kb_per_split - 1) / T.kb_per_split;  // no empty part
+            T.across = thin[i].across ? 1 : 0;
+            c.items += (T.I + kTpTile - 1) / kTpTile * T.splits;
+            if (i == 0) c.items0 = c.items;
+        }
+        c.busy = rest;
+        for (c.c_busy = 0; c.c_busy <= (rest > 0 ? 1 : 0); ++c.c_busy) {
+            c.c_idle = std::max(0, (c.items - c.c_busy * rest + idle - 1) / idle);
+            if (c.c_idle > 2) continue;
+            const double cost = 10.0 + 1.1 * piece, end = std::max(c.c_idle * cost, c.c_busy ? extra + c.c_busy * cost : extra);
+            if (best >= 0.0 && end >= best) continue;
+            best = end;
+            *t = c;
+        }
+    }
+    if (best >= 0.0 && 0.22 * (best - extra) <= 0.75 * alone) return true;
+    *t = TcThinArgs{};
+    return false;
+}
+
+// (for the tests: how n thin products of I[i] rows over contractions Cn[i] are dealt behind num_work tiles of kb_all blocks, the last n_half of
+// them halves; out: items, items0, busy, c_idle, c_busy, then splits and kb_per_split of each)
+extern "C" int hgf_internal_tc_deal_thin(const int32_t *I, const int32_t *Cn, int32_t n, int32_t num_work, int32_t n_half, int32_t kb_all, int32_t pairs, int32_t *out) {
+    TcThinProduct thin[kTcThinMax] = {};
+    for (int i = 0; i < n && i < kTcThinMax; ++i) { thin[i].I = I[i]; thin[i].Cn = Cn[i]; thin[i].J = 16; }
+    TcThinArgs t = {};
+    const bool ride = tc_deal_thin(&t, thin, n, num_work, n_half, kb_all, pairs);
+    out[0] = t.items; out[1] = t.items0; out[2] = t.busy; out[3] = t.c_idle; out[4] = t.c_busy;
+    for (int i = 0; i < n; ++i) { out[5 + 2 * i] = t.job[i].splits; out[6 + 2 * i] = t.job[i].kb_per_split; }
+    return ride ? 1 : 0;
+}
+
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
 // operand forms.  `partials` (splits_max * I * ldc floats) enables splitting the contraction when the
 // output has fewer tiles than the device has SMs; ldc must then be J.  With `splits_out` they are left there for the kernel that
-// reads the product next (*splits_out of them; 1: the product is in C).  Bases 16-byte aligned, ld % 8 == 0.
+// reads the product next (*splits_out of them; 1: the product is in C).  `thin`: products that may ride in a launch by pairs; `splits` is 0
+// afterwards for those that did not.  Bases 16-byte aligned, ld % 8 == 0.
 static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J,
-                           float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, cudaStream_t stream) {
+                           float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, TcThinProduct *thin, int n_thin, cudaStream_t stream) {
     const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64), sms = device_sm_count();
     const int kb1 = (Cn + kTBK - 1) / kTBK, kb2 = A2.p ? (Cn2 + kTBK - 1) / kTBK : 0, kb_all = kb1 + kb2;
     int pairs = I > kTBM && J > 128 && kb_all >= kTpMinBlocks && sms > 0 ? tc_pairs_at_once() : 0;
@@ -617,10 +796,21 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
         g.C = C; g.alpha = alpha; g.accumulate = accumulate ? 1 : 0;
         if (splits_out) *splits_out = 1;
         const int work = tiles + g.n_half / 2;
+        TcThinArgs t = {};
+        TcThinMaps thin_maps;
+        if (n_thin && !tc_deal_thin(&t, thin, n_thin, work, g.n_half, kb_all, pairs)) n_thin = 0;
+        for (int i = 0; i < kTcThinMax; ++i) {
+            thin_maps.a[i] = maps[0];
+            thin_maps.b[i] = maps[1];
+            if (i >= n_thin) continue;
+            if (!tc_map(&thin_maps.a[i], thin[i].A, thin[i].I, thin[i].Cn, kTBM, &t.job[i].a_mn) || !tc_map(&thin_maps.b[i], thin[i].B, thin[i].J, thin[i].Cn, 0))
+                return cudaErrorInvalidValue;
+            thin[i].splits = t.job[i].splits;
+        }
         unsigned int *status = device_status_word();
         if (!status) return cudaErrorMemoryAllocation;
-        return launch_chained(tc_pair_gemm_kernel, 2u * (unsigned)(work < pairs ? work : pairs), kTThreads, TpCfg::SMEM_BYTES, stream, maps[0], maps[1],
-                              maps[2], maps[3], g, status);
+        return launch_chained(tc_pair_gemm_kernel, 2u * (unsigned)(work < pairs && !n_thin ? work : pairs), kTThreads, TpCfg::SMEM_BYTES, stream, maps[0], maps[1],
+                              maps[2], maps[3], g, thin_maps, t, status);
     }
     const int tiles = ((I + kTBM - 1) / kTBM) * ((J + BN - 1) / BN);
     int splits = 1;
@@ -865,34 +1055,13 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     float *partials = (float *)(ws + L.partials);
     bool ok = true;
     auto gemm = [&](TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J, float alpha,
-                    bool acc, bool may_split, int *splits_out = nullptr) {
-        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, splits_out, stream) == cudaSuccess;
+                    bool acc, bool may_split, int *splits_out = nullptr, TcThinProduct *thin = nullptr, int n_thin = 0) {
+        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, splits_out, thin, n_thin, stream) == cudaSuccess;
     };
     const TcOperand dy_k = {(const __nv_bfloat16 *)dy, N, false};  // dY as [M rows][N contraction]
     const TcOperand dy_mn = {(const __nv_bfloat16 *)dy, N, true};  // dY as [N rows] contracted over its M stored rows
     const TcOperand x_k = {(const __nv_bfloat16 *)x, K, false}, x_mn = {(const __nv_bfloat16 *)x, K, true};
 
-    if (grads->dW) {  // Algorithm 1, steps 1-2 again, then dW[n][k] = sum_m dY[m][n] Xd[m][k]
-        if (K <= kBwQuantMaxK) {
-            const unsigned rows8 = (unsigned)((Mi + 7) / 8);
-            const __nv_bfloat16 *xp = (const __nv_bfloat16 *)x;
-            ok = (K <= kBwQuantMaxK / 2 ? launch_chained(bw_quant_kernel<8>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))
-                            : launch_chained(bw_quant_kernel<16>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))) == cudaSuccess;
-        } else {
-            PrologueParams pp = {};
-            pp.x = (const __nv_bfloat16 *)x;
-            pp.xq = (int8_t *)(ws + L.xq);
-            pp.gamma_x = (float *)(ws + L.gamma_x);
-            pp.M = Mi;
-            pp.K = K;
-            pp.flags = HGF_FLAG_NO_PDL;
-            if (launch_quant(pp, GemmPrologueExtra{}, stream) != cudaSuccess) return HGF_ERR_CUDA;
-            const size_t n8 = (size_t)M * K / 8;
-            ok = launch_chained(bw_dequant_kernel, blocks1(n8), 256, 0, stream, pp.xq, pp.gamma_x, K, n8, bf(L.xd)) == cudaSuccess;
-        }
-        gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false);
-    }
-    const bool fold = gamma > 1e-20f;  // the low-rank term of dX rides in the same contraction, pre-divided by gamma_W
     {
         BwWeights p = {};
         p.packed = (const uint32_t *)packed;
@@ -909,32 +1078,79 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         const unsigned blocks = p.blocks_t + p.blocks_at + blocks1(p.n_bt);
         if (blocks) ok = ok && launch_chained(bw_weights_kernel, blocks, 256, 0, stream, p) == cudaSuccess;
     }
+    float *z = (float *)(ws + L.z), *dh = (float *)(ws + L.dh), *G = grads->dBt ? grads->dBt : (float *)(ws + L.G);
+    const TcOperand At_k = {bf(L.At_b), K, false}, At_mn = {bf(L.At_b), K, true};
+    int sp = 1;
+    if (r) {                                                                                                 // Z = x A
+        gemm(x_k, At_k, K, none, none, 0, z, r, Mi, r, 1.0f, false, true, &sp);
+        ok = ok && launch_chained(bw_act_kernel, blocks1((size_t)M * r), 256, 0, stream, sp > 1 ? partials : z, sp, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, z, bf(L.h_b)) == cudaSuccess;
+    }
+    // The products with dY and H: dH = dY (g (.) B^T), and G[n][j] = sum_m dY[m][n] H[m][j], behind dW's tiles where tc_deal_thin has room there,
+    // else as launches of their own.
+    const bool want_g = r && (grads->dBt || grads->dgate);
+    const size_t half = (size_t)(kBwSplitsMax / 2) * std::max({Mi, N, K}) * r;  // (two sets of partial sums at a time)
+    TcThinProduct with_dw[2] = {{dy_k, TcOperand{bf(L.gBt), r, true}, Mi, r, N, false, partials, 0},
+                                {dy_mn, TcOperand{bf(L.h_b), r, true}, N, r, Mi, false, partials + half, 0}};
+    if (grads->dW) {  // Algorithm 1, steps 1-2 again, then dW[n][k] = sum_m dY[m][n] Xd[m][k]
+        if (K <= kBwQuantMaxK) {
+            const unsigned rows8 = (unsigned)((Mi + 7) / 8);
+            const __nv_bfloat16 *xp = (const __nv_bfloat16 *)x;
+            ok = ok && (K <= kBwQuantMaxK / 2 ? launch_chained(bw_quant_kernel<8>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))
+                            : launch_chained(bw_quant_kernel<16>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))) == cudaSuccess;
+        } else {
+            PrologueParams pp = {};
+            pp.x = (const __nv_bfloat16 *)x;
+            pp.xq = (int8_t *)(ws + L.xq);
+            pp.gamma_x = (float *)(ws + L.gamma_x);
+            pp.M = Mi;
+            pp.K = K;
+            pp.flags = HGF_FLAG_NO_PDL;
+            if (launch_quant(pp, GemmPrologueExtra{}, stream) != cudaSuccess) return HGF_ERR_CUDA;
+            const size_t n8 = (size_t)M * K / 8;
+            ok = ok && launch_chained(bw_dequant_kernel, blocks1(n8), 256, 0, stream, pp.xq, pp.gamma_x, K, n8, bf(L.xd)) == cudaSuccess;
+        }
+        gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false, nullptr, with_dw, r ? (want_g ? 2 : 1) : 0);
+    }
+    const bool fold = gamma > 1e-20f;  // the low-rank term of dX rides in the same contraction, pre-divided by gamma_W
     const TcOperand T_mn = {bf(L.T), K, true};  // T [N][K]: rows k of the product, contracted over n
     if (!r) {
         if (grads->dx) gemm(dy_k, T_mn, N, none, none, 0, grads->dx, K, Mi, K, gamma, false, false);
         return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
     }
-    float *z = (float *)(ws + L.z), *dh = (float *)(ws + L.dh), *G = grads->dBt ? grads->dBt : (float *)(ws + L.G);
-    const TcOperand At_k = {bf(L.At_b), K, false}, At_mn = {bf(L.At_b), K, true};
-    int sp = 1;
-    gemm(x_k, At_k, K, none, none, 0, z, r, Mi, r, 1.0f, false, true, &sp);                                  // Z = x A
-    ok = ok && launch_chained(bw_act_kernel, blocks1((size_t)M * r), 256, 0, stream, sp > 1 ? partials : z, sp, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, z, bf(L.h_b)) == cudaSuccess;
-    gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true, &sp);       // dH = dY (g (.) B^T)
-    ok = ok && launch_chained(bw_dz_kernel, blocks1((size_t)M * r), 256, 0, stream, sp > 1 ? partials : dh, sp, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b)) == cudaSuccess;
+    const float *dh_sums = partials;
+    sp = with_dw[0].splits;
+    if (!sp) {
+        gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true, &sp);
+        if (sp == 1) dh_sums = dh;
+    }
+    ok = ok && launch_chained(bw_dz_kernel, blocks1((size_t)M * r), 256, 0, stream, dh_sums, sp, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b)) == cudaSuccess;
+    // dA^T[j][k] = sum_m dZ[m][j] x[m][k]
+    TcThinProduct with_dx = {x_mn, TcOperand{bf(L.dz_b), r, true}, K, r, Mi, true, partials, 0};
     if (grads->dx) {                                                                                         // dX = gamma_W dY T + dZ A^T
         const TcOperand dzs_k = {bf(L.dzs_b), r, false};
         if (fold) {
-            gemm(dy_k, T_mn, N, dzs_k, At_mn, r, grads->dx, K, Mi, K, gamma, false, false);
+            gemm(dy_k, T_mn, N, dzs_k, At_mn, r, grads->dx, K, Mi, K, gamma, false, false, nullptr, &with_dx, grads->dAt ? 1 : 0);
         } else {
             gemm(dy_k, T_mn, N, none, none, 0, grads->dx, K, Mi, K, gamma, false, false);
             gemm(dzs_k, At_mn, r, none, none, 0, grads->dx, K, Mi, K, 1.0f, true, false);
         }
     }
-    if (grads->dAt)                                                                                          // dA^T[j][k] = sum_m dZ[m][j] x[m][k]
-        gemm(TcOperand{bf(L.dz_b), r, true}, x_mn, Mi, none, none, 0, grads->dAt, K, r, K, 1.0f, false, true);
-    if (grads->dBt || grads->dgate) {                                                                        // G[n][j] = sum_m dY[m][n] H[m][j]
-        gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true, &sp);
-        ok = ok && launch_chained(bw_gate_kernel, (unsigned)((N + 7) / 8), 256, 0, stream, sp > 1 ? partials : G, sp, (const __half *)Bt, gate, N, r, G, grads->dgate) == cudaSuccess;
+    if (grads->dAt) {
+        if (!with_dx.splits) {
+            gemm(TcOperand{bf(L.dz_b), r, true}, x_mn, Mi, none, none, 0, grads->dAt, K, r, K, 1.0f, false, true);
+        } else {
+            const size_t n4 = (size_t)r * K / 4;
+            ok = ok && launch_chained(tc_reduce_kernel, blocks1(n4), 256, 0, stream, (const float4 *)partials, with_dx.splits, n4, 1.0f, 0, (float4 *)grads->dAt) == cudaSuccess;
+        }
+    }
+    if (want_g) {
+        const float *g_sums = partials + half;
+        sp = with_dw[1].splits;
+        if (!sp) {
+            gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true, &sp);
+            g_sums = sp > 1 ? partials : G;
+        }
+        ok = ok && launch_chained(bw_gate_kernel, (unsigned)((N + 7) / 8), 256, 0, stream, g_sums, sp, (const __half *)Bt, gate, N, r, G, grads->dgate) == cudaSuccess;
     }
     return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
 }
