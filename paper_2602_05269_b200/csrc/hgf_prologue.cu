@@ -943,7 +943,8 @@ __global__ void __launch_bounds__(kThreads, 4) round_rows_kernel(const PrologueP
 // What it replaces there: a block walked its tokens' columns in a chain of 256-column chunks (a barrier and most of
 // a memory latency each, K / 256 of them, on M / 8 blocks), rounded in a second pass from L2, and a LayerNorm took a
 // launch of its own.
-constexpr int kRpThreads = 256, kRpWarps = kRpThreads / 32, kRpTokens = 16;
+constexpr int kRpTokens = 16;
+constexpr int kRpParts = 8;  // warps that share out the slice for x A; of sixteen warps two sets, half of the columns of H each
 struct RpLayout {
     int per, pitch;              // columns of a slice (a multiple of 64), bytes per staged row
     int off_stat, off_amax, off_sum, off_slots, off_part, off_x, smem;
@@ -957,8 +958,8 @@ __host__ __device__ inline RpLayout rp_layout(int K, int r, int log2_c) {
     L.off_amax = L.off_stat + C * kRpTokens * 16;         // [rank][token] patterns
     L.off_sum = L.off_amax + C * kRpTokens * 4;           // [rank][token] ints
     L.off_slots = L.off_sum + C * kRpTokens * 4;          // [rank][token][r]
-    L.off_part = L.off_slots + C * kRpTokens * r * 4;     // [warp][token][r]
-    L.off_x = (L.off_part + kRpWarps * kRpTokens * r * 4 + 127) / 128 * 128;
+    L.off_part = L.off_slots + C * kRpTokens * r * 4;     // [part][token][r]
+    L.off_x = (L.off_part + kRpParts * kRpTokens * r * 4 + 127) / 128 * 128;
     L.smem = L.off_x + kRpTokens * L.pitch;
     return L;
 }
@@ -966,11 +967,11 @@ __host__ __device__ inline RpLayout rp_layout(int K, int r, int log2_c) {
 // PER_SM: CTAs an SM that its registers leave room for (0: as they come).  All forms fit two but the widest behind a LayerNorm, which takes 154 registers
 // and spills 36 bytes at 128: in launches of more CTAs than SMs two an SM are worth that (r = 64, 2048 -> 1024: 26.3 -> 21.1 us
 // at M = 1000, 34.5 -> 27.8 at M = 2048), in smaller ones not (22.1 -> 26.4 at M = 1184).
-template <int JT, bool LN, int PER_SM>
-__global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x, const FrontEnd fe,
+template <int JT, bool LN, int TPW, int PER_SM>
+__global__ void __launch_bounds__(512 / TPW, PER_SM) rows_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x, const FrontEnd fe,
                                                                    const int log2_c, unsigned int *status) {
     extern __shared__ __align__(128) uint8_t rp_smem[];
-    constexpr int r = 8 * JT;
+    constexpr int r = 8 * JT, kRpThreads = 512 / TPW, W = kRpTokens / TPW;  // W warps: warp w works tokens w (and w + W) of the block
     const int C = 1 << log2_c, token_blocks = (p.M + kRpTokens - 1) / kRpTokens;
     const int cluster = (int)blockIdx.x >> log2_c, rank = (int)blockIdx.x & (C - 1);
     if (cluster >= token_blocks) {
@@ -1007,33 +1008,37 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
         cluster_arrive_relaxed();
     }
     const int nch = cols >> 5;
-    const __half *arow = JT > 0 ? p.At + (size_t)g * K + k0 + 8 * t : nullptr;
-    uint4 av[JT > 0 ? JT : 1];
+    constexpr int JH = JT * kRpParts / W;  // a warp's column tiles of H
+    const int part = warp & (kRpParts - 1), j0 = (warp / kRpParts) * 8 * JH;
+    const __half *arow = JT > 0 ? p.At + (size_t)(j0 + g) * K + k0 + 8 * t : nullptr;
+    uint4 av[JT > 0 ? JH : 1];
     auto load_a = [&](int c) {
         if constexpr (JT > 0)
 #pragma unroll
-            for (int jt = 0; jt < JT; ++jt) av[jt] = c < nch ? *reinterpret_cast<const uint4 *>(arow + (size_t)8 * jt * K + 32 * c) : make_uint4(0u, 0u, 0u, 0u);
+            for (int jt = 0; jt < JH; ++jt) av[jt] = c < nch ? *reinterpret_cast<const uint4 *>(arow + (size_t)8 * jt * K + 32 * c) : make_uint4(0u, 0u, 0u, 0u);
     };
     __syncthreads();
     pdl_wait();
-    load_a(warp);  // this warp's first chunk of A^T (like every read of this path, after the wait)
+    pdl_launch_dependents();  // (the launch that follows finds room only as these blocks leave; let in at the end it came 0.1 to 0.4 us later)
+    load_a(part);  // this warp's first chunk of A^T (like every read of this path, after the wait)
     bool ok = warp_wait(bar_x, status, 0x680u);
     cluster_wait_acquire();  // every CTA of the cluster has started
 
-    // ---- statistics: warp w works tokens w and w + 8 of the block --------------------------------------------
+    // ---- statistics --------------------------------------------------------------------------------------------
     const int nu = cols >> 3;  // 16-byte units of a row's slice
-    auto unit = [&](int ml, int i) { return *reinterpret_cast<const uint4 *>(x_s + ml * L.pitch + 16 * i); };
-    float mean[2] = {0.0f, 0.0f}, rstd[2] = {0.0f, 0.0f};
-    // the normalised values of unit i of both tokens (the weights are read once for the two)
-    auto ln_both = [&](int i, auto &&body) {
+    auto has_row = [&](int q) { return warp + W * q < rows; };
+    auto unit = [&](int q, int i) { return *reinterpret_cast<const uint4 *>(x_s + (warp + W * q) * L.pitch + 16 * i); };
+    float mean[TPW] = {}, rstd[TPW] = {};
+    // the normalised values of unit i of the warp's tokens (the weights are read once for all of them)
+    auto ln_each = [&](int i, auto &&body) {
         const float4 *w4 = reinterpret_cast<const float4 *>(fe.ln_w + k0 + 8 * i), *b4 = reinterpret_cast<const float4 *>(fe.ln_b + k0 + 8 * i);
         const float4 w0 = w4[0], w1 = w4[1], b0 = b4[0], b1 = b4[1];
         const float w[8] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w}, b[8] = {b0.x, b0.y, b0.z, b0.w, b1.x, b1.y, b1.z, b1.w};
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            if (warp + kRpWarps * q >= rows) continue;
+        for (int q = 0; q < TPW; ++q) {
+            if (!has_row(q)) continue;
             float f[8], xn[8];
-            unpack8(unit(warp + kRpWarps * q, i), f);
+            unpack8(unit(q, i), f);
 #pragma unroll
             for (int e = 0; e < 8; ++e) xn[e] = ln_value(f[e], mean[q], rstd[q], w[e], b[e]);
             body(q, xn);
@@ -1044,15 +1049,15 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
         // of a double is x 2^-896 (subnormals too), so one fused multiply-add gives x - x[0] without a conversion; infinities and
         // NaNs, which that would miss, make the sum a NaN.
         // (four partial sums each: the additions of one are a chain)
-        double first[2], sum[2][4] = {}, sum2[2][4] = {};
-        uint32_t top[2] = {0u, 0u};
+        double first[TPW], sum[TPW][4] = {}, sum2[TPW][4] = {};
+        uint32_t top[TPW] = {};
 #pragma unroll
-        for (int q = 0; q < 2; ++q) first[q] = warp + kRpWarps * q < rows ? (double)__bfloat162float(p.x[(size_t)(m0 + warp + kRpWarps * q) * K]) : 0.0;
+        for (int q = 0; q < TPW; ++q) first[q] = has_row(q) ? (double)__bfloat162float(p.x[(size_t)(m0 + warp + W * q) * K]) : 0.0;
         for (int i = lane; i < nu; i += 32)
 #pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                if (warp + kRpWarps * q >= rows) continue;
-                const uint4 u = unit(warp + kRpWarps * q, i);
+            for (int q = 0; q < TPW; ++q) {
+                if (!has_row(q)) continue;
+                const uint4 u = unit(q, i);
                 top[q] = absmax8_bits(top[q], u);
                 const uint32_t w[4] = {u.x, u.y, u.z, u.w};
 #pragma unroll
@@ -1065,8 +1070,7 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
                 }
             }
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int ml = warp + kRpWarps * q;
+        for (int q = 0; q < TPW; ++q) {
             double s = (top[q] & 0xffffu) >= 0x7f80u || top[q] >= 0x7f800000u ? __longlong_as_double(0x7ff8000000000000ll)
                                                                                          : (sum[q][0] + sum[q][1]) + (sum[q][2] + sum[q][3]),
                    ss = (sum2[q][0] + sum2[q][1]) + (sum2[q][2] + sum2[q][3]);
@@ -1076,18 +1080,17 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
                 ss += __shfl_xor_sync(0xffffffffu, ss, o);
             }
             if (lane < C) {
-                const uint32_t dst = s0 + L.off_stat + (rank * kRpTokens + ml) * 16;
+                const uint32_t dst = s0 + L.off_stat + (rank * kRpTokens + warp + W * q) * 16;
                 st_async_b64(dst, bar_stat, (uint32_t)lane, (uint64_t)__double_as_longlong(s));
                 st_async_b64(dst + 8, bar_stat, (uint32_t)lane, (uint64_t)__double_as_longlong(ss));
             }
         }
         ok = warp_wait(bar_stat, status, 0x681u) && ok;
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
-            const int ml = warp + kRpWarps * q;
+        for (int q = 0; q < TPW; ++q) {
             double s = 0.0, ss = 0.0;
             for (int k = 0; k < C; ++k) {
-                const double2 v = *reinterpret_cast<const double2 *>(rp_smem + L.off_stat + (k * kRpTokens + ml) * 16);
+                const double2 v = *reinterpret_cast<const double2 *>(rp_smem + L.off_stat + (k * kRpTokens + warp + W * q) * 16);
                 s += v.x;
                 ss += v.y;
             }
@@ -1096,72 +1099,72 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
             rstd[q] = (float)rsqrt(var + (double)fe.eps);
         }
     }
-    uint32_t bits[2] = {0u, 0u};
+    uint32_t bits[TPW] = {};
     if constexpr (LN) {
-        float a[2] = {0.0f, 0.0f};
+        float a[TPW] = {};
 #pragma unroll 2
         for (int i = lane; i < nu; i += 32)
-            ln_both(i, [&](int q, const float (&xn)[8]) {
+            ln_each(i, [&](int q, const float (&xn)[8]) {
 #pragma unroll
                 for (int e = 0; e < 8; ++e) a[q] = fmaxf(a[q], fabsf(xn[e]));
             });
 #pragma unroll
-        for (int q = 0; q < 2; ++q) bits[q] = __float_as_uint(a[q]);
+        for (int q = 0; q < TPW; ++q) bits[q] = __float_as_uint(a[q]);
     } else {
-        uint32_t acc[2] = {0u, 0u};
+        uint32_t acc[TPW] = {};
         for (int i = lane; i < nu; i += 32)
 #pragma unroll
-            for (int q = 0; q < 2; ++q)
-                if (warp + kRpWarps * q < rows) acc[q] = absmax8_bits(acc[q], unit(warp + kRpWarps * q, i));
+            for (int q = 0; q < TPW; ++q)
+                if (has_row(q)) acc[q] = absmax8_bits(acc[q], unit(q, i));
 #pragma unroll
-        for (int q = 0; q < 2; ++q) {
+        for (int q = 0; q < TPW; ++q) {
             bits[q] = __float_as_uint(absmax_bits_to_float(acc[q]));
             if (bits[q] > 0x7f800000u) bits[q] = 0u;  // a NaN does not count, as in fmaxf
         }
     }
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < TPW; ++q) {
         bits[q] = __reduce_max_sync(0xffffffffu, bits[q]);
-        if (lane < C) st_async_f32(s0 + L.off_amax + (rank * kRpTokens + warp + kRpWarps * q) * 4, bar_amax, (uint32_t)lane, __uint_as_float(bits[q]));
+        if (lane < C) st_async_f32(s0 + L.off_amax + (rank * kRpTokens + warp + W * q) * 4, bar_amax, (uint32_t)lane, __uint_as_float(bits[q]));
     }
 
     // ---- x A over the slice, while the maxima travel: tokens are the 16-row operand, 8 columns of H the 8-column operand --
     if constexpr (JT > 0) {
-        float acc[JT][4];
+        float acc[JH][4];
 #pragma unroll
-        for (int jt = 0; jt < JT; ++jt)
+        for (int jt = 0; jt < JH; ++jt)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[jt][c] = 0.0f;
-        for (int c = warp; c < nch; c += kRpWarps) {
+        for (int c = part; c < nch; c += kRpParts) {
             const uint8_t *xr = x_s + g * L.pitch + 64 * c + 16 * t;
             const uint4 x0 = *reinterpret_cast<const uint4 *>(xr), x1 = *reinterpret_cast<const uint4 *>(xr + 8 * L.pitch);
-            uint4 a_now[JT];
+            uint4 a_now[JH];
 #pragma unroll
-            for (int jt = 0; jt < JT; ++jt) a_now[jt] = av[jt];
-            load_a(c + kRpWarps);
+            for (int jt = 0; jt < JH; ++jt) a_now[jt] = av[jt];
+            load_a(c + kRpParts);
 #pragma unroll
             for (int i = 0; i < 4; ++i) {
                 // elements 2 i and 2 i + 1 of this lane's eight take the k slots t and t + 4 of MMA i
                 const uint32_t w0 = (&x0.x)[i], w1 = (&x1.x)[i];
 #pragma unroll
-                for (int jt = 0; jt < JT; ++jt) {
+                for (int jt = 0; jt < JH; ++jt) {
                     const float2 bf = __half22float2(*reinterpret_cast<const __half2 *>(&(&a_now[jt].x)[i]));
                     mma_tf32(acc[jt], w0 << 16, w1 << 16, w0 & 0xffff0000u, w1 & 0xffff0000u, __float_as_uint(bf.x), __float_as_uint(bf.y));
                 }
             }
         }
-        float *part = reinterpret_cast<float *>(rp_smem + L.off_part) + (size_t)warp * kRpTokens * r;
+        float *sums = reinterpret_cast<float *>(rp_smem + L.off_part) + (size_t)part * kRpTokens * r + j0;
 #pragma unroll
-        for (int jt = 0; jt < JT; ++jt) {
-            *reinterpret_cast<float2 *>(part + g * r + 8 * jt + 2 * t) = make_float2(acc[jt][0], acc[jt][1]);
-            *reinterpret_cast<float2 *>(part + (g + 8) * r + 8 * jt + 2 * t) = make_float2(acc[jt][2], acc[jt][3]);
+        for (int jt = 0; jt < JH; ++jt) {
+            *reinterpret_cast<float2 *>(sums + g * r + 8 * jt + 2 * t) = make_float2(acc[jt][0], acc[jt][1]);
+            *reinterpret_cast<float2 *>(sums + (g + 8) * r + 8 * jt + 2 * t) = make_float2(acc[jt][2], acc[jt][3]);
         }
         __syncthreads();
         const float *all = reinterpret_cast<const float *>(rp_smem + L.off_part);
         for (int e = tid; e < kRpTokens * r; e += kRpThreads) {  // to the CTA that owns the token, in warp order
             float z = 0.0f;
 #pragma unroll
-            for (int w = 0; w < kRpWarps; ++w) z += all[w * kRpTokens * r + e];
+            for (int w = 0; w < kRpParts; ++w) z += all[w * kRpTokens * r + e];
             st_async_f32(s0 + L.off_slots + (rank * kRpTokens * r + e) * 4, bar_h, (uint32_t)((e / r) >> (4 - log2_c)), z);
         }
         __syncwarp();
@@ -1169,44 +1172,43 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
 
     // ---- codes ------------------------------------------------------------------------------------------------
     ok = warp_wait(bar_amax, status, 0x682u) && ok;
-    float gm[2], scale[2];
-    int sums[2] = {0, 0};
+    float gm[TPW], scale[TPW];
+    int sums[TPW] = {};
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
+    for (int q = 0; q < TPW; ++q) {
         uint32_t most = 0u;
         for (int k = 0; k < C; ++k) {
-            const uint32_t v = *reinterpret_cast<const uint32_t *>(rp_smem + L.off_amax + (k * kRpTokens + warp + kRpWarps * q) * 4);
+            const uint32_t v = *reinterpret_cast<const uint32_t *>(rp_smem + L.off_amax + (k * kRpTokens + warp + W * q) * 4);
             most = v > most ? v : most;
         }
         gm[q] = fmaxf(__uint_as_float(most), 1e-5f);
         scale[q] = __fdiv_rn(127.0f, gm[q]);
     }
     auto store = [&](int q, int i, const uint2 &o) {
-        const size_t at = ((size_t)(m0 + warp + kRpWarps * q) * K + k0) / 8 + i;
+        const size_t at = ((size_t)(m0 + warp + W * q) * K + k0) / 8 + i;
         reinterpret_cast<uint2 *>(p.xq)[at] = o;
         if (p.dbg_xq) reinterpret_cast<uint2 *>(p.dbg_xq)[at] = o;
     };
     if (ok) {
         if constexpr (LN) {
 #pragma unroll 2
-            for (int i = lane; i < nu; i += 32) ln_both(i, [&](int q, const float (&xn)[8]) { store(q, i, ln_codes8(xn, scale[q], sums[q])); });
+            for (int i = lane; i < nu; i += 32) ln_each(i, [&](int q, const float (&xn)[8]) { store(q, i, ln_codes8(xn, scale[q], sums[q])); });
         } else {
-            const QuantScale qs[2] = {make_quant_scale(gm[0]), make_quant_scale(gm[1])};
+            QuantScale qs[TPW];
+#pragma unroll
+            for (int q = 0; q < TPW; ++q) qs[q] = make_quant_scale(gm[q]);
             for (int i = lane; i < nu; i += 32)
 #pragma unroll
-                for (int q = 0; q < 2; ++q)
-                    if (warp + kRpWarps * q < rows) store(q, i, quant8(unit(warp + kRpWarps * q, i), qs[q], sums[q]));
+                for (int q = 0; q < TPW; ++q)
+                    if (has_row(q)) store(q, i, quant8(unit(q, i), qs[q], sums[q]));
         }
     }
 #pragma unroll
-    for (int q = 0; q < 2; ++q) {
-        const int ml = warp + kRpWarps * q;
-        int sum = sums[q];
-        sum = __reduce_add_sync(0xffffffffu, sum);
-        if (lane == 0)
-            st_async_f32(s0 + L.off_sum + (rank * kRpTokens + ml) * 4, bar_sum, (uint32_t)(ml >> (4 - log2_c)), __int_as_float(sum));
+    for (int q = 0; q < TPW; ++q) {
+        const int ml = warp + W * q, owner = ml >> (4 - log2_c), sum = __reduce_add_sync(0xffffffffu, sums[q]);
+        if (lane == 0) st_async_f32(s0 + L.off_sum + (rank * kRpTokens + ml) * 4, bar_sum, (uint32_t)owner, __int_as_float(sum));
         // (the CTA that owns the token writes its values)
-        if (lane == 0 && (ml >> (4 - log2_c)) == rank && ml < rows && ok) {
+        if (lane == 0 && owner == rank && ml < rows && ok) {
             const int m = m0 + ml;
             p.gamma_x[m] = gm[q];
             if (x.tok_sc) x.tok_sc[m] = gm[q] * x.gw_over_127;
@@ -1217,7 +1219,6 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
             }
         }
     }
-    pdl_launch_dependents();  // late: see gemm_prologue_kernel
 
     const int own = kRpTokens >> log2_c, t0 = rank * own;  // this CTA's tokens of the block
     if constexpr (JT > 0) {
@@ -1254,12 +1255,13 @@ __global__ void __launch_bounds__(kRpThreads, PER_SM) rows_prologue_kernel(const
         }
 }
 
-// Where it is used, and the cluster size: see launch_rows_prologue.
-template <int JT, bool LN, int PER_SM = 0>
-static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, int log2_c, cudaStream_t stream) {
+// Where it is used, the cluster size and `least` (bytes of shared memory): see launch_rows_prologue.
+template <int JT, bool LN, int TPW, int PER_SM = 0>
+static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd &fe, int log2_c, size_t least, cudaStream_t stream) {
+    constexpr int kRpThreads = 512 / TPW;
     static std::atomic<unsigned long long> attr_done{0};
     const RpLayout L = rp_layout(p.K, p.r, log2_c);
-    cudaError_t e = ensure_dynamic_smem(rows_prologue_kernel<JT, LN, PER_SM>, kRpSmemLimit, attr_done);
+    cudaError_t e = ensure_dynamic_smem(rows_prologue_kernel<JT, LN, TPW, PER_SM>, kRpSmemLimit, attr_done);
     if (e != cudaSuccess) return e;
     unsigned int *status = device_status_word();
     if (!status) return cudaErrorMemoryAllocation;
@@ -1267,13 +1269,13 @@ static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPr
     cudaLaunchAttribute attr[2];
     cudaLaunchConfig_t cfg = prologue_cfg(((p.M + kRpTokens - 1) / kRpTokens) * C + (gate_blocks + C - 1) / C * C, !(p.flags & HGF_FLAG_NO_PDL), stream, attr);
     cfg.blockDim = dim3(kRpThreads);
-    cfg.dynamicSmemBytes = (size_t)L.smem;
+    cfg.dynamicSmemBytes = (size_t)L.smem > least ? (size_t)L.smem : least;
     attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
     attr[cfg.numAttrs].val.clusterDim.x = (unsigned)C;
     attr[cfg.numAttrs].val.clusterDim.y = 1;
     attr[cfg.numAttrs].val.clusterDim.z = 1;
     ++cfg.numAttrs;
-    e = cudaLaunchKernelEx(&cfg, rows_prologue_kernel<JT, LN, PER_SM>, p, x, fe, log2_c, status);
+    e = cudaLaunchKernelEx(&cfg, rows_prologue_kernel<JT, LN, TPW, PER_SM>, p, x, fe, log2_c, status);
     count_launch();
     return e != cudaSuccess ? e : cudaGetLastError();
 }
@@ -1312,6 +1314,17 @@ static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPr
 //    11.1 / 13.9 at M = 500 (96 output tiles), 12.7 / 13.6 at 640 (120), 16.5 / 13.9 at 700 (144); 512 -> 5632 12.5 / 14.2 at M = 300 (132);
 //    768 -> 1024 12.9 / 11.7 at M = 700, 15.4 / 18.1 at 1500, 22.9 / 21.4 at 3000; 768 -> 3040 13.0 / 14.3 at M = 500, a quarter less
 //    at 700 to 1168.  Long rows in one CTA: K = 3072 72 / 68 at M = 5000, 80.4 / 82.6 at 8192.
+// At most two CTAs an SM (by asking for 80 KB) where that many run at once: CTAs start as the SMs come free at the end of the launch before, and
+// with room for three the first SMs took three and others none.  As they come / two: 2048 -> 2048, r = 32, LayerNorm 32.0 / 26.7 at M = 2000, without a
+// correction 24.1 / 18.0, r = 32 without a LayerNorm 16.6 / 14.9 at M = 1000.  29 clusters of eight and more do need room for three: 4096 -> 2048
+// 18.0 / 19.9 at M = 500 (K <= 2048 takes clusters of four there: 1024 -> 2048, r = 16 12.0 / 10.2).
+// Sixteen warps a CTA, a token each, or eight with two each, eight / sixteen: r = 32 2048 -> 2048 13.0 / 12.4 at M = 17, 14.9 / 14.7 at 1000, 20.6 / 19.9 at 1184,
+// 22.3 / 21.4 at 2300; with a LayerNorm 12.9 / 12.4, 18.5 / 18.4, 25.7 / 26.1, 27.4 / 27.7 (slices of 1024 columns), 4096 -> 4096 31.7 / 32.5 at M = 800 and
+// 49.3 / 48.5 at 1184 (of 2048); without a correction 2048 -> 1024 11.8 / 11.4 at M = 200, 17.4 / 17.9 at 1184.  Ranks of 64 leave room for one CTA of
+// sixteen warps an SM: 13.3 / 11.6 at M = 200, 13.6 / 15.9 at 440, 23.3 / 21.1 at 1184, 24.1 / 28.4 at 2000; with a LayerNorm 15.0 / 13.6, 17.1 / 19.6, 25.8 / 23.9,
+// 30.6 / 33.5; rank 48 11.4 / 10.7 at M = 17, 12.7 / 12.7 at 440, 15.1 / 15.4 at 800.
+// Batches: as many blocks of tokens as SMs; the other kernels / this one at M = 2200 26.9 / 21.8 for 2048 -> 2048, 52.5 / 45.5 for 5632 -> 2048, 37.9 / 28.7 with a
+// LayerNorm, r = 64 28.3 / 25.0; at M = 3000 31.6 / 32.5, 64.0 / 65.2, 44.4 / 42.5, 35.6 / 38.3; with a LayerNorm 51.2 / 48.5 at 4096, 65.4 / 70.4 at 6000.
 // Cluster size: CTAs for every SM, two of them on one if they fit; one step smaller where that many don't run at once: 1024 -> 1024,
 // M = 1168, r = 48 16.4 -> 15.0 us, M = 570 15.4 -> 13.9; 8192 -> 1024, M = 525 26.6 -> 28.5.
 static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd *fe, cudaStream_t stream) {
@@ -1323,6 +1336,8 @@ static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmProlo
     // (registers: two CTAs an SM at most; 33 clusters of eight or 71 of four run at once on 148 SMs, more take a second round, which
     // only long slices are worth)
     if ((p.r >= 48 || (fe && p.r == 32)) && ((c == 3 && p.K <= 2048 && (blocks << c) > 2 * sms - sms / 4) || (c == 2 && (blocks << c) > 2 * sms - sms / 16))) --c;
+    const int crowded = 2 * sms - 2 * sms / 5;  // (29 clusters of eight and more, with the blocks for the up-projection's operand)
+    if (p.r > 0 && p.r <= 32 && c == 3 && p.K <= 2048 && (blocks << 3) > crowded) --c;
     while (c < 3 && rp_layout(p.K, p.r, c).smem > 110 * 1024) ++c;  // two CTAs on an SM
     if (rp_layout(p.K, p.r, c).smem > kRpSmemLimit) return cudaErrorNotSupported;
     bool take;
@@ -1335,19 +1350,38 @@ static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmProlo
             else take = take && (p.K <= 512 || p.M >= 1800 || tiles > sms);
         }
     } else {
-        take = p.M <= 2048 && p.K >= 1024;
+        take = (blocks <= sms || (fe && p.r <= 32 && p.M <= 4096)) && p.K >= 1024;
         if (!fe) take = take && (blocks << c) <= 4 * sms && (p.r > 16 || p.K > 2048 || p.M <= 1280);
     }
     if (!take) return cudaErrorNotSupported;
     const FrontEnd none = {};
+    // sixteen warps a CTA (a token each) or eight
+    const int ctas = blocks << c, slice = p.K >> c;
+    const bool three = p.r > 0 && p.r <= 32 && c == 3 && ctas > crowded;  // CTAs an SM
+    bool wide;
+    if (three) wide = false;
+    else if (p.r <= 32) wide = !fe || c == 3 || slice <= 512 || (p.r > 0 && slice >= 2048);
+    else if (fe) wide = ctas <= sms;
+    else if (p.r == 48) wide = c == 3;
+    else wide = ctas <= (c == 3 ? sms - sms / 6 : (c == 2 ? sms - sms / 10 : sms));
+    const size_t least = !three && ctas <= 2 * sms ? 80 * 1024 : 0;
     switch (p.r) {
-        case 0: return fe ? launch_rows_prologue_jt<0, true>(p, x, *fe, c, stream) : cudaErrorNotSupported;
-        case 16: return fe ? launch_rows_prologue_jt<2, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<2, false>(p, x, none, c, stream);
-        case 32: return fe ? launch_rows_prologue_jt<4, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<4, false>(p, x, none, c, stream);
-        case 48: return fe ? launch_rows_prologue_jt<6, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<6, false>(p, x, none, c, stream);
+        case 0:
+            if (!fe) return cudaErrorNotSupported;
+            return wide ? launch_rows_prologue_jt<0, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<0, true, 2>(p, x, *fe, c, least, stream);
+        case 16:
+            if (fe) return wide ? launch_rows_prologue_jt<2, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<2, true, 2>(p, x, *fe, c, least, stream);
+            return wide ? launch_rows_prologue_jt<2, false, 1>(p, x, none, c, least, stream) : launch_rows_prologue_jt<2, false, 2>(p, x, none, c, least, stream);
+        case 32:
+            if (fe) return wide ? launch_rows_prologue_jt<4, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<4, true, 2>(p, x, *fe, c, least, stream);
+            return wide ? launch_rows_prologue_jt<4, false, 1>(p, x, none, c, least, stream) : launch_rows_prologue_jt<4, false, 2>(p, x, none, c, least, stream);
+        case 48:
+            if (fe) return wide ? launch_rows_prologue_jt<6, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<6, true, 2>(p, x, *fe, c, least, stream);
+            return wide ? launch_rows_prologue_jt<6, false, 1>(p, x, none, c, least, stream) : launch_rows_prologue_jt<6, false, 2>(p, x, none, c, least, stream);
         case 64:
-            if (!fe) return launch_rows_prologue_jt<8, false>(p, x, none, c, stream);
-            return (blocks << c) <= sms ? launch_rows_prologue_jt<8, true>(p, x, *fe, c, stream) : launch_rows_prologue_jt<8, true, 2>(p, x, *fe, c, stream);
+            if (!fe) return wide ? launch_rows_prologue_jt<8, false, 1>(p, x, none, c, least, stream) : launch_rows_prologue_jt<8, false, 2>(p, x, none, c, least, stream);
+            if (wide) return launch_rows_prologue_jt<8, true, 1>(p, x, *fe, c, least, stream);
+            return (blocks << c) <= sms ? launch_rows_prologue_jt<8, true, 2>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<8, true, 2, 2>(p, x, *fe, c, least, stream);
         default: return cudaErrorInvalidValue;
     }
 }
