@@ -286,8 +286,8 @@ tc_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constant
 // Barriers: both CTAs' copies count on the first one's FULL; its commits reach both CTAs' EMPTY and ACCFULL; both epilogues
 // arrive on its ACCEMPTY.
 // Which products it takes: tc_pairs_pay.  The tiles of 128 x 256 by single CTAs held the two large products of
-// 2048 x 5632 at M = 8192 at 1.14 and 1.22 PFLOP/s (166, 155 us), pairs at 1.25 and 1.42 (152, 133 us), where the power limit is
-// near (library bf16 products for seconds on end: 1.37).  Whole backward pass in a captured chain: 425 -> 380 us, 8192 x 5632 -> 2048
+// 2048 x 5632 at M = 8192 at 1.14 and 1.22 PFLOP/s (166, 155 us), pairs at 1.25 and 1.42 (152, 133 us; 143 and 127 since a stage comes in
+// fewer copies: tc_map), where the power limit is near (library bf16 products for seconds on end: 1.37).  Whole backward pass in a captured chain: 425 -> 380 us, 8192 x 5632 -> 2048
 // 547 -> 451, 2048 -> 2048 215 -> 186, 1500 x 3200 -> 2000 93 -> 75.
 struct TpCfg {
     static constexpr int STAGES = 6, A_BYTES = kTBM * 128, STAGE_BYTES = 2 * A_BYTES;
@@ -879,7 +879,7 @@ __global__ void __launch_bounds__(256) bw_quant_kernel(const __nv_bfloat16 *x, i
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         if (lane + 32 * u < nv) {
-            const uint2 c = quant8(v[u], qs, sum);
+            const uint2 c = quant8<true>(v[u], qs, sum);
             const uint32_t w[2] = {c.x ^ 0x80808080u, c.y ^ 0x80808080u};  // code + 128
             uint32_t o[4];
 #pragma unroll

@@ -268,7 +268,7 @@ __global__ void __launch_bounds__(kThreads) quant_rows_kernel(const ProloguePara
 #pragma unroll
     for (int u = 0; u < U; ++u) {
         if (lane + 32 * u < nv) {
-            const uint2 o = quant8(v[u], qs, sum);
+            const uint2 o = quant8<true>(v[u], qs, sum);
             qv[lane + 32 * u] = o;
             if (dq) dq[lane + 32 * u] = o;
         }
@@ -886,12 +886,12 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
         int i = lane;
         for (; i + 96 < nv; i += 128) {  // four units in flight per lane
             const uint4 v0 = xv[i], v1 = xv[i + 32], v2 = xv[i + 64], v3 = xv[i + 96];
-            const uint2 o0 = quant8(v0, qs, sum), o1 = quant8(v1, qs, sum), o2 = quant8(v2, qs, sum), o3 = quant8(v3, qs, sum);
+            const uint2 o0 = quant8<true>(v0, qs, sum), o1 = quant8<true>(v1, qs, sum), o2 = quant8<true>(v2, qs, sum), o3 = quant8<true>(v3, qs, sum);
             qv[i] = o0; qv[i + 32] = o1; qv[i + 64] = o2; qv[i + 96] = o3;
             if (dq) { dq[i] = o0; dq[i + 32] = o1; dq[i + 64] = o2; dq[i + 96] = o3; }
         }
         for (; i < nv; i += 32) {
-            const uint2 o = quant8(xv[i], qs, sum);
+            const uint2 o = quant8<true>(xv[i], qs, sum);
             qv[i] = o;
             if (dq) dq[i] = o;
         }
@@ -922,12 +922,12 @@ __global__ void __launch_bounds__(kThreads, 4) round_rows_kernel(const PrologueP
     int i = lane;
     for (; i + 96 < nv; i += 128) {  // four units in flight per lane
         const uint4 v0 = xv[i], v1 = xv[i + 32], v2 = xv[i + 64], v3 = xv[i + 96];
-        const uint2 o0 = quant8(v0, qs, sum), o1 = quant8(v1, qs, sum), o2 = quant8(v2, qs, sum), o3 = quant8(v3, qs, sum);
+        const uint2 o0 = quant8<true>(v0, qs, sum), o1 = quant8<true>(v1, qs, sum), o2 = quant8<true>(v2, qs, sum), o3 = quant8<true>(v3, qs, sum);
         qv[i] = o0; qv[i + 32] = o1; qv[i + 64] = o2; qv[i + 96] = o3;
         if (dq) { dq[i] = o0; dq[i + 32] = o1; dq[i + 64] = o2; dq[i + 96] = o3; }
     }
     for (; i < nv; i += 32) {
-        const uint2 o = quant8(xv[i], qs, sum);
+        const uint2 o = quant8<true>(xv[i], qs, sum);
         qv[i] = o;
         if (dq) dq[i] = o;
     }

@@ -67,20 +67,41 @@ __device__ __forceinline__ float absmax_bits_to_float(uint32_t acc) {
 // the bytes are packed straight from those patterns, and the tie test of all eight values is one
 // predicate; only a unit that holds an exact tie (rare) goes back over its values to move the odd
 // candidates to their even neighbours.
+// PAIRS: two values an instruction (f32x2), each rounded as by itself, the same bytes: for the kernels that are bound by the number of
+// instructions (layer calls, one at a time / pairs: 4096 -> 4096 without a correction at M = 4000 75.4 / 74.2 us, 2048 -> 2048 at M = 100 11.05 / 10.8,
+// 6144 -> 1024, r = 64 at M = 6000 121.1 / 119.2, 2048 -> 5632 at M = 8192 equal, at the power limit).  Where a warp has one unit and waits for
+// the result the pairs' latency shows (32 decode launches in a row 217 / 222 us), and rows_prologue_kernel's registers would no longer leave room for
+// three CTAs an SM (5632 -> 2048 at M = 512 20.1 / 22.6): those take one value at a time.
+template <bool PAIRS = false>
 __device__ __forceinline__ uint2 quant8(const uint4 &v, const QuantScale &s, int &sum) {
     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
     uint32_t b[8];
     if (s.fast) {
         constexpr float kMagic = 12582912.0f;  // 1.5 * 2^23
-        float xf[8], res[8];
+        float res[8];
         bool tie = false;
+        if constexpr (PAIRS) {
+            const uint64_t magic = pack_f32x2(kMagic, kMagic), inv = pack_f32x2(s.inv127, s.inv127), gamma = pack_f32x2(s.gamma, s.gamma);
 #pragma unroll
-        for (int e = 0; e < 8; ++e) {
-            xf[e] = (e & 1) ? bf16hi_to_float(w[e >> 1]) : bf16lo_to_float(w[e >> 1]);
-            const float tm = fmaf(xf[e], s.inv127, kMagic);
-            res[e] = fmaf(kMagic - tm, s.gamma, 127.0f * xf[e]);  // 127 x - q gamma, exact
-            tie = tie || fabsf(res[e]) == s.half_gamma;
-            b[e] = __float_as_uint(tm);
+            for (int e = 0; e < 8; e += 2) {
+                const uint64_t x = pack_f32x2(bf16lo_to_float(w[e >> 1]), bf16hi_to_float(w[e >> 1])), tm = fma_f32x2(x, inv, magic);
+                float t0, t1;
+                unpack_f32x2(tm, t0, t1);
+                b[e] = __float_as_uint(t0);
+                b[e + 1] = __float_as_uint(t1);
+                // 127 x - q gamma, exact (magic - tm = -q is, too)
+                unpack_f32x2(fma_f32x2(fma_f32x2(tm, pack_f32x2(-1.0f, -1.0f), magic), gamma, mul_f32x2(x, pack_f32x2(127.0f, 127.0f))), res[e], res[e + 1]);
+                tie = tie || fabsf(res[e]) == s.half_gamma || fabsf(res[e + 1]) == s.half_gamma;
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) {
+                const float x = (e & 1) ? bf16hi_to_float(w[e >> 1]) : bf16lo_to_float(w[e >> 1]);
+                const float tm = fmaf(x, s.inv127, kMagic);
+                res[e] = fmaf(kMagic - tm, s.gamma, 127.0f * x);  // 127 x - q gamma, exact
+                tie = tie || fabsf(res[e]) == s.half_gamma;
+                b[e] = __float_as_uint(tm);
+            }
         }
         if (tie) {
 #pragma unroll
