@@ -18,11 +18,12 @@
 //   then four or eight warps that stage a problem's activations (one problem ahead where shared memory has the room), H and scales
 // What bounds it is the chain of the MMA issuer.  Stamped on one B200, 36 blocks of 2048, 16 tokens: of 241 thousand clocks in the middle
 // CTA the issuer waits 13 for the first x~, 10 for x~ at changes of problem, 46 for operands and 33 for accumulators that the epilogue
-// still reads; the rest is 360 clocks for the 8 MMAs of a column tile, their commits and loops, where HBM alone would take 330.  The CTAs
-// end 123 to 143 us after the first one's start: shares are cut in 16-row tiles, but a run costs whole blocks of eight.  8 blocks of
+// still reads; the rest is 360 clocks for the 8 MMAs of a column tile, their commits and loops, where HBM alone would take 330.  8 blocks of
 // 4096 on base-3 weights, one token: 199 thousand, 9 for x~, 50 for operands, 7 for accumulators, 490 a column tile of 10 MMAs.
-// Against the warp MMA, one launch with its prologue, 2048-wide blocks with r = 32: 16 tokens, 36 blocks 167 -> 155 us, 2 blocks
-// 31.2 -> 26.2; base-3 weights, 4096-wide, r = 64, one token, 8 blocks 153.5 -> 133; 2048-wide, 8 tokens, 36 blocks 212 -> 165.
+// A run costs whole blocks of eight row tiles, so the shares are cut by them (plan_decode_tc): cut by row tiles the CTAs ended 123 to 143 us
+// after the first one's start, the busiest with 418 column tiles for an even 381, and the groups took 155.4 -> 151.9 and 133.2 -> 121.7 us.
+// Against the warp MMA, one launch with its prologue, 2048-wide blocks with r = 32: 16 tokens, 36 blocks 167 -> 152 us, 2 blocks
+// 31.2 -> 26.2; base-3 weights, 4096-wide, r = 64, one token, 8 blocks 153.5 -> 122; 2048-wide, 8 tokens, 36 blocks 212 -> 165.
 //
 // Two-bit codes: masked in place they are codes times 1, 4, 16 (the fourth position is shifted down by two: 64 times a code
 // would not fit a signed byte), and each scale has an accumulator; the scaled sums are exact multiples.  The order of K

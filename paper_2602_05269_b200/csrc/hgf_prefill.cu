@@ -233,7 +233,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
         // uniform registers: eight MMAs take 230 clocks to issue, a stage 750 with its two barriers.  (One thread in a
         // divergent branch needed 1100, two such threads taking stages in turns 890.)  Large layers are then held by
         // the power limit: 1.75 GHz at 985 W, 8192 x 2048 x 5632 in 122.4 us against 126.1, 4096 x 4096 x 11008 in 201.5
-        // against 209.8; two issuing warps, or asking for the next stage ahead of time, change neither.
+        // against 209.8 (with the swizzled weight tiles of launch_prefill_gemm 118.6 and 194); two issuing warps, or asking for the next stage ahead of time, change neither.
         {
             auto wait = [&](int i, uint32_t par, unsigned int code) { return __all_sync(0xffffffffu, mbar_wait_poll(bar(i), par, abort_flag, status, code)) != 0; };
             bool ok = true;
