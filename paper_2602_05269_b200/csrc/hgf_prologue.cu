@@ -663,7 +663,7 @@ static cudaLaunchConfig_t prologue_cfg(int blocks, bool pdl, cudaStream_t stream
 constexpr int kRpSmemLimit = 200 * 1024;
 
 // ---- GEMM-path prologue in one kernel -------------------------------------------------------------
-// Quantisation (Algorithm 1, steps 1-2) and the LoRA down-projection (steps 5-6) of a block of 32
+// Quantisation (Algorithm 1, steps 1-2) and the LoRA down-projection (steps 5-6) of a block of TOK
 // tokens, reading x from HBM once.  First pass: x and the rows of A^T travel through a three-stage
 // ring of 256-column chunks (16-byte asynchronous copies); every warp takes 32 columns of a chunk,
 // feeds them to the tf32 MMA (tokens are the 16-row operand, 8 columns of H the 8-column operand;
@@ -671,16 +671,21 @@ constexpr int kRpSmemLimit = 200 * 1024;
 // lane's registers on the way, keeps the running maximum of |x| of its rows.  Then the warps' partial
 // sums of x A are added in a fixed order, and the block's rows - still in L2 - are read again and
 // rounded with the now known scales.  JT = r / 8 column tiles of H; JT = 0 quantises only.
-constexpr int kFpThreads = 256;
-constexpr int kFpWarps = kFpThreads / 32;
-constexpr int kFpTokens = 32;
+// W: eight warps of two token tiles each, two blocks an SM; from rank 48 on, where a block's ring takes an SM's shared memory, sixteen
+// warps (the second eight take every other token tile), so that the MMA and its conversions have as many warps there.  Layer calls,
+// eight / sixteen: r = 64, 6144 -> 1024 at M = 6000 119.1 / 115.5 us, 4096 -> 1024 with a LayerNorm at M = 8192 131.5 / 128.9, 1024 -> 1024 at M = 4000
+// 23.3 / 21.2, 512 -> 512 at M = 300 11.7 / 10.75; r = 48, 512 -> 1024 at M = 4736 19.4 / 17.6, 768 -> 768 at M = 700 12.4 / 11.5.  Ranks up to 32 have sixteen warps
+// an SM as it is and are bound by the MMA's rate: with 32 warps 2048 -> 5632 at M = 8192 117.9 / 119.6, 5632 -> 2048 135.0 / 140.4.
+// TOK: 64 tokens a block halve the reads of A^T and need fewer rounds; that is worth it at rank 48 beyond one round of 32 tokens
+// (3072 -> 1024 at M = 5000 58.0 / 50.0 us, 1024 -> 512 at M = 16384 53.1 / 47.8).  Rank 64 would spill at 128 registers (6144 -> 1024 at M = 6000
+// 115.5 / 133.1), for ranks up to 32 it is the same time (2048 -> 5632 at M = 8192 118.6 / 119.3).
+constexpr int kFpWarps = 8;                          // warps that share a chunk's columns
 constexpr int kFpChunk = 256;                        // columns per stage
 constexpr int kFpPitch = kFpChunk * 2 + 64;          // bytes per staged row: neighbouring rows on the other 16 banks
 constexpr int kFpStages = 3;
-__host__ __device__ constexpr int fp_stage_bytes(int r) { return (kFpTokens + r) * kFpPitch; }
-__host__ __device__ constexpr int fp_smem_bytes(int r) {
-    return kFpStages * fp_stage_bytes(r) > kFpWarps * kFpTokens * r * 4 ? kFpStages * fp_stage_bytes(r)
-                                                                         : kFpWarps * kFpTokens * r * 4;
+__host__ __device__ constexpr int fp_stage_bytes(int tokens, int r) { return (tokens + r) * kFpPitch; }
+__host__ __device__ constexpr int fp_smem_bytes(int tokens, int r) {
+    return kFpStages * fp_stage_bytes(tokens, r) > kFpWarps * tokens * r * 4 ? kFpStages * fp_stage_bytes(tokens, r) : kFpWarps * tokens * r * 4;
 }
 
 // The up-projection's operand: row n of B^T times its channel's gate, fp16, padded to 64 columns; piece `idx` is 16 bytes.
@@ -701,65 +706,59 @@ __device__ __forceinline__ void gate_operand(const GemmPrologueExtra &x, int r, 
     *reinterpret_cast<uint4 *>(x.gb16 + (size_t)n * 64 + c * 8) = v;
 }
 
-template <int JT>
-__global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x) {
+template <int JT, int W, int TOK>
+__global__ void __launch_bounds__(32 * W, 1) gemm_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x) {
     extern __shared__ __align__(128) uint8_t fp_smem[];
-    __shared__ float s_amax[kFpWarps][kFpTokens];
-    __shared__ float s_gamma[kFpTokens];
+    constexpr int THREADS = 32 * W, SETS = W / kFpWarps, TILES = TOK / 16 / SETS;  // (token tiles a warp)
+    __shared__ float s_amax[kFpWarps][TOK];
+    __shared__ float s_gamma[TOK];
     constexpr int r = 8 * JT;
     pdl_wait();  // x, and the workspace this kernel overwrites, belong to earlier work
-    const int tpb = x.tokens_per_block;  // tokens this launch gives a block (at most kFpTokens)
+    const int tpb = x.tokens_per_block;  // tokens this launch gives a block (at most TOK)
     const int token_blocks = (p.M + tpb - 1) / tpb;
     if ((int)blockIdx.x >= token_blocks) {
         // the remaining blocks prepare the up-projection's operand
         if constexpr (JT > 0) {
-            gate_operand(x, r, ((int)blockIdx.x - token_blocks) * kFpThreads + (int)threadIdx.x);
+            gate_operand(x, r, ((int)blockIdx.x - token_blocks) * THREADS + (int)threadIdx.x);
         }
         return;
     }
     const int K = p.K, M = p.M;
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, g = lane >> 2, t = lane & 3;
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5, part = warp % kFpWarps, mt0 = warp / kFpWarps, g = lane >> 2, t = lane & 3;
     const int m0 = blockIdx.x * tpb;
     const uint32_t smem_u32 = (uint32_t)__cvta_generic_to_shared(fp_smem);
-    constexpr int kStage = fp_stage_bytes(r);
+    constexpr int kStage = fp_stage_bytes(TOK, r);
     const int nchunks = (K + kFpChunk - 1) / kFpChunk;
 
-    // One chunk into one stage: 32 (+ r) rows of 32 16-byte units; rows past M and columns past K are
-    // zeros.  A thread copies unit `lane` of rows warp, warp + 8, ...: the same ones in every chunk.
-    constexpr int kRowsPerThread = (kFpTokens + r) / kFpWarps;
-    const uint8_t *src_row[kRowsPerThread];
-    bool row_ok[kRowsPerThread];
-#pragma unroll
-    for (int q = 0; q < kRowsPerThread; ++q) {
-        const int row = warp + kFpWarps * q;
-        if (row < kFpTokens) {
-            row_ok[q] = row < tpb && m0 + row < M;
-            src_row[q] = reinterpret_cast<const uint8_t *>(p.x + (size_t)(row_ok[q] ? m0 + row : 0) * K) + 16 * lane;
-        } else {
-            row_ok[q] = true;
-            src_row[q] = reinterpret_cast<const uint8_t *>(p.At + (size_t)(row - kFpTokens) * K) + 16 * lane;
-        }
-    }
+    // One chunk into one stage: TOK (+ r) rows of 32 16-byte units; rows past M and columns past K are
+    // zeros.  A thread copies unit `lane` of rows warp, warp + W, ... (tokens first: TOK and r are multiples of 16): the same
+    // ones in every chunk.
+    constexpr int kRowsPerThread = (TOK + r) / W;
+    const uint8_t *src_x = reinterpret_cast<const uint8_t *>(p.x + (size_t)(m0 + warp) * K) + 16 * lane;
+    const uint8_t *src_a = JT > 0 ? reinterpret_cast<const uint8_t *>(p.At + (size_t)warp * K) + 16 * lane : nullptr;
+    const int rows_x = M - m0 < tpb ? M - m0 : tpb;
     auto fetch = [&](int c, int stage) {
         const uint32_t dst = smem_u32 + stage * kStage + warp * kFpPitch + 16 * lane;
         const int k = c * kFpChunk + 8 * lane;
         const bool col_ok = k < K;
 #pragma unroll
         for (int q = 0; q < kRowsPerThread; ++q) {
-            const bool in = col_ok && row_ok[q];
-            cp_async_16(dst + q * kFpWarps * kFpPitch, src_row[q] + (in ? (size_t)c * kFpChunk * 2 : 0), in ? 16u : 0u);
+            constexpr int kTokenRows = TOK / W;
+            const bool token = q < kTokenRows, in = col_ok && (!token || warp + W * q < rows_x);
+            const uint8_t *src = token ? src_x + (size_t)(q * W) * K * 2 : src_a + (size_t)((q - kTokenRows) * W) * K * 2;
+            cp_async_16(dst + q * W * kFpPitch, in ? src + (size_t)c * kFpChunk * 2 : reinterpret_cast<const uint8_t *>(p.x), in ? 16u : 0u);
         }
         asm volatile("cp.async.commit_group;\n" ::: "memory");
     };
 
-    float acc[2][JT > 0 ? JT : 1][4];
+    float acc[TILES][JT > 0 ? JT : 1][4];
 #pragma unroll
-    for (int a = 0; a < 2; ++a)
+    for (int a = 0; a < TILES; ++a)
 #pragma unroll
         for (int b = 0; b < (JT > 0 ? JT : 1); ++b)
 #pragma unroll
             for (int c = 0; c < 4; ++c) acc[a][b][c] = 0.0f;
-    uint32_t amax[2][2] = {{0u, 0u}, {0u, 0u}};  // rows 16 mt + 8 hh + g, packed maxima of the bit patterns
+    uint32_t amax[TILES][2] = {};  // rows 16 mt + 8 hh + g, packed maxima of the bit patterns
 
 #pragma unroll
     for (int sg = 0; sg < kFpStages - 1; ++sg) {
@@ -772,13 +771,14 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
         if (c + kFpStages - 1 < nchunks) fetch(c + kFpStages - 1, (c + kFpStages - 1) % kFpStages);
         else asm volatile("cp.async.commit_group;\n" ::: "memory");
 
-        const uint32_t st = smem_u32 + (c % kFpStages) * kStage + 64 * warp + 16 * t;
+        const uint32_t st = smem_u32 + (c % kFpStages) * kStage + 64 * part + 16 * t;
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt) {
+        for (int i_mt = 0; i_mt < TILES; ++i_mt) {
+            const int mt = mt0 + SETS * i_mt;
             if (16 * mt >= tpb) break;  // a block of up to 16 tokens has no second tile
             const uint4 x0 = pg_lds_u4(st + (16 * mt + g) * kFpPitch), x1 = pg_lds_u4(st + (16 * mt + 8 + g) * kFpPitch);
-            amax[mt][0] = absmax8_bits(amax[mt][0], x0);
-            amax[mt][1] = absmax8_bits(amax[mt][1], x1);
+            amax[i_mt][0] = absmax8_bits(amax[i_mt][0], x0);
+            amax[i_mt][1] = absmax8_bits(amax[i_mt][1], x1);
             if constexpr (JT > 0) {
                 // elements 2 i and 2 i + 1 of this lane's eight take the k slots t and t + 4 of MMA i
                 uint32_t xs[4][4];
@@ -789,11 +789,11 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
                 }
 #pragma unroll
                 for (int jt = 0; jt < JT; ++jt) {
-                    const uint4 a4 = pg_lds_u4(st + (kFpTokens + 8 * jt + g) * kFpPitch);
+                    const uint4 a4 = pg_lds_u4(st + (TOK + 8 * jt + g) * kFpPitch);
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const float2 bf = __half22float2(*reinterpret_cast<const __half2 *>(&(&a4.x)[i]));
-                        mma_tf32(acc[mt][jt], xs[i][0], xs[i][1], xs[i][2], xs[i][3], __float_as_uint(bf.x), __float_as_uint(bf.y));
+                        mma_tf32(acc[i_mt][jt], xs[i][0], xs[i][1], xs[i][2], xs[i][3], __float_as_uint(bf.x), __float_as_uint(bf.y));
                     }
                 }
             }
@@ -803,16 +803,16 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
 
     // the rows' maxima: over the four lanes that share a row, then over the warps
 #pragma unroll
-    for (int mt = 0; mt < 2; ++mt)
+    for (int mt = 0; mt < TILES; ++mt)
 #pragma unroll
         for (int hh = 0; hh < 2; ++hh) {
             float a = absmax_bits_to_float(amax[mt][hh]);
             a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 1));
             a = fmaxf(a, __shfl_xor_sync(0xffffffffu, a, 2));
-            if (t == 0) s_amax[warp][16 * mt + 8 * hh + g] = a;
+            if (t == 0) s_amax[part][16 * (mt0 + SETS * mt) + 8 * hh + g] = a;
         }
     __syncthreads();  // also: every warp is done with the ring, which the partial sums now reuse
-    if (tid < kFpTokens) {
+    if (tid < TOK) {
         float a = s_amax[0][tid];
 #pragma unroll
         for (int w = 1; w < kFpWarps; ++w) a = fmaxf(a, s_amax[w][tid]);
@@ -821,10 +821,10 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
     if constexpr (JT > 0) {
         float *s_acc = reinterpret_cast<float *>(fp_smem);  // [warps][32 tokens][r]
 #pragma unroll
-        for (int mt = 0; mt < 2; ++mt)
+        for (int mt = 0; mt < TILES; ++mt)
 #pragma unroll
             for (int jt = 0; jt < JT; ++jt) {
-                float *base = s_acc + ((size_t)warp * kFpTokens + 16 * mt) * r + 8 * jt;
+                float *base = s_acc + ((size_t)part * TOK + 16 * (mt0 + SETS * mt)) * r + 8 * jt;
                 base[g * r + 2 * t] = acc[mt][jt][0];
                 base[g * r + 2 * t + 1] = acc[mt][jt][1];
                 base[(g + 8) * r + 2 * t] = acc[mt][jt][2];
@@ -834,11 +834,11 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
     __syncthreads();
     if constexpr (JT > 0) {
         const float *s_acc = reinterpret_cast<const float *>(fp_smem);
-        for (int e = tid; e < kFpTokens * r; e += kFpThreads) {
+        for (int e = tid; e < TOK * r; e += THREADS) {
             const int ml = e / r, j = e % r, m = m0 + ml;
             float z = 0.0f;
 #pragma unroll
-            for (int w = 0; w < kFpWarps; ++w) z += s_acc[w * kFpTokens * r + e];
+            for (int w = 0; w < kFpWarps; ++w) z += s_acc[w * TOK * r + e];
             const float h = (p.flags & HGF_FLAG_NO_SILU) ? z : silu_f(z);
             if (ml < tpb && m < M) {
                 p.h[(size_t)m * r + j] = h;
@@ -848,7 +848,7 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
         }
         if constexpr (JT < 8) {  // zero padding of the fp16 copy up to 64 columns
             if (p.h16)
-                for (int e = tid; e < kFpTokens * (64 - r); e += kFpThreads) {
+                for (int e = tid; e < TOK * (64 - r); e += THREADS) {
                     const int ml = e / (64 - r), j = r + e % (64 - r), m = m0 + ml;
                     if (ml < tpb && m < M) p.h16[(size_t)m * 64 + j] = __float2half_rn(0.0f);
                 }
@@ -871,11 +871,11 @@ __global__ void __launch_bounds__(kFpThreads) gemm_prologue_kernel(const Prologu
         return;
     }
 
-    // second pass: the warps round the block's rows, warp w rows w, w + 8, ...
+    // second pass: the warps round the block's rows, warp w rows w, w + W, ...
     const int nv = K / 8;
 #pragma unroll 1
-    for (int rr = 0; rr < kFpTokens / kFpWarps; ++rr) {
-        const int ml = warp + kFpWarps * rr, m = m0 + ml;
+    for (int rr = 0; rr < TOK / W; ++rr) {
+        const int ml = warp + W * rr, m = m0 + ml;
         if (ml >= tpb || m >= M) break;
         const float gm = s_gamma[ml];
         const QuantScale qs = make_quant_scale(gm);
@@ -1280,22 +1280,22 @@ static cudaError_t launch_rows_prologue_jt(const PrologueParams &p, const GemmPr
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
-template <int JT>
+template <int JT, int W, int TOK>
 static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPrologueExtra &x, int blocks, cudaStream_t stream) {
     // Never more than two blocks per SM (the launcher spreads the rows over twice the SM count of
-    // blocks): blocks that start as SMs come free at the tail of the preceding launch would otherwise
+    // blocks, from rank 48 on one): blocks that start as SMs come free at the tail of the preceding launch would otherwise
     // pile up four to an SM on the first SMs free and leave the others idle.
-    constexpr int smem = fp_smem_bytes(8 * JT) > 80 * 1024 ? fp_smem_bytes(8 * JT) : 80 * 1024;
+    constexpr int smem = fp_smem_bytes(TOK, 8 * JT) > 80 * 1024 ? fp_smem_bytes(TOK, 8 * JT) : 80 * 1024;
     static std::atomic<unsigned long long> attr_done{0};
     {
-        cudaError_t e = ensure_dynamic_smem(gemm_prologue_kernel<JT>, smem, attr_done);
+        cudaError_t e = ensure_dynamic_smem(gemm_prologue_kernel<JT, W, TOK>, smem, attr_done);
         if (e != cudaSuccess) return e;
     }
     cudaLaunchAttribute attr[1];
     cudaLaunchConfig_t cfg = prologue_cfg(blocks, !(p.flags & HGF_FLAG_NO_PDL), stream, attr);
-    cfg.blockDim = dim3(kFpThreads);
+    cfg.blockDim = dim3(32 * W);
     cfg.dynamicSmemBytes = smem;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_prologue_kernel<JT>, p, x);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, gemm_prologue_kernel<JT, W, TOK>, p, x);
     return e != cudaSuccess ? e : cudaGetLastError();
 }
 
@@ -1393,13 +1393,15 @@ cudaError_t launch_gemm_prologue(const PrologueParams &p, const GemmPrologueExtr
         if (e != cudaErrorNotSupported) return e;
     }
     // Tokens per block: as many blocks as are resident at once share the rows evenly; beyond that a
-    // block takes its full 32.
+    // block takes its full 32 (rank 48: as many rounds as blocks of 64 need, evenly; see the kernel).
     const int sm_count = device_sm_count();
     if (!sm_count) return cudaErrorInvalidDevice;
-    const int per_sm = p.r >= 48 ? 1 : 2;  // blocks that fit an SM (shared memory: 138 KB and more from rank 48 on)
-    int tpb = (p.M + per_sm * sm_count - 1) / (per_sm * sm_count);
+    const bool wide = p.r >= 48, big = p.r == 48 && p.M > 32 * sm_count;
+    const int per_sm = wide ? 1 : 2, most = big ? 64 : 32;  // blocks that fit an SM (shared memory: 138 KB and more from rank 48 on)
+    const int rounds = big ? (p.M + 64 * sm_count - 1) / (64 * sm_count) : 1, shares = per_sm * sm_count * rounds;
+    int tpb = (p.M + shares - 1) / shares;
     tpb = (tpb + 3) / 4 * 4;
-    tpb = tpb < 8 ? 8 : (tpb > kFpTokens ? kFpTokens : tpb);
+    tpb = tpb < 8 ? 8 : (tpb > most ? most : tpb);
     GemmPrologueExtra xx = x;
     xx.tokens_per_block = tpb;
     // The rounding pass as a second launch where there is enough of x to pay for a launch: it then runs at twice
@@ -1407,14 +1409,15 @@ cudaError_t launch_gemm_prologue(const PrologueParams &p, const GemmPrologueExtr
     // K = 2048, 141.3 -> 134.3 us at K = 5632; M = 4096: 209.7 -> 205.1 us at K = 11008, unchanged at K = 4096).
     const size_t x_bytes = (size_t)p.M * p.K * 2;
     xx.split_round = (p.xq && p.r > 0 && x_bytes >= ((size_t)8 << 20)) ? 1 : 0;
-    const int blocks = (p.M + tpb - 1) / tpb + ((p.r > 0 && x.gb16) ? (x.N * 8 + kFpThreads - 1) / kFpThreads : 0);
+    const int threads = wide ? 512 : 256;
+    const int blocks = (p.M + tpb - 1) / tpb + ((p.r > 0 && x.gb16) ? (x.N * 8 + threads - 1) / threads : 0);
     cudaError_t e;
     switch (p.r) {
-        case 0: e = launch_gemm_prologue_jt<0>(p, xx, blocks, stream); break;
-        case 16: e = launch_gemm_prologue_jt<2>(p, xx, blocks, stream); break;
-        case 32: e = launch_gemm_prologue_jt<4>(p, xx, blocks, stream); break;
-        case 48: e = launch_gemm_prologue_jt<6>(p, xx, blocks, stream); break;
-        case 64: e = launch_gemm_prologue_jt<8>(p, xx, blocks, stream); break;
+        case 0: e = launch_gemm_prologue_jt<0, 8, 32>(p, xx, blocks, stream); break;
+        case 16: e = launch_gemm_prologue_jt<2, 8, 32>(p, xx, blocks, stream); break;
+        case 32: e = launch_gemm_prologue_jt<4, 8, 32>(p, xx, blocks, stream); break;
+        case 48: e = big ? launch_gemm_prologue_jt<6, 16, 64>(p, xx, blocks, stream) : launch_gemm_prologue_jt<6, 16, 32>(p, xx, blocks, stream); break;
+        case 64: e = launch_gemm_prologue_jt<8, 16, 32>(p, xx, blocks, stream); break;
         default: return cudaErrorInvalidValue;
     }
     count_launch();
@@ -1442,7 +1445,7 @@ cudaError_t launch_quant(const PrologueParams &p, const GemmPrologueExtra &x, cu
         cudaLaunchConfig_t cfg = prologue_cfg(row_blocks, !(p.flags & HGF_FLAG_NO_PDL), stream, attr);
         cudaError_t e = cudaLaunchKernelEx(&cfg, quant_rows_kernel<16>, p, x);
         if (e != cudaSuccess) return e;
-    } else if (p.M >= 2 * kFpTokens) {
+    } else if (p.M >= 64) {
         PrologueParams q = p;
         q.r = 0;
         return launch_gemm_prologue(q, x, stream);
