@@ -457,14 +457,14 @@ def run_ours(args):
 # DRAM traffic of the decode GEMV launch from one ncu capture (dram__bytes_read.sum + dram__bytes_write.sum
 # of a config-1, M = 1 group launch): bytes moved per algorithmic byte.  It is only reported while the
 # kernel source is the one that was captured.
-DECODE_TRAFFIC = {"source_sha1": "44eb0003e0499940df9fd74a941b599545d6a00d",
-                  "dram_bytes_per_algorithmic_byte": (517.350656e6 + 5.821696e6) / 518805504.0}
+DECODE_TRAFFIC = {"source_sha1": "bb299d90944092f2d46485e50576d12d0bd16fed",
+                  "dram_bytes_per_algorithmic_byte": (517.360128e6 + 5.661952e6) / 518805504.0}
 
 
 # DRAM traffic of the prefill GEMM launch from one ncu capture of the very shape the bench times
 # (2048 -> 5632, r = 32, M = 8192, bf16 y): dram__bytes_read.sum + dram__bytes_write.sum of one launch.  Below
 # the launch's algorithmic bytes because most of y is still in L2 when the kernel ends.
-PREFILL_TRAFFIC = {"source_sha1": "d63d4d700369fb6bb26571622ae28e0b0029d6fc", "dram_bytes_per_launch": 21.574912e6 + 43.079680e6}
+PREFILL_TRAFFIC = {"source_sha1": "a767dc2ba520744b4e1bc2bf911cd245bc5d128e", "dram_bytes_per_launch": 21.575168e6 + 43.553024e6}
 
 
 def prefill_traffic():
