@@ -18,9 +18,12 @@ struct AbsScratch {
 
 // mean |W| into s->gamma.  Per-block sums in double (fixed grid-stride order, fixed tree), then the block that
 // finishes last adds the partials with one warp (lane-strided, then a fixed shuffle tree) and rounds the mean
-// once to fp32: the same order every time, whichever block is last.  13.7 us for 2048 x 5632, where HBM needs 7 (4 bytes per weight):
-// the rest is the start and the end of the launch.  As long as the sums and their addition took as two launches (11.1 + 2.5 us);
+// once to fp32: the same order every time, whichever block is last.  As long as the sums and their addition took as two launches;
 // what a packing call gained came from its scratch (below).  Four 16-byte loads in flight per thread, added in index order.
+// What is beyond the bytes (5632 x 2048: 13.7 us where HBM needs 7) is the chain at either end: a thread's last loads, the partial sums
+// of the last block and the start of the packing kernel were each waited for in turn.  Asked for together, and the packing kernel let in
+// when the weights are read: whole calls, host to host, 5632 x 2048 51.3 -> 44.8 us, 1000 x 2048 40.4 -> 37.6, 333 x 1088 40.3 -> 32.7, 11008 x 4096
+// 93.7 -> 91.8; 2048 x 2048 and 4096 x 4096, with no last loads, as before.  A training step of 64 x 512 -> 512 71.5 -> 64.7, 512 x 2048 -> 2048 112.6 -> 107.
 __global__ void __launch_bounds__(kAbsThreads) abs_mean_kernel(const float4 *W4, size_t n4, double count, AbsScratch *s) {
     double acc = 0.0;
     const size_t stride = (size_t)gridDim.x * kAbsThreads;
@@ -30,8 +33,14 @@ __global__ void __launch_bounds__(kAbsThreads) abs_mean_kernel(const float4 *W4,
         const float4 v0 = W4[i], v1 = W4[i + stride], v2 = W4[i + 2 * stride], v3 = W4[i + 3 * stride];
         add(v0); add(v1); add(v2); add(v3);
     }
-    for (; i < n4; i += stride) add(W4[i]);
-    __shared__ double red[kAbsThreads];
+    float4 rest[3];  // (fewer than four left: asked for together, too)
+#pragma unroll
+    for (int u = 0; u < 3; ++u) rest[u] = i + u * stride < n4 ? W4[i + u * stride] : make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+#pragma unroll
+    for (int u = 0; u < 3; ++u)
+        if (i + u * stride < n4) add(rest[u]);
+    pdl_launch_dependents();  // the packing kernel may ask for its weights
+    __shared__ double red[kAbsBlocks];
     __shared__ bool last;
     red[threadIdx.x] = acc;
     __syncthreads();
@@ -45,11 +54,15 @@ __global__ void __launch_bounds__(kAbsThreads) abs_mean_kernel(const float4 *W4,
         last = atomicAdd(&s->done, 1u) + 1u == gridDim.x;
     }
     __syncthreads();
-    if (!last || threadIdx.x >= 32) return;
+    if (!last) return;
     __threadfence();
+#pragma unroll
+    for (int k = 0; k < kAbsBlocks; k += kAbsThreads) red[k + threadIdx.x] = __ldcg(&s->partials[k + threadIdx.x]);
+    __syncthreads();
+    if (threadIdx.x >= 32) return;
     double sum = 0.0;
 #pragma unroll 8
-    for (int k = threadIdx.x; k < kAbsBlocks; k += 32) sum += __ldcg(&s->partials[k]);
+    for (int k = threadIdx.x; k < kAbsBlocks; k += 32) sum += red[k];
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
     if (threadIdx.x == 0) {
@@ -72,30 +85,36 @@ __device__ __forceinline__ WordPos word_pos(size_t w, int64_t steps) {
     return p;
 }
 
-// One thread per 32-bit packed word (16 weights).  Weight k0 + 4 j + b goes to bits
+// Sixteen lanes a row of a tile, 16 words of 16 weights.  Weight k0 + 4 j + b goes to bits
 // 8 b + 2 j of the word; code = t + 1; t = sign(w) * [|w| > gamma/2].  Padding words hold code 1.
+// Lane l asks for the 16 bytes l, l + 16, l + 32, l + 48 of the row, neighbours next to each other, before it waits for the scale;
+// four lanes have the quarters of a word.  (A word a lane, 64 bytes apart, left the reading to the L1's tag look-ups.)
 __global__ void __launch_bounds__(256) ternarise_pack_kernel(const float *W, int64_t N, int64_t K, int64_t steps,
-                                                             size_t n_words, const float *gamma, uint32_t *packed) {
-    size_t w = (size_t)blockIdx.x * 256 + threadIdx.x;
-    if (w >= n_words) return;
-    const WordPos p = word_pos(w, steps);
-    uint32_t word = 0x55555555u;
-    if (p.n < N && p.k0 < K) {
-        const float half = 0.5f * *gamma;  // exact
-        const float4 *src = reinterpret_cast<const float4 *>(W + p.n * K + p.k0);
-        word = 0;
+                                                             const float *gamma, uint32_t *packed) {
+    const size_t w = (size_t)blockIdx.x * 256 + threadIdx.x;  // (a block is a tile)
+    const int l = threadIdx.x & 15;
+    const WordPos p = word_pos(w - l, steps);
+    float4 v[4];
 #pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float4 v = src[j];
-            float e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-            for (int b = 0; b < 4; ++b) {
-                uint32_t c = e[b] > half ? 2u : (e[b] < -half ? 0u : 1u);
-                word |= c << (8 * b + 2 * j);
-            }
-        }
+    for (int i = 0; i < 4; ++i) {
+        const int64_t k = p.k0 + 64 * i + 4 * l;
+        v[i] = p.n < N && k < K ? *reinterpret_cast<const float4 *>(W + p.n * K + k) : make_float4(0.0f, 0.0f, 0.0f, 0.0f);  // (0: code 1)
     }
-    packed[w] = word;
+    pdl_wait();
+    const float half = 0.5f * __ldcg(gamma);  // exact
+    uint32_t mine = 0u;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const float e[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        uint32_t word = 0u;
+#pragma unroll
+        for (int b = 0; b < 4; ++b) word |= (e[b] > half ? 2u : (e[b] < -half ? 0u : 1u)) << (8 * b);
+        word <<= 2 * (l & 3);
+        word |= __shfl_xor_sync(0xffffffffu, word, 1);
+        word |= __shfl_xor_sync(0xffffffffu, word, 2);
+        if ((l & 3) == i) mine = word;
+    }
+    packed[w - l + 4 * (l & 3) + (l >> 2)] = mine;
 }
 
 __global__ void __launch_bounds__(256) unpack_kernel(const uint32_t *packed, int64_t N, int64_t K, int64_t steps,
@@ -300,12 +319,12 @@ static hgf_status pack_with_scale(const float *W, int64_t d_out, int64_t d_in, f
     if (!scratch.p) return HGF_ERR_CUDA;
     const size_t n = (size_t)d_out * (size_t)d_in;
     abs_mean_kernel<<<kAbsBlocks, kAbsThreads, 0, stream>>>((const float4 *)W, n / 4, (double)n, scratch.p);
-    pack(&scratch.p->gamma);
+    const cudaError_t e0 = pack(&scratch.p->gamma);
     count_launch(2);
     cudaError_t e = cudaMemcpyAsync(gamma_out, &scratch.p->gamma, sizeof(float), cudaMemcpyDeviceToHost, stream);
     const cudaError_t e1 = cudaStreamSynchronize(stream);  // also after a failed copy: the slot must be idle
     const cudaError_t e2 = cudaGetLastError();
-    return (e == cudaSuccess && e1 == cudaSuccess && e2 == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
+    return (e0 == cudaSuccess && e == cudaSuccess && e1 == cudaSuccess && e2 == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
 }
 
 }  // namespace hgf
@@ -328,6 +347,7 @@ extern "C" hgf_status hgf_pack_ternary_b3(const float *W, int64_t d_out, int64_t
     return pack_with_scale(W, d_out, d_in, gamma_out, stream, [&](const float *gamma) {
         ternarise_pack_b3_kernel<<<(unsigned)((n_bytes + 255) / 256), 256, 0, stream>>>(W, d_out, d_in, steps, n_bytes, gamma,
                                                                                         (uint8_t *)packed);
+        return cudaGetLastError();
     });
 }
 
@@ -355,8 +375,16 @@ extern "C" hgf_status hgf_pack_ternary(const float *W, int64_t d_out, int64_t d_
     const int64_t steps = padded_k(d_in) / 256;
     const size_t n_words = (size_t)row_tiles(d_out) * (size_t)steps * 256;
     return pack_with_scale(W, d_out, d_in, gamma_out, stream, [&](const float *gamma) {
-        ternarise_pack_kernel<<<(unsigned)((n_words + 255) / 256), 256, 0, stream>>>(W, d_out, d_in, steps, n_words, gamma,
-                                                                                     (uint32_t *)packed);
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // (after the scale's kernel alone, which starts when all work before it is done)
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3((unsigned)(n_words / 256));
+        cfg.blockDim = dim3(256);
+        cfg.stream = stream;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, ternarise_pack_kernel, W, d_out, d_in, steps, gamma, (uint32_t *)packed);
     });
 }
 
