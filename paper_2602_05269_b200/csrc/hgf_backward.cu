@@ -8,6 +8,7 @@
 // quantiser again, its codes times their scale), the ternary codes as a bf16 matrix of exact -1 / 0 / +1, A and
 // g (.) B in bf16.  gamma_W is applied to the fp32 accumulator.
 #include <algorithm>
+#include <vector>
 
 #include "hgf_tc.cuh"
 #include "hgf_warp.cuh"
@@ -766,26 +767,39 @@ extern "C" int hgf_internal_tc_deal_thin(const int32_t *I, const int32_t *Cn, in
     return ride ? 1 : 0;
 }
 
+// (for the tests) What a pass does with its room for partial sums, in the order of its launches, of which none is enqueued.
+struct BwTrace {
+    int sms, pairs;
+    const float *room;
+    struct Use { bool write; int64_t first, end; };
+    std::vector<Use> uses;
+    struct Rides { bool dx; int n, n_half, c_idle, c_busy; };
+    std::vector<Rides> rides;  // of each launch by pairs
+    void use(bool write, const float *p, size_t n) { uses.push_back({write, p - room, p - room + (int64_t)n}); }
+};
+
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
 // operand forms.  `partials` (splits_max * I * ldc floats) enables splitting the contraction when the
 // output has fewer tiles than the device has SMs; ldc must then be J.  With `splits_out` they are left there for the kernel that
 // reads the product next (*splits_out of them; 1: the product is in C).  `thin`: products that may ride in a launch by pairs; `splits` is 0
 // afterwards for those that did not.  Bases 16-byte aligned, ld % 8 == 0.
 static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J,
-                           float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, TcThinProduct *thin, int n_thin, cudaStream_t stream) {
-    const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64), sms = device_sm_count();
+                           float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, TcThinProduct *thin, int n_thin, cudaStream_t stream, BwTrace *trace) {
+    const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64), sms = trace ? trace->sms : device_sm_count();
     const int kb1 = (Cn + kTBK - 1) / kTBK, kb2 = A2.p ? (Cn2 + kTBK - 1) / kTBK : 0, kb_all = kb1 + kb2;
-    int pairs = I > kTBM && J > 128 && kb_all >= kTpMinBlocks && sms > 0 ? tc_pairs_at_once() : 0;
+    int pairs = I > kTBM && J > 128 && kb_all >= kTpMinBlocks && sms > 0 ? (trace ? trace->pairs : tc_pairs_at_once()) : 0;
     if (!tc_pairs_pay(I, J, kb_all, B.mn, sms, pairs)) pairs = 0;
     CUtensorMap maps[4];
     const int rows_b = pairs ? 128 : BN;
     TcGemmArgs g = {};
-    if (!tc_map(&maps[0], A, I, Cn, kTBM, &g.a_mn) || !tc_map(&maps[1], B, J, Cn, rows_b, &g.b_mn)) return cudaErrorInvalidValue;
-    maps[2] = maps[0];
-    maps[3] = maps[1];
-    int form_a = g.a_mn, form_b = g.b_mn;  // (by the extents I and J and the row pitches' alignment: alike for both pairs)
-    if (A2.p && (!tc_map(&maps[2], A2, I, Cn2, kTBM, &form_a) || !tc_map(&maps[3], B2, J, Cn2, rows_b, &form_b))) return cudaErrorInvalidValue;
-    if (form_a != g.a_mn || form_b != g.b_mn) return cudaErrorInvalidValue;
+    if (!trace) {
+        if (!tc_map(&maps[0], A, I, Cn, kTBM, &g.a_mn) || !tc_map(&maps[1], B, J, Cn, rows_b, &g.b_mn)) return cudaErrorInvalidValue;
+        maps[2] = maps[0];
+        maps[3] = maps[1];
+        int form_a = g.a_mn, form_b = g.b_mn;  // (by the extents I and J and the row pitches' alignment: alike for both pairs)
+        if (A2.p && (!tc_map(&maps[2], A2, I, Cn2, kTBM, &form_a) || !tc_map(&maps[3], B2, J, Cn2, rows_b, &form_b))) return cudaErrorInvalidValue;
+        if (form_a != g.a_mn || form_b != g.b_mn) return cudaErrorInvalidValue;
+    }
     g.I = I; g.J = J; g.ldc = ldc;
     g.kb1 = kb1;
     g.kb2 = kb2;
@@ -799,6 +813,14 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
         TcThinArgs t = {};
         TcThinMaps thin_maps;
         if (n_thin && !tc_deal_thin(&t, thin, n_thin, work, g.n_half, kb_all, pairs)) n_thin = 0;
+        if (trace) {
+            for (int i = 0; i < n_thin; ++i) {
+                thin[i].splits = t.job[i].splits;
+                trace->use(true, thin[i].P, (size_t)thin[i].splits * thin[i].I * thin[i].J);
+            }
+            trace->rides.push_back({!A.mn, n_thin, g.n_half, t.c_idle, t.c_busy});
+            return cudaSuccess;
+        }
         for (int i = 0; i < kTcThinMax; ++i) {
             thin_maps.a[i] = maps[0];
             thin_maps.b[i] = maps[1];
@@ -831,10 +853,15 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
     } else {
         g.C = partials; g.alpha = 1.0f; g.accumulate = 0;
     }
-    cudaError_t e = BN == 256 ? tc_gemm_bn<256>(maps, g, stream) : (BN == 128 ? tc_gemm_bn<128>(maps, g, stream) : tc_gemm_bn<64>(maps, g, stream));
     if (splits_out) *splits_out = g.splits;  // the caller adds the partial sums
-    if (e != cudaSuccess || g.splits == 1 || splits_out) return e;
     const size_t n4 = (size_t)I * J / 4;
+    if (trace) {
+        if (g.splits > 1) trace->use(true, partials, 4 * n4 * g.splits);
+        if (g.splits > 1 && !splits_out) trace->use(false, partials, 4 * n4 * g.splits);
+        return cudaSuccess;
+    }
+    cudaError_t e = BN == 256 ? tc_gemm_bn<256>(maps, g, stream) : (BN == 128 ? tc_gemm_bn<128>(maps, g, stream) : tc_gemm_bn<64>(maps, g, stream));
+    if (e != cudaSuccess || g.splits == 1 || splits_out) return e;
     return launch_chained(tc_reduce_kernel, (unsigned)((n4 + 255) / 256), 256, 0, stream, (const float4 *)partials, g.splits, n4, alpha, accumulate ? 1 : 0, (float4 *)C);
 }
 
@@ -1030,10 +1057,9 @@ extern "C" size_t hgf_backward_workspace_bytes(int64_t M, int64_t d_in, int64_t 
     return bw_layout(M, d_in, d_out, r).total;
 }
 
-extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *packed, float gamma, int64_t d_in, int64_t d_out,
-                                          const void *At, const void *Bt, int32_t r, const float *gate, const void *dy,
-                                          const hgf_grads *grads, void *workspace, size_t workspace_bytes, uint32_t flags,
-                                          void *stream_) {
+static hgf_status backward(const void *x, int64_t M, const void *packed, float gamma, int64_t d_in, int64_t d_out, const void *At, const void *Bt,
+                           int32_t r, const float *gate, const void *dy, const hgf_grads *grads, void *workspace, size_t workspace_bytes,
+                           uint32_t flags, void *stream_, BwTrace *trace) {
     if (!x || !packed || !dy || !grads || M <= 0 || d_in <= 0 || d_out <= 0 || r < 0) return HGF_ERR_INVALID_ARG;
     if (flags & ~HGF_FLAG_NO_SILU) return HGF_ERR_INVALID_ARG;
     if (!At || !Bt || !gate) r = 0;
@@ -1053,10 +1079,20 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     auto blocks1 = [](size_t n) { return (unsigned)((n + 255) / 256); };
     const TcOperand none = {nullptr, 0, false};
     float *partials = (float *)(ws + L.partials);
+    if (trace) trace->room = partials;
     bool ok = true;
+    auto launch = [&](auto *kernel, unsigned blocks, auto... args) {
+        if (!trace) ok = ok && launch_chained(kernel, blocks, 256, 0, stream, args...) == cudaSuccess;
+    };
+    auto done = [&] { return ok && (trace || cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA; };
     auto gemm = [&](TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J, float alpha,
                     bool acc, bool may_split, int *splits_out = nullptr, TcThinProduct *thin = nullptr, int n_thin = 0) {
-        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, splits_out, thin, n_thin, stream) == cudaSuccess;
+        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, splits_out, thin, n_thin, stream, trace) == cudaSuccess;
+    };
+    // The partial sums of a product, or the product itself, for the launch that comes next; the room may be used again after it.
+    auto read = [&](const float *sums, const float *product, int splits, size_t n) {
+        if (trace && splits > 0 && sums != product) trace->use(false, sums, n * splits);
+        return sums;
     };
     const TcOperand dy_k = {(const __nv_bfloat16 *)dy, N, false};  // dY as [M rows][N contraction]
     const TcOperand dy_mn = {(const __nv_bfloat16 *)dy, N, true};  // dY as [N rows] contracted over its M stored rows
@@ -1076,14 +1112,14 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
             p.blocks_at = blocks1(p.n_at);
         }
         const unsigned blocks = p.blocks_t + p.blocks_at + blocks1(p.n_bt);
-        if (blocks) ok = ok && launch_chained(bw_weights_kernel, blocks, 256, 0, stream, p) == cudaSuccess;
+        if (blocks) launch(bw_weights_kernel, blocks, p);
     }
     float *z = (float *)(ws + L.z), *dh = (float *)(ws + L.dh), *G = grads->dBt ? grads->dBt : (float *)(ws + L.G);
     const TcOperand At_k = {bf(L.At_b), K, false}, At_mn = {bf(L.At_b), K, true};
     int sp = 1;
     if (r) {                                                                                                 // Z = x A
         gemm(x_k, At_k, K, none, none, 0, z, r, Mi, r, 1.0f, false, true, &sp);
-        ok = ok && launch_chained(bw_act_kernel, blocks1((size_t)M * r), 256, 0, stream, sp > 1 ? partials : z, sp, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, z, bf(L.h_b)) == cudaSuccess;
+        launch(bw_act_kernel, blocks1((size_t)M * r), read(sp > 1 ? partials : z, z, sp, (size_t)M * r), sp, (size_t)M * r, (flags & HGF_FLAG_NO_SILU) ? 1 : 0, z, bf(L.h_b));
     }
     // The products with dY and H: dH = dY (g (.) B^T), and G[n][j] = sum_m dY[m][n] H[m][j], behind dW's tiles where tc_deal_thin has room there,
     // else as launches of their own.
@@ -1095,8 +1131,7 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         if (K <= kBwQuantMaxK) {
             const unsigned rows8 = (unsigned)((Mi + 7) / 8);
             const __nv_bfloat16 *xp = (const __nv_bfloat16 *)x;
-            ok = ok && (K <= kBwQuantMaxK / 2 ? launch_chained(bw_quant_kernel<8>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))
-                            : launch_chained(bw_quant_kernel<16>, rows8, 256, 0, stream, xp, Mi, K, bf(L.xd))) == cudaSuccess;
+            launch(K <= kBwQuantMaxK / 2 ? bw_quant_kernel<8> : bw_quant_kernel<16>, rows8, xp, Mi, K, bf(L.xd));
         } else {
             PrologueParams pp = {};
             pp.x = (const __nv_bfloat16 *)x;
@@ -1105,9 +1140,9 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
             pp.M = Mi;
             pp.K = K;
             pp.flags = HGF_FLAG_NO_PDL;
-            if (launch_quant(pp, GemmPrologueExtra{}, stream) != cudaSuccess) return HGF_ERR_CUDA;
+            if (!trace && launch_quant(pp, GemmPrologueExtra{}, stream) != cudaSuccess) return HGF_ERR_CUDA;
             const size_t n8 = (size_t)M * K / 8;
-            ok = ok && launch_chained(bw_dequant_kernel, blocks1(n8), 256, 0, stream, pp.xq, pp.gamma_x, K, n8, bf(L.xd)) == cudaSuccess;
+            launch(bw_dequant_kernel, blocks1(n8), pp.xq, pp.gamma_x, K, n8, bf(L.xd));
         }
         gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false, nullptr, with_dw, r ? (want_g ? 2 : 1) : 0);
     }
@@ -1115,7 +1150,7 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
     const TcOperand T_mn = {bf(L.T), K, true};  // T [N][K]: rows k of the product, contracted over n
     if (!r) {
         if (grads->dx) gemm(dy_k, T_mn, N, none, none, 0, grads->dx, K, Mi, K, gamma, false, false);
-        return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
+        return done();
     }
     const float *dh_sums = partials;
     sp = with_dw[0].splits;
@@ -1123,7 +1158,11 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
         gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true, &sp);
         if (sp == 1) dh_sums = dh;
     }
-    ok = ok && launch_chained(bw_dz_kernel, blocks1((size_t)M * r), 256, 0, stream, dh_sums, sp, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b)) == cudaSuccess;
+    launch(bw_dz_kernel, blocks1((size_t)M * r), read(dh_sums, dh, sp, (size_t)M * r), sp, z, (size_t)M * r, fold ? 1.0f / gamma : 1.0f, bf(L.dz_b), bf(L.dzs_b));
+    auto from_g = [&](const float *sums, int splits) {  // dBt and dgate
+        launch(bw_gate_kernel, (unsigned)((N + 7) / 8), read(sums, G, splits, (size_t)N * r), splits, (const __half *)Bt, gate, N, r, G, grads->dgate);
+    };
+    if (with_dw[1].splits) from_g(with_dw[1].P, with_dw[1].splits);  // (ahead of dA, whose partial sums may take all of the room)
     // dA^T[j][k] = sum_m dZ[m][j] x[m][k]
     TcThinProduct with_dx = {x_mn, TcOperand{bf(L.dz_b), r, true}, K, r, Mi, true, partials, 0};
     if (grads->dx) {                                                                                         // dX = gamma_W dY T + dZ A^T
@@ -1140,17 +1179,47 @@ extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *
             gemm(TcOperand{bf(L.dz_b), r, true}, x_mn, Mi, none, none, 0, grads->dAt, K, r, K, 1.0f, false, true);
         } else {
             const size_t n4 = (size_t)r * K / 4;
-            ok = ok && launch_chained(tc_reduce_kernel, blocks1(n4), 256, 0, stream, (const float4 *)partials, with_dx.splits, n4, 1.0f, 0, (float4 *)grads->dAt) == cudaSuccess;
+            launch(tc_reduce_kernel, blocks1(n4), (const float4 *)read(partials, nullptr, with_dx.splits, 4 * n4), with_dx.splits, n4, 1.0f, 0, (float4 *)grads->dAt);
         }
     }
-    if (want_g) {
-        const float *g_sums = partials + half;
-        sp = with_dw[1].splits;
-        if (!sp) {
-            gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true, &sp);
-            g_sums = sp > 1 ? partials : G;
-        }
-        ok = ok && launch_chained(bw_gate_kernel, (unsigned)((N + 7) / 8), 256, 0, stream, g_sums, sp, (const __half *)Bt, gate, N, r, G, grads->dgate) == cudaSuccess;
+    if (want_g && !with_dw[1].splits) {
+        gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true, &sp);
+        from_g(sp > 1 ? partials : G, sp);
     }
-    return (ok && cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA;
+    return done();
+}
+
+extern "C" hgf_status hgf_linear_backward(const void *x, int64_t M, const void *packed, float gamma, int64_t d_in, int64_t d_out,
+                                          const void *At, const void *Bt, int32_t r, const float *gate, const void *dy,
+                                          const hgf_grads *grads, void *workspace, size_t workspace_bytes, uint32_t flags,
+                                          void *stream) {
+    return backward(x, M, packed, gamma, d_in, d_out, At, Bt, r, gate, dy, grads, workspace, workspace_bytes, flags, stream, nullptr);
+}
+
+// (for the tests, without a GPU: what the pass does with its room for partial sums, `floats` of it, on a device of that many SMs and pairs;
+// want: bits 0 to 4 for dx, dW, dAt, dBt, dgate.  uses: [write, first, end] each, at most `most`, their number is returned, -1 if the call is
+// refused; rides: [thin products taken, half tiles, c_idle, c_busy] of dW's launch by pairs and of dX's, zeros where there is none)
+extern "C" int hgf_internal_backward_trace(int64_t M, int64_t d_in, int64_t d_out, int32_t r, float gamma, int32_t want, int32_t sms, int32_t pairs,
+                                           int64_t *floats, int64_t *uses, int32_t most, int32_t *rides) {
+    BwTrace trace = {};
+    trace.sms = sms;
+    trace.pairs = pairs;
+    char *at = (char *)((uintptr_t)1 << 40);  // (addresses that nothing reads)
+    const hgf_grads g = {(float *)(want & 1 ? at : nullptr), (float *)(want & 2 ? at : nullptr), (float *)(want & 4 ? at : nullptr),
+                         (float *)(want & 8 ? at : nullptr), (float *)(want & 16 ? at : nullptr)};
+    const size_t bytes = hgf_backward_workspace_bytes(M, d_in, d_out, r);
+    if (backward(at, M, at, gamma, d_in, d_out, at, at, r, (const float *)at, at, &g, at, bytes, 0, nullptr, &trace) != HGF_OK) return -1;
+    *floats = (int64_t)((bytes - bw_layout(M, d_in, d_out, r).partials) / 4);
+    int n = 0;
+    for (const BwTrace::Use &u : trace.uses) {
+        if (n == most) break;
+        uses[3 * n] = u.write; uses[3 * n + 1] = u.first; uses[3 * n + 2] = u.end;
+        ++n;
+    }
+    for (int k = 0; k < 8; ++k) rides[k] = 0;
+    for (const BwTrace::Rides &t : trace.rides) {
+        int32_t *to = rides + (t.dx ? 4 : 0);
+        to[0] = t.n; to[1] = t.n_half; to[2] = t.c_idle; to[3] = t.c_busy;
+    }
+    return n;
 }

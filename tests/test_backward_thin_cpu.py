@@ -60,3 +60,40 @@ def test_where_they_ride(lib, M, K, N, dw, dx):
         return deal(lib, thin, tiles + half // 2, half, blocks, 74)[0]
     assert product(N, K, -(-M // 64), [(M, N), (N, M)]) == dw
     assert product(M, K, -(-N // 64) + 1, [(K, M)]) == dx
+
+
+GRADIENTS = ("dx", "dW", "dAt", "dBt", "dgate")
+
+
+def trace(lib, M, K, N, r, want=GRADIENTS, gamma=0.02, sms=148, pairs=74):
+    """A backward pass of which nothing is enqueued: its room for partial sums, what its launches do with it, who rides with dW and with dX."""
+    uses, rides, floats = (ctypes.c_int64 * 300)(), (ctypes.c_int32 * 8)(), ctypes.c_int64()
+    bits = sum(1 << GRADIENTS.index(n) for n in want)
+    n = lib.hgf_internal_backward_trace(ctypes.c_int64(M), ctypes.c_int64(K), ctypes.c_int64(N), r, ctypes.c_float(gamma), bits, sms, pairs, ctypes.byref(floats), uses, 100, rides)
+    assert 0 <= n < 100
+    return floats.value, [tuple(uses[3 * i:3 * i + 3]) for i in range(n)], list(rides)
+
+
+SIZES = [(4096, 2112, 2048), (3300, 2048, 2048), (2656, 3456, 3456), (2500, 2112, 512), (4096, 2176, 3072), (3456, 3968, 3200), (3072, 3072, 3072), (4096, 2560, 2560),
+         (2560, 2560, 2560), (2261, 1024, 2048), (8192, 2048, 5632), (64, 512, 512), (1, 64, 8)]
+WANTS = [GRADIENTS, ("dW", "dAt", "dBt", "dgate"), ("dW", "dAt", "dgate"), ("dx", "dAt", "dBt"), ("dW", "dBt"), ("dgate",)]
+
+
+@pytest.mark.parametrize("gamma", [0.02, 0.0])
+@pytest.mark.parametrize("want", WANTS, ids="-".join)
+@pytest.mark.parametrize("sms", [148, 132, 20])
+def test_partial_sums_are_read_before_their_room_is_written_again(lib, sms, want, gamma):
+    rng = random.Random(sms)
+    sizes = SIZES + [(rng.randint(1, 9000), 64 * rng.randint(1, 130), 8 * rng.randint(1, 1000)) for _ in range(60)]
+    sizes += [(256 * m, 256 * k, 256 * n) for m in (4, 8, 10, 16) for k in (4, 8, 10, 16) for n in (2, 8, 12)]
+    for M, K, N in sizes:
+        floats, uses, rides = trace(lib, M, K, N, rng.choice([16, 32, 48, 64]), want, gamma, sms, sms // 2)
+        unread = {}  # first float -> end, of the sums that are still to be read
+        for write, first, end in uses:
+            assert 0 <= first < end <= floats
+            if write:
+                assert all(end <= a or first >= b for a, b in unread.items()), f"{M} x {K} -> {N}, {rides}: sums written over others that are still to be read"
+                unread[first] = end
+            else:
+                assert unread.pop(first, None) == end, f"{M} x {K} -> {N}, {rides}: other sums are read than were written"
+        assert not unread

@@ -25,3 +25,36 @@ def test_gradients(M, K, N, r):
     for n in ref:
         err = np.abs(got[n].cpu().numpy().astype(np.float64) - ref[n]).max() / np.abs(ref[n]).max()
         assert err <= 1e-2, f"{n}: normalised error {err:.3e}"
+
+
+def _exact(M, K, N, r):
+    """The arguments of a pass and its four gradients that do not take quantised activations, in 64 bits."""
+    from paper_2602_05269_b200 import hgf
+    g = torch.Generator(device="cuda")
+    g.manual_seed(M + 7 * K + 13 * N + r)
+    rand = lambda *shape: torch.randn(shape, generator=g, device="cuda")  # noqa: E731
+    x, dy = rand(M, K).to(torch.bfloat16), rand(M, N).to(torch.bfloat16)
+    packed, gamma = hgf.pack_ternary(0.02 * rand(N, K))
+    At, Bt, gate = (K ** -0.5 * rand(r, K)).half(), (r ** -0.5 * rand(N, r)).half(), rand(N).abs()
+    z = x.double() @ At.double().t()
+    s = torch.sigmoid(z)
+    G = dy.double().t() @ (z * s)
+    dz = ((dy.double() * gate.double()) @ Bt.double()) * (s * (1 + z * (1 - s)))
+    ref = {"dx": gamma * (dy.double() @ hgf.unpack_ternary(packed, N, K).double()) + dz @ At.double(), "dAt": dz.t() @ x.double(),
+           "dBt": gate.double()[:, None] * G, "dgate": (G * Bt.double()).sum(1)}
+    return (x, packed, gamma, K, N, dy, At, Bt, gate), ref
+
+
+# dW's launch takes dH and G along, and dA is a launch of its own whose contraction is split often enough to fill the room for partial sums
+@pytest.mark.parametrize("without_dx,M,K,N,r", [(False, 4096, 2112, 2048, 32), (False, 2656, 3456, 3456, 16), (False, 2500, 2112, 512, 48), (False, 4096, 2176, 3072, 64),
+                                                (True, 3072, 3072, 3072, 32), (True, 4096, 2560, 2560, 16), (True, 2560, 2560, 2560, 48)])
+def test_partial_sums_of_two_products_at_a_time(without_dx, M, K, N, r):
+    """Tolerance as in test_gpu_backward.py, 2^-9 of a typical term, here in the 2-norm: within 5e-3 of the gradient's."""
+    from paper_2602_05269_b200 import hgf
+    args, ref = _exact(M, K, N, r)
+    got = hgf.linear_backward(*args, want=("dW", "dAt", "dBt", "dgate") if without_dx else None)
+    hgf.check_status()
+    for n in ref:
+        if n in got:
+            err = float((got[n].double() - ref[n]).norm() / ref[n].norm())
+            assert err <= 5e-3, f"{n}: {err:.3e}"
