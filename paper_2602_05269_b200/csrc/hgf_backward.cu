@@ -67,10 +67,12 @@ struct TcGemmArgs {
 };
 
 // A product with one extent of at most 64 that rides in a launch by pairs (tc_pair_gemm_kernel): output tiles of 256 x 64, the
-// contraction in `splits` parts, each with partial sums of its own.  B is stored with its row index contiguous.
+// contraction in `splits` parts, each of one or several partial sums of kb_per_sum blocks: those of a launch of its own (tc_split_blocks), added
+// in the same order, so the results are the same bits either way.  The sums of the first part are added before they are written; the
+// others are left to the reader.  B is stored with its row index contiguous.
 struct TcThin {
-    float *P;                    // [splits][I][J], or [splits][J][I] when `across`
-    int I, J, kb, splits, kb_per_split;
+    float *P;                    // [1 + sums of the parts past the first][I][J], or [..][J][I] when `across`
+    int I, J, kb, splits, kb_per_split, kb_per_sum;  // (kb_per_split a multiple of kb_per_sum)
     int a_mn, across;            // (a_mn as in TcGemmArgs)
 };
 constexpr int kTcThinMax = 2;
@@ -505,26 +507,28 @@ tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
                 warp_commit_pair(bar(C::BAR_ACCFULL + b));
             }
             Piece t;
-            for (int q = 0; ok && piece_of(q, t); ++q, ++it) {
-                const int b = it & 1;
-                const uint32_t acc = tmem_base + b * kTpTile;
-                if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x890u))) break;
-                tc_fence_after();
+            for (int q = 0; ok && piece_of(q, t); ++q) {
                 const bool a_mn = thin.job[t.job].a_mn != 0;
                 const uint32_t idesc_w = C::IDESC | (a_mn ? 1u << 15 : 0u) | (1u << 16) | ((uint32_t)(kThinCols >> 3) << 17), step = a_mn ? (16 * 128) >> 4 : 32 >> 4;
-                for (int kb = t.kb0; kb < t.kb1; ++kb) {
-                    if (!(ok = wait(C::BAR_FULL + s, ph, 0x8a0u + s))) break;
+                for (int k0 = t.kb0; ok && k0 < t.kb1; k0 += thin.job[t.job].kb_per_sum, ++it) {
+                    const int b = it & 1, k1 = min(k0 + thin.job[t.job].kb_per_sum, t.kb1);
+                    const uint32_t acc = tmem_base + b * kTpTile;
+                    if (it >= 2 && !(ok = wait(C::BAR_ACCEMPTY + b, (uint32_t)((it >> 1) - 1) & 1u, 0x890u))) break;
                     tc_fence_after();
-                    const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
-                    const uint64_t adesc = a_mn ? make_sw128_mn_desc(sa, kTBox) : make_sw128_desc(sa), bdesc = make_sw128_mn_desc(sb, kTBox);
+                    for (int kb = k0; kb < k1; ++kb) {
+                        if (!(ok = wait(C::BAR_FULL + s, ph, 0x8a0u + s))) break;
+                        tc_fence_after();
+                        const uint32_t sa = sbase + s * C::STAGE_BYTES, sb = sa + C::A_BYTES;
+                        const uint64_t adesc = a_mn ? make_sw128_mn_desc(sa, kTBox) : make_sw128_desc(sa), bdesc = make_sw128_mn_desc(sb, kTBox);
 #pragma unroll
-                    for (int kk = 0; kk < kTBK / 16; ++kk)
-                        warp_mma_f16_pair(acc, adesc + (uint64_t)(step * kk), bdesc + (uint64_t)(((16 * 128) >> 4) * kk), idesc_w, (kb > t.kb0 || kk) ? 1u : 0u);
-                    warp_commit_pair(bar(C::BAR_EMPTY + s));
-                    if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+                        for (int kk = 0; kk < kTBK / 16; ++kk)
+                            warp_mma_f16_pair(acc, adesc + (uint64_t)(step * kk), bdesc + (uint64_t)(((16 * 128) >> 4) * kk), idesc_w, (kb > k0 || kk) ? 1u : 0u);
+                        warp_commit_pair(bar(C::BAR_EMPTY + s));
+                        if (++s == C::STAGES) { s = 0; ph ^= 1u; }
+                    }
+                    if (!ok) break;
+                    warp_commit_pair(bar(C::BAR_ACCFULL + b));
                 }
-                if (!ok) break;
-                warp_commit_pair(bar(C::BAR_ACCFULL + b));
             }
         }
     } else {
@@ -565,33 +569,42 @@ tc_pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_con
             if (lane == 0) mbar_arrive_cluster(cluster_address(bar(C::BAR_ACCEMPTY + b), 0));
         }
         Piece t;
-        for (int n = 0; ok && piece_of(n, t); ++n, ++it) {
+        for (int n = 0; ok && piece_of(n, t); ++n) {
             const TcThin &T = thin.job[t.job];
-            const int b = it & 1;
-            ok = mbar_wait(bar(C::BAR_ACCFULL + b), (uint32_t)(it >> 1) & 1u, abort_flag, status, 0x8b0u);
-            if (!(ok = __all_sync(0xffffffffu, ok))) break;
-            tc_fence_after();
-            const int i = t.i0 + rank * kTBM + 32 * q + lane;
-            const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16) + b * kTpTile;
-            for (int cc = 0; cc < T.J; cc += 16) {  // (J is a multiple of 16)
-                uint32_t v[16];
-                tmem_ld16(lane_base + cc, v);
-                tmem_ld_wait();
-                if (i < T.I) {
-                    if (T.across) {
+            int out = t.part ? 1 + (t.kb0 - T.kb_per_split) / T.kb_per_sum : 0;
+            float run[64];
+            for (int k0 = t.kb0; ok && k0 < t.kb1; k0 += T.kb_per_sum, ++it) {
+                const int b = it & 1;
+                ok = mbar_wait(bar(C::BAR_ACCFULL + b), (uint32_t)(it >> 1) & 1u, abort_flag, status, 0x8b0u);
+                if (!(ok = __all_sync(0xffffffffu, ok))) break;
+                tc_fence_after();
+                const int i = t.i0 + rank * kTBM + 32 * q + lane;
+                const uint32_t lane_base = tmem_base + ((uint32_t)(32 * q) << 16) + b * kTpTile;
+                const bool add = t.part == 0 && k0 > 0, store = t.part > 0 || k0 + T.kb_per_sum >= t.kb1;
 #pragma unroll
-                        for (int u = 0; u < 16; ++u) T.P[((size_t)t.part * T.J + cc + u) * T.I + i] = __uint_as_float(v[u]);
-                    } else {
-                        float4 *dst = reinterpret_cast<float4 *>(T.P + ((size_t)t.part * T.I + i) * T.J + cc);
+                for (int cc = 0; cc < 64; cc += 16) {
+                    if (cc >= T.J) break;  // (J is a multiple of 16)
+                    uint32_t v[16];
+                    tmem_ld16(lane_base + cc, v);
+                    tmem_ld_wait();
 #pragma unroll
-                        for (int u = 0; u < 4; ++u)
-                            dst[u] = make_float4(__uint_as_float(v[4 * u]), __uint_as_float(v[4 * u + 1]), __uint_as_float(v[4 * u + 2]), __uint_as_float(v[4 * u + 3]));
+                    for (int u = 0; u < 16; ++u) run[cc + u] = add ? run[cc + u] + __uint_as_float(v[u]) : __uint_as_float(v[u]);
+                    if (store && i < T.I) {
+                        if (T.across) {
+#pragma unroll
+                            for (int u = 0; u < 16; ++u) T.P[((size_t)out * T.J + cc + u) * T.I + i] = run[cc + u];
+                        } else {
+                            float4 *dst = reinterpret_cast<float4 *>(T.P + ((size_t)out * T.I + i) * T.J + cc);
+#pragma unroll
+                            for (int u = 0; u < 4; ++u) dst[u] = make_float4(run[cc + 4 * u], run[cc + 4 * u + 1], run[cc + 4 * u + 2], run[cc + 4 * u + 3]);
+                        }
                     }
                 }
+                out += store;
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive_cluster(cluster_address(bar(C::BAR_ACCEMPTY + b), 0));
             }
-            tc_fence_before();
-            __syncwarp();
-            if (lane == 0) mbar_arrive_cluster(cluster_address(bar(C::BAR_ACCEMPTY + b), 0));
         }
     }
 
@@ -700,13 +713,29 @@ extern "C" int hgf_internal_tc_pairs_pay(int32_t I, int32_t J, int32_t contracti
     return tc_pairs_pay(I, J, (contraction + kTBK - 1) / kTBK, true, sms, pairs) ? 1 : 0;
 }
 
-// A thin product as the caller describes it: P as in TcThin, room for splits_max partial sums; splits: as many as it was given.
+constexpr int kBwSplitsMax = 16;  // partial sums of a product that may be split
+
+// Output columns of a single CTA's tile.
+static int tc_tile_columns(int J) { return J > 128 ? 256 : (J > 64 ? 128 : 64); }
+// An I x J product over kb blocks of 64 by single CTAs that may split its contraction: blocks of a partial sum.
+static int tc_split_blocks(int I, int J, int kb, int sms) {
+    const int BN = tc_tile_columns(J), tiles = ((I + kTBM - 1) / kTBM) * ((J + BN - 1) / BN);
+    int splits = 1;
+    if (sms > 0 && tiles * 2 <= sms) splits = std::max(1, std::min({sms / tiles, kBwSplitsMax, kb / 4}));  // at least four blocks per split
+    return (kb + splits - 1) / splits;
+}
+
+// A thin product as the caller describes it: P as in TcThin, room for all of its partial sums; `rides` is set by tc_gemm: to how many sums
+// there are in P then, 0 if it did not ride.
 struct TcThinProduct {
     TcOperand A, B;      // B.mn
     int I, J, Cn;
     bool across;
     float *P;
-    int splits;
+    int kb_per_sum;      // those of a launch of its own
+    int rides;
+    int sums() const { return ((Cn + kTBK - 1) / kTBK + kb_per_sum - 1) / kb_per_sum; }
+    int sums_left(const TcThin &t) const { return 1 + std::max(0, sums() - t.kb_per_split / kb_per_sum); }
 };
 
 // The thin products' pieces over the pairs; false where launches of their own are the better way.  In half blocks of the product (64 of the
@@ -714,8 +743,10 @@ struct TcThinProduct {
 // for its start and end.  The pairs that have a tile of the last round less take pieces first; contractions are split, up to four
 // times, where that brings the last pair's end forward.  A launch of its own takes 4 us and its first operand's bytes at 4.5 TB/s; the
 // estimate has to stay below three quarters of that, since a pair streams what has left L2 by then more slowly than all SMs together do.
-// Training steps, launches of their own / this: 700 x 1024 -> 3000 130 / 112 us, 2048 x 2048 -> 2048 147 / 128, 1500 x 3200 -> 2000, r = 64 191 / 166,
-// 8000 x 768 -> 1536, r = 64 214 / 185, 4096 x 4096 -> 4096, r = 16 430 / 414, 8192 x 4096 -> 1024, r = 64 370 / 354, 8192 x 2048 -> 5632 565 / 559.
+// Backward passes in a captured chain, launches of their own / this: 700 x 1024 -> 3000, r = 32 72 / 54 us, 2048 x 2048 -> 2048 91 / 76,
+// 1500 x 3200 -> 2000, r = 64 129 / 106, 8000 x 768 -> 1536, r = 64 133 / 106, 4096 x 4096 -> 4096, r = 16 287 / 268, 8192 x 4096 -> 1024, r = 64
+// 228 / 220, 8192 x 2048 -> 5632 391 / 390.  A part is whole partial sums of a launch of its own, for the same bits.  Parts of any size would be 0 to
+// 11 per cent faster (geometric mean of 30 passes 2.8), but their longer sums are others: gradients moved by 1e-4.
 static bool tc_deal_thin(TcThinArgs *t, const TcThinProduct *thin, int n, int num_work, int n_half, int kb_all, int pairs) {
     const int rest = num_work % pairs, idle = pairs - rest;
     const double extra = rest ? (n_half ? kb_all : 2.0 * kb_all) : 0.0;
@@ -726,16 +757,19 @@ static bool tc_deal_thin(TcThinArgs *t, const TcThinProduct *thin, int n, int nu
         alone += 4.0 + 2.0 * thin[i].I * thin[i].Cn / 4.5e6;
     }
     for (int parts = 1; parts <= 4; ++parts) {
-        const int piece = (longest + parts - 1) / parts;
+        const int share = (longest + parts - 1) / parts;
+        int piece = 0;  // blocks of the longest
         TcThinArgs c = {};
         for (int i = 0; i < n; ++i) {
             TcThin &T = c.job[i];
             T.P = thin[i].P;
             T.I = thin[i].I; T.J = thin[i].J;
             T.kb = (thin[i].Cn + kTBK - 1) / kTBK;
-            T.splits = (T.kb + piece - 1) / piece;
-            T.kb_per_split = (T.kb + T.splits - 1) / T.splits;
+            T.kb_per_sum = thin[i].kb_per_sum;
+            T.splits = (T.kb + share - 1) / share;
+            T.kb_per_split = ((T.kb + T.splits - 1) / T.splits + T.kb_per_sum - 1) / T.kb_per_sum * T.kb_per_sum;  // whole partial sums
             T.splits = (T.kb + T.kb_per_split - 1) / T.kb_per_split;  // no empty part
+            piece = std::max(piece, std::min(T.kb_per_split, T.kb));
             T.across = thin[i].across ? 1 : 0;
             c.items += (T.I + kTpTile - 1) / kTpTile * T.splits;
             if (i == 0) c.items0 = c.items;
@@ -759,7 +793,10 @@ static bool tc_deal_thin(TcThinArgs *t, const TcThinProduct *thin, int n, int nu
 // them halves; out: items, items0, busy, c_idle, c_busy, then splits and kb_per_split of each)
 extern "C" int hgf_internal_tc_deal_thin(const int32_t *I, const int32_t *Cn, int32_t n, int32_t num_work, int32_t n_half, int32_t kb_all, int32_t pairs, int32_t *out) {
     TcThinProduct thin[kTcThinMax] = {};
-    for (int i = 0; i < n && i < kTcThinMax; ++i) { thin[i].I = I[i]; thin[i].Cn = Cn[i]; thin[i].J = 16; }
+    for (int i = 0; i < n && i < kTcThinMax; ++i) {
+        thin[i].I = I[i]; thin[i].Cn = Cn[i]; thin[i].J = 16;
+        thin[i].kb_per_sum = tc_split_blocks(I[i], 16, (Cn[i] + kTBK - 1) / kTBK, 2 * pairs);
+    }
     TcThinArgs t = {};
     const bool ride = tc_deal_thin(&t, thin, n, num_work, n_half, kb_all, pairs);
     out[0] = t.items; out[1] = t.items0; out[2] = t.busy; out[3] = t.c_idle; out[4] = t.c_busy;
@@ -779,13 +816,13 @@ struct BwTrace {
 };
 
 // C[I][J] = alpha * (A B^T + A2 B2^T) (+ C).  A2.p == nullptr: one pair only.  Both pairs have the same
-// operand forms.  `partials` (splits_max * I * ldc floats) enables splitting the contraction when the
+// operand forms.  `partials` (kBwSplitsMax * I * ldc floats) enables splitting the contraction when the
 // output has fewer tiles than the device has SMs; ldc must then be J.  With `splits_out` they are left there for the kernel that
-// reads the product next (*splits_out of them; 1: the product is in C).  `thin`: products that may ride in a launch by pairs; `splits` is 0
-// afterwards for those that did not.  Bases 16-byte aligned, ld % 8 == 0.
+// reads the product next (*splits_out of them; 1: the product is in C).  `thin`: products that may ride in a launch by pairs; those that
+// did have `rides` afterwards.  Bases 16-byte aligned, ld % 8 == 0.
 static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J,
-                           float alpha, bool accumulate, float *partials, int splits_max, int *splits_out, TcThinProduct *thin, int n_thin, cudaStream_t stream, BwTrace *trace) {
-    const int BN = J > 128 ? 256 : (J > 64 ? 128 : 64), sms = trace ? trace->sms : device_sm_count();
+                           float alpha, bool accumulate, float *partials, int *splits_out, TcThinProduct *thin, int n_thin, cudaStream_t stream, BwTrace *trace) {
+    const int BN = tc_tile_columns(J), sms = trace ? trace->sms : device_sm_count();
     const int kb1 = (Cn + kTBK - 1) / kTBK, kb2 = A2.p ? (Cn2 + kTBK - 1) / kTBK : 0, kb_all = kb1 + kb2;
     int pairs = I > kTBM && J > 128 && kb_all >= kTpMinBlocks && sms > 0 ? (trace ? trace->pairs : tc_pairs_at_once()) : 0;
     if (!tc_pairs_pay(I, J, kb_all, B.mn, sms, pairs)) pairs = 0;
@@ -815,8 +852,8 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
         if (n_thin && !tc_deal_thin(&t, thin, n_thin, work, g.n_half, kb_all, pairs)) n_thin = 0;
         if (trace) {
             for (int i = 0; i < n_thin; ++i) {
-                thin[i].splits = t.job[i].splits;
-                trace->use(true, thin[i].P, (size_t)thin[i].splits * thin[i].I * thin[i].J);
+                thin[i].rides = thin[i].sums_left(t.job[i]);
+                trace->use(true, thin[i].P, (size_t)thin[i].rides * thin[i].I * thin[i].J);
             }
             trace->rides.push_back({!A.mn, n_thin, g.n_half, t.c_idle, t.c_busy});
             return cudaSuccess;
@@ -827,7 +864,7 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
             if (i >= n_thin) continue;
             if (!tc_map(&thin_maps.a[i], thin[i].A, thin[i].I, thin[i].Cn, kTBM, &t.job[i].a_mn) || !tc_map(&thin_maps.b[i], thin[i].B, thin[i].J, thin[i].Cn, 0))
                 return cudaErrorInvalidValue;
-            thin[i].splits = t.job[i].splits;
+            thin[i].rides = thin[i].sums_left(t.job[i]);
         }
         unsigned int *status = device_status_word();
         if (!status) return cudaErrorMemoryAllocation;
@@ -835,19 +872,13 @@ static cudaError_t tc_gemm(TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOpe
                               maps[2], maps[3], g, thin_maps, t, status);
     }
     const int tiles = ((I + kTBM - 1) / kTBM) * ((J + BN - 1) / BN);
-    int splits = 1;
-    if (partials && ldc == J && sms > 0 && tiles * 2 <= sms) {
-        splits = sms / tiles;
-        if (splits > splits_max) splits = splits_max;
-        if (splits > kb_all / 4) splits = kb_all / 4 > 0 ? kb_all / 4 : 1;   // at least four blocks per split
-    }
+    g.kb_per_split = partials && ldc == J ? tc_split_blocks(I, J, kb_all, sms) : kb_all;
+    g.splits = (kb_all + g.kb_per_split - 1) / g.kb_per_split;  // no empty split
     // Tail of the tile schedule: when the tiles left for the last round of the persistent CTAs would keep at most
     // half of the SMs busy, they are worked as twice as many tiles of half the width, which fills the round.
-    if (splits == 1 && BN == 256 && B.mn && sms > 0 && tiles > sms && tiles % sms != 0 && 2 * (tiles % sms) <= sms &&
+    if (g.splits == 1 && BN == 256 && B.mn && sms > 0 && tiles > sms && tiles % sms != 0 && 2 * (tiles % sms) <= sms &&
         J % 256 == 0)
         g.n_half = 2 * (tiles % sms);
-    g.kb_per_split = (kb_all + splits - 1) / splits;
-    g.splits = (kb_all + g.kb_per_split - 1) / g.kb_per_split;  // no empty split
     if (g.splits == 1) {
         g.C = C; g.alpha = alpha; g.accumulate = accumulate ? 1 : 0;
     } else {
@@ -1019,7 +1050,6 @@ __global__ void __launch_bounds__(256) bw_gate_kernel(const float *P, int splits
     if (dgate && lane == 0) dgate[n] = dg;
 }
 
-constexpr int kBwSplitsMax = 16;
 constexpr int kBwQuantMaxK = 4096;  // up to here a row fits a warp's registers (bw_quant_kernel): no codes and scales in memory
 
 struct BwLayout {
@@ -1087,7 +1117,7 @@ static hgf_status backward(const void *x, int64_t M, const void *packed, float g
     auto done = [&] { return ok && (trace || cudaGetLastError() == cudaSuccess) ? HGF_OK : HGF_ERR_CUDA; };
     auto gemm = [&](TcOperand A, TcOperand B, int Cn, TcOperand A2, TcOperand B2, int Cn2, float *C, int ldc, int I, int J, float alpha,
                     bool acc, bool may_split, int *splits_out = nullptr, TcThinProduct *thin = nullptr, int n_thin = 0) {
-        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, kBwSplitsMax, splits_out, thin, n_thin, stream, trace) == cudaSuccess;
+        ok = ok && tc_gemm(A, B, Cn, A2, B2, Cn2, C, ldc, I, J, alpha, acc, may_split ? partials : nullptr, splits_out, thin, n_thin, stream, trace) == cudaSuccess;
     };
     // The partial sums of a product, or the product itself, for the launch that comes next; the room may be used again after it.
     auto read = [&](const float *sums, const float *product, int splits, size_t n) {
@@ -1124,9 +1154,14 @@ static hgf_status backward(const void *x, int64_t M, const void *packed, float g
     // The products with dY and H: dH = dY (g (.) B^T), and G[n][j] = sum_m dY[m][n] H[m][j], behind dW's tiles where tc_deal_thin has room there,
     // else as launches of their own.
     const bool want_g = r && (grads->dBt || grads->dgate);
-    const size_t half = (size_t)(kBwSplitsMax / 2) * std::max({Mi, N, K}) * r;  // (two sets of partial sums at a time)
-    TcThinProduct with_dw[2] = {{dy_k, TcOperand{bf(L.gBt), r, true}, Mi, r, N, false, partials, 0},
-                                {dy_mn, TcOperand{bf(L.h_b), r, true}, N, r, Mi, false, partials + half, 0}};
+    const int sms = trace ? trace->sms : device_sm_count();
+    auto blocks64 = [](int n) { return (n + kTBK - 1) / kTBK; };
+    TcThinProduct with_dw[2] = {{dy_k, TcOperand{bf(L.gBt), r, true}, Mi, r, N, false, partials, r ? tc_split_blocks(Mi, r, blocks64(N), sms) : 1, 0},
+                                {dy_mn, TcOperand{bf(L.h_b), r, true}, N, r, Mi, false, nullptr, r ? tc_split_blocks(N, r, blocks64(Mi), sms) : 1, 0}};
+    // G's partial sums lie behind dH's; where there is no room for both (M just above N, both above K: 2261 x 1024 -> 2048) G has a launch of its own.
+    const size_t h_floats = (size_t)with_dw[0].sums() * Mi * r, g_floats = (size_t)with_dw[1].sums() * N * r;
+    const bool both = want_g && h_floats + g_floats <= (size_t)kBwSplitsMax * std::max({Mi, N, K}) * r;
+    with_dw[1].P = partials + h_floats;
     if (grads->dW) {  // Algorithm 1, steps 1-2 again, then dW[n][k] = sum_m dY[m][n] Xd[m][k]
         if (K <= kBwQuantMaxK) {
             const unsigned rows8 = (unsigned)((Mi + 7) / 8);
@@ -1144,7 +1179,7 @@ static hgf_status backward(const void *x, int64_t M, const void *packed, float g
             const size_t n8 = (size_t)M * K / 8;
             launch(bw_dequant_kernel, blocks1(n8), pp.xq, pp.gamma_x, K, n8, bf(L.xd));
         }
-        gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false, nullptr, with_dw, r ? (want_g ? 2 : 1) : 0);
+        gemm(dy_mn, TcOperand{bf(L.xd), K, true}, Mi, none, none, 0, grads->dW, K, N, K, 1.0f, false, false, nullptr, with_dw, r ? (both ? 2 : 1) : 0);
     }
     const bool fold = gamma > 1e-20f;  // the low-rank term of dX rides in the same contraction, pre-divided by gamma_W
     const TcOperand T_mn = {bf(L.T), K, true};  // T [N][K]: rows k of the product, contracted over n
@@ -1153,7 +1188,7 @@ static hgf_status backward(const void *x, int64_t M, const void *packed, float g
         return done();
     }
     const float *dh_sums = partials;
-    sp = with_dw[0].splits;
+    sp = with_dw[0].rides;
     if (!sp) {
         gemm(dy_k, TcOperand{bf(L.gBt), r, true}, N, none, none, 0, dh, r, Mi, r, 1.0f, false, true, &sp);
         if (sp == 1) dh_sums = dh;
@@ -1162,9 +1197,9 @@ static hgf_status backward(const void *x, int64_t M, const void *packed, float g
     auto from_g = [&](const float *sums, int splits) {  // dBt and dgate
         launch(bw_gate_kernel, (unsigned)((N + 7) / 8), read(sums, G, splits, (size_t)N * r), splits, (const __half *)Bt, gate, N, r, G, grads->dgate);
     };
-    if (with_dw[1].splits) from_g(with_dw[1].P, with_dw[1].splits);  // (ahead of dA, whose partial sums may take all of the room)
+    if (with_dw[1].rides) from_g(with_dw[1].P, with_dw[1].rides);  // (ahead of dA, whose partial sums may take all of the room)
     // dA^T[j][k] = sum_m dZ[m][j] x[m][k]
-    TcThinProduct with_dx = {x_mn, TcOperand{bf(L.dz_b), r, true}, K, r, Mi, true, partials, 0};
+    TcThinProduct with_dx = {x_mn, TcOperand{bf(L.dz_b), r, true}, K, r, Mi, true, partials, tc_split_blocks(r, K, blocks64(Mi), sms), 0};
     if (grads->dx) {                                                                                         // dX = gamma_W dY T + dZ A^T
         const TcOperand dzs_k = {bf(L.dzs_b), r, false};
         if (fold) {
@@ -1175,14 +1210,14 @@ static hgf_status backward(const void *x, int64_t M, const void *packed, float g
         }
     }
     if (grads->dAt) {
-        if (!with_dx.splits) {
+        if (!with_dx.rides) {
             gemm(TcOperand{bf(L.dz_b), r, true}, x_mn, Mi, none, none, 0, grads->dAt, K, r, K, 1.0f, false, true);
         } else {
             const size_t n4 = (size_t)r * K / 4;
-            launch(tc_reduce_kernel, blocks1(n4), (const float4 *)read(partials, nullptr, with_dx.splits, 4 * n4), with_dx.splits, n4, 1.0f, 0, (float4 *)grads->dAt);
+            launch(tc_reduce_kernel, blocks1(n4), (const float4 *)read(partials, nullptr, with_dx.rides, 4 * n4), with_dx.rides, n4, 1.0f, 0, (float4 *)grads->dAt);
         }
     }
-    if (want_g && !with_dw[1].splits) {
+    if (want_g && !with_dw[1].rides) {
         gemm(dy_mn, TcOperand{bf(L.h_b), r, true}, Mi, none, none, 0, G, r, N, r, 1.0f, false, true, &sp);
         from_g(sp > 1 ? partials : G, sp);
     }

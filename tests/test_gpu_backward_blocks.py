@@ -27,8 +27,7 @@ def test_gradients(M, K, N, r):
         assert err <= 1e-2, f"{n}: normalised error {err:.3e}"
 
 
-def _exact(M, K, N, r):
-    """The arguments of a pass and its four gradients that do not take quantised activations, in 64 bits."""
+def _arguments(M, K, N, r):
     from paper_2602_05269_b200 import hgf
     g = torch.Generator(device="cuda")
     g.manual_seed(M + 7 * K + 13 * N + r)
@@ -36,13 +35,19 @@ def _exact(M, K, N, r):
     x, dy = rand(M, K).to(torch.bfloat16), rand(M, N).to(torch.bfloat16)
     packed, gamma = hgf.pack_ternary(0.02 * rand(N, K))
     At, Bt, gate = (K ** -0.5 * rand(r, K)).half(), (r ** -0.5 * rand(N, r)).half(), rand(N).abs()
+    return x, packed, gamma, K, N, dy, At, Bt, gate
+
+
+def _exact(x, packed, gamma, K, N, dy, At, Bt, gate):
+    """The four gradients that do not take quantised activations, in 64 bits."""
+    from paper_2602_05269_b200 import hgf
     z = x.double() @ At.double().t()
     s = torch.sigmoid(z)
     G = dy.double().t() @ (z * s)
     dz = ((dy.double() * gate.double()) @ Bt.double()) * (s * (1 + z * (1 - s)))
     ref = {"dx": gamma * (dy.double() @ hgf.unpack_ternary(packed, N, K).double()) + dz @ At.double(), "dAt": dz.t() @ x.double(),
            "dBt": gate.double()[:, None] * G, "dgate": (G * Bt.double()).sum(1)}
-    return (x, packed, gamma, K, N, dy, At, Bt, gate), ref
+    return ref
 
 
 # dW's launch takes dH and G along, and dA is a launch of its own whose contraction is split often enough to fill the room for partial sums
@@ -51,10 +56,25 @@ def _exact(M, K, N, r):
 def test_partial_sums_of_two_products_at_a_time(without_dx, M, K, N, r):
     """Tolerance as in test_gpu_backward.py, 2^-9 of a typical term, here in the 2-norm: within 5e-3 of the gradient's."""
     from paper_2602_05269_b200 import hgf
-    args, ref = _exact(M, K, N, r)
+    args = _arguments(M, K, N, r)
+    ref = _exact(*args)
     got = hgf.linear_backward(*args, want=("dW", "dAt", "dBt", "dgate") if without_dx else None)
     hgf.check_status()
     for n in ref:
         if n in got:
             err = float((got[n].double() - ref[n]).norm() / ref[n].norm())
             assert err <= 5e-3, f"{n}: {err:.3e}"
+
+
+# dW's launch takes dH and G along, dX's takes dA, or not; asked for without dW and dx the same products are launches of their own
+@pytest.mark.parametrize("M,K,N,r", [(8192, 2048, 5632, 32), (2048, 2048, 2048, 32), (700, 1024, 3000, 32), (8000, 768, 1536, 64), (4096, 4096, 4096, 16),
+                                     (1500, 3200, 2000, 64), (512, 2048, 2048, 48), (5000, 4160, 1000, 32)])
+def test_a_gradient_has_the_same_bits_whichever_others_are_asked_for(M, K, N, r):
+    from paper_2602_05269_b200 import hgf
+    args = _arguments(M, K, N, r)
+    got = hgf.linear_backward(*args)
+    for want in (("dBt", "dgate"), ("dAt",), ("dx",), ("dW",), ("dx", "dAt"), ("dW", "dAt")):
+        alone = hgf.linear_backward(*args, want=want)
+        for n in want:
+            assert torch.equal(alone[n], got[n]), f"{n} by itself as {want}: {(alone[n] - got[n]).norm() / got[n].norm():.1e} apart"
+    hgf.check_status()
