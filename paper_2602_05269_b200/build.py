@@ -1,15 +1,15 @@
-"""Build libhgf_b200.so (sm_100a, nvcc) and _hgf_python.so (the binding's native part) in-tree.  Run as `python -m paper_2602_05269_b200.build`."""
+"""Build libhgf_b200.so (sm_100a, nvcc) and the binding's native part (_hgf_python, g++) in-tree.  Run as `python -m paper_2602_05269_b200.build`."""
 from __future__ import annotations
 
 import os
 import subprocess
 import sys
+import sysconfig
 from concurrent.futures import ThreadPoolExecutor
 
 HERE = os.path.dirname(os.path.abspath(__file__))
 CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libhgf_b200.so")
-MODULE = os.path.join(HERE, "_hgf_python.so")
 OBJ_DIR = os.path.join(HERE, "_build")
 SOURCES = ["hgf_api.cu", "hgf_pack.cu", "hgf_prologue.cu", "hgf_decode.cu", "hgf_decode_small.cu", "hgf_decode_tc.cu", "hgf_prefill.cu", "hgf_attention.cu", "hgf_backward.cu"]
 NVCC_FLAGS = ["-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo", "-O3", "-std=c++17",
@@ -21,6 +21,12 @@ def _nvcc() -> str:
         if cand and (os.path.isabs(cand) and os.path.exists(cand) or not os.path.isabs(cand)):
             return cand
     return "nvcc"
+
+
+def module_path() -> str:
+    """The binding's native part: one for each Python and torch, whose binary interfaces it is compiled against."""
+    import torch
+    return os.path.join(HERE, f"_hgf_python.{sysconfig.get_config_var('SOABI')}.torch-{torch.__version__}.so")
 
 
 def _deps(src: str):
@@ -48,7 +54,7 @@ def build(force: bool = False, verbose: bool = False) -> str:
         if verbose or r.returncode:
             sys.stderr.write(" ".join(cmd) + "\n" + r.stdout + r.stderr)
         if r.returncode:
-            raise RuntimeError("nvcc failed: " + " ".join(cmd))
+            raise RuntimeError(f"{os.path.basename(cmd[0])} failed: " + " ".join(cmd))
 
     with ThreadPoolExecutor(max_workers=4) as ex:
         list(ex.map(run, jobs))
@@ -60,17 +66,16 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
     src = os.path.join(CSRC, "hgf_python.cpp")
     newest = max(os.path.getmtime(d) for d in (src, os.path.join(HERE, "..", "include", "hgf.h")))
-    if force or not os.path.exists(MODULE) or os.path.getmtime(MODULE) < newest:
-        import sysconfig
-
+    module = module_path()
+    if force or not os.path.exists(module) or os.path.getmtime(module) < newest:
         import torch
         t = os.path.dirname(torch.__file__)
         cuda = os.path.join(os.path.dirname(os.path.dirname(nvcc)) if os.path.isabs(nvcc) else "/usr/local/cuda", "include")
-        tmp = MODULE + f".tmp{os.getpid()}"
+        tmp = module + f".tmp{os.getpid()}"
         run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", f"-I{t}/include", f"-I{t}/include/torch/csrc/api/include", f"-I{cuda}",
              f"-I{sysconfig.get_paths()['include']}", f"-D_GLIBCXX_USE_CXX11_ABI={int(torch.compiled_with_cxx11_abi())}", src, "-o", tmp,
              f"-L{t}/lib", "-ltorch_python", "-lc10", "-lc10_cuda", "-ltorch_cpu", "-ltorch_cuda"])
-        os.replace(tmp, MODULE)
+        os.replace(tmp, module)
     return LIB
 
 

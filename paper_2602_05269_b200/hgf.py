@@ -7,9 +7,13 @@ library's kernels.  If the library is missing, or a call fails, this raises: the
 from __future__ import annotations
 
 import ctypes
+import importlib.machinery
+import importlib.util
 import os
 
 import torch
+
+from . import build as _build
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libhgf_b200.so")
@@ -143,11 +147,14 @@ def lib() -> ctypes.CDLL:
 
 def _marshal():
     """The native module beside the library, built with it."""
+    path = _build.module_path()
+    loader = importlib.machinery.ExtensionFileLoader("_hgf_python", path)
     try:
-        from . import _hgf_python
+        module = importlib.util.module_from_spec(importlib.util.spec_from_loader("_hgf_python", loader))
+        loader.exec_module(module)
     except ImportError as e:
-        raise RuntimeError(f"{_HERE}/_hgf_python.so is missing or does not load ({e}): run `python -m paper_2602_05269_b200.build`") from e
-    return _hgf_python
+        raise RuntimeError(f"{path} is missing or does not load ({e}): run `python -m paper_2602_05269_b200.build`") from e
+    return module
 
 
 def _ptr(t):

@@ -65,3 +65,32 @@ def test_arguments_of_another_type_raise(call, changed):
 def test_wrong_number_of_arguments(call):
     with pytest.raises(TypeError):
         call(*arguments()[:-1])
+
+
+def test_another_torch_or_python_has_a_module_of_its_own(monkeypatch):
+    hgf_build.build()
+    compiled = []
+
+    class Done:
+        returncode, stdout, stderr = 0, "", ""
+
+    def run(cmd, **_):
+        compiled.append(cmd)
+        return Done()
+    monkeypatch.setattr(hgf_build.subprocess, "run", run)
+    monkeypatch.setattr(hgf_build.os, "replace", lambda a, b: None)
+    hgf_build.build()
+    assert not compiled
+    monkeypatch.setattr(torch, "__version__", "1.2.3")
+    hgf_build.build()
+    assert [c[0] for c in compiled] == ["g++"] and "1.2.3" in compiled[0][compiled[0].index("-o") + 1]
+    monkeypatch.undo()
+    monkeypatch.setattr(hgf_build.subprocess, "run", run)
+    monkeypatch.setattr(hgf_build.os, "replace", lambda a, b: None)
+    tag = hgf_build.sysconfig.get_config_var("SOABI")
+    monkeypatch.setattr(hgf_build.sysconfig, "get_config_var", lambda name: "cpython-399" if name == "SOABI" else tag)
+    hgf_build.build()
+    assert len(compiled) == 2 and "cpython-399" in compiled[1][compiled[1].index("-o") + 1]
+    Done.returncode = 1
+    with pytest.raises(RuntimeError, match=r"g\+\+ failed"):
+        hgf_build.build()
