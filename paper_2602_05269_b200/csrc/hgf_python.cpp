@@ -15,12 +15,21 @@ decltype(&hgf_linear_forward_ln) g_forward_ln = nullptr;
 // A tensor that is exactly one (or a Parameter); anything else answers through its own methods.
 const at::Tensor *plain_tensor(PyObject *o) { return THPVariable_CheckExact(o) ? &THPVariable_Unpack(o) : nullptr; }
 
+// A Python int, nothing that turns into one (TypeError: the caller goes through ctypes then, which takes ints alone, too).
+bool integer(PyObject *o, unsigned long long *out) {
+    if (!PyLong_Check(o)) {
+        PyErr_SetString(PyExc_TypeError, "int expected");
+        return false;
+    }
+    *out = PyLong_AsUnsignedLongLongMask(o);
+    return true;
+}
 bool method_value(PyObject *o, const char *name, unsigned long long *out) {
     PyObject *v = PyObject_CallMethod(o, name, nullptr);
     if (!v) return false;
-    *out = PyLong_AsUnsignedLongLongMask(v);
+    const bool ok = integer(v, out);
     Py_DECREF(v);
-    return !PyErr_Occurred();
+    return ok;
 }
 bool address(PyObject *o, void **out) {
     *out = nullptr;
@@ -54,13 +63,17 @@ bool rows(PyObject *o, int64_t *out) {  // shape[0]
     PyObject *first = shape ? PySequence_GetItem(shape, 0) : nullptr;
     Py_XDECREF(shape);
     if (!first) return false;
-    *out = (int64_t)PyLong_AsUnsignedLongLongMask(first);
+    unsigned long long v = 0;
+    const bool ok = integer(first, &v);
+    *out = (int64_t)v;
     Py_DECREF(first);
-    return !PyErr_Occurred();
+    return ok;
 }
 bool integer(PyObject *o, int64_t *out) {
-    *out = (int64_t)PyLong_AsUnsignedLongLongMask(o);
-    return !PyErr_Occurred();
+    unsigned long long v = 0;
+    const bool ok = integer(o, &v);
+    *out = (int64_t)v;
+    return ok;
 }
 
 // linear_forward(x, packed, gamma, d_in, d_out, At, Bt, gate, y, workspace, flags, stream, ln_weight, ln_bias, eps, gate_group) -> status
@@ -74,7 +87,7 @@ PyObject *linear_forward(PyObject *, PyObject *const *a, Py_ssize_t n) try {
     size_t workspace_bytes = 0;
     if (!rows(a[0], &M) || !address(a[0], &x) || !address(a[1], &packed) || !integer(a[3], &d_in) || !integer(a[4], &d_out) ||
         !address(a[5], &At) || !address(a[6], &Bt) || !address(a[7], &gate) || !address(a[8], &y) || !address(a[9], &workspace) ||
-        !elements(a[9], &workspace_bytes) || !integer(a[10], &flags) || !address(a[12], &ln_weight) || !address(a[13], &ln_bias))
+        !elements(a[9], &workspace_bytes) || !integer(a[10], &flags))
         return nullptr;
     if (a[5] != Py_None && !rows(a[5], &r)) return nullptr;
     const float gamma = (float)PyFloat_AsDouble(a[2]);
@@ -84,13 +97,16 @@ PyObject *linear_forward(PyObject *, PyObject *const *a, Py_ssize_t n) try {
     } else {
         PyObject *s = PyObject_GetAttrString(a[11], "cuda_stream");
         if (!s) return nullptr;
-        stream = PyLong_AsVoidPtr(s);
+        unsigned long long v = 0;
+        const bool ok = integer(s, &v);
         Py_DECREF(s);
-        if (PyErr_Occurred()) return nullptr;
+        if (!ok) return nullptr;
+        stream = reinterpret_cast<void *>(v);
     }
     hgf_front_end fe = {};
     const bool front_end = a[12] != Py_None || a[15] != Py_None;
     if (front_end) {
+        if (!address(a[12], &ln_weight) || !address(a[13], &ln_bias)) return nullptr;
         fe.ln_weight = (const float *)ln_weight;
         fe.ln_bias = (const float *)ln_bias;
         fe.eps = (float)PyFloat_AsDouble(a[14]);
