@@ -433,7 +433,10 @@ static std::vector<int4> gemv_ranges(const std::vector<DecodeProblem> &dps, long
 // (`longest`, in column tiles) and by whether a GEMV share holds several problems.  Where only the GEMV's shares do (`runs`: the most
 // problems of a share if the row tiles are dealt evenly) it is always this kernel's (1.10 to 1.53); on base-3 weights short rows on less than half of the SMs are too
 // (0.96 to 1.16, mean 1.05).  Captured chains, warp MMA's time over this kernel's, 1650 groups: one to three equal problems, blocks of
-// transformers (one to twelve, 512 to 4096 wide), mixed sizes.
+// transformers (one to twelve, 512 to 4096 wide), mixed sizes.  All of these were measured with this kernel's shares cut by row tiles, as
+// evenly as they go; `runs` is of that deal still.  Cut by blocks of eight (plan_decode_tc) this kernel's groups are faster than in those figures (60 of
+// them: the time before over the time now 0.98 and more, mean 1.065), and some that stay on the GEMV would be, too: three of 5632 -> 2048 at
+// M = 16 take 27.5 us there and 21.2 here.
 //   base-3, shares of one problem:   taken 0.96 to 1.42, mean 1.17; left 0.73 to 1.07, mean 0.91  (2048 -> 2048, M = 1: 10.9 us, here 12.0)
 //   base-3, several problems:        taken 0.90 to 1.53, mean 1.20; left 0.82 to 1.22, mean 0.96
 //   two-bit, shares of one problem:  taken 0.95 to 1.18, mean 1.05; left 0.86 to 1.17, mean 0.95  (5632 -> 2048, M = 16: 19.1 us, here 22.1)

@@ -100,7 +100,7 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
     auto bar = [&](int i) { return bar0 + 8u * i; };
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(smem + C::OFF_BAR + C::BAR_COUNT * 8);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + C::OFF_BAR + C::BAR_COUNT * 8 + 4);
-    static_assert(TILE_T == 128, "the epilogue's staging loops are written for 128-token tiles");
+    static_assert(TILE_T == 128, "a tile has 128 tokens or 64: the epilogue's warps take half of them each, in steps of 32 or 16");
 
     // the next launch in the stream, if it asks for it, may be set up while this one runs (it waits
     // for this grid's completion before it touches memory)
@@ -167,9 +167,8 @@ prefill_gemm_kernel(const __grid_constant__ CUtensorMap tmap_x, const __grid_con
 
     if (warp == 0) {
         // ------------------------------------------------------------------ TMA producer
-        // The whole warp walks the loop (a single thread issuing ten copies per two k blocks, each
-        // with its address arithmetic, cannot keep up with the MMAs): every lane polls the barriers,
-        // lane 0 posts the byte counts and the activation tile, lanes 0-7 one weight tile each.
+        // The whole warp walks the loop: every lane polls the barriers, lane 0 posts the byte counts and issues the copies, two a
+        // stage (the activation tile's halves) and up to four a tile (the epilogue's operands).
         {
             int s = 0;
             uint32_t ph = 0;

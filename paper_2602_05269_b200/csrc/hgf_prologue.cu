@@ -819,7 +819,7 @@ __global__ void __launch_bounds__(32 * W, 1) gemm_prologue_kernel(const Prologue
         s_gamma[tid] = fmaxf(a, 1e-5f);
     }
     if constexpr (JT > 0) {
-        float *s_acc = reinterpret_cast<float *>(fp_smem);  // [warps][32 tokens][r]
+        float *s_acc = reinterpret_cast<float *>(fp_smem);  // [part of the columns, kFpWarps of them][TOK][r]
 #pragma unroll
         for (int mt = 0; mt < TILES; ++mt)
 #pragma unroll

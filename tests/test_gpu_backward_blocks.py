@@ -6,6 +6,7 @@ import torch
 
 import oracle
 from paper_2602_05269_b200 import inputs as syn
+from test_backward_thin_cpu import trace
 
 pytestmark = pytest.mark.gpu
 
@@ -58,7 +59,9 @@ def test_partial_sums_of_two_products_at_a_time(without_dx, M, K, N, r):
     from paper_2602_05269_b200 import hgf
     args = _arguments(M, K, N, r)
     ref = _exact(*args)
-    got = hgf.linear_backward(*args, want=("dW", "dAt", "dBt", "dgate") if without_dx else None)
+    want = ("dW", "dAt", "dBt", "dgate") if without_dx else ("dx", "dW", "dAt", "dBt", "dgate")
+    assert trace(hgf.lib(), M, K, N, r, want)[2][::4] == [2, 0]
+    got = hgf.linear_backward(*args, want=want)
     hgf.check_status()
     for n in ref:
         if n in got:
@@ -77,4 +80,28 @@ def test_a_gradient_has_the_same_bits_whichever_others_are_asked_for(M, K, N, r)
         alone = hgf.linear_backward(*args, want=want)
         for n in want:
             assert torch.equal(alone[n], got[n]), f"{n} by itself as {want}: {(alone[n] - got[n]).norm() / got[n].norm():.1e} apart"
+    hgf.check_status()
+
+
+# [thin products, half tiles, c_idle, c_busy] of dW's launch and of dX's: pairs that go from a tile to a piece, that take several pieces, and that go
+# from half a tile to a piece; parts of one partial sum and of several, a last one that is shorter
+@pytest.mark.parametrize("M,K,N,r,rides", [
+    (466, 512, 520, 16, [2, 0, 1, 0, 1, 0, 1, 0]), (1102, 640, 4104, 48, [2, 0, 1, 1, 1, 0, 1, 0]), (2314, 576, 4560, 32, [2, 0, 2, 1, 1, 0, 1, 0]),
+    (577, 2304, 2904, 64, [2, 68, 0, 1, 1, 0, 1, 0]), (1426, 1280, 4784, 16, [2, 42, 1, 1, 1, 0, 1, 0]), (1681, 2304, 2720, 32, [2, 50, 2, 0, 1, 0, 1, 0]),
+    (2063, 2048, 3128, 48, [2, 60, 2, 1, 0, 0, 0, 0]), (2200, 4864, 936, 64, [2, 4, 1, 0, 1, 46, 2, 1]), (1835, 3328, 560, 16, [2, 0, 1, 0, 1, 60, 0, 1]),
+    (3189, 2048, 2600, 32, [2, 28, 2, 0, 1, 60, 2, 0]), (5777, 512, 512, 64, [2, 0, 1, 0, 0, 0, 0, 0]), (408, 4992, 792, 32, [0, 0, 0, 0, 1, 0, 1, 0]),
+    (1774, 4864, 600, 48, [2, 0, 1, 0, 1, 0, 2, 1]), (3072, 3072, 3072, 16, [2, 0, 1, 1, 1, 0, 0, 1])])
+def test_pairs_that_take_tiles_and_pieces(M, K, N, r, rides):
+    """Against 64 bits (tolerance as above); dW and what rides beside it are the bits that they are without each other."""
+    from paper_2602_05269_b200 import hgf
+    assert trace(hgf.lib(), M, K, N, r)[2] == rides
+    args = _arguments(M, K, N, r)
+    ref, got = _exact(*args), hgf.linear_backward(*args)
+    for n in ref:
+        err = float((got[n].double() - ref[n]).norm() / ref[n].norm())
+        assert err <= 5e-3, f"{n}: {err:.3e}"
+    assert torch.equal(got["dW"], hgf.linear_backward(*args[:6], want=("dW",))["dW"])
+    for want in (("dBt", "dgate"), ("dAt",), ("dx",)):
+        alone = hgf.linear_backward(*args, want=want)
+        assert all(torch.equal(alone[n], got[n]) for n in want), want
     hgf.check_status()
