@@ -464,7 +464,7 @@ DECODE_TRAFFIC = {"source_sha1": "bb299d90944092f2d46485e50576d12d0bd16fed",
 # DRAM traffic of the prefill GEMM launch from one ncu capture of the very shape the bench times
 # (2048 -> 5632, r = 32, M = 8192, bf16 y): dram__bytes_read.sum + dram__bytes_write.sum of one launch.  Below
 # the launch's algorithmic bytes because most of y is still in L2 when the kernel ends.
-PREFILL_TRAFFIC = {"source_sha1": "a767dc2ba520744b4e1bc2bf911cd245bc5d128e", "dram_bytes_per_launch": 21.575168e6 + 43.553024e6}
+PREFILL_TRAFFIC = {"source_sha1": "f24e441faca673b71c3e2d72a3d73c62b3cf83b2", "dram_bytes_per_launch": 21.572864e6 + 43.299584e6}
 
 
 def prefill_traffic():
