@@ -966,7 +966,7 @@ __host__ __device__ inline RpLayout rp_layout(int K, int r, int log2_c) {
 
 // PER_SM: CTAs an SM that its registers leave room for (0: as they come).  All forms fit two but the widest behind a LayerNorm, which takes 154 registers
 // and spills 36 bytes at 128: in launches of more CTAs than SMs two an SM are worth that (r = 64, 2048 -> 1024: 26.3 -> 21.1 us
-// at M = 1000, 34.5 -> 27.8 at M = 2048), in smaller ones not (22.1 -> 26.4 at M = 1184).
+// at M = 1000, 34.5 -> 27.8 at M = 2048), in smaller ones not (22.1 -> 26.4 at M = 1184; they run sixteen warps a CTA now).
 template <int JT, bool LN, int TPW, int PER_SM>
 __global__ void __launch_bounds__(512 / TPW, PER_SM) rows_prologue_kernel(const PrologueParams p, const GemmPrologueExtra x, const FrontEnd fe,
                                                                    const int log2_c, unsigned int *status) {
@@ -1327,47 +1327,68 @@ static cudaError_t launch_gemm_prologue_jt(const PrologueParams &p, const GemmPr
 // LayerNorm, r = 64 28.3 / 25.0; at M = 3000 31.6 / 32.5, 64.0 / 65.2, 44.4 / 42.5, 35.6 / 38.3; with a LayerNorm 51.2 / 48.5 at 4096, 65.4 / 70.4 at 6000.
 // Cluster size: CTAs for every SM, two of them on one if they fit; one step smaller where that many don't run at once: 1024 -> 1024,
 // M = 1168, r = 48 16.4 -> 15.0 us, M = 570 15.4 -> 13.9; 8192 -> 1024, M = 525 26.6 -> 28.5.
-static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd *fe, cudaStream_t stream) {
-    const int sms = device_sm_count();
-    if (!sms) return cudaErrorInvalidDevice;
-    const int blocks = (p.M + kRpTokens - 1) / kRpTokens;
+struct RpForm {
+    int c;         // log2 of the CTAs of a cluster
+    bool wide;     // sixteen warps a CTA (a token each), or eight
+    size_t least;  // bytes of shared memory at least
+};
+// Whether rows_prologue_kernel takes a batch, and in which form.
+static bool rp_form(int M, int K, int N, int r, bool ln, int sms, RpForm *f) {
+    const int blocks = (M + kRpTokens - 1) / kRpTokens;
     int c = 0;
     while (c < 3 && (blocks << c) < sms) ++c;
     // (registers: two CTAs an SM at most; 33 clusters of eight or 71 of four run at once on 148 SMs, more take a second round, which
     // only long slices are worth)
-    if ((p.r >= 48 || (fe && p.r == 32)) && ((c == 3 && p.K <= 2048 && (blocks << c) > 2 * sms - sms / 4) || (c == 2 && (blocks << c) > 2 * sms - sms / 16))) --c;
+    if ((r >= 48 || (ln && r == 32)) && ((c == 3 && K <= 2048 && (blocks << c) > 2 * sms - sms / 4) || (c == 2 && (blocks << c) > 2 * sms - sms / 16))) --c;
     const int crowded = 2 * sms - 2 * sms / 5;  // (29 clusters of eight and more, with the blocks for the up-projection's operand)
-    if (p.r > 0 && p.r <= 32 && c == 3 && p.K <= 2048 && (blocks << 3) > crowded) --c;
-    while (c < 3 && rp_layout(p.K, p.r, c).smem > 110 * 1024) ++c;  // two CTAs on an SM
-    if (rp_layout(p.K, p.r, c).smem > kRpSmemLimit) return cudaErrorNotSupported;
+    if (r > 0 && r <= 32 && c == 3 && K <= 2048 && (blocks << 3) > crowded) --c;
+    while (c < 3 && rp_layout(K, r, c).smem > 110 * 1024) ++c;  // two CTAs on an SM
+    if (rp_layout(K, r, c).smem > kRpSmemLimit) return false;
+    const int ctas = blocks << c, slice = K >> c;
     bool take;
-    if (p.r == 0) {
-        take = p.M >= 64 && (p.M <= 7168 || c > 0 || p.K <= 2048);
-        if (p.K < 896) {  // (by the output tiles of the launch that follows: in one round of them or more)
-            const int tiles = ((p.M + 127) / 128) * ((x.N + 127) / 128);
-            if (p.M < 640) take = take && tiles > sms;
-            else if (2 * blocks < sms) take = take && (p.K >= 640 || tiles > sms * 5 / 6);
-            else take = take && (p.K <= 512 || p.M >= 1800 || tiles > sms);
+    if (r == 0) {
+        take = M >= 64 && (M <= 7168 || c > 0 || K <= 2048);
+        if (K < 896) {  // (by the output tiles of the launch that follows: in one round of them or more)
+            const int tiles = ((M + 127) / 128) * ((N + 127) / 128);
+            if (M < 640) take = take && tiles > sms;
+            else if (2 * blocks < sms) take = take && (K >= 640 || tiles > sms * 5 / 6);
+            else take = take && (K <= 512 || M >= 1800 || tiles > sms);
         }
+        take = take && ln;
     } else {
-        take = (blocks <= sms || (fe && p.r <= 32 && p.M <= 4096)) && p.K >= 1024;
-        if (!fe) take = take && (blocks << c) <= 4 * sms && (p.r > 16 || p.K > 2048 || p.M <= 1280);
+        take = (blocks <= sms || (ln && r <= 32 && M <= 4096)) && K >= 1024;
+        if (!ln) take = take && ctas <= 4 * sms && (r > 16 || K > 2048 || M <= 1280);
     }
-    if (!take) return cudaErrorNotSupported;
+    if (!take) return false;
+    const bool three = r > 0 && r <= 32 && c == 3 && ctas > crowded;  // CTAs an SM
+    f->c = c;
+    if (three) f->wide = false;
+    else if (r <= 32) f->wide = !ln || c == 3 || slice <= 512 || (r > 0 && slice >= 2048);
+    else if (ln) f->wide = ctas <= sms;
+    else if (r == 48) f->wide = c == 3;
+    else f->wide = ctas <= (c == 3 ? sms - sms / 6 : (c == 2 ? sms - sms / 10 : sms));
+    f->least = !three && ctas <= 2 * sms ? 80 * 1024 : 0;
+    return true;
+}
+// (for the tests; out: log2 of the CTAs of a cluster, sixteen warps, bytes of shared memory at least)
+extern "C" int hgf_internal_rows_prologue_form(int32_t M, int32_t K, int32_t N, int32_t r, int32_t ln, int32_t sms, int32_t *out) {
+    RpForm f = {};
+    if (!rp_form(M, K, N, r, ln != 0, sms, &f)) return 0;
+    out[0] = f.c; out[1] = f.wide; out[2] = (int32_t)f.least;
+    return 1;
+}
+
+static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmPrologueExtra &x, const FrontEnd *fe, cudaStream_t stream) {
+    const int sms = device_sm_count();
+    if (!sms) return cudaErrorInvalidDevice;
+    RpForm f = {};
+    if (!rp_form(p.M, p.K, x.N, p.r, fe != nullptr, sms, &f)) return cudaErrorNotSupported;
     const FrontEnd none = {};
-    // sixteen warps a CTA (a token each) or eight
-    const int ctas = blocks << c, slice = p.K >> c;
-    const bool three = p.r > 0 && p.r <= 32 && c == 3 && ctas > crowded;  // CTAs an SM
-    bool wide;
-    if (three) wide = false;
-    else if (p.r <= 32) wide = !fe || c == 3 || slice <= 512 || (p.r > 0 && slice >= 2048);
-    else if (fe) wide = ctas <= sms;
-    else if (p.r == 48) wide = c == 3;
-    else wide = ctas <= (c == 3 ? sms - sms / 6 : (c == 2 ? sms - sms / 10 : sms));
-    const size_t least = !three && ctas <= 2 * sms ? 80 * 1024 : 0;
+    const int c = f.c;
+    const bool wide = f.wide;
+    const size_t least = f.least;
     switch (p.r) {
         case 0:
-            if (!fe) return cudaErrorNotSupported;
             return wide ? launch_rows_prologue_jt<0, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<0, true, 2>(p, x, *fe, c, least, stream);
         case 16:
             if (fe) return wide ? launch_rows_prologue_jt<2, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<2, true, 2>(p, x, *fe, c, least, stream);
@@ -1380,8 +1401,7 @@ static cudaError_t launch_rows_prologue(const PrologueParams &p, const GemmProlo
             return wide ? launch_rows_prologue_jt<6, false, 1>(p, x, none, c, least, stream) : launch_rows_prologue_jt<6, false, 2>(p, x, none, c, least, stream);
         case 64:
             if (!fe) return wide ? launch_rows_prologue_jt<8, false, 1>(p, x, none, c, least, stream) : launch_rows_prologue_jt<8, false, 2>(p, x, none, c, least, stream);
-            if (wide) return launch_rows_prologue_jt<8, true, 1>(p, x, *fe, c, least, stream);
-            return (blocks << c) <= sms ? launch_rows_prologue_jt<8, true, 2>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<8, true, 2, 2>(p, x, *fe, c, least, stream);
+            return wide ? launch_rows_prologue_jt<8, true, 1>(p, x, *fe, c, least, stream) : launch_rows_prologue_jt<8, true, 2, 2>(p, x, *fe, c, least, stream);
         default: return cudaErrorInvalidValue;
     }
 }

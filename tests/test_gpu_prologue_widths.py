@@ -1,5 +1,7 @@
 """rows_prologue_kernel with eight and with sixteen warps a CTA, and the batches at which launch_rows_prologue changes its mind, against the
 oracle: codes and integer sums bit for bit, y within the GEMM path's tolerance."""
+import ctypes
+
 import numpy as np
 import pytest
 import torch
@@ -36,3 +38,17 @@ def test_against_the_oracle(M, K, r, ln):
     assert np.array_equal(dbg["xq"].cpu().numpy(), ref["xq"])
     assert np.array_equal(dbg["y_int"].cpu().numpy(), ref["y_int"])
     assert np.abs(y.cpu().numpy() - ref["y"]).max() / np.abs(ref["y"]).max() <= 6e-4
+
+
+# each rank, with and without a LayerNorm: [log2 of the CTAs of a cluster, sixteen warps, shared memory for at most two CTAs an SM]
+@pytest.mark.parametrize("M,K,r,ln,form", [
+    (468, 2112, 16, False, [3, 0, 0]), (1186, 6336, 16, False, [2, 1, 0]), (2365, 2112, 16, False, [0, 1, 1]), (1170, 1088, 16, True, [1, 0, 1]),
+    (467, 2112, 16, True, [3, 0, 0]), (2420, 3200, 16, True, [1, 0, 0]), (2427, 4160, 16, True, [1, 1, 0]), (588, 2112, 32, True, [2, 0, 1]),
+    (2370, 2048, 32, True, [0, 1, 1]), (466, 2112, 32, True, [3, 0, 0]), (598, 9024, 48, False, [3, 1, 0]), (2363, 1024, 48, True, [0, 1, 1]),
+    (295, 1024, 48, True, [3, 0, 1]), (1188, 1024, 48, True, [1, 0, 1]), (519, 1024, 64, False, [2, 1, 1]), (596, 7616, 64, False, [3, 0, 0]),
+    (515, 1024, 64, True, [2, 1, 1]), (292, 1024, 64, True, [3, 0, 1]), (598, 7552, 64, True, [3, 0, 0]), (595, 2112, 0, True, [2, 0, 1]), (1186, 6976, 0, True, [2, 0, 0])])
+def test_every_form(M, K, r, ln, form):
+    from paper_2602_05269_b200 import hgf
+    out = (ctypes.c_int32 * 3)()
+    assert hgf.lib().hgf_internal_rows_prologue_form(M, K, 64, r, int(ln), 148, out) and [out[0], out[1], int(out[2] > 0)] == form
+    test_against_the_oracle(M, K, r, ln)
